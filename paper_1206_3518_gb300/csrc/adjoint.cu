@@ -34,7 +34,7 @@ constexpr int kQChunk = 32;         // q points per direct-term chunk
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct BwdLayout {
-  size_t spec, eps2, ab, done, scal, Y, Mh, Mf, Vf, Zf, Gh, Xv, Xc, Yd, total;
+  size_t spec, eps2, ab, done, scal, Y, Mh, Mf, Vf, Zf, Gh, Xv, Xc, Yd, split, total;
   long long rows_v, rows_c;
 };
 
@@ -60,6 +60,8 @@ BwdLayout bwd_layout(const DevSys& d, long long nsteps) {
   L.Xv = o; o = a256(o + 8 * (size_t)L.rows_v * d.ng_max);
   L.Xc = o; o = a256(o + 8 * (size_t)L.rows_c * d.ng_max);
   L.Yd = o; o = a256(o + 8 * (size_t)L.rows_c * d.ng_max);
+  const long long w = d.nv > d.nc ? d.nv * d.nv : d.nc * d.nc;
+  L.split = o; o = a256(o + wr32_split_bytes(d, qc, w));
   L.total = o;
   return L;
 }
@@ -350,8 +352,8 @@ int launch_backward(const DevSys& d, const long long* h_qblk_off, const long lon
       const int q1 = (q0 + kQChunk) < d.nq ? q0 + kQChunk : d.nq;
       long long maxb = 0;
       for (int q = q0; q < q1; ++q) maxb = std::max(maxb, h_qblk_off[q + 1] - h_qblk_off[q]);
-      if ((e = launch_gemm_wr(d, rho_dir, q0, q1, 0, maxb * d.nv * d.nv, W, Xv, 0, stream))) return e;
-      if ((e = launch_gemm_wr(d, rho_dir, q0, q1, 0, maxb * d.nc * d.nc, W, Xc, 1, stream))) return e;
+      if ((e = launch_gemm_wr(d, rho_dir, q0, q1, 0, maxb * d.nv * d.nv, W, Xv, base + L.split, 0, status, stream))) return e;
+      if ((e = launch_gemm_wr(d, rho_dir, q0, q1, 0, maxb * d.nc * d.nc, W, Xc, base + L.split, 1, status, stream))) return e;
       const long long nb = h_qblk_off[q1] - h_qblk_off[q0];
       if (nb > 0)
         block_grad_kernel<<<(unsigned)nb, 256, 0, st>>>(d, Gh, (const float2*)rho_dir, Xv, Xc, (float2*)drho_dir, Yd,

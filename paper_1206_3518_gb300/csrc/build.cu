@@ -6,8 +6,8 @@
 //
 // init_kernel   : 2K^x + diag on every tile that touches the upper block triangle; the
 //                 exchange scale sqrt(2 vbar/(Omega Nk)) is applied to both operands.
-// gemm_wr       : per q, X = W(q) R for the smaller band side (grouped over the q chunk),
-//                 stored as X^T rows [col][G] (G contiguous); its own register-blocked tile.
+// W.rho         : per q, X = W(q) R for the smaller band side (grouped over the q chunk), stored as
+//                 X^T rows [col][G] (G contiguous); on the tensor cores (tcwr32.cu, FP32 accuracy).
 // block_kernel  : per upper block (k <= k'), M = X^H R of the other side (K = NG_q),
 //                 H_kk' = H_kk' - M/(Omega Nk) and the mirror H_k'k = H_kk'^H;
 //                 diagonal blocks become (B + B^H)/2.
@@ -54,115 +54,6 @@ __global__ __launch_bounds__(kGemmThreads) void init_kernel(DevSys d, const floa
         v.x += (float)(e[(size_t)k * d.nb + d.nv + ic] + delta - e[(size_t)k * d.nb + iv]);
       }
       H[(size_t)S * d.dim + S2] = v;
-    }
-  }
-}
-
-// Grouped over the q chunk: X_q^T[col][G] = sum_G' R_q[col][G'] W_q[G][G']  (W Hermitian).
-// Tile 128 rows x 64 columns, K in steps of 16 complex; 256 threads, each 8 rows x 4 columns.
-// Operands are staged transposed ([k][row]) in shared memory so that a thread reads its 8
-// A values and 4 B values of one k with float4 loads; the next K step is prefetched into
-// registers while the current one is consumed (two shared buffers, one barrier per step).
-namespace wr {
-constexpr int TM = 128, TN = 64, TK = 16, kThreads = 256;
-struct Smem {                   // 48 KB: two K steps of both operands
-  float2 a[2][TK][TM];
-  float2 b[2][TK][TN];
-};
-}  // namespace wr
-
-__global__ __launch_bounds__(wr::kThreads, 2) void gemm_wr(DevSys d, const float2* __restrict__ rho_dir,
-                                                          const float2* __restrict__ W, float2* __restrict__ X,
-                                                          int q_begin, long long vbase, int side_c) {
-  using namespace wr;
-  const int q = q_begin + blockIdx.z;
-  const long long b0 = d.qblk_off[q_begin];
-  const long long nblk = d.qblk_off[q + 1] - d.qblk_off[q];
-  const int w = side_width(d, side_c);
-  const int M = (int)(nblk * w), NG = d.ngq[q];
-  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-  if (m0 >= M || n0 >= NG) return;
-  const float2* A = rho_dir + (size_t)side_rows_offset(d, q, side_c, vbase) * d.ng_max;
-  const float2* B = W + (size_t)q * d.ng_max * d.ng_max;
-  float2* C = X + (size_t)((d.qblk_off[q] - b0) * w) * d.ng_max;
-  __shared__ __align__(16) Smem sm;
-  const int t = threadIdx.x;
-  const int tm = t / 16, tn = t % 16;
-  // staging assignment: A row t/2, K half t%2 (8 values); B row t/4, K quarter t%4 (4 values)
-  const int ar = t >> 1, ah = (t & 1) * 8, br = t >> 2, bq = (t & 3) * 4;
-  const bool a_in = m0 + ar < M, b_in = n0 + br < NG;
-  const float2* Ap = A + (size_t)(m0 + ar) * d.ng_max;
-  const float2* Bp = B + (size_t)(n0 + br) * d.ng_max;
-  float2 ra[8], rb[4];
-  auto fetch = [&](int k0) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int k = k0 + ah + i;
-      ra[i] = (a_in && k < NG) ? Ap[k] : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int k = k0 + bq + i;
-      rb[i] = (b_in && k < NG) ? Bp[k] : make_float2(0.f, 0.f);
-    }
-  };
-  auto put = [&](int buf) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) sm.a[buf][ah + i][ar] = ra[i];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) sm.b[buf][bq + i][br] = rb[i];
-  };
-  float2 acc[8][4];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
-  fetch(0);
-  put(0);
-  __syncthreads();
-  int buf = 0;
-  for (int k0 = 0; k0 < NG; k0 += TK) {
-    const bool more = k0 + TK < NG;
-    if (more) fetch(k0 + TK);
-#pragma unroll
-    for (int k = 0; k < TK; ++k) {
-      float2 av[8], bv[4];
-      const float4* pa = reinterpret_cast<const float4*>(&sm.a[buf][k][tm * 8]);
-      const float4* pb = reinterpret_cast<const float4*>(&sm.b[buf][k][tn * 4]);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float4 v = pa[i];
-        av[2 * i] = make_float2(v.x, v.y);
-        av[2 * i + 1] = make_float2(v.z, v.w);
-      }
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const float4 v = pb[j];
-        bv[2 * j] = make_float2(v.x, v.y);
-        bv[2 * j + 1] = make_float2(v.z, v.w);
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc[i][j].x = fmaf(av[i].x, bv[j].x, fmaf(-av[i].y, bv[j].y, acc[i][j].x));
-          acc[i][j].y = fmaf(av[i].x, bv[j].y, fmaf(av[i].y, bv[j].x, acc[i][j].y));
-        }
-    }
-    if (more) {
-      put(buf ^ 1);
-      __syncthreads();
-      buf ^= 1;
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int r = m0 + tm * 8 + i;
-    if (r >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = n0 + tn * 4 + j;
-      if (c < NG) C[(size_t)r * d.ng_max + c] = acc[i][j];
     }
   }
 }
@@ -464,7 +355,7 @@ int launch_mirror(const DevSys& d, void* H, void* stream) {
   return (int)cudaGetLastError();
 }
 
-// FP32 W.rho rows of a q chunk (w rows per block), then (for BSE_PREC_BF16X3) the split BF16 tile images.
+// FP32 W.rho rows of a q chunk (w rows per block), followed by the split tile images of the products.
 static size_t x_bytes(const DevSys& d, long long qchunk, long long w) {
   long long nb = qchunk * d.nkpt;
   if (nb > d.nblocks) nb = d.nblocks;
@@ -475,11 +366,17 @@ static long long direct_width(const DevSys& d) {
   return (d.nv * d.nv <= d.nc * d.nc) ? d.nv * d.nv : d.nc * d.nc;
 }
 
+// Split operand images of the W.rho products, in either precision.
+static size_t split_bytes(const DevSys& d, long long qchunk, long long w) {
+  const size_t a = tc_split_bytes(d, qchunk, w), b = wr32_split_bytes(d, qchunk, w);
+  return a > b ? a : b;
+}
+
 // The direct stage's W.rho rows and split images of a q chunk; at least the exchange stage's split images of
 // rho_x (BSE_BK_INIT with BSE_PREC_BF16X3).
 size_t kernel_ws_bytes(const DevSys& d, long long qchunk) {
   const long long w = direct_width(d);
-  const size_t direct = x_bytes(d, qchunk, w) + tc_split_bytes(d, qchunk, w);
+  const size_t direct = x_bytes(d, qchunk, w) + split_bytes(d, qchunk, w);
   const size_t init = gram_ws_bytes(d);
   return direct > init ? direct : init;
 }
@@ -487,7 +384,7 @@ size_t kernel_ws_bytes(const DevSys& d, long long qchunk) {
 // Coupling build: W.rho_cv' rows and split images of a q chunk, or (init) conj(rho_x(-G)) rows.
 size_t coupling_ws_bytes(const DevSys& d, long long qchunk) {
   const long long w = (long long)d.nv * d.nc;
-  const size_t direct = qchunk > 0 ? x_bytes(d, qchunk, w) + tc_split_bytes(d, qchunk, w) : 0;
+  const size_t direct = qchunk > 0 ? x_bytes(d, qchunk, w) + split_bytes(d, qchunk, w) : 0;
   const size_t init = (((size_t)d.dim * d.ng_max * sizeof(float2)) + 255) & ~(size_t)255;
   return direct > init ? direct : init;
 }
@@ -496,14 +393,6 @@ int launch_kernel_init(const DevSys& d, const void* rho_x, const double* energie
                        void* stream) {
   dim3 grid((d.dim + BN - 1) / BN, (d.dim + BM - 1) / BM);
   init_kernel<<<grid, kGemmThreads, 0, (cudaStream_t)stream>>>(d, (const float2*)rho_x, energies, delta, (float2*)H);
-  return (int)cudaGetLastError();
-}
-
-int launch_gemm_wr(const DevSys& d, const void* rho_dir, int q_begin, int q_end, long long vbase, long long max_rows,
-                   const void* W, void* X, int side_c, void* stream) {
-  dim3 grid((d.ng_max + wr::TN - 1) / wr::TN, (unsigned)((max_rows + wr::TM - 1) / wr::TM), q_end - q_begin);
-  gemm_wr<<<grid, wr::kThreads, 0, (cudaStream_t)stream>>>(d, (const float2*)rho_dir, (const float2*)W, (float2*)X,
-                                                          q_begin, vbase, side_c);
   return (int)cudaGetLastError();
 }
 
@@ -519,10 +408,8 @@ int launch_kernel_direct_range(const DevSys& d, const void* rho_dir, int q_begin
     void* split_ws = (char*)ws + x_bytes(d, q_end - q_begin, direct_width(d));
     e = launch_gemm_wr_tc(d, rho_dir, q_begin, q_end, vbase, max_rows, W, ws, split_ws, side_c, status, stream);
   } else if (prec == BSE_PREC_FP32) {
-    dim3 grid((d.ng_max + wr::TN - 1) / wr::TN, (unsigned)((max_rows + wr::TM - 1) / wr::TM), q_end - q_begin);
-    gemm_wr<<<grid, wr::kThreads, 0, st>>>(d, (const float2*)rho_dir, (const float2*)W, (float2*)ws, q_begin, vbase,
-                                           side_c);
-    e = (int)cudaGetLastError();
+    void* split_ws = (char*)ws + x_bytes(d, q_end - q_begin, direct_width(d));
+    e = launch_gemm_wr(d, rho_dir, q_begin, q_end, vbase, max_rows, W, ws, split_ws, side_c, status, stream);
   } else {
     return -1;
   }
@@ -556,10 +443,8 @@ int launch_coupling_direct_range(const DevSys& d, const void* rho_cpl, int q_beg
     void* split_ws = (char*)ws + x_bytes(d, q_end - q_begin, w);
     e = launch_gemm_wr_tc(d, rho_cpl, q_begin, q_end, vbase, max_rows, W, ws, split_ws, 2, status, stream);
   } else if (prec == BSE_PREC_FP32) {
-    dim3 grid((d.ng_max + wr::TN - 1) / wr::TN, (unsigned)((max_rows + wr::TM - 1) / wr::TM), q_end - q_begin);
-    gemm_wr<<<grid, wr::kThreads, 0, st>>>(d, (const float2*)rho_cpl, (const float2*)W, (float2*)ws, q_begin, vbase,
-                                           2);
-    e = (int)cudaGetLastError();
+    void* split_ws = (char*)ws + x_bytes(d, q_end - q_begin, w);
+    e = launch_gemm_wr(d, rho_cpl, q_begin, q_end, vbase, max_rows, W, ws, split_ws, 2, status, stream);
   } else {
     return -1;
   }

@@ -143,7 +143,8 @@ int launch_spectrum_coupled(const DevSys& d, const void* A, const void* Bm, cons
                             void* ws, int* status, void* stream);
 size_t kernel_ws_bytes(const DevSys& d, long long qchunk);
 int launch_gemm_wr(const DevSys& d, const void* rho_dir, int q_begin, int q_end, long long vbase, long long max_rows,
-                   const void* W, void* X, int side_c, void* stream);
+                   const void* W, void* X, void* split_ws, int side, int* status, void* stream);
+size_t wr32_split_bytes(const DevSys& d, long long qchunk, long long w);
 
 // Streams n elements of elem_bytes (4: float / complex64 parts, 8: double) through a NaN/Inf check;
 // a hit sets BSE_ERR_NONFINITE in *status.  n <= 0 launches nothing.
