@@ -45,11 +45,9 @@ constexpr size_t kTcSmem = (size_t)kStages * kStage + 1024 + 256;   // ring, 1 K
 
 using umma::gtimer;
 using umma::idesc_of;
-using umma::kNegA;
 using umma::mbar_arrive;
 using umma::mbar_init;
 using umma::mbar_wait;
-using umma::mma_bf16;
 using umma::mma_commit;
 using umma::smem_desc;
 using umma::smem_u32;
@@ -196,7 +194,7 @@ __global__ __launch_bounds__(kTcThreads, 1) void tc_gemm_wr(DevSys d, TcArgs a) 
   const int w = side_width(d, g.side_c);
   const long long b0 = d.qblk_off[g.q_begin];
   const long long ntiles = (long long)g.nq * g.mt_max * g.nt_max;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = umma::uniform(tid >> 5), lane = tid & 31;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -244,54 +242,50 @@ __global__ __launch_bounds__(kTcThreads, 1) void tc_gemm_wr(DevSys d, TcArgs a) 
         *issued = c + 1;
       }
     }
-  } else if (warp == 1 && lane == 0) {          // MMA issuer
-    const uint32_t idesc = idesc_of(N), idesc_neg = idesc | kNegA;
+  } else if (warp == 1) {                       // MMA issue: the whole warp runs the loop, one lane issues
+    const bool leader = umma::elect_one();
+    const uint32_t idesc = idesc_of(N);
+    const uint64_t d0 = smem_desc(umma::uniform(smem_u32(sm)));
+    const uint32_t a_lo = (uint32_t)(kTileA >> 4), b_lo = (uint32_t)(N * kRow) >> 4, tm = umma::uniform(tmem);
     unsigned c = 0, j = 0;
     Tile t;
     bool ok = true;
     for (long long ti = blockIdx.x; ti < ntiles && ok; ti += gridDim.x) {
       if (!tile_of(d, g, w, ti, t)) continue;
+      const int NG = umma::uniform(t.NG), nch = (NG + TKC - 1) / TKC;
       const int buf = (int)(j & 1);
-      if (j >= 2 && !mbar_wait(smem_u32(tempty + buf), ((j >> 1) - 1) & 1u)) {
-        fail_now(fail, a.status);
-        ok = false;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t d_re = tmem + (uint32_t)(buf * kAccCols), d_im = d_re + 128;
-      for (int kc = 0; kc < t.nch; ++kc, ++c) {
+      if (j >= 2) ok = umma::uniform(mbar_wait(smem_u32(tempty + buf), ((j >> 1) - 1) & 1u));
+      if (ok) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d_re = tm + (uint32_t)(buf * kAccCols), d_im = d_re + 128;
+      for (int kc = 0; kc < nch && ok; ++kc, ++c) {
         const int st = (int)(c % kStages);
-        if (!mbar_wait(smem_u32(full + st), (c / kStages) & 1u) || *fail) {
-          fail_now(fail, a.status);
-          ok = false;
-          break;
-        }
+        ok = umma::uniform(mbar_wait(smem_u32(full + st), (c / kStages) & 1u) && !*fail);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sah = smem_u32(sm + st * kStage), sal = sah + kTileA;
-        const uint32_t sbh = sah + 2 * kTileA, sbl = sbh + (uint32_t)(N * kRow);
-        const int nkk = (t.NG - kc * TKC > 16) ? 2 : 1;   // the last chunk may need one K16 step only
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-          if (kk >= nkk) break;
-#pragma unroll
-          for (int s = 0; s < 3; ++s) {           // hi.hi, hi.lo, lo.hi
-            const uint32_t pa = ((s == 2) ? sal : sah) + kk * 32, pb = ((s == 1) ? sbl : sbh) + kk * 32;
-            const uint32_t acc = (kc | kk | s) != 0 ? 1u : 0u;
-            mma_bf16(d_re, smem_desc(pa), smem_desc(pb), idesc, acc);                // Re R Re W
-            mma_bf16(d_re, smem_desc(pa + 64), smem_desc(pb + 64), idesc_neg, 1u);   // - Im R Im W
-            mma_bf16(d_im, smem_desc(pa), smem_desc(pb + 64), idesc, acc);           // Re R Im W
-            mma_bf16(d_im, smem_desc(pa + 64), smem_desc(pb), idesc, 1u);            // Im R Re W
-          }
+        const uint64_t da = d0 + (uint64_t)((st * kStage) >> 4), db = da + (uint64_t)((2 * kTileA) >> 4);
+        if (leader) {
+          umma::mma_cplx_k16_desc<false>(d_re, d_im, da, a_lo, db, b_lo, 0, idesc, kc == 0);
+          if (NG - kc * TKC > 16)               // the last chunk may need one K16 step only
+            umma::mma_cplx_k16_desc<false>(d_re, d_im, da, a_lo, db, b_lo, 1, idesc, false);
+          mma_commit(smem_u32(empty + st));
+          *consumed = c + 1;
         }
-        mma_commit(smem_u32(empty + st));
-        *consumed = c + 1;
+        __syncwarp();
       }
-      if (!ok) break;
-      mma_commit(smem_u32(tfull + buf));
+      if (leader) {
+        if (ok)
+          mma_commit(smem_u32(tfull + buf));
+        else
+          fail_now(fail, a.status);
+      }
+      __syncwarp();
       ++j;
     }
-    mma_commit(smem_u32(drain));                // tracks every MMA issued above
-    if (!mbar_wait(smem_u32(drain), 0u)) fail_now(fail, a.status);
+    if (leader) {
+      mma_commit(smem_u32(drain));              // tracks every MMA issued above
+      if (!mbar_wait(smem_u32(drain), 0u)) fail_now(fail, a.status);
+    }
+    __syncwarp();
   } else if (warp >= 4) {                       // epilogue: TMEM lanes 32(w-4).. -> output rows
     const int ew = warp - 4;
     const bool even = (d.ng_max & 1) == 0;

@@ -141,7 +141,7 @@ __global__ __launch_bounds__(kThreads, 1) void gram_kernel(DevSys d, const unsig
   volatile int* fail = (volatile int*)(tmem_slot + 1);
   volatile unsigned* issued = (volatile unsigned*)(tmem_slot + 2);
   volatile unsigned* consumed = (volatile unsigned*)(tmem_slot + 3);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = umma::uniform(tid >> 5), lane = tid & 31;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -188,41 +188,45 @@ __global__ __launch_bounds__(kThreads, 1) void gram_kernel(DevSys d, const unsig
         *issued = c + 1;
       }
     }
-  } else if (warp == 1 && lane == 0) {          // MMA issuer
+  } else if (warp == 1) {                       // MMA issue: the whole warp runs the loop, one lane issues
+    const bool leader = umma::elect_one();
     const uint32_t idesc = umma::idesc_of(kTM);
-    const uint64_t d0 = umma::smem_desc(smem_u32(sm));
-    const uint32_t lo = (uint32_t)(kTile >> 4);
+    const uint64_t d0 = umma::smem_desc(umma::uniform(smem_u32(sm)));
+    const uint32_t lo = (uint32_t)(kTile >> 4), tm = umma::uniform(tmem);
     unsigned c = 0, j = 0;
     bool ok = true;
     for (long long t = blockIdx.x; t < g.ntiles && ok; t += gridDim.x, ++j) {
       const int buf = (int)(j & 1);
-      if (j >= 2 && !mbar_wait(smem_u32(tempty + buf), ((j >> 1) - 1) & 1u)) {
-        fail_now(fail, status);
-        ok = false;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t d_re = tmem + (uint32_t)(buf * kAcc), d_im = d_re + 128;
-      for (int kc = 0; kc < g.nkc; ++kc, ++c) {
+      if (j >= 2) ok = umma::uniform(mbar_wait(smem_u32(tempty + buf), ((j >> 1) - 1) & 1u));
+      if (ok) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d_re = tm + (uint32_t)(buf * kAcc), d_im = d_re + 128;
+      for (int kc = 0; kc < g.nkc && ok; ++kc, ++c) {
         const int st = (int)(c % kStages);
-        if (!mbar_wait(smem_u32(full + st), (c / kStages) & 1u) || *fail) {
-          fail_now(fail, status);
-          ok = false;
-          break;
-        }
+        ok = umma::uniform(mbar_wait(smem_u32(full + st), (c / kStages) & 1u) && !*fail);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t da = d0 + (uint64_t)((st * kStage) >> 4), db = da + (uint64_t)(kImg >> 4);
-        const int nkk = (d.ng0 - kc * kTKC > 16) ? 2 : 1;
-        for (int kk = 0; kk < nkk; ++kk)
-          umma::mma_cplx_conj_k16_desc(d_re, d_im, da, lo, db, lo, kk, idesc, kc == 0 && kk == 0);
-        mma_commit(smem_u32(empty + st));
-        *consumed = c + 1;
+        if (leader) {
+          umma::mma_cplx_k16_desc<true>(d_re, d_im, da, lo, db, lo, 0, idesc, kc == 0);
+          if (d.ng0 - kc * kTKC > 16) umma::mma_cplx_k16_desc<true>(d_re, d_im, da, lo, db, lo, 1, idesc, false);
+          mma_commit(smem_u32(empty + st));
+          *consumed = c + 1;
+        }
+        __syncwarp();
       }
-      if (!ok) break;
-      mma_commit(smem_u32(tfull + buf));
+      if (leader) {
+        if (ok)
+          mma_commit(smem_u32(tfull + buf));
+        else
+          fail_now(fail, status);
+      }
+      __syncwarp();
     }
-    mma_commit(smem_u32(drain));                // tracks every MMA issued above
-    if (!mbar_wait(smem_u32(drain), 0u)) fail_now(fail, status);
+    if (leader) {
+      mma_commit(smem_u32(drain));              // tracks every MMA issued above
+      if (!mbar_wait(smem_u32(drain), 0u)) fail_now(fail, status);
+    }
+    __syncwarp();
   } else if (warp >= 4) {                       // epilogue: TMEM lanes 32 (w - 4) .. -> rows of H
     const int ew = warp - 4;
     const int nvc = d.nv * d.nc;

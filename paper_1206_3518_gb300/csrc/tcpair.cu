@@ -31,6 +31,9 @@
 // brings the B rows into a ring of shared-memory stages with bulk copies (the region's panel of the chunk:
 // its hi rows and its lo rows, counted on the stage's mbarrier); the columns of a region's points without
 // a block in the tile are computed and dropped.
+// The MMA warp issues warp-uniformly (umma.cuh): from one thread of a divergent branch each MMA took 105 cycles
+// against the 48 of N = 96 and the issue loop was the bound (fcc 8x8x8 3v4c 22.0 -> 15.2 ms, fcc 12x12x12 4v4c 511 ->
+// 388 ms).
 // Two accumulators (Re | Im, 2 N <= 192 TMEM columns each) alternate between passes (one band n, 128
 // rows), so the epilogue of one pass overlaps the MMAs of the next.  Every mbarrier wait is bounded (2 s); on expiry the CTA
 // records BSE_ERR_TIMEOUT, stops issuing, waits (bounded) for its MMAs in flight, frees its tensor
@@ -212,7 +215,7 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
   long long* bvec = (long long*)(sm + g.o_bvec);
   short* ptab = (short*)(sm + g.o_ptab);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = umma::uniform(tid >> 5), lane = tid & 31;
   const int ntiles = d.nkpt * d.tc_nreg, rs = d.tc_rsize;
   const int f0 = d.fwf[0], f1 = d.fwf[1], f2 = d.fwf[2];
   const int kb1 = 2 * f1 + 1, kb2 = 2 * f2 + 1;
@@ -470,48 +473,47 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
               umma::bulk_g2s(bh + (uint32_t)(g.nmax * umma::kRow), p + half_bytes, half_bytes, smem_u32(full_b + st));
             }
       }
-    } else if (warp == kMmaWarp) {               // ---- MMA issue
-      if (lane == 0) {
-        unsigned s = sc, p = pc;
-        bool ok = !*fail;
-        const uint64_t dstage0 = umma::smem_desc(smem_u32(sm));     // B stage st: + st stage_bytes / 16
-        const uint32_t blo = (uint32_t)((g.nmax * umma::kRow) >> 4);
-        for (int set = 0; set < 2; ++set) {
-          const int nset = set ? nc : nv;
-          const int N = (rs * nset + 15) & ~15;
-          const uint32_t idesc = umma::idesc_of(N);
-          for (int nn = 0; nn < nset; ++nn)
-            for (int mt = 0; mt < nmt; ++mt, ++p) {
-              const int buf = (int)(p & 1u);
-              if (ok && p >= 2 && !mbar_wait(smem_u32(tempty + buf), ((p >> 1) - 1) & 1u)) {
-                fail_now(fail, status);
-                ok = false;
-              }
-              if (ok) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              const uint32_t d_re = tmem + (uint32_t)buf * acc_cols, d_im = d_re + half;
-              for (int c = 0; c < nch; ++c, ++s) {
-                if (!ok || *fail) {
-                  ok = false;
-                  continue;
-                }
-                const int st = (int)(s % (unsigned)g.stages), sa = (int)(s & 1u);
-                if (!mbar_wait(smem_u32(full_a + sa), (s >> 1) & 1u) ||
-                    !mbar_wait(smem_u32(full_b + st), (s / g.stages) & 1u) || *fail) {
-                  fail_now(fail, status);
-                  ok = false;
-                  continue;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint64_t db = dstage0 + (uint64_t)((st * g.stage_bytes) >> 4);
-                const uint32_t a = tmem + a_col0 + (uint32_t)(sa * kACols);
-                const int nkk = (kc - c * kTKC > 16) ? 2 : 1;
-                for (int kk = 0; kk < nkk; ++kk)
-                  umma::mma_cplx_k16_ts(d_re, d_im, a + (uint32_t)(kk * 32), db, blo, kk, idesc, c == 0 && kk == 0);
-                mma_commit(smem_u32(empty_a + sa));
-                mma_commit(smem_u32(empty_b + st));
-              }
-              if (ok) mma_commit(smem_u32(tfull + buf));
+    } else if (warp == kMmaWarp) {               // ---- MMA issue: the whole warp runs the loop, one lane issues
+      const bool leader = umma::elect_one();
+      unsigned s = sc, p = pc;
+      bool ok = umma::uniform(!*fail);
+      const uint64_t dstage0 = umma::smem_desc(umma::uniform(smem_u32(sm)));   // B stage st: + st stage_bytes / 16
+      const uint32_t blo = (uint32_t)((g.nmax * umma::kRow) >> 4), tm = umma::uniform(tmem);
+      const int kcu = umma::uniform(kc), nmtu = umma::uniform(nmt), nchu = (kcu + kTKC - 1) / kTKC;
+      for (int set = 0; set < 2; ++set) {
+        const int nset = set ? nc : nv;
+        const int N = (rs * nset + 15) & ~15;
+        const uint32_t idesc = umma::idesc_of(N);
+        for (int pass = 0; pass < nset * nmtu; ++pass, ++p) {
+          const int buf = (int)(p & 1u);
+          if (ok && p >= 2) {
+            ok = umma::uniform(mbar_wait(smem_u32(tempty + buf), ((p >> 1) - 1) & 1u));
+            if (!ok && leader) fail_now(fail, status);
+          }
+          if (ok) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t d_re = tm + (uint32_t)buf * acc_cols, d_im = d_re + half;
+          for (int c = 0; c < nchu; ++c, ++s) {
+            if (!ok) continue;
+            const int st = (int)(s % (unsigned)g.stages), sa = (int)(s & 1u);
+            ok = umma::uniform(!*fail && mbar_wait(smem_u32(full_a + sa), (s >> 1) & 1u) &&
+                               mbar_wait(smem_u32(full_b + st), (s / g.stages) & 1u) && !*fail);
+            if (!ok) {
+              if (leader) fail_now(fail, status);
+              continue;
             }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint64_t db = dstage0 + (uint64_t)((st * g.stage_bytes) >> 4);
+            const uint32_t a = tm + a_col0 + (uint32_t)(sa * kACols);
+            if (leader) {
+              umma::mma_cplx_k16_ts(d_re, d_im, a, db, blo, 0, idesc, c == 0);
+              if (kcu - c * kTKC > 16) umma::mma_cplx_k16_ts(d_re, d_im, a + 32u, db, blo, 1, idesc, false);
+              mma_commit(smem_u32(empty_a + sa));
+              mma_commit(smem_u32(empty_b + st));
+            }
+            __syncwarp();
+          }
+          if (ok && leader) mma_commit(smem_u32(tfull + buf));
+          __syncwarp();
         }
       }
     } else {                                     // ---- epilogue: TMEM lanes 32 warp .. -> rows

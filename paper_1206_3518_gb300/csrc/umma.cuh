@@ -92,39 +92,27 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// The twelve MMAs of 16 complex K values in BF16x3 split-complex form, A and B tiles (hi, lo) at
-// shared addresses ah/al, bh/bl (kk selects the K16 half of the 32-value row):
-//   Re D += Re A Re B - Im A Im B,   Im D += Re A Im B + Im A Re B,   each as hi.hi + hi.lo + lo.hi.
-// init != 0 starts both accumulators.
-__device__ __forceinline__ void mma_cplx_k16(uint32_t d_re, uint32_t d_im, uint32_t ah, uint32_t al, uint32_t bh,
-                                             uint32_t bl, int kk, uint32_t idesc, bool init) {
-  const uint32_t idesc_neg = idesc | kNegA;
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {                 // hi.hi, hi.lo, lo.hi
-    const uint32_t pa = ((s == 2) ? al : ah) + kk * 32, pb = ((s == 1) ? bl : bh) + kk * 32;
-    const uint32_t acc = (init && s == 0) ? 0u : 1u;
-    mma_bf16(d_re, smem_desc(pa), smem_desc(pb), idesc, acc);                // Re A Re B
-    mma_bf16(d_re, smem_desc(pa + 64), smem_desc(pb + 64), idesc_neg, 1u);   // - Im A Im B
-    mma_bf16(d_im, smem_desc(pa), smem_desc(pb + 64), idesc, acc);           // Re A Im B
-    mma_bf16(d_im, smem_desc(pa + 64), smem_desc(pb), idesc, 1u);            // Im A Re B
-  }
-}
-
-// The same twelve MMAs with precomputed descriptors: da / db of the hi tiles, a_lo / b_lo the offsets (in
-// 16-byte units) of the lo tiles; K16 half kk at +2, the Im half at +4 (a descriptor's start address is
-// its low 14 bits, address / 16, so a byte offset o adds o / 16).
+// The twelve MMAs of 16 complex K values in BF16x3 split-complex form,
+//   Re D += Re A Re B - Im A Im B,   Im D += Re A Im B + Im A Re B   (CONJ: conj(A) B),
+// each as hi.hi + hi.lo + lo.hi; Re D before Im D (a change of accumulator costs 5 cycles).  da / db: descriptors of
+// the hi tiles, a_lo / b_lo the offsets (in 16-byte units) of the lo tiles; K16 half kk at +2, the Im half at +4 (a
+// descriptor's start address is its low 14 bits, address / 16, so a byte offset o adds o / 16).  init starts both
+// accumulators.
+template <bool CONJ>
 __device__ __forceinline__ void mma_cplx_k16_desc(uint32_t d_re, uint32_t d_im, uint64_t da, uint32_t a_lo, uint64_t db,
                                                   uint32_t b_lo, int kk, uint32_t idesc, bool init) {
-  const uint32_t idesc_neg = idesc | kNegA;
+  const uint32_t neg = idesc | kNegA;
 #pragma unroll
-  for (int s = 0; s < 3; ++s) {                 // hi.hi, hi.lo, lo.hi
-    const uint64_t pa = da + ((s == 2) ? a_lo : 0u) + (uint32_t)kk * 2u;
-    const uint64_t pb = db + ((s == 1) ? b_lo : 0u) + (uint32_t)kk * 2u;
-    const uint32_t acc = (init && s == 0) ? 0u : 1u;
-    mma_bf16(d_re, pa, pb, idesc, acc);                 // Re A Re B
-    mma_bf16(d_re, pa + 4u, pb + 4u, idesc_neg, 1u);    // - Im A Im B
-    mma_bf16(d_im, pa, pb + 4u, idesc, acc);            // Re A Im B
-    mma_bf16(d_im, pa + 4u, pb, idesc, 1u);             // Im A Re B
+  for (int im = 0; im < 2; ++im) {
+    const uint32_t d = im ? d_im : d_re, sign = (im != 0) == CONJ ? neg : idesc;   // of the product with Im A
+    const uint32_t b0 = im ? 4u : 0u, b1 = 4u - b0;                            // plane of B met by Re A, by Im A
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {                 // hi.hi, hi.lo, lo.hi
+      const uint64_t pa = da + ((s == 2) ? a_lo : 0u) + (uint32_t)kk * 2u;
+      const uint64_t pb = db + ((s == 1) ? b_lo : 0u) + (uint32_t)kk * 2u;
+      mma_bf16(d, pa, pb + b0, idesc, (init && s == 0) ? 0u : 1u);
+      mma_bf16(d, pa + 4u, pb + b1, sign, 1u);
+    }
   }
 }
 
@@ -137,21 +125,22 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, ui
       : "memory");
 }
 
-// The twelve MMAs of 16 complex K values with the A planes in tensor memory at columns a + 0 (Re hi),
-// a + 8 (Im hi), a + 16 (Re lo), a + 24 (Im lo) (two BF16 per 32-bit column, lane = row), B in shared
-// memory as for mma_cplx_k16_desc.
+// The same with the A planes in tensor memory at columns a + 0 (Re hi), a + 8 (Im hi), a + 16 (Re lo), a + 24 (Im lo)
+// (two BF16 per 32-bit column, lane = row).
 __device__ __forceinline__ void mma_cplx_k16_ts(uint32_t d_re, uint32_t d_im, uint32_t a, uint64_t db, uint32_t b_lo,
                                                 int kk, uint32_t idesc, bool init) {
-  const uint32_t idesc_neg = idesc | kNegA;
+  const uint32_t neg = idesc | kNegA;
 #pragma unroll
-  for (int s = 0; s < 3; ++s) {                 // hi.hi, hi.lo, lo.hi
-    const uint32_t ar = a + ((s == 2) ? 16u : 0u), ai = ar + 8u;
-    const uint64_t pb = db + ((s == 1) ? b_lo : 0u) + (uint32_t)kk * 2u;
-    const uint32_t acc = (init && s == 0) ? 0u : 1u;
-    mma_bf16_ts(d_re, ar, pb, idesc, acc);              // Re A Re B
-    mma_bf16_ts(d_re, ai, pb + 4u, idesc_neg, 1u);      // - Im A Im B
-    mma_bf16_ts(d_im, ar, pb + 4u, idesc, acc);         // Re A Im B
-    mma_bf16_ts(d_im, ai, pb, idesc, 1u);               // Im A Re B
+  for (int im = 0; im < 2; ++im) {
+    const uint32_t d = im ? d_im : d_re, sign = im ? idesc : neg;
+    const uint32_t b0 = im ? 4u : 0u, b1 = 4u - b0;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {                 // hi.hi, hi.lo, lo.hi
+      const uint32_t ar = a + ((s == 2) ? 16u : 0u);
+      const uint64_t pb = db + ((s == 1) ? b_lo : 0u) + (uint32_t)kk * 2u;
+      mma_bf16_ts(d, ar, pb + b0, idesc, (init && s == 0) ? 0u : 1u);
+      mma_bf16_ts(d, ar + 8u, pb + b1, sign, 1u);
+    }
   }
 }
 
@@ -165,23 +154,6 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32
       "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
       "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
       : "memory");
-}
-
-// The twelve MMAs of 16 complex K values for conj(A) B (descriptors as mma_cplx_k16_desc):
-//   Re D += Re A Re B + Im A Im B,   Im D += Re A Im B - Im A Re B.
-__device__ __forceinline__ void mma_cplx_conj_k16_desc(uint32_t d_re, uint32_t d_im, uint64_t da, uint32_t a_lo,
-                                                       uint64_t db, uint32_t b_lo, int kk, uint32_t idesc, bool init) {
-  const uint32_t idesc_neg = idesc | kNegA;
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {                 // hi.hi, hi.lo, lo.hi
-    const uint64_t pa = da + ((s == 2) ? a_lo : 0u) + (uint32_t)kk * 2u;
-    const uint64_t pb = db + ((s == 1) ? b_lo : 0u) + (uint32_t)kk * 2u;
-    const uint32_t acc = (init && s == 0) ? 0u : 1u;
-    mma_bf16(d_re, pa, pb, idesc, acc);                 // Re A Re B
-    mma_bf16(d_re, pa + 4u, pb + 4u, idesc, 1u);        // + Im A Im B
-    mma_bf16(d_im, pa, pb + 4u, idesc, acc);            // Re A Im B
-    mma_bf16(d_im, pa + 4u, pb, idesc_neg, 1u);         // - Im A Re B
-  }
 }
 
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
