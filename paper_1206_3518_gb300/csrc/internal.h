@@ -81,7 +81,7 @@ bse_status cuda_check(int err, const char* what);
 // Kernel launchers (defined in the .cu files); all return cudaError_t as int.
 int launch_realspace(const DevSys& d, const void* coef, void* u, void* stream);
 int launch_pair_exchange(const DevSys& d, const void* u, void* rho_x, int* status, void* stream);
-int launch_pair_direct(const DevSys& d, const void* u, void* rho_dir, int q_begin, int q_end, long long vbase,
+int launch_pair_direct(const DevSys& d, void* u, void* rho_dir, int q_begin, int q_end, long long vbase,
                        int* status, void* stream);
 int launch_dipole(const DevSys& d, const void* coef, const double* energies, double gap_floor, void* P, void* stream);
 int launch_pair_chi0(const DevSys& d, const void* u, void* rho, int q_begin, int q_end, int* status, void* stream);
@@ -92,6 +92,7 @@ int pair_supported(const DevSys& d);
 size_t pair_ws_bytes(const DevSys& d);
 int gcorr_valid(const DevSys& d);
 int tcpair_valid(const DevSys& d);
+int tcpair_preferred(const DevSys& d, int q_begin, int q_end);
 size_t tcpair_ws_bytes(const DevSys& d);
 int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, int q_begin, int q_end,
                   long long vbase, int* status, void* stream);

@@ -566,8 +566,10 @@ static long long job_cells(const DevSys& d, int nqc, bool merged) {
   return ntq * ntk * kTQ * kTK * (merged ? 1 : 2);
 }
 
-int launch_pair_direct(const DevSys& d, const void* u, void* rho_dir, int q_begin, int q_end, long long vbase,
+int launch_pair_direct(const DevSys& d, void* u, void* rho_dir, int q_begin, int q_end, long long vbase,
                        int* status, void* stream) {
+  if (d.pair_variant == -1 && use_gcorr(d) && tcpair_preferred(d, q_begin, q_end))   // no variant asked for
+    return launch_pair_direct_tensor(d, u, rho_dir, q_begin, q_end, vbase, status, stream);
   if (use_gcorr(d))
     return gcorr_split(d)
                ? launch_gcorr(d, coef_copy(d, u), rho_dir, 3, 1, q_begin, q_end - q_begin, vbase,

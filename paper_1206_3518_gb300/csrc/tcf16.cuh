@@ -190,6 +190,28 @@ __device__ __forceinline__ void chunk_mmas(uint32_t d_re, uint32_t d_im, uint64_
   }
 }
 
+// The same with the A planes in tensor memory at columns a + 0 (Re hi), a + 8 (Im hi), a + 16 (Re lo), a + 24 (Im lo) of
+// the first K16 half, + 32 of the second (two FP16 per 32-bit column, lane = row); A as it is (no conjugation).
+template <int NKK>
+__device__ __forceinline__ void chunk_mmas_ts(uint32_t d_re, uint32_t d_im, uint32_t a, uint64_t db, uint32_t b_lo,
+                                              uint32_t idesc) {
+  const uint32_t neg = idesc | umma::kNegA;
+#pragma unroll
+  for (int im = 0; im < 2; ++im) {
+    const uint32_t d = im ? d_im : d_re, sign = im ? idesc : neg;
+    const uint32_t b0 = im ? 4u : 0u, b1 = 4u - b0;
+#pragma unroll
+    for (int s = 0; s < 3; ++s)                  // hi.lo, lo.hi, hi.hi
+#pragma unroll
+      for (int kk = NKK - 1; kk >= 0; --kk) {
+        const uint32_t pa = a + (uint32_t)kk * 32u + (s == 1 ? 16u : 0u);
+        const uint64_t pb = db + (s == 0 ? b_lo : 0u) + (uint32_t)kk * 2u;
+        umma::mma_bf16_ts(d, pa, pb + b0, idesc, (s != 0 || kk != NKK - 1) ? 1u : 0u);
+        umma::mma_bf16_ts(d, pa + 8u, pb + b1, sign, 1u);
+      }
+  }
+}
+
 __device__ __forceinline__ void fail_now(volatile int* fail, int* status) {
   *fail = 1;
   atomicCAS(status, 0, (int)BSE_ERR_TIMEOUT);

@@ -14,36 +14,46 @@
 //   K          the region's layout, the union of the spheres S(k') of its points;
 //   columns    the tile's blocks times the bands m of the set.
 //
-// A_n is gathered into shared memory from a dense index box of S(k) (points outside S(k) read a zero
-// row); B comes from packed panels of the coefficients of each region's points in its K layout (zero off
-// S(k')), written once per call.  The epilogue keeps, for every block, the rows on its own sphere and writes
-// them at their sphere positions, so the output is the direct set of the correlation kernels.
+// A_n is gathered from a dense difference box in shared memory that holds the coefficients of band n themselves
+// (zero off S(k)): one 8-byte lookup per element.  B comes from packed panels of the coefficients of each
+// region's points in its K layout (zero off S(k')), written once per call.  The epilogue keeps, for every block,
+// the rows on its own sphere and writes them at their sphere positions, so the output is the direct set of
+// the correlation kernels.
 //
-// Arithmetic (BF16x3): every operand is split x = hi + lo in BF16 and each real product accumulates
-// hi.hi + hi.lo + lo.hi in FP32 in tensor memory (relative error ~2^-16 per product, as for the
-// W.rho products of the mixed build).  The G = 0 overlaps of the diagonal blocks (k' = k), which
-// meet the q = 0 head of W, are summed again in FP64 afterwards (tcpair_diag_kernel).
+// Arithmetic (FP16x3, tcf16.cuh): the coefficients of every (k, band) are scaled by a power of two and split
+// hi + lo in FP16 (22 bits); each real product is hi.lo + lo.hi + hi.hi, and the tensor core's accumulator holds
+// one K chunk (32 complex values) at a time, which the epilogue warps add to FP32 registers.  The result has the
+// accuracy of the FP32 correlation kernel, so one kernel serves both precisions of the build.  The G = 0 overlaps
+// of the diagonal blocks (k' = k), which meet the q = 0 head of W, are summed again in FP64
+// afterwards (tcpair_diag_kernel).
 //
-// tcpair_kernel is persistent (one CTA per SM) and takes tiles (k, region) from a counter, region-major.
-// Warps 0-3 drain the accumulators, warp 4 issues the MMAs (12 per 16 complex K, A from tensor memory,
-// B from shared memory), warps 5-12 gather the A tile of each K chunk (32 complex K values) straight into
-// tensor memory (two A slots, tcgen05.st; warps 5-8 the even stages, 9-12 the odd ones), and warp 13
-// brings the B rows into a ring of shared-memory stages with bulk copies (the region's panel of the chunk:
-// its hi rows and its lo rows, counted on the stage's mbarrier); the columns of a region's points without
-// a block in the tile are computed and dropped.
-// The MMA warp issues warp-uniformly (umma.cuh): from one thread of a divergent branch each MMA took 105 cycles
-// against the 48 of N = 96 and the issue loop was the bound (fcc 8x8x8 3v4c 22.0 -> 15.2 ms, fcc 12x12x12 4v4c 511 ->
-// 388 ms).
-// Two accumulators (Re | Im, 2 N <= 192 TMEM columns each) alternate between passes (one band n, 128
-// rows), so the epilogue of one pass overlaps the MMAs of the next.  Every mbarrier wait is bounded (2 s); on expiry the CTA
-// records BSE_ERR_TIMEOUT, stops issuing, waits (bounded) for its MMAs in flight, frees its tensor
-// memory and returns.
-#include <cuda_bf16.h>
+// tcpair_kernel is persistent (one CTA per SM) and takes tiles (k, region) from a counter, region-major; a pass is
+// one band n and 128 rows.  Four warpgroups share the registers (setmaxnreg):
+//   0, 1  promote the chunks of the even / odd passes into registers and write the pass's densities while the
+//         other group promotes the next pass (the scattered 8-byte stores, one cache line each, take most of
+//         a pass);
+//   2     gathers the A tile of each K chunk straight into tensor memory (four slots, tcgen05.st);
+//   3     two warps issue the MMAs (12 per 16 complex K, A from tensor memory, B from shared memory; warp-uniform,
+//         umma.cuh), one warp brings the B rows into a ring of shared-memory stages with bulk copies (the region's
+//         panel of the chunk: its hi rows and its lo rows); the columns of a region's points without a block in
+//         the tile are computed and dropped.
+// At most 64 columns per pass: a group's sums are 2 x 64 registers a thread, and two accumulators (Re | Im, 128 TMEM
+// columns each) and four A slots fill tensor memory.  Every mbarrier wait is bounded (2 s); on expiry the CTA records
+// BSE_ERR_TIMEOUT, stops issuing, waits (bounded) for its MMAs in flight, frees its tensor memory and returns.
+//
+// What bounds it: the MMAs of a chunk (24 of 40 cycles at N = 64) against the gather (~300 cycles of shared-memory
+// bandwidth a chunk) and
+// the promotion; without promotion and stores fcc 8x8x8 3v4c takes 8.2 ms of 10.5.  Measured (ms; before: the FP32
+// correlation kernel / BF16x3 tensor kernel with 96 columns, two lookups an element and one accumulator a pass):
+// fcc 8x8x8 3v4c 10.5 (50.1 / 15.2), fcc 12x12x12 4v4c, 144 q 49.4 (- / 59), 27x27 sheet 2v3c, 64 q 1.33 (1.52 / -).  Error
+// against 64 bits (2-norm): 1.3e-7 to 1.5e-7 (correlation kernel 2.0e-7 to 4.0e-7).
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
 #include "internal.h"
+#include "tcf16.cuh"
 #include "umma.cuh"
 
 namespace bse {
@@ -56,15 +66,17 @@ using umma::mma_commit;
 using umma::smem_u32;
 using umma::swz;
 
-constexpr int kEpiWarps = 4;                   // warps 0-3: TMEM lane quarters 0-3
-constexpr int kMmaWarp = 4;
-constexpr int kG0 = 5;                         // first gather warp
-constexpr int kGWarps = 8;
-constexpr int kB0 = kG0 + kGWarps;             // the B producer warp (bulk copies)
+constexpr int kGroups = 2;                     // epilogue warpgroups (warps 0-3, 4-7)
+constexpr int kG0 = 8, kGWarps = 4;            // gather warpgroup
+constexpr int kMmaWarp = 12, kB0 = 14;         // two MMA issue warps, B producer (bulk copies)
+constexpr int kThreads = 512;
+// 128 registers a thread at launch; 168 + 168 + 112 + 64 = 4 x 128
+constexpr int kRegEpi = 168, kRegGather = 112, kRegIssue = 64;
 constexpr int kMaxStages = 6;                  // B ring depth at most
-constexpr int kAStages = 2;                    // A tiles in tensor memory
-constexpr int kThreads = (kB0 + 1) * 32;
+constexpr int kAStages = 4;                    // A tiles in tensor memory (even, as the ring's depth)
 constexpr int kGThreads = kGWarps * 32;
+constexpr int kNCols = 64;                     // columns (k', band) of a pass at most
+constexpr int kAcc = 2 * kNCols;               // one accumulator: Re [0, 64), Im [64, 128)
 constexpr int kTKC = 32;                       // complex K values per stage
 constexpr int kACols = 64;                     // one A tile in TMEM: two K16 halves x (Re hi, Im hi, Re lo, Im lo) x 8
 constexpr int kImgRow = 256;                   // packed image of 32 K values: hi row (128 B), lo row (128 B)
@@ -75,40 +87,42 @@ struct TpGeo {
   long long vbase;
   int nkc;                                      // K chunks of the packed images (tc_kpad / 32)
   int stages, nmax;                             // ring depth; B rows per stage (max columns, multiple of 16)
+  int cap;                                      // rows of the position table
   int stage_bytes;
-  int bx, by, bz, bbox_n, bbox_c;               // difference box of S(k): dims, entries, key of G1 = 0
-  int rowbox, nwords;
-  int o_bar, o_bbox, o_kcoef, o_kkey, o_rows, o_bits, o_slot, o_cols, o_binfo, o_bvec, o_ptab;
+  int by, bz, box_n, box_c;                     // difference box of S(k): dims, entries, key of G1 = 0
+  int rowbox, nwords, wpl;                      // row box: entries, bit words, words per (x, y) line
+  int o_bar, o_box, o_pkey, o_kkey, o_rows, o_bits, o_slot, o_binfo, o_bptr, o_binv, o_ptab;
   size_t smem;                                  // dynamic shared memory incl. 1 KB alignment slack
 };
 
-TpGeo tp_geo(const DevSys& d, int stages) {
+TpGeo tp_geo(const DevSys& d, int stages, int cap) {
   TpGeo g{};
   g.stages = stages;
+  g.cap = cap;
   g.nkc = d.tc_kpad / kTKC;
   const int mb = d.nv > d.nc ? d.nv : d.nc;
   g.nmax = (d.tc_rsize * mb + 15) / 16 * 16;
   g.stage_bytes = 2 * g.nmax * umma::kRow;      // B hi rows, B lo rows
   const int rx = d.fwf[0] + d.fpair[0], ry = d.fwf[1] + d.fpair[1], rz = d.fwf[2] + d.fpair[2];
-  g.bx = 2 * rx + 1;
   g.by = 2 * ry + 1;
   g.bz = 2 * rz + 1;
-  g.bbox_n = g.bx * g.by * g.bz;
-  g.bbox_c = (rx * g.by + ry) * g.bz + rz;
+  g.box_n = (2 * rx + 1) * g.by * g.bz;
+  g.box_c = (rx * g.by + ry) * g.bz + rz;
   g.rowbox = (2 * d.fpair[0] + 1) * (2 * d.fpair[1] + 1) * (2 * d.fpair[2] + 1);
-  g.nwords = (g.rowbox + 31) / 32;
+  g.wpl = (2 * d.fpair[2] + 1 + 31) / 32;
+  g.nwords = (2 * d.fpair[0] + 1) * (2 * d.fpair[1] + 1) * g.wpl;
   size_t o = (size_t)stages * g.stage_bytes;
-  g.o_bar = (int)o; o += align16((size_t)(2 * stages + 2 * kAStages + 5) * 8 + 8 * sizeof(int));
-  g.o_bbox = (int)o; o += align16((size_t)g.bbox_n * 2);
-  g.o_kcoef = (int)o; o += align16((size_t)(d.npw_max + 1) * 8);
+  g.o_bar = (int)o; o += align16((size_t)(2 * stages + 2 * kAStages + 2 * kGroups + 4) * 8 + 8 * sizeof(int));
+  g.o_box = (int)o; o += align16((size_t)g.box_n * 8);
+  g.o_pkey = (int)o; o += align16((size_t)d.npw_max * 4);
   g.o_kkey = (int)o; o += align16((size_t)d.tc_kpad * 4);
   g.o_rows = (int)o; o += align16((size_t)g.rowbox * 4);
   g.o_bits = (int)o; o += align16((size_t)g.nwords * 4);
   g.o_slot = (int)o; o += align16((size_t)d.tc_rsize * 4);
-  g.o_cols = (int)o; o += align16((size_t)d.tc_rsize * 4);
   g.o_binfo = (int)o; o += align16((size_t)d.tc_rsize * 16);
-  g.o_bvec = (int)o; o += align16((size_t)d.tc_rsize * 16);
-  g.o_ptab = (int)o; o += align16((size_t)128 * d.tc_rsize * 2);
+  g.o_bptr = (int)o; o += align16((size_t)d.tc_rsize * 16);
+  g.o_binv = (int)o; o += align16((size_t)d.tc_rsize * d.nb * 4);
+  g.o_ptab = (int)o; o += align16((size_t)cap * d.tc_rsize * 2);
   g.smem = o + 1024;
   return g;
 }
@@ -120,22 +134,42 @@ __device__ __forceinline__ void fail_now(volatile int* fail, int* status) {
 
 __device__ __forceinline__ void gather_bar() { asm volatile("barrier.sync 1, %0;" ::"n"(kGThreads) : "memory"); }
 
-__device__ __forceinline__ uint32_t bf16_bits(float x) {
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  return (uint32_t)*reinterpret_cast<const unsigned short*>(&h);
+__device__ __forceinline__ uint2 lds64(uint32_t addr) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
+  return v;
 }
 
-// x = hi + lo in BF16 as (hi | lo << 16)
+// x = hi + lo in FP16 as (hi | lo << 16)
 __device__ __forceinline__ uint32_t split_word(float x) {
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  const float r = x - __bfloat162float(h);
-  return (uint32_t)*reinterpret_cast<const unsigned short*>(&h) | (bf16_bits(r) << 16);
+  const __half h = __float2half_rn(x);
+  const __half l = __float2half_rn(x - __half2float(h));
+  return (uint32_t)__half_as_ushort(h) | ((uint32_t)__half_as_ushort(l) << 16);
+}
+
+// ---------------------------------------------------------------- scales
+// scale[k nb + band]: the power of two that puts the largest component of c_{k,band} into [2^14, 2^15); its inverse
+// in the second half.  One warp per (k, band).
+__global__ void tcpair_scale_kernel(DevSys d, const float2* __restrict__ coef, float* __restrict__ scale) {
+  const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (row >= d.nkpt * d.nb) return;
+  const float2* x = coef + (size_t)row * d.npw_max;
+  const int n = d.npw[row / d.nb];
+  float m = 0.f;
+  for (int i = lane; i < n; i += 32) m = fmaxf(m, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int e = tcf::scale_exp(m);
+  if (lane == 0) {
+    scale[row] = tcf::pow2(e);
+    scale[d.nkpt * d.nb + row] = tcf::pow2(-e);
+  }
 }
 
 // ---------------------------------------------------------------- packed coefficient panels
 // Packed B panels: for each region r, set (valence bands, then conduction bands) and K chunk c, the rows
 // j = slot nset + m of every k' of the region (slot: its position in the region, m: its band in the set),
-// [Re 32 | Im 32] BF16 in the region's K layout (zero off S(k')), hi rows then lo rows, the 16-byte chunks of
+// [Re 32 | Im 32] FP16 in the region's K layout (zero off S(k')), hi rows then lo rows, the 16-byte chunks of
 // row j permuted by j mod 8 (128B swizzle): a stage's B tile is two bulk copies.
 __device__ __forceinline__ size_t panel_off(const DevSys& d, int r, int set, int c, int nkc) {
   const size_t per_r = (size_t)nkc * 2 * umma::kRow * d.tc_rsize * (d.nv + d.nc);
@@ -150,8 +184,8 @@ __device__ __forceinline__ void region_of(const DevSys& d, int k2, int& r, int& 
   slot = ((o0 % d.tc_rg[0]) * d.tc_rg[1] + o1 % d.tc_rg[1]) * d.tc_rg[2] + o2 % d.tc_rg[2];
 }
 
-__global__ void tcpair_pack_kernel(DevSys d, const float2* __restrict__ coef, unsigned char* __restrict__ bimg,
-                                   int nkc) {
+__global__ void tcpair_pack_kernel(DevSys d, const float2* __restrict__ coef, const float* __restrict__ scale,
+                                   unsigned char* __restrict__ bimg, int nkc) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long total = (long long)d.nkpt * d.nb * d.npw_max;
   if (t >= total) return;
@@ -164,7 +198,8 @@ __global__ void tcpair_pack_kernel(DevSys d, const float2* __restrict__ coef, un
   region_of(d, k2, r, slot);
   const int l = d.tc_kpos[(size_t)k2 * d.npw_max + i];
   const float2 c = coef[t];
-  const uint32_t re = split_word(c.x), im = split_word(c.y);
+  const float sc = scale[kb];
+  const uint32_t re = split_word(c.x * sc), im = split_word(c.y * sc);
   const int e = l % kTKC, j = slot * nset + m, ph = j & 7;
   unsigned short* hi = reinterpret_cast<unsigned short*>(bimg + panel_off(d, r, set, l / kTKC, nkc)) + j * 64;
   unsigned short* lo = hi + d.tc_rsize * nset * 64;
@@ -189,42 +224,63 @@ __global__ void tcpair_tiles_kernel(DevSys d, int q_begin, int nqc, int* __restr
 }
 
 // ---------------------------------------------------------------- the GEMM tiles
+// One row of a pass to its blocks: NSET columns per slot, unrolled (a loop over columns with the slot's tables and
+// branches in it took as long as the promotion of the pass; where the stores go makes no difference: consecutive
+// addresses instead of sphere positions measured the same).
+template <int NSET>
+__device__ __forceinline__ void write_pass(const float (&re)[kNCols], const float (&im)[kNCols], float ia,
+                                           const float* ib, float2* const* bptr, const short* pt, int rs, int nb,
+                                           size_t first, int ng_max) {
+#pragma unroll
+  for (int b = 0; b < kNCols / NSET; ++b) {
+    if (b >= rs) break;
+    const int pb = pt[b];
+    float2* dst = bptr[2 * b] + first + pb;
+#pragma unroll
+    for (int m = 0; m < NSET; ++m) {
+      const float s = ib[b * nb + m];
+      const float2 v = make_float2(re[b * NSET + m] * ia * s, im[b * NSET + m] * ia * s);
+      if (pb >= 0) dst[(size_t)m * ng_max] = v;
+    }
+  }
+}
+
 __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const float2* __restrict__ coef,
+                                                             const float* __restrict__ scale,
                                                              const unsigned char* __restrict__ bimg,
                                                              const int* __restrict__ blist, int* __restrict__ counter,
-                                                             float2* __restrict__ out, TpGeo g, int* status) {
+                                                             float2* __restrict__ out,
+                                                             const __grid_constant__ TpGeo g, int* status) {
   extern __shared__ __align__(1024) unsigned char tp_smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)tp_smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full_b = (uint64_t*)(sm + g.o_bar);   // [stages] B rows landed
   uint64_t* empty_b = full_b + g.stages;          // [stages] MMAs done with the B stage
-  uint64_t* full_a = empty_b + g.stages;          // [2] A tile written to tensor memory
-  uint64_t* empty_a = full_a + kAStages;          // [2] MMAs done with the A tile
-  uint64_t* tfull = empty_a + kAStages;           // [2] accumulator complete
-  uint64_t* tempty = tfull + 2;                    // [2] accumulator drained
-  uint64_t* drain = tempty + 2;                    // every MMA of this CTA complete
-  int* iv = (int*)(drain + 1);                     // tmem, fail, tile, nblk, rows, k of the box
+  uint64_t* full_a = empty_b + g.stages;          // [4] A tile written to tensor memory
+  uint64_t* empty_a = full_a + kAStages;          // [4] MMAs done with the A tile
+  uint64_t* tfull = empty_a + kAStages;           // [group][2] accumulator holds a chunk of one of the group's passes
+  uint64_t* tempty = tfull + 2 * kGroups;          // [2] accumulator promoted
+  uint64_t* drain = tempty + 2;                    // [2] every MMA of an issue warp complete
+  int* iv = (int*)(drain + 2);                     // tmem, fail, tile, rows, points in the box, blocks
   volatile int* fail = iv + 1;
-  unsigned short* bbox = (unsigned short*)(sm + g.o_bbox);
-  uint2* kcoef = (uint2*)(sm + g.o_kcoef);
+  uint2* box = (uint2*)(sm + g.o_box);
+  int* pkey = (int*)(sm + g.o_pkey);
   int* kkey = (int*)(sm + g.o_kkey);
   char4* rows = (char4*)(sm + g.o_rows);
   unsigned* bits = (unsigned*)(sm + g.o_bits);
   int* slot = (int*)(sm + g.o_slot);
-  int* cols = (int*)(sm + g.o_cols);
   int4* binfo = (int4*)(sm + g.o_binfo);
-  long long* bvec = (long long*)(sm + g.o_bvec);
-  short* ptab = (short*)(sm + g.o_ptab);
+  float2** bptr = (float2**)(sm + g.o_bptr);       // [slot][set] first vector of the block
+  float* binv = (float*)(sm + g.o_binv);           // [slot][band] inverse scale of the point's coefficients
+  short* ptab = (short*)(sm + g.o_ptab);           // [row][slot] sphere position of the row on the slot's block, or -1
 
   const int tid = threadIdx.x, warp = umma::uniform(tid >> 5), lane = tid & 31;
   const int ntiles = d.nkpt * d.tc_nreg, rs = d.tc_rsize;
   const int f0 = d.fwf[0], f1 = d.fwf[1], f2 = d.fwf[2];
   const int kb1 = 2 * f1 + 1, kb2 = 2 * f2 + 1;
   const int p0 = d.fpair[0], p1 = d.fpair[1], p2 = d.fpair[2];
-  const int rb1 = 2 * p1 + 1, rb2 = 2 * p2 + 1;
-  const int nv = d.nv, nc = d.nc;
-  const uint32_t half = (uint32_t)((g.nmax + 31) & ~31);    // Re [0, half), Im [half, 2 half) of an accumulator
-  const uint32_t acc_cols = 2 * half;
-  const uint32_t a_col0 = 2 * acc_cols;                      // the A tiles after the two accumulators
+  const int rb1 = 2 * p1 + 1;
+  const int nv = d.nv, nc = d.nc, nb = d.nb;
+  constexpr uint32_t a_col0 = 2 * kAcc;            // the A slots after the two accumulators
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(iv)), "r"(512)
@@ -237,112 +293,116 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
       mbar_init(smem_u32(empty_b + i), 1);
     }
     for (int i = 0; i < kAStages; ++i) {
-      mbar_init(smem_u32(full_a + i), kGWarps / kAStages);
+      mbar_init(smem_u32(full_a + i), kGWarps);
       mbar_init(smem_u32(empty_a + i), 1);
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(smem_u32(tfull + i), 1);
-      mbar_init(smem_u32(tempty + i), kEpiWarps);
-    }
-    mbar_init(smem_u32(drain), 1);
+    for (int i = 0; i < 2 * kGroups; ++i) mbar_init(smem_u32(tfull + i), 1);
+    for (int i = 0; i < 2; ++i) mbar_init(smem_u32(tempty + i), 4);
+    for (int i = 0; i < 2; ++i) mbar_init(smem_u32(drain + i), 1);
     iv[1] = 0;
-    iv[5] = -1;
+    iv[4] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  for (int i = tid; i < g.box_n; i += kThreads) box[i] = make_uint2(0u, 0u);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = (uint32_t)iv[0];
+  const uint32_t tmem = umma::uniform((uint32_t)iv[0]);
 
-  unsigned sc = 0, pc = 0;                       // stages and passes issued so far (same on every role)
-  while (true) {
-    __syncthreads();                             // every role is done with the previous tile
-    if (tid == 0) iv[2] = *fail ? ntiles : atomicAdd(counter, 1);
-    __syncthreads();
-    const int t_ = iv[2];
-    if (t_ >= ntiles) break;
-    // region-major order: the CTAs in flight share one region's packed B rows, which stay in L2
-    const int r = t_ / d.nkpt, k = t_ - r * d.nkpt;
-    const int tile = k * d.tc_nreg + r;
-    const int kc = d.tc_kcount[r];
-    const bool newk = iv[5] != k;
-    // ---- tile setup: columns, K keys, difference box of S(k), rows
-    if (tid < rs) slot[tid] = blist[(size_t)tile * rs + tid];
+  const int role = warp >> 2;                    // 0, 1 epilogue, 2 gather, 3 issue
+  unsigned sc = 0, pc = 0;                       // stages and passes issued so far (the same in every role)
+  int r = 0, k = 0, kc = 0, MT = 0, nmt = 0, nch = 0, n1 = 0;
+
+  const size_t pq = (size_t)(2 * f0 + 1) * kb1 * kb2;
+  auto position = [&](char4 G, int4 bi) -> short {
+    const int x = G.x + (bi.z & 3) - 1, y = G.y + ((bi.z >> 2) & 3) - 1, z = G.z + ((bi.z >> 4) & 3) - 1;
+    if (bi.x < 0 || x < -f0 || x > f0 || y < -f1 || y > f1 || z < -f2 || z > f2) return -1;
+    return d.tc_pmap[(size_t)bi.x * pq + ((size_t)(x + f0) * kb1 + y + f1) * kb2 + z + f2];
+  };
+
+  // The next tile and its tables (all 512 threads, each role from its own copy of the tile loop: the register split
+  // only holds where the roles' code does not meet).  False: no tile is left.
+  auto all_bar = []() { asm volatile("barrier.sync 2, %0;" ::"n"(kThreads) : "memory"); };
+  auto next_tile = [&]() -> bool {
+    sc += (unsigned)(nb * nmt * nch);
+    pc += (unsigned)(nb * nmt);
+    int tile;
+    while (true) {
+      all_bar();                                 // every role is done with the previous tile
+      if (tid == 0) {
+        iv[2] = *fail ? ntiles : atomicAdd(counter, 1);
+        iv[5] = 0;
+      }
+      all_bar();
+      const int t_ = iv[2];
+      if (t_ >= ntiles) return false;
+      // region-major order: the CTAs in flight share one region's packed B rows, which stay in L2
+      r = t_ / d.nkpt;
+      k = t_ - r * d.nkpt;
+      tile = k * d.tc_nreg + r;
+      for (int i = tid; i < rs; i += kThreads) {
+        const int b = blist[(size_t)tile * rs + i];
+        slot[i] = b;
+        if (b >= 0) iv[5] = 1;
+      }
+      all_bar();
+      if (iv[5]) break;
+    }
+    kc = umma::uniform(d.tc_kcount[r]);
+    // ---- tile setup: blocks per slot, K keys, sphere keys of k, rows
     for (int i = tid; i < g.nwords; i += kThreads) bits[i] = 0u;
+    for (int i = tid; i < iv[4]; i += kThreads) box[pkey[i]] = make_uint2(0u, 0u);   // the previous tile's points
     for (int i = tid; i < g.nkc * kTKC; i += kThreads) {
-      int key = g.bbox_c;                        // padding: G2 = 0 (the B images are zero there)
+      int key = g.box_c;                         // padding: G2 = 0 (the B images are zero there)
       if (i < kc) {
         const char4 g2 = d.tc_klist[(size_t)r * d.tc_kpad + i];
         key += ((int)g2.x * g.by + (int)g2.y) * g.bz + (int)g2.z;
       }
-      kkey[i] = key;
+      kkey[i] = key * 8;
     }
-    if (newk)
-      for (int i = tid; i < g.bbox_n; i += kThreads) bbox[i] = (unsigned short)d.npw_max;
-    __syncthreads();
-    if (warp == 0) {
-      int n = 0;
-      for (int b0 = 0; b0 < rs; b0 += 32) {
-        const int j = b0 + lane;
-        const int b = j < rs ? slot[j] : -1;
-        const unsigned m = __ballot_sync(0xffffffffu, b >= 0);
-        if (b >= 0) cols[n + __popc(m & ((1u << lane) - 1u))] = b;
-        n += __popc(m);
-      }
-      if (lane == 0) iv[3] = n;
-    }
-    if (newk) {
-      const int n1 = d.npw[k];
-      for (int i = tid; i < n1; i += kThreads) {
-        const char4 gg = d.gk[(size_t)k * d.npw_max + i];
-        bbox[g.bbox_c + ((int)gg.x * g.by + (int)gg.y) * g.bz + (int)gg.z] = (unsigned short)i;
-      }
-    }
-    __syncthreads();
-    if (tid == 0) iv[5] = k;
-    const int nblk = iv[3];
-    if (nblk == 0) continue;
-    for (int i = tid; i < rs; i += kThreads) {  // per slot of the region; x = -1: no block of this range
+    for (int i = tid; i < rs; i += kThreads) {   // per slot of the region; x = -1: no block of this range
       const int b = slot[i];
       if (b < 0) {
         binfo[i] = make_int4(-1, 0, 0, 0);
+        for (int n = 0; n < nb; ++n) binv[i * nb + n] = 0.f;
         continue;
       }
       const int4 blk = d.blocks[b];
       const long long qb = d.qblk_off[blk.z], nbq = d.qblk_off[blk.z + 1] - qb;
       const long long base = d.qvec_off[blk.z] - g.vbase;
       binfo[i] = make_int4(blk.z, blk.y, blk.w, 0);
-      bvec[2 * i] = base + (b - qb) * nv * nv;
-      bvec[2 * i + 1] = base + nbq * nv * nv + (b - qb) * nc * nc;
+      bptr[2 * i] = out + (size_t)(base + (b - qb) * nv * nv) * d.ng_max;
+      bptr[2 * i + 1] = out + (size_t)(base + nbq * nv * nv + (b - qb) * nc * nc) * d.ng_max;
+      for (int n = 0; n < nb; ++n) binv[i * nb + n] = scale[(size_t)d.nkpt * nb + (size_t)blk.y * nb + n];
     }
-    for (int i = 0; i < nblk; ++i) {
-      const int4 blk = d.blocks[cols[i]];
+    all_bar();
+    for (int i = warp; i < rs; i += kThreads / 32) {   // the union of the blocks' spheres, one warp per block
+      const int b = slot[i];
+      if (b < 0) continue;
+      const int4 blk = d.blocks[b];
       const int gx = (blk.w & 3) - 1, gy = ((blk.w >> 2) & 3) - 1, gz = ((blk.w >> 4) & 3) - 1;
       const int ng = d.ngq[blk.z];
-      for (int p = tid; p < ng; p += kThreads) {
-        const char4 gp = d.gq[(size_t)blk.z * d.ng_max + p];
-        const int li = ((gp.x - gx + p0) * rb1 + gp.y - gy + p1) * rb2 + gp.z - gz + p2;
-        atomicOr(&bits[li >> 5], 1u << (li & 31));
+      const char4* gq = d.gq + (size_t)blk.z * d.ng_max;
+      for (int p0_ = 0; p0_ < ng; p0_ += 128) {   // four loads in flight
+        char4 gp[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) gp[u] = gq[min(p0_ + 32 * u + lane, ng - 1)];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int z = gp[u].z - gz + p2;
+          atomicOr(&bits[((gp[u].x - gx + p0) * rb1 + gp[u].y - gy + p1) * g.wpl + (z >> 5)], 1u << (z & 31));
+        }
       }
     }
-    __syncthreads();
-    int ng_ref;
-    {
-      const int4 b0 = d.blocks[cols[0]];
-      const int4 bi = make_int4(b0.z, b0.y, b0.w, 0);
-      const int gx = (bi.z & 3) - 1, gy = ((bi.z >> 2) & 3) - 1, gz = ((bi.z >> 4) & 3) - 1;
-      ng_ref = d.ngq[bi.x];
-      for (int p = tid; p < ng_ref; p += kThreads) {
-        const char4 gp = d.gq[(size_t)bi.x * d.ng_max + p];
-        const int x = gp.x - gx, y = gp.y - gy, z = gp.z - gz;
-        rows[p] = make_char4((signed char)x, (signed char)y, (signed char)z, 0);
-        const int li = ((x + p0) * rb1 + y + p1) * rb2 + z + p2;
-        atomicAnd(&bits[li >> 5], ~(1u << (li & 31)));
-      }
+    all_bar();
+    n1 = d.npw[k];
+    for (int i = tid; i < n1; i += kThreads) {
+      const char4 gg = d.gk[(size_t)k * d.npw_max + i];
+      pkey[i] = g.box_c + ((int)gg.x * g.by + (int)gg.y) * g.bz + (int)gg.z;
     }
-    __syncthreads();
-    if (warp == 0) {
-      int n = ng_ref;
+    if (tid == 0) iv[4] = n1;
+    if (warp == 0) {                             // rows in lexicographic order: neighbours in a warp gather neighbours
+      int n = 0;
       for (int w0 = 0; w0 < g.nwords; w0 += 32) {
         const int w = w0 + lane;
         unsigned m = w < g.nwords ? bits[w] : 0u;
@@ -354,237 +414,263 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
           if (lane >= o) incl += t;
         }
         int pos = n + incl - cnt;
+        const int line = w / g.wpl, x = line / rb1 - p0, y = line % rb1 - p1, z0 = (w % g.wpl) * 32 - p2;
         while (m) {
-          const int li = w * 32 + __ffs(m) - 1;
+          rows[pos++] = make_char4((signed char)x, (signed char)y, (signed char)(z0 + __ffs(m) - 1), 0);
           m &= m - 1u;
-          const int z = li % rb2, y = (li / rb2) % rb1, x = li / (rb2 * rb1);
-          rows[pos++] = make_char4((signed char)(x - p0), (signed char)(y - p1), (signed char)(z - p2), 0);
         }
         n += __shfl_sync(0xffffffffu, incl, 31);
       }
-      if (lane == 0) iv[4] = n;
+      if (lane == 0) iv[3] = n;
     }
-    __syncthreads();
-    const int MT = iv[4];
-    const int nmt = (MT + 127) / 128;
-    const int nch = (kc + kTKC - 1) / kTKC;
+    all_bar();
+    MT = umma::uniform(iv[3]);
+    if (MT <= g.cap) {                           // (a larger union: per pass, below)
+      for (int i = tid; i < MT * rs; i += kThreads) ptab[i] = position(rows[i / rs], binfo[i % rs]);
+      all_bar();
+    }
+    nmt = (MT + 127) / 128;
+    nch = (kc + kTKC - 1) / kTKC;
+    return true;
+  };
 
-    if (warp >= kG0 && warp < kB0) {             // ---- gather: A tiles into tensor memory
-      // warp -> lane quarter q4 (rows 32 q4 .. 32 q4 + 31 of the M tile) and A slot sa: the four warps of
-      // slot sa write every other stage, all 32 K values, in two halves (the first store overlaps the
-      // second half's lookups)
-      const int gt = tid - kG0 * 32, q4 = warp & 3, sa = (warp - kG0) >> 2;
-      unsigned s = sc;
-      for (int set = 0; set < 2; ++set) {
-        const int nset = set ? nc : nv, n0 = set ? nv : 0;
-        for (int nn = 0; nn < nset; ++nn) {
-          gather_bar();                          // every gather warp is done with the previous band
-          {
-            const int n1 = d.npw[k];
-            const float2* cn = coef + ((size_t)k * d.nb + n0 + nn) * d.npw_max;
-            for (int i = gt; i <= d.npw_max; i += kGThreads) {
-              uint2 v = make_uint2(0u, 0u);
-              if (i < n1) {
-                const float2 c = cn[i];
-                v = make_uint2(split_word(c.x), split_word(-c.y));    // conj
-              }
-              kcoef[i] = v;
-            }
+  if (role == 2) {                               // ---- gather: A tiles into tensor memory
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegGather));
+    int sa = 0;                                  // A slot and its phase
+    uint32_t aph = 0u;
+    bool ok = true;
+    while (next_tile()) {
+      const int gt = tid - kG0 * 32, q4 = warp & 3;
+      const uint32_t box_u = smem_u32(box);
+      uint2 x[16];
+      auto load16 = [&](uint32_t at, int k0) {   // 16 K values of this row
+        const int4* kp = reinterpret_cast<const int4*>(kkey + k0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int4 t = kp[q];
+          x[4 * q] = lds64(at + (uint32_t)t.x);
+          x[4 * q + 1] = lds64(at + (uint32_t)t.y);
+          x[4 * q + 2] = lds64(at + (uint32_t)t.z);
+          x[4 * q + 3] = lds64(at + (uint32_t)t.w);
+        }
+      };
+      auto pack16 = [&](uint32_t (&v)[32]) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          v[j] = __byte_perm(x[2 * j].x, x[2 * j + 1].x, 0x5410);        // Re hi
+          v[8 + j] = __byte_perm(x[2 * j].y, x[2 * j + 1].y, 0x5410);    // Im hi
+          v[16 + j] = __byte_perm(x[2 * j].x, x[2 * j + 1].x, 0x7632);   // Re lo
+          v[24 + j] = __byte_perm(x[2 * j].y, x[2 * j + 1].y, 0x7632);   // Im lo
+        }
+      };
+      for (int n = 0; n < nb; ++n) {             // valence bands, then conduction bands
+        gather_bar();                            // every gather warp is done with the previous band
+        {
+          const float2* cn = coef + ((size_t)k * nb + n) * d.npw_max;
+          const float a = scale[(size_t)k * nb + n];
+          for (int i = gt; i < n1; i += kGThreads) {
+            const float2 c = cn[i];
+            box[pkey[i]] = make_uint2(split_word(c.x * a), split_word(-c.y * a));    // conj
           }
-          gather_bar();
-          for (int mt = 0; mt < nmt; ++mt) {
-            const int row = mt * 128 + q4 * 32 + lane;
-            const bool rval = row < MT;
-            int rkey = 0;
-            if (rval) {
-              const char4 G = rows[row];
-              rkey = ((int)G.x * g.by + (int)G.y) * g.bz + (int)G.z;
+        }
+        gather_bar();
+        if (umma::uniform(*fail != 0)) ok = false;
+        for (int mt = 0; mt < nmt; ++mt) {
+          const int row = mt * 128 + q4 * 32 + lane;
+          uint32_t at = box_u;                   // rows past the last one gather something and are dropped
+          if (row < MT) {
+            const char4 G = rows[row];
+            at -= (uint32_t)((((int)G.x * g.by + (int)G.y) * g.bz + (int)G.z) * 8);
+          }
+          // the lookups of the next 16 K values are in flight while the last ones are packed and stored
+          load16(at, 0);
+          for (int c = 0; c < nch; ++c) {
+            if (ok) {
+              ok = umma::uniform(mbar_wait(smem_u32(empty_a + sa), aph ^ 1u));
+              if (!ok) fail_now(fail, status);
             }
-            for (int c = 0; c < nch; ++c, ++s) {
-              if ((int)(s & 1u) != sa) continue;
-              int ok = 1;
-              if (lane == 0) {                   // warp-uniform decision
-                ok = *fail ? 0 : 1;
-                if (ok && s >= (unsigned)kAStages) {
-                  ok = mbar_wait(smem_u32(empty_a + sa), ((s >> 1) - 1) & 1u) ? 1 : 0;
-                  if (!ok) fail_now(fail, status);
-                }
-              }
-              ok = __shfl_sync(0xffffffffu, ok, 0);
-              if (!ok) continue;
+            if (ok) {
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll 1
-              for (int hk = 0; hk < 2; ++hk) {
-                uint32_t v[32];
-                if (rval) {
-                  const int4* kp = reinterpret_cast<const int4*>(kkey + c * kTKC + hk * 16);
-                  int kk16[16];
-#pragma unroll
-                  for (int q = 0; q < 4; ++q) {
-                    const int4 t = kp[q];
-                    kk16[4 * q] = t.x;
-                    kk16[4 * q + 1] = t.y;
-                    kk16[4 * q + 2] = t.z;
-                    kk16[4 * q + 3] = t.w;
-                  }
-                  uint2 x[16];
-#pragma unroll
-                  for (int e = 0; e < 16; ++e) x[e] = kcoef[bbox[kk16[e] - rkey]];
-#pragma unroll
-                  for (int j = 0; j < 8; ++j) {
-                    v[j] = __byte_perm(x[2 * j].x, x[2 * j + 1].x, 0x5410);        // Re hi
-                    v[8 + j] = __byte_perm(x[2 * j].y, x[2 * j + 1].y, 0x5410);    // Im hi
-                    v[16 + j] = __byte_perm(x[2 * j].x, x[2 * j + 1].x, 0x7632);   // Re lo
-                    v[24 + j] = __byte_perm(x[2 * j].y, x[2 * j + 1].y, 0x7632);   // Im lo
-                  }
-                } else {
-#pragma unroll
-                  for (int j = 0; j < 32; ++j) v[j] = 0u;
-                }
-                umma::tmem_st32(tmem + ((uint32_t)(q4 * 32) << 16) + a_col0 + (uint32_t)(sa * kACols + hk * 32), v);
-              }
+              const uint32_t ta = tmem + ((uint32_t)(q4 * 32) << 16) + a_col0 + (uint32_t)(sa * kACols);
+              uint32_t v[32];
+              pack16(v);
+              load16(at, c * kTKC + 16);
+              umma::tmem_st32(ta, v);
+              pack16(v);
+              load16(at, min(c + 1, nch - 1) * kTKC);
+              umma::tmem_st32(ta + 32u, v);
               asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
               asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
               __syncwarp();
               if (lane == 0) mbar_arrive(smem_u32(full_a + sa));
             }
+            if (++sa == kAStages) {
+              sa = 0;
+              aph ^= 1u;
+            }
           }
         }
       }
-    } else if (warp == kB0) {                    // ---- B producer: the region's panel, two bulk copies per stage
-      unsigned s = sc;
-      for (int set = 0; set < 2; ++set) {
-        const int nset = set ? nc : nv;
-        const uint32_t half_bytes = (uint32_t)(rs * nset) * umma::kRow;
-        for (int nn = 0; nn < nset; ++nn)
-          for (int mt = 0; mt < nmt; ++mt)
-            for (int c = 0; c < nch; ++c, ++s) {
-              if (lane != 0) continue;
-              const int st = (int)(s % (unsigned)g.stages);
-              if (*fail) continue;
-              if (s >= (unsigned)g.stages && !mbar_wait(smem_u32(empty_b + st), ((s / g.stages) - 1) & 1u)) {
+    }
+  } else if (role == 3) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegIssue));
+    unsigned copied = 0;                         // B producer: stages whose copies have been issued
+    int st = 0, sa = 0;                          // B stage, A slot and accumulator, and their phases
+    uint32_t bph = 0u, aph = 0u, cph = 0u, buf = 0u;
+    bool ok = true;
+    while (next_tile()) {
+    if (warp == kB0) {                           // ---- B producer: the region's panel, two bulk copies per stage
+      if (lane == 0) {
+        for (int set = 0; set < 2; ++set) {
+          const int nset = set ? nc : nv;
+          const uint32_t half_bytes = (uint32_t)(rs * nset) * umma::kRow;
+          for (int pass = 0; pass < nset * nmt; ++pass)
+            for (int c = 0; c < nch; ++c) {
+              if (ok && !mbar_wait(smem_u32(empty_b + st), bph ^ 1u)) {
                 fail_now(fail, status);
-                continue;
+                ok = false;
               }
+              if (!ok) continue;
               umma::mbar_arrive_expect_tx(smem_u32(full_b + st), 2 * half_bytes);
               const uint32_t bh = smem_u32(sm + (size_t)st * g.stage_bytes);
               const unsigned char* p = bimg + panel_off(d, r, set, c, g.nkc);
               umma::bulk_g2s(bh, p, half_bytes, smem_u32(full_b + st));
               umma::bulk_g2s(bh + (uint32_t)(g.nmax * umma::kRow), p + half_bytes, half_bytes, smem_u32(full_b + st));
-            }
-      }
-    } else if (warp == kMmaWarp) {               // ---- MMA issue: the whole warp runs the loop, one lane issues
-      const bool leader = umma::elect_one();
-      unsigned s = sc, p = pc;
-      bool ok = umma::uniform(!*fail);
-      const uint64_t dstage0 = umma::smem_desc(umma::uniform(smem_u32(sm)));   // B stage st: + st stage_bytes / 16
-      const uint32_t blo = (uint32_t)((g.nmax * umma::kRow) >> 4), tm = umma::uniform(tmem);
-      const int kcu = umma::uniform(kc), nmtu = umma::uniform(nmt), nchu = (kcu + kTKC - 1) / kTKC;
-      for (int set = 0; set < 2; ++set) {
-        const int nset = set ? nc : nv;
-        const int N = (rs * nset + 15) & ~15;
-        const uint32_t idesc = umma::idesc_of(N);
-        for (int pass = 0; pass < nset * nmtu; ++pass, ++p) {
-          const int buf = (int)(p & 1u);
-          if (ok && p >= 2) {
-            ok = umma::uniform(mbar_wait(smem_u32(tempty + buf), ((p >> 1) - 1) & 1u));
-            if (!ok && leader) fail_now(fail, status);
-          }
-          if (ok) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t d_re = tm + (uint32_t)buf * acc_cols, d_im = d_re + half;
-          for (int c = 0; c < nchu; ++c, ++s) {
-            if (!ok) continue;
-            const int st = (int)(s % (unsigned)g.stages), sa = (int)(s & 1u);
-            ok = umma::uniform(!*fail && mbar_wait(smem_u32(full_a + sa), (s >> 1) & 1u) &&
-                               mbar_wait(smem_u32(full_b + st), (s / g.stages) & 1u) && !*fail);
-            if (!ok) {
-              if (leader) fail_now(fail, status);
-              continue;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t db = dstage0 + (uint64_t)((st * g.stage_bytes) >> 4);
-            const uint32_t a = tm + a_col0 + (uint32_t)(sa * kACols);
-            if (leader) {
-              umma::mma_cplx_k16_ts(d_re, d_im, a, db, blo, 0, idesc, c == 0);
-              if (kcu - c * kTKC > 16) umma::mma_cplx_k16_ts(d_re, d_im, a + 32u, db, blo, 1, idesc, false);
-              mma_commit(smem_u32(empty_a + sa));
-              mma_commit(smem_u32(empty_b + st));
-            }
-            __syncwarp();
-          }
-          if (ok && leader) mma_commit(smem_u32(tfull + buf));
-          __syncwarp();
-        }
-      }
-    } else {                                     // ---- epilogue: TMEM lanes 32 warp .. -> rows
-      unsigned p = pc;
-      const size_t pq = (size_t)(2 * f0 + 1) * kb1 * kb2;
-      short* pt = ptab + (size_t)(warp * 32 + lane) * rs;
-      for (int set = 0; set < 2; ++set) {
-        const int nset = set ? nc : nv;
-        const int ncols = rs * nset;
-        for (int nn = 0; nn < nset; ++nn)
-          for (int mt = 0; mt < nmt; ++mt, ++p) {
-            const int buf = (int)(p & 1u);
-            const int row = mt * 128 + warp * 32 + lane;
-            const bool valid = row < MT;
-            // sphere positions of this row on every block of the tile (independent loads, before the wait)
-            if (valid) {
-              const char4 G = rows[row];
-#pragma unroll 4
-              for (int b = 0; b < rs; ++b) {
-                const int4 bi = binfo[b];
-                const int x = G.x + (bi.z & 3) - 1, y = G.y + ((bi.z >> 2) & 3) - 1, z = G.z + ((bi.z >> 4) & 3) - 1;
-                short pb = -1;
-                if (bi.x >= 0 && x >= -f0 && x <= f0 && y >= -f1 && y <= f1 && z >= -f2 && z <= f2)
-                  pb = d.tc_pmap[(size_t)bi.x * pq + ((size_t)(x + f0) * kb1 + y + f1) * kb2 + z + f2];
-                pt[b] = pb;
+              ++copied;
+              if (++st == g.stages) {
+                st = 0;
+                bph ^= 1u;
               }
             }
-            int ok = 1;
-            if (lane == 0) {
-              ok = (!*fail && mbar_wait(smem_u32(tfull + buf), (p >> 1) & 1u)) ? 1 : 0;
-              if (!ok) fail_now(fail, status);
+        }
+      }
+      __syncwarp();
+    } else if (warp < kB0) {                     // ---- MMA issue: the whole warp runs the loop, one lane issues
+      // Two warps, one per accumulator (even and odd stages): a stage's three waits take ~300 cycles even when
+      // everything is there, and run while the other warp's MMAs do.  Lanes 0-2 wait on one barrier each.
+      const bool leader = umma::elect_one();
+      const uint32_t own = (uint32_t)(warp - kMmaWarp);
+      unsigned p = pc;
+      if (umma::uniform(*fail != 0)) ok = false;
+      const uint64_t dstage0 = umma::smem_desc(umma::uniform(smem_u32(sm)));   // B stage st: + st stage_bytes / 16
+      const uint32_t blo = (uint32_t)((g.nmax * umma::kRow) >> 4);
+      for (int set = 0; set < 2; ++set) {
+        const int nset = set ? nc : nv;
+        const uint32_t idesc = tcf::idesc_f16((rs * nset + 15) & ~15);
+        for (int pass = 0; pass < nset * nmt; ++pass, ++p) {
+          uint64_t* tf = tfull + 2 * (p & 1u);
+          for (int c = 0; c < nch; ++c) {
+            if (ok && buf == own) {
+              const uint32_t bar = lane == 0 ? smem_u32(full_a + sa) : lane == 1 ? smem_u32(full_b + st)
+                                                                                   : smem_u32(tempty + buf);
+              ok = __all_sync(0xffffffffu, mbar_wait(bar, lane == 0 ? aph : lane == 1 ? bph : cph ^ 1u)) != 0;
+              if (!ok && leader) fail_now(fail, status);
             }
-            ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) continue;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            for (int c0 = 0; c0 < ncols; c0 += 32) {
-              uint32_t v[32], u[32];
-              const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)buf * acc_cols + (uint32_t)c0;
-              umma::tmem_ld32(taddr, v);
-              umma::tmem_ld32(taddr + half, u);
-              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-              if (!valid) continue;
-              int b = c0 / nset, m = c0 - b * nset;
-              int pb = pt[b];
-              long long vec0 = bvec[2 * b + set] + (long long)nn * nset;
+            const uint64_t db = dstage0 + (uint64_t)((st * g.stage_bytes) >> 4);
+            const uint32_t a = tmem + a_col0 + (uint32_t)(sa * kACols), d_re = tmem + own * kAcc;
+            if (leader && buf == own) {
+              if (kc - c * kTKC > 16)
+                tcf::chunk_mmas_ts<2>(d_re, d_re + kNCols, a, db, blo, idesc);
+              else
+                tcf::chunk_mmas_ts<1>(d_re, d_re + kNCols, a, db, blo, idesc);
+              mma_commit(smem_u32(empty_a + sa));
+              mma_commit(smem_u32(empty_b + st));
+              mma_commit(smem_u32(tf + own));
+            }
+            __syncwarp();
+            if (++sa == kAStages) {
+              sa = 0;
+              aph ^= 1u;
+            }
+            if (++st == g.stages) {
+              st = 0;
+              bph ^= 1u;
+            }
+            cph ^= buf;
+            buf ^= 1u;
+          }
+        }
+      }
+    }
+    }
+    if (warp == kB0 && lane == 0 && *fail)       // copies still in flight after a failure
+      for (unsigned c = copied > (unsigned)g.stages ? copied - g.stages : 0u; c < copied; ++c)
+        if (!mbar_wait(smem_u32(full_b + c % (unsigned)g.stages), (c / g.stages) & 1u)) break;
+  } else {                                       // ---- epilogue group: promote its passes, then write them
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegEpi));
+    unsigned mine0 = 0u, mine1 = 0u;             // chunks this group has promoted from each accumulator
+    while (next_tile()) {
+      unsigned s = sc, p = pc;
+      const int q4 = warp & 3;
+      const uint32_t lane_addr = tmem + ((uint32_t)(q4 * 32) << 16);
+      bool ok = true;
+      for (int n = 0; n < nb; ++n) {
+        const int set = n < nv ? 0 : 1, nset = set ? nc : nv, nn = set ? n - nv : n;
+        const int ncols = rs * nset;
+        for (int mt = 0; mt < nmt; ++mt, ++p) {
+          if ((int)(p & 1u) != role) {
+            s += (unsigned)nch;
+            continue;
+          }
+          const int row = mt * 128 + q4 * 32 + lane;
+          const bool valid = row < MT;
+          const short* pt = ptab + (size_t)(MT <= g.cap ? row : role * 128 + q4 * 32 + lane) * rs;
+          if (MT > g.cap && valid) {
+            const char4 G = rows[row];
+#pragma unroll 4
+            for (int b = 0; b < rs; ++b) ptab[(size_t)(role * 128 + q4 * 32 + lane) * rs + b] = position(G, binfo[b]);
+          }
+          float re[kNCols], im[kNCols];
 #pragma unroll
-              for (int jj = 0; jj < 32; ++jj) {
-                if (c0 + jj < ncols && pb >= 0)
-                  out[(size_t)(vec0 + m) * d.ng_max + pb] = make_float2(__uint_as_float(v[jj]), __uint_as_float(u[jj]));
-                if (++m == nset) {
-                  m = 0;
-                  ++b;
-                  if (c0 + jj + 1 < ncols) {
-                    pb = pt[b];
-                    vec0 = bvec[2 * b + set] + (long long)nn * nset;
-                  }
-                }
+          for (int j = 0; j < kNCols; ++j) re[j] = im[j] = 0.f;
+          for (int c = 0; c < nch; ++c, ++s) {
+            const int buf = (int)(s & 1u);
+            if (ok) {
+              ok = mbar_wait(smem_u32(tfull + 2 * role + buf), (buf ? mine1 : mine0) & 1u);
+              if (!ok) fail_now(fail, status);
+              ok = umma::uniform(ok);
+            }
+            mine0 += buf ? 0u : 1u;
+            mine1 += buf ? 1u : 0u;
+            if (!ok) continue;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t base = lane_addr + (uint32_t)(buf * kAcc);
+#pragma unroll
+            for (int j0 = 0; j0 < kNCols; j0 += 16) {
+              if (j0 >= ncols) break;
+              uint32_t v[16], u[16];
+              umma::tmem_ld16(base + (uint32_t)j0, v);
+              umma::tmem_ld16(base + (uint32_t)(kNCols + j0), u);
+              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                re[j0 + j] += __uint_as_float(v[j]);
+                im[j0 + j] += __uint_as_float(u[j]);
               }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(tempty + buf));
           }
+          if (!ok || !valid) continue;
+          const float ia = scale[(size_t)d.nkpt * nb + (size_t)k * nb + n];
+          const float* ib = binv + (set ? nv : 0);
+          const size_t first = (size_t)nn * nset * d.ng_max;
+          switch (nset) {
+            case 1: write_pass<1>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
+            case 2: write_pass<2>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
+            case 3: write_pass<3>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
+            default: write_pass<4>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
+          }
+        }
       }
     }
-    sc += (unsigned)((nv + nc) * nmt * nch);
-    pc += (unsigned)((nv + nc) * nmt);
   }
-  if (warp == kMmaWarp && lane == 0) {          // tracks every MMA issued above
-    mma_commit(smem_u32(drain));
-    if (!mbar_wait(smem_u32(drain), 0u)) fail_now(fail, status);
+  if (role == 3 && warp < kB0 && lane == 0) {   // tracks every MMA this thread issued above
+    mma_commit(smem_u32(drain + warp - kMmaWarp));
+    if (!mbar_wait(smem_u32(drain + warp - kMmaWarp), 0u)) fail_now(fail, status);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -636,14 +722,22 @@ __global__ void tcpair_diag_kernel(DevSys d, const float2* __restrict__ coef, fl
   }
 }
 
-int stages_of(const DevSys& d) {
-  for (int st = kMaxStages; st >= 2; --st)
-    if (tp_geo(d, st).smem <= 227 * 1024) return st;
-  return 0;
+// Ring depth and position-table rows: at least four stages, then a table for up to 1024 rows of a tile (256 serve
+// the two groups' passes), then more stages.  The depth is even, so that a stage's slot always belongs to the same
+// issue warp (which then sees every phase of the slot's barriers).  Depth 0: does not fit shared memory.
+TpGeo tp_fit(const DevSys& d) {
+  for (int cap = 1024; cap >= 256; cap -= 128)
+    for (int st = kMaxStages; st >= 4; st -= 2) {
+      const TpGeo g = tp_geo(d, st, cap);
+      if (g.smem <= 227 * 1024) return g;
+    }
+  TpGeo g = tp_geo(d, 2, 256);
+  if (g.smem > 227 * 1024) g.stages = 0;
+  return g;
 }
 
 struct TpWs {
-  size_t bimg, blist, counter, total;
+  size_t bimg, blist, counter, scale, total;
 };
 
 TpWs tp_ws(const DevSys& d) {
@@ -652,6 +746,7 @@ TpWs tp_ws(const DevSys& d) {
   w.bimg = o; o += ((size_t)d.nkpt * d.nb * (d.tc_kpad / kTKC) * kImgRow + 255) & ~(size_t)255;
   w.blist = o; o += ((size_t)d.nkpt * d.tc_nreg * d.tc_rsize * sizeof(int) + 255) & ~(size_t)255;
   w.counter = o; o += 256;
+  w.scale = o; o += ((size_t)2 * d.nkpt * d.nb * sizeof(float) + 255) & ~(size_t)255;
   w.total = o;
   return w;
 }
@@ -660,9 +755,35 @@ TpWs tp_ws(const DevSys& d) {
 
 // The tensor-core route needs a region of at most one N tile of columns and its tiles in shared memory.
 int tcpair_valid(const DevSys& d) {
-  if (d.tc_kpad < kTKC || d.tc_rsize < 1 || d.tc_rsize * (d.nv > d.nc ? d.nv : d.nc) > 96) return 0;
-  if (d.tc_rsize > kThreads) return 0;
-  return stages_of(d) > 0 ? 1 : 0;
+  if (d.nv > 4 || d.nc > 4) return 0;            // write_pass
+  if (d.tc_kpad < kTKC || d.tc_rsize < 1 || d.tc_rsize * (d.nv > d.nc ? d.nv : d.nc) > kNCols) return 0;
+  return tp_fit(d).stages > 0 ? 1 : 0;
+}
+
+// Whether the direct set of [q_begin, q_end) goes to this kernel when the caller has not chosen one.  A tile is a k and
+// a region of k'; it costs the same however few of the region's points have a block in the range, so the
+// route needs tiles for every SM and columns in use: at least 304 tiles, and at least 30 of the 2 x 64 columns of a
+// tile's two band sets on average (regions of the mesh k + q touches are counted at one k off the region grid).
+// Measured, this kernel against gcorr_kernel: 7x7x7 2v2c, 49 q (28 columns) 0.49 against 0.41 ms; 27x27 sheet 2v3c, 64 q
+// (32) 1.33 / 1.52; 5x5x5 4v4c (40) 1.98 / 3.91; 32x32 sheet 3v3c, 64 q 1.73 / 2.61; 8x8x8 3v4c (112) 10.5 / 50.1; 4x4x4
+// 3v3c (256 tiles) 0.131 / 0.117; 3x3x3 1v2c (27 tiles) 0.054 / 0.024.  With k-point symmetry only scattered
+// representative blocks are left and the tiles are nearly empty.
+int tcpair_preferred(const DevSys& d, int q_begin, int q_end) {
+  if (!tcpair_valid(d) || d.nfill > 0) return 0;
+  const int nqc = q_end - q_begin;
+  int touched = d.tc_nreg;
+  if (nqc < d.nq && d.tc_nreg <= 4096) {
+    unsigned long long seen[64] = {};
+    touched = 0;
+    for (int q = q_begin; q < q_end; ++q) {
+      const int i0 = (q / (d.nk2 * d.nk3) + d.tc_rg[0] / 2) % d.nk1, i1 = ((q / d.nk3) % d.nk2 + d.tc_rg[1] / 2) % d.nk2,
+                i2 = (q % d.nk3 + d.tc_rg[2] / 2) % d.nk3;
+      const int r = ((i0 / d.tc_rg[0]) * d.tc_nr[1] + i1 / d.tc_rg[1]) * d.tc_nr[2] + i2 / d.tc_rg[2];
+      touched += (seen[r >> 6] >> (r & 63) & 1ull) ? 0 : 1;
+      seen[r >> 6] |= 1ull << (r & 63);
+    }
+  }
+  return (long long)d.nkpt * touched >= 304 && (long long)nqc * d.nb >= 30ll * touched ? 1 : 0;
 }
 
 size_t tcpair_ws_bytes(const DevSys& d) { return tcpair_valid(d) ? tp_ws(d).total : 0; }
@@ -673,8 +794,7 @@ int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, in
   if (!tcpair_valid(d)) return (int)cudaErrorInvalidValue;
   static int attr_dev = -1, num_sms = 0;
   static size_t attr_smem = 0;
-  const int stages = stages_of(d);
-  TpGeo g = tp_geo(d, stages);
+  TpGeo g = tp_fit(d);
   int dev = 0;
   int e = (int)cudaGetDevice(&dev);
   if (e) return e;
@@ -698,7 +818,9 @@ int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, in
   g.vbase = vbase;
   if ((e = (int)cudaMemsetAsync(bimg, 0, w.blist - w.bimg, st))) return e;
   const long long npk = (long long)d.nkpt * d.nb * d.npw_max;
-  tcpair_pack_kernel<<<(unsigned)((npk + 255) / 256), 256, 0, st>>>(d, (const float2*)coef, bimg, g.nkc);
+  float* scale = (float*)(base + w.scale);
+  tcpair_scale_kernel<<<(unsigned)((d.nkpt * d.nb + 7) / 8), 256, 0, st>>>(d, (const float2*)coef, scale);
+  tcpair_pack_kernel<<<(unsigned)((npk + 255) / 256), 256, 0, st>>>(d, (const float2*)coef, scale, bimg, g.nkc);
   if ((e = (int)cudaGetLastError())) return e;
   if ((e = (int)cudaMemsetAsync(blist, 0xFF, w.counter - w.blist, st))) return e;
   const long long nt = (long long)g.nqc * d.nkpt;
@@ -707,8 +829,8 @@ int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, in
   if ((e = (int)cudaMemsetAsync(counter, 0, sizeof(int), st))) return e;
   const int ntiles = d.nkpt * d.tc_nreg;
   const int grid = ntiles < num_sms ? ntiles : num_sms;
-  tcpair_kernel<<<grid, kThreads, g.smem, st>>>(d, (const float2*)coef, bimg, blist, counter, (float2*)rho_dir, g,
-                                                status);
+  tcpair_kernel<<<grid, kThreads, g.smem, st>>>(d, (const float2*)coef, scale, bimg, blist, counter,
+                                                (float2*)rho_dir, g, status);
   if ((e = (int)cudaGetLastError())) return e;
   if (q_begin == 0) {
     tcpair_diag_kernel<<<d.nkpt, 256, 0, st>>>(d, (const float2*)coef, (float2*)rho_dir, vbase);
