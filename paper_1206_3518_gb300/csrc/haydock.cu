@@ -14,6 +14,14 @@
 // matrix-vector product keeps compensated FP32 partial sums.  Only O(dim) per step and
 // the coefficient reductions use native FP64.
 //
+// The recursion amplifies a change in the last bit: from one rounding of v_j to FP32 that falls the other way the a_j, b_j
+// drift apart by a factor of ~10 every few steps up to the rounding level of the FP32 products, and eps_2 by 3e-7.  So
+// the order of every sum that reaches w, h or v is fixed: rows per CTA, chains per basis vector, lanes per partial.
+// What a step takes beside the H stream (dim 6144: 45 of 82 us) is latency: five barriers, FP64 scalars, sums over few
+// rows.  Within that order: one FP64 warp for the scalars, the chains of a vector on up to four threads, eight to sixteen
+// loads in flight everywhere, the growing barrier counter.  Measured before and after, the same bits: dim 576, 100 steps
+// 3.30 -> 2.42 ms; dim 6144, 300 steps 24.9 -> 22.9 ms; six sheets of dim 882 to 5400, 300 steps 60.4 -> 45.8 ms.
+//
 // One persistent cooperative launch runs every step.  Each CTA owns a
 // contiguous slice of rows for the product, the projections and the updates,
 // so the only global exchanges are the projection coefficients and two norms
@@ -48,11 +56,6 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned v) {
-  unsigned old;
-  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-  return old;
-}
 __device__ __forceinline__ void red_add_release(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -60,25 +63,22 @@ __device__ __forceinline__ void red_add_release(unsigned* p, unsigned v) {
 // Limit of one grid-barrier wait (ns); settable per device for failure-injection tests.
 __device__ unsigned long long g_wait_limit_ns = 2000000000ull;
 
-// Barrier over the gsize CTAs of one system's group, on a (count, generation) pair: arrivals are
-// acquire-release atomics, the last arrival resets the count and releases the generation, the
-// others poll it with acquire loads.  False if the wait timed out or another CTA already
-// reported an error.
-__device__ bool grid_barrier(unsigned* bar, int* status, unsigned gsize) {
+// Barrier over the gsize CTAs of one system's group: a counter that only grows; every CTA adds one (release) and polls
+// it (acquire) until all arrivals of this and the earlier barriers (target) are in.  (A generation word that the last
+// arrival updates adds an atomic's latency; a flag word per CTA, polled by a warp, costs more in polling traffic:
+// 300 steps of five barriers at dim 6144 took 24.9 and 27.3 ms against 24.3.)  False if the wait timed out or another CTA
+// already reported an error.
+__device__ bool grid_barrier(unsigned* count, unsigned& target, int* status, unsigned gsize) {
   __shared__ int ok;
+  target += gsize;
   __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned* gen = bar + 1;
-    const unsigned g = ld_acquire(gen);
-    const unsigned arrived = atom_add_acq_rel(bar, 1u);
+    red_add_release(count, 1u);
     int good = 1;
-    if (arrived == gsize - 1) {
-      atomicExch(bar, 0u);
-      red_add_release(gen, 1u);
-    } else {
+    if ((int)(ld_acquire(count) - target) < 0) {
       const unsigned long long t0 = globaltimer();
       unsigned it = 0;
-      while (ld_acquire(gen) == g) {
+      while ((int)(ld_acquire(count) - target) < 0) {
         if ((it++ & 31u) == 0) {             // the first poll and every 32nd: a zero limit expires at once
           if (*(volatile int*)status != 0) {
             good = 0;
@@ -90,7 +90,6 @@ __device__ bool grid_barrier(unsigned* bar, int* status, unsigned gsize) {
             break;
           }
         }
-        __nanosleep(32);
       }
     }
     ok = good;
@@ -270,22 +269,22 @@ __device__ __forceinline__ void seg_dot(const float2* __restrict__ Hr, const flo
         }
       }
     }
-    float2 s = make_float2(0.f, 0.f);
-    int cnt = 0;
-    for (; i < n4; i += 32) {
-      const float4 h = __ldcs(h4 + i);
-      const float4 v = x4[i];
-      s.x = fmaf(h.x, v.x, fmaf(-h.y, v.y, s.x));
-      s.y = fmaf(h.x, v.y, fmaf(h.y, v.x, s.y));
-      s.x = fmaf(h.z, v.z, fmaf(-h.w, v.w, s.x));
-      s.y = fmaf(h.z, v.w, fmaf(h.w, v.z, s.y));
-      if (++cnt == 8) {
-        carry(s);
-        s = make_float2(0.f, 0.f);
-        cnt = 0;
-      }
+    for (; i < n4; i += 32 * 8) {           // the rest, eight loads in flight
+      float4 h[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) h[u] = i + 32 * u < n4 ? __ldcs(h4 + i + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (i + 32 * u < n4) {
+          const float4 v = x4[i + 32 * u];
+          s.x = fmaf(h[u].x, v.x, fmaf(-h[u].y, v.y, s.x));
+          s.y = fmaf(h[u].x, v.y, fmaf(h[u].y, v.x, s.y));
+          s.x = fmaf(h[u].z, v.z, fmaf(-h[u].w, v.w, s.x));
+          s.y = fmaf(h[u].z, v.w, fmaf(h[u].w, v.z, s.y));
+        }
+      carry(s);
     }
-    carry(s);
     if ((cols & 1) && lane == 0) {          // odd tail element
       const float2 h = __ldcs(Hr + cols - 1), v = xs[cols - 1];
       carry(make_float2(h.x * v.x - h.y * v.y, h.x * v.y + h.y * v.x));
@@ -304,6 +303,41 @@ __device__ __forceinline__ void seg_dot(const float2* __restrict__ Hr, const flo
       }
     }
     carry(s);
+  }
+}
+
+// Two short rows (fewer than 1024 columns, both 16-byte aligned) at once: sixteen loads in flight instead of eight, every
+// row's sums as in seg_dot.
+__device__ __forceinline__ void seg_dot2(const float2* __restrict__ H0, const float2* __restrict__ H1, const float2* xs,
+                                         int cols, int lane, float2 (&ar)[2], float2 (&ai)[2]) {
+  const float4* x4 = reinterpret_cast<const float4*>(xs);
+  const int n4 = cols >> 1;
+  for (int i = lane; i < n4; i += 32 * 8) {
+    float4 h[2][8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const bool in = i + 32 * u < n4;
+      h[0][u] = in ? __ldcs(reinterpret_cast<const float4*>(H0) + i + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+      h[1][u] = in ? __ldcs(reinterpret_cast<const float4*>(H1) + i + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float2 s[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (i + 32 * u < n4) {
+        const float4 v = x4[i + 32 * u];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          s[k].x = fmaf(h[k][u].x, v.x, fmaf(-h[k][u].y, v.y, s[k].x));
+          s[k].y = fmaf(h[k][u].x, v.y, fmaf(h[k][u].y, v.x, s[k].y));
+          s[k].x = fmaf(h[k][u].z, v.z, fmaf(-h[k][u].w, v.w, s[k].x));
+          s[k].y = fmaf(h[k][u].z, v.w, fmaf(h[k][u].w, v.z, s[k].y));
+        }
+      }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      df_add(ar[k], make_float2(s[k].x, 0.f));
+      df_add(ai[k], make_float2(s[k].y, 0.f));
+    }
   }
 }
 
@@ -327,12 +361,12 @@ struct HayArgs {
   double2* h1;      // [nsteps]
   double2* h2;      // [nsteps]
   double* npart;    // [grid][2]
-  unsigned* bar;    // [2]
+  unsigned* bar;    // [1] barrier arrivals
   int* status;
 };
 
 // hpart[cta][i] = sum over own rows conj(V[i][r]) w[r], i in [0, n) (double-float products).
-// One thread per basis vector walks the CTA's rows with independent, unrolled loads (the rows of
+// One to four threads per basis vector walk the CTA's rows with independent, unrolled loads (the rows of
 // V owned by a CTA are written and read by that CTA only, so plain cached loads are coherent).
 // This CTA's rows of basis vector i: the shared copy for i < vsk (row stride vrows), else global.
 struct BasisRows {
@@ -344,12 +378,20 @@ struct BasisRows {
   }
 };
 
-__device__ void project_partial(const HayArgs& A, const BasisRows& Vb, const float4* wsm, int nrows, int n) {
-  for (int i = threadIdx.x; i < n; i += kThreads) {
-    const float4* Vi = Vb.row(i);
-    float2 sr[4], si[4];                    // four independent chains (rows mod 4) hide the add latency
+// A vector's sum runs in four chains (rows mod 4; the last nrows mod 4 rows go to the first), added in order at the end;
+// T = 1, 2 or 4 threads share the chains of a vector, as many as there are threads for.
+template <int T>
+__device__ __forceinline__ void project_chains(const HayArgs& A, const BasisRows& Vb, const float4* wsm, int nrows, int n) {
+  constexpr int C = 4 / T;                  // chains per thread
+  const int t = threadIdx.x % T;
+  for (int i0 = 0; i0 < n; i0 += kThreads / T) {
+    const int i = i0 + threadIdx.x / T;
+    const bool live = i < n;
+    const float4* Vi = Vb.row(live ? i : 0);
+    const int rows = live ? nrows : 0;
+    float2 sr[C], si[C];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) sr[u] = si[u] = make_float2(0.f, 0.f);
+    for (int u = 0; u < C; ++u) sr[u] = si[u] = make_float2(0.f, 0.f);
     auto mac = [&](float2& ar, float2& ai, float4 v, float4 w) {
       const float2 vr = make_float2(v.x, v.y), vi = make_float2(v.z, v.w);
       const float2 wr = make_float2(w.x, w.y), wi = make_float2(w.z, w.w);
@@ -360,21 +402,47 @@ __device__ void project_partial(const HayArgs& A, const BasisRows& Vb, const flo
       df_mac(ai, df_neg(vi), wr);
     };
     int r = 0;
-    for (; r + 4 <= nrows; r += 4) {
-      float4 v[4];
+    for (; r + 16 <= rows; r += 16) {        // 4 C loads in flight
+      float4 v[4][C];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = Vi[r + u];
+      for (int b = 0; b < 4; ++b)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) mac(sr[u], si[u], v[u], wsm[r + u]);
+        for (int u = 0; u < C; ++u) v[b][u] = Vi[r + 4 * b + t * C + u];
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int u = 0; u < C; ++u) mac(sr[u], si[u], v[b][u], wsm[r + 4 * b + t * C + u]);
     }
-    for (; r < nrows; ++r) mac(sr[0], si[0], Vi[r], wsm[r]);
+    for (; r + 4 <= rows; r += 4)
 #pragma unroll
-    for (int u = 1; u < 4; ++u) {
-      df_add(sr[0], sr[u]);
-      df_add(si[0], si[u]);
+      for (int u = 0; u < C; ++u) mac(sr[u], si[u], Vi[r + t * C + u], wsm[r + t * C + u]);
+    if (t == 0)
+      for (; r < rows; ++r) mac(sr[0], si[0], Vi[r], wsm[r]);
+#pragma unroll
+    for (int u = 1; u < 4; ++u) {            // chain u: thread u / C of the vector, its slot u % C
+      float4 x = make_float4(sr[u % C].x, sr[u % C].y, si[u % C].x, si[u % C].y);
+      if (u / C > 0) {
+        const int src = (int)(threadIdx.x & 31 & ~(T - 1)) + u / C;
+        x = make_float4(__shfl_sync(0xffffffffu, x.x, src), __shfl_sync(0xffffffffu, x.y, src),
+                        __shfl_sync(0xffffffffu, x.z, src), __shfl_sync(0xffffffffu, x.w, src));
+      }
+      if (t == 0) {
+        df_add(sr[0], make_float2(x.x, x.y));
+        df_add(si[0], make_float2(x.z, x.w));
+      }
     }
-    A.hpart[(size_t)A.grank * A.nsteps + i] = cdf_val(make_float4(sr[0].x, sr[0].y, si[0].x, si[0].y));
+    if (live && t == 0)
+      A.hpart[(size_t)A.grank * A.nsteps + i] = cdf_val(make_float4(sr[0].x, sr[0].y, si[0].x, si[0].y));
   }
+}
+
+__device__ void project_partial(const HayArgs& A, const BasisRows& Vb, const float4* wsm, int nrows, int n) {
+  if (4 * n <= kThreads)
+    project_chains<4>(A, Vb, wsm, nrows, n);
+  else if (2 * n <= kThreads)
+    project_chains<2>(A, Vb, wsm, nrows, n);
+  else
+    project_chains<1>(A, Vb, wsm, nrows, n);
 }
 
 // h[i] = sum_cta hpart[cta][i] for the i owned by this CTA (deterministic order, FP64).
@@ -382,10 +450,16 @@ __device__ void reduce_coeffs(const HayArgs& A, double2* h, int n) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int i = A.grank + A.gsize * warp; i < n; i += A.gsize * kWarps) {
     double2 s = make_double2(0.0, 0.0);
-    for (int c = lane; c < A.gsize; c += 32) {
-      const double2 v = __ldcg(A.hpart + (size_t)c * A.nsteps + i);
-      s.x += v.x;
-      s.y += v.y;
+    for (int c0 = lane; c0 < A.gsize; c0 += 32 * 5) {      // five loads in flight
+      double2 v[5];
+#pragma unroll
+      for (int u = 0; u < 5; ++u)
+        v[u] = c0 + 32 * u < A.gsize ? __ldcg(A.hpart + (size_t)(c0 + 32 * u) * A.nsteps + i) : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int u = 0; u < 5; ++u) {
+        s.x += v[u].x;
+        s.y += v[u].y;
+      }
     }
     s = warp_sum(s);
     if (lane == 0) h[i] = s;
@@ -418,6 +492,13 @@ __device__ void subtract_projection(const BasisRows& Vb, float4* wsm, float4* re
       };
       const int rr = rb + r;
       int i = ig;
+      for (; i + 7 * ng < n; i += 8 * ng) {
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = Vb.row(i + u * ng)[rr];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mac(sr[u & 3], si[u & 3], v[u], hs[i + u * ng]);
+      }
       for (; i + 3 * ng < n; i += 4 * ng) {
         float4 v[4];
 #pragma unroll
@@ -436,7 +517,8 @@ __device__ void subtract_projection(const BasisRows& Vb, float4* wsm, float4* re
     __syncthreads();
     if (threadIdx.x < nr) {
       float2 tr = make_float2(0.f, 0.f), ti = make_float2(0.f, 0.f);
-      for (int q = 0; q < ng; ++q) {
+#pragma unroll 8
+      for (int q = 0; q < min(ng, n); ++q) {               // groups past the last vector have nothing
         const float4 t = red[q * nr + threadIdx.x];
         df_add(tr, make_float2(t.x, t.y));
         df_add(ti, make_float2(t.z, t.w));
@@ -477,29 +559,12 @@ __device__ double all_cta_sum(const HayArgs& A, int which, double* red1) {
   return bc;
 }
 
-// both sums of npart[c][0] and npart[c][1] in one pass by warp 0 (identical order in every CTA)
-__device__ double2 all_cta_sum2(const HayArgs& A, double2* red2) {
-  if (threadIdx.x < 32) {
-    double2 v = make_double2(0.0, 0.0);
-    for (int c = threadIdx.x; c < A.gsize; c += 32) {
-      const double2 p = __ldcg(reinterpret_cast<const double2*>(A.npart) + c);
-      v.x += p.x;
-      v.y += p.y;
-    }
-    v = warp_sum(v);
-    if (threadIdx.x == 0) red2[0] = v;
-  }
-  __syncthreads();
-  const double2 t = red2[0];
-  __syncthreads();
-  return t;
-}
-
 constexpr int kMaxBatch = 24;
 
 // One system of a batched launch (pointers into that system's workspace).
 struct HaySys {
   int dim, cta0, ncta;
+  int rows, vsk;        // rows per CTA; basis vectors whose own rows are kept in shared memory
   double prefactor;
   const float2* H;
   const double2* P;
@@ -516,16 +581,15 @@ struct HaySys {
 };
 
 struct HayBatch {
-  int nsys, nsteps, nw, rows_max;   // rows_max: largest rows-per-CTA over the systems
+  int nsys, nsteps, nw;
   int xtile;                        // columns of v_j staged per pass
-  int vsk;                          // basis vectors whose own rows are kept in shared memory
   double eta;
   const double* omega;
   int* status;
   HaySys s[kMaxBatch];
 };
 
-// The CTA's rows of the first B.vsk basis vectors also live in shared memory (they are read only by
+// The CTA's rows of the first vsk basis vectors also live in shared memory (they are read only by
 // this CTA), so most projections and updates read shared memory; the global copy serves the rest
 // and the adjoint.
 __global__ __launch_bounds__(kThreads, 1) void haydock_kernel(const __grid_constant__ HayBatch B) {
@@ -558,20 +622,23 @@ __global__ __launch_bounds__(kThreads, 1) void haydock_kernel(const __grid_const
   A.status = B.status;
   extern __shared__ float4 dyn[];
   float4* wsm = dyn;                                // own rows of w (double-float)
-  float4* hs = dyn + B.rows_max;                    // projection coefficients (double-float)
+  float4* hs = dyn + S.rows;                        // projection coefficients (double-float)
   float2* xs = reinterpret_cast<float2*>(hs + B.nsteps);   // column tile of v_j (FP32)
-  float4* vsm = reinterpret_cast<float4*>(xs + B.xtile);   // [vsk][rows_max] own rows of the first basis vectors
-  if (B.vsk > 0 && (reinterpret_cast<uintptr_t>(vsm) & 15) != 0) {   // float4 rows must be 16-byte aligned
+  float4* vsm = reinterpret_cast<float4*>(xs + B.xtile);   // [vsk][rows] own rows of the first basis vectors
+  if (S.vsk > 0 && (reinterpret_cast<uintptr_t>(vsm) & 15) != 0) {   // float4 rows must be 16-byte aligned
     if (threadIdx.x == 0) atomicCAS(B.status, 0, (int)BSE_ERR_CUDA);
     return;
   }
   __shared__ float4 red[kThreads];
   __shared__ double red1[kWarps];
+  __shared__ double step_out[2];
   const int dim = A.dim;
   const int rows_per = (dim + A.gsize - 1) / A.gsize;
   const int row0 = min(dim, A.grank * rows_per);
   const int nrows = min(dim, row0 + rows_per) - row0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  unsigned arrivals = 0;                    // barrier arrivals so far
 
   // v_0 = P / |P|
   double pp = 0.0;
@@ -581,18 +648,18 @@ __global__ __launch_bounds__(kThreads, 1) void haydock_kernel(const __grid_const
   }
   pp = block_sum(pp, red1);
   if (threadIdx.x == 0) A.npart[2 * A.grank] = pp;
-  if (!grid_barrier(A.bar, A.status, (unsigned)A.gsize)) return;
+  if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
   const double pn2 = all_cta_sum(A, 0, red1);
   const double pinv = 1.0 / sqrt(pn2);
   for (int r = threadIdx.x; r < nrows; r += kThreads) {
     const double2 p = A.P[row0 + r];
     const double2 v = make_double2(p.x * pinv, p.y * pinv);
     A.V[row0 + r] = cdf_split(v);
-    if (B.vsk > 0) vsm[r] = cdf_split(v);
+    if (S.vsk > 0) vsm[r] = cdf_split(v);
     A.vf[row0 + r] = make_float2((float)v.x, (float)v.y);
   }
-  const BasisRows Vb{vsm, A.V + row0, B.vsk, B.rows_max, dim};
-  if (!grid_barrier(A.bar, A.status, (unsigned)A.gsize)) return;
+  const BasisRows Vb{vsm, A.V + row0, S.vsk, S.rows, dim};
+  if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
 
   int done = A.nsteps;
   float vscale = 1.0f;                      // vf holds v_j / vscale: w_j unnormalised, scaled when staged
@@ -607,9 +674,7 @@ __global__ __launch_bounds__(kThreads, 1) void haydock_kernel(const __grid_const
         xs[c] = make_float2(x.x * vscale, x.y * vscale);
       }
       __syncthreads();
-      for (int r = warp; r < nrows; r += kWarps) {
-        float2 ar = make_float2(0.f, 0.f), ai = make_float2(0.f, 0.f);
-        seg_dot(A.H + (size_t)(row0 + r) * dim + col0, xs, cols, lane, ar, ai);
+      auto add_row = [&](int r, float2 ar, float2 ai) {
         const float4 t = cdf_warp_sum(make_float4(ar.x, ar.y, ai.x, ai.y));
         if (lane == 0) {
           const float4 o = wsm[r];
@@ -620,6 +685,20 @@ __global__ __launch_bounds__(kThreads, 1) void haydock_kernel(const __grid_const
           im = df_norm(im);
           wsm[r] = make_float4(re.x, re.y, im.x, im.y);
         }
+      };
+      int r = warp;
+      if (cols < 1024 && ((dim | cols) & 1) == 0 && (reinterpret_cast<uintptr_t>(A.H) & 15) == 0)
+        for (; r + kWarps < nrows; r += 2 * kWarps) {
+          float2 ar[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, ai[2] = {ar[0], ar[0]};
+          const float2* h = A.H + (size_t)(row0 + r) * dim + col0;
+          seg_dot2(h, h + (size_t)kWarps * dim, xs, cols, lane, ar, ai);
+          add_row(r, ar[0], ai[0]);
+          add_row(r + kWarps, ar[1], ai[1]);
+        }
+      for (; r < nrows; r += kWarps) {
+        float2 ar = make_float2(0.f, 0.f), ai = make_float2(0.f, 0.f);
+        seg_dot(A.H + (size_t)(row0 + r) * dim + col0, xs, cols, lane, ar, ai);
+        add_row(r, ar, ai);
       }
     }
     __syncthreads();
@@ -634,14 +713,14 @@ __global__ __launch_bounds__(kThreads, 1) void haydock_kernel(const __grid_const
       if (lane == 0) A.npart[2 * A.grank + 1] = hv2;
     }
     project_partial(A, Vb, wsm, nrows, j + 1);
-    if (!grid_barrier(A.bar, A.status, (unsigned)A.gsize)) return;
+    if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
     reduce_coeffs(A, A.h1, j + 1);
-    if (!grid_barrier(A.bar, A.status, (unsigned)A.gsize)) return;
+    if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
     subtract_projection(Vb, wsm, red, hs, A.h1, nrows, j + 1);
     project_partial(A, Vb, wsm, nrows, j + 1);
-    if (!grid_barrier(A.bar, A.status, (unsigned)A.gsize)) return;
+    if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
     reduce_coeffs(A, A.h2, j + 1);
-    if (!grid_barrier(A.bar, A.status, (unsigned)A.gsize)) return;
+    if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
     subtract_projection(Vb, wsm, red, hs, A.h2, nrows, j + 1);
     for (int r = threadIdx.x; r < nrows; r += kThreads) {     // published unnormalised
       const float4 w = wsm[r];
@@ -657,35 +736,55 @@ __global__ __launch_bounds__(kThreads, 1) void haydock_kernel(const __grid_const
       for (int o = 16; o > 0; o >>= 1) ww += __shfl_xor_sync(0xffffffffu, ww, o);
       if (lane == 0) A.npart[2 * A.grank] = ww;
     }
-    if (!grid_barrier(A.bar, A.status, (unsigned)A.gsize)) return;
-    const double2 sums = all_cta_sum2(A, reinterpret_cast<double2*>(red));
-    const double bn2 = sums.x, sc2 = sums.y;
-    const double2 c1 = __ldcg(A.h1 + j), c2 = __ldcg(A.h2 + j);
-    const double aj = c1.x + c2.x;
-    const double bn = sqrt(bn2);
+    if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
+    // norms, coefficients and the breakdown test in FP64 by one warp: by every thread the square roots and the division
+    // took ~10 us a step (FP64 issues at two lanes a cycle)
     const bool last = (j + 1 == A.nsteps);
-    const bool brk = !last && !(bn > kBreakdownRel * sqrt(sc2));
-    if (A.grank == 0 && threadIdx.x == 0) {
-      A.ab[j] = aj;
-      if (j == 0) A.ab[A.nsteps] = 0.0;
-      if (!last) A.ab[A.nsteps + j + 1] = brk ? 0.0 : bn;
+    if (warp == 0) {
+      double2 v = make_double2(0.0, 0.0);
+      for (int c0 = lane; c0 < A.gsize; c0 += 32 * 5) {
+        double2 p[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+          p[u] = c0 + 32 * u < A.gsize ? __ldcg(reinterpret_cast<const double2*>(A.npart) + c0 + 32 * u)
+                                       : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int u = 0; u < 5; ++u) {
+          v.x += p[u].x;
+          v.y += p[u].y;
+        }
+      }
+      v = warp_sum(v);
+      if (lane == 0) {
+        const double bn = sqrt(v.x);
+        const bool stop = !last && !(v.x > kBreakdownRel * kBreakdownRel * v.y);
+        step_out[0] = 1.0 / bn;
+        step_out[1] = stop ? 1.0 : 0.0;
+        if (A.grank == 0) {
+          A.ab[j] = __ldcg(A.h1 + j).x + __ldcg(A.h2 + j).x;
+          if (j == 0) A.ab[A.nsteps] = 0.0;
+          if (!last) A.ab[A.nsteps + j + 1] = stop ? 0.0 : bn;
+        }
+      }
     }
+    __syncthreads();
+    const double binv = step_out[0];
+    const bool brk = step_out[1] != 0.0;
     if (last) break;
     if (brk) {
       done = j + 1;
       break;
     }
-    const double binv = 1.0 / bn;
     float4* Vn = A.V + (size_t)(j + 1) * dim + row0;   // own rows only: no grid barrier needed
     for (int r = threadIdx.x; r < nrows; r += kThreads) {
       const double2 w = cdf_val(wsm[r]);
       const float4 v = cdf_split(make_double2(w.x * binv, w.y * binv));
       Vn[r] = v;
-      if (j + 1 < B.vsk) vsm[(size_t)(j + 1) * B.rows_max + r] = v;
+      if (j + 1 < S.vsk) vsm[(size_t)(j + 1) * S.rows + r] = v;
     }
     vscale = (float)binv;
   }
-  if (!grid_barrier(A.bar, A.status, (unsigned)A.gsize)) return;
+  if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
   if (A.grank == 0 && threadIdx.x == 0) *A.steps_done = done;
   // continued fraction from the bottom: g = 1/(z - a_j - b_{j+1}^2 g)
   const double C = A.prefactor * pn2;
@@ -773,7 +872,6 @@ int run_haydock_batch(const HayJob* jobs, int n, int nsteps, const double* omega
   B.eta = eta;
   B.omega = omega;
   B.status = status;
-  B.rows_max = 0;
   int cta = 0;
   for (int i = 0; i < n; ++i) {
     const DevSys& d = *jobs[i].d;
@@ -797,21 +895,23 @@ int run_haydock_batch(const HayJob* jobs, int n, int nsteps, const double* omega
     S.h2 = (double2*)(base + L.h2);
     S.npart = (double*)(base + L.npart);
     S.bar = (unsigned*)(base + L.bar);
-    const int rows = (d.dim + ncta[i] - 1) / ncta[i];
-    if (rows > B.rows_max) B.rows_max = rows;
-    const int e = (int)cudaMemsetAsync(S.bar, 0, 2 * sizeof(unsigned), st);
+    S.rows = (d.dim + ncta[i] - 1) / ncta[i];
+    const int e = (int)cudaMemsetAsync(S.bar, 0, sizeof(unsigned), st);
     if (e) return e;
   }
   // x tile of up to 8192 columns, then as many basis vectors' own rows in shared memory as fit
   int dim_max = 0;
   for (int i = 0; i < n; ++i) dim_max = jobs[i].d->dim > dim_max ? jobs[i].d->dim : dim_max;
   B.xtile = dim_max < kXTile ? (dim_max + 1) / 2 * 2 : kXTile;   // even: the basis rows after it stay 16-byte aligned
-  const size_t fixed = ((size_t)B.rows_max + (size_t)nsteps) * sizeof(float4) + (size_t)B.xtile * sizeof(float2);
-  if (fixed > kDynMax || fixed % sizeof(float4) != 0) return -1;
-  const size_t per_vec = (size_t)B.rows_max * sizeof(float4);
-  const size_t fit = (kDynMax - fixed) / per_vec;
-  B.vsk = (int)(fit < (size_t)nsteps ? fit : (size_t)nsteps);
-  const size_t dyn = fixed + (size_t)B.vsk * per_vec;
+  size_t dyn = 0;
+  for (int i = 0; i < n; ++i) {
+    HaySys& S = B.s[i];
+    const size_t fixed = ((size_t)S.rows + (size_t)nsteps) * sizeof(float4) + (size_t)B.xtile * sizeof(float2);
+    if (fixed > kDynMax || fixed % sizeof(float4) != 0) return -1;
+    const size_t per_vec = (size_t)S.rows * sizeof(float4), fit = (kDynMax - fixed) / per_vec;
+    S.vsk = (int)(fit < (size_t)nsteps ? fit : (size_t)nsteps);
+    if (fixed + (size_t)S.vsk * per_vec > dyn) dyn = fixed + (size_t)S.vsk * per_vec;
+  }
   cudaFuncSetAttribute((const void*)haydock_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, haydock_kernel, kThreads, dyn);
   if (occ < 1) return -1;
