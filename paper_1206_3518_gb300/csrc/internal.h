@@ -87,7 +87,7 @@ int launch_dipole(const DevSys& d, const void* coef, const double* energies, dou
 int launch_pair_chi0(const DevSys& d, const void* u, void* rho, int q_begin, int q_end, int* status, void* stream);
 size_t screen_ws_bytes(const DevSys& d, long long qchunk);
 int launch_screening(const DevSys& d, void* rho_chi, const double* energies, const void* P, int q_begin, int q_end,
-                     int iterations, void* W, float* residual, void* ws, double gap_floor, void* stream);
+                     int iterations, void* W, float* residual, void* ws, double gap_floor, int* status, void* stream);
 int pair_supported(const DevSys& d);
 size_t pair_ws_bytes(const DevSys& d);
 int gcorr_valid(const DevSys& d);

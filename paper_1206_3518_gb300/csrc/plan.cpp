@@ -1096,7 +1096,7 @@ bse_status bse_screening(bse_plan* plan, int s, void* rho_chi, const double* ene
   if ((st = scan_input(plan, energies, (long long)d.nkpt * d.nb, 8, stream)) != BSE_OK) return st;
   if (q_begin == 0 && (st = scan_input(plan, P, 2LL * d.dim, 8, stream)) != BSE_OK) return st;
   return cuda_check(launch_screening(d, rho_chi, energies, P, q_begin, q_end, iterations, W, residual, ws,
-                                     sp.sys.gap_floor, stream),
+                                     sp.sys.gap_floor, plan->d_status, stream),
                     "screening");
 }
 

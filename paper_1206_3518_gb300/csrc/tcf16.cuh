@@ -19,6 +19,9 @@
 // (umma.cuh).  Rows past the operand's last row are not written: they only reach accumulator rows or columns
 // that are not stored.  K past the operand's length is zero.
 //
+// Real products (Op::kReal) use the same pipeline: 128-byte rows of 64 real K, B tiles of up to 256 rows, 12 MMAs of
+// M128 N256 K16 per chunk into one accumulator of 256 columns, two stages.
+//
 // gemm_kernel is persistent (one CTA per SM, static round-robin over tiles): warps 0-7 promote and store (two
 // warps per TMEM lane quarter, 64 columns each), warp 8 brings the images with bulk copies into a 3-stage
 // ring, warp 9 issues the 24 MMAs of a chunk.  M128 x N <= 128: 64 KB per stage, two accumulators of 256 TMEM
@@ -46,10 +49,13 @@ constexpr int kStage = 2 * kTileA + 2 * kNMax * umma::kRow;
 constexpr int kEpiWarps = 8, kProdWarp = 8, kMmaWarp = 9;
 constexpr int kThreads = (kMmaWarp + 1) * 32;
 constexpr int kAccCols = 256;                  // one accumulator: Re [0, 128), Im [128, 256)
+constexpr int kRealK = 64, kRealN = 256;        // real products: K per chunk, rows of a B tile at most
+constexpr int kRealStages = 2;
+static_assert(kRealStages * (2 * kTileA + 2 * kRealN * umma::kRow) <= kStages * kStage, "ring");
 constexpr int kXpose = 32 * 16 * 8;            // one epilogue warp's 32 x 16 complex outputs on their way out
 constexpr size_t kSmem = (size_t)kStages * kStage + kEpiWarps * kXpose + 1024 + 256;
 
-// One output tile: images of its first K chunk, bytes from chunk to chunk, complex K, B rows (a multiple of
+// One output tile: images of its first K chunk, bytes from chunk to chunk, K (complex, or real), B rows (a multiple of
 // 16) and what the epilogue needs (origin of the tile, valid rows and columns, batch index).
 struct Tile {
   const unsigned char *a, *b;
@@ -190,7 +196,19 @@ __device__ __forceinline__ void chunk_mmas(uint32_t d_re, uint32_t d_im, uint64_
   }
 }
 
-// The same with the A planes in tensor memory at columns a + 0 (Re hi), a + 8 (Im hi), a + 16 (Re lo), a + 24 (Im lo) of
+// The 3 nkk MMAs of one chunk of a real product.
+__device__ __forceinline__ void chunk_mmas_real(uint32_t d, uint64_t da, uint32_t a_lo, uint64_t db, uint32_t b_lo, int nkk,
+                                                uint32_t idesc) {
+#pragma unroll
+  for (int s = 0; s < 3; ++s)                    // hi.lo, lo.hi, hi.hi
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk)
+      if (kk < nkk)
+        umma::mma_bf16(d, da + (s == 1 ? a_lo : 0u) + (uint32_t)kk * 2u, db + (s == 0 ? b_lo : 0u) + (uint32_t)kk * 2u,
+                       idesc, (s | kk) != 0 ? 1u : 0u);
+}
+
+// The MMAs of a complex chunk with the A planes in tensor memory at columns a + 0 (Re hi), a + 8 (Im hi), a + 16 (Re lo), a + 24 (Im lo) of
 // the first K16 half, + 32 of the second (two FP16 per 32-bit column, lane = row); A as it is (no conjugation).
 template <int NKK>
 __device__ __forceinline__ void chunk_mmas_ts(uint32_t d_re, uint32_t d_im, uint32_t a, uint64_t db, uint32_t b_lo,
@@ -217,17 +235,21 @@ __device__ __forceinline__ void fail_now(volatile int* fail, int* status) {
   atomicCAS(status, 0, (int)BSE_ERR_TIMEOUT);
 }
 
-// Op: long long ntiles; int* status; static constexpr bool kConj; bool tile(long long t, Tile&) (false: nothing
+// Op: long long ntiles; int* status; static constexpr bool kReal, kConj, kHerm (tiles m0 <= n0
+// of a Hermitian result: the upper triangle is stored with its mirror image, float2* mirror_out(...)); bool tile(long long t, Tile&) (false: nothing
 // to do); float2* row_out(const Tile&, int row) the address of column 0 of a row of the tile; float row_scale(const
 // Tile&, int row), col_scale(const Tile&, int col) the inverse scales; float2 value(const Tile&, int row, int col,
-// float2 sum) the output from the unscaled sum.  Outputs go out through shared memory, 16 columns
+// float2 sum) the output from the unscaled sum (real: float* row_out, no value()).  Outputs go out through shared memory, 16 columns
 // at a time, so that eight lanes write 128 contiguous bytes of a row (rows stored lane by lane cost 2.8 times the
 // time of the whole product at 115 columns: 294 us against 106 us without stores).
 template <class Op>
 __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant__ Op op) {
+  constexpr bool R = Op::kReal;
+  constexpr int kChunk = R ? kRealK : kTKC, kRing = R ? kRealStages : kStages;
+  constexpr int kStageB = 2 * kTileA + 2 * (R ? kRealN : kNMax) * umma::kRow;
   extern __shared__ __align__(1024) unsigned char tcf_smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)tcf_smem_raw + 1023) & ~(uintptr_t)1023);
-  unsigned char* xpose = sm + kStages * kStage;
+  unsigned char* xpose = sm + kStages * kStage;   // after the ring (the larger of the two)
   uint64_t* full = (uint64_t*)(xpose + kEpiWarps * kXpose);   // [3] stage landed
   uint64_t* empty = full + kStages;                       // [3] MMAs done with the stage
   uint64_t* tfull = empty + kStages;                      // [2] accumulator holds a chunk
@@ -247,7 +269,7 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 32) {
-    for (int i = 0; i < kStages; ++i) {
+    for (int i = 0; i < kRing; ++i) {
       umma::mbar_init(smem_u32(full + i), 1);
       umma::mbar_init(smem_u32(empty + i), 1);
     }
@@ -272,16 +294,16 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
       Tile t;
       for (long long ti = blockIdx.x; ti < op.ntiles && !*fail; ti += gridDim.x) {
         if (!op.tile(ti, t)) continue;
-        const int nch = (t.K + kTKC - 1) / kTKC;
+        const int nch = (t.K + kChunk - 1) / kChunk;
         const uint32_t bbytes = (uint32_t)(2 * t.n * umma::kRow);
         for (int kc = 0; kc < nch; ++kc, ++c) {
-          const int st = (int)(c % kStages);
-          if (c >= kStages && !umma::mbar_wait(smem_u32(empty + st), ((c / kStages) - 1) & 1u)) {
+          const int st = (int)(c % kRing);
+          if (c >= kRing && !umma::mbar_wait(smem_u32(empty + st), ((c / kRing) - 1) & 1u)) {
             fail_now(fail, op.status);
             break;
           }
           if (*fail) break;
-          const uint32_t base = smem_u32(sm + st * kStage);
+          const uint32_t base = smem_u32(sm + st * kStageB);
           umma::mbar_arrive_expect_tx(smem_u32(full + st), (uint32_t)(2 * kTileA) + bbytes);
           umma::bulk_g2s(base, t.a + (size_t)kc * t.a_step, 2 * kTileA, smem_u32(full + st));
           umma::bulk_g2s(base + 2 * kTileA, t.b + (size_t)kc * t.b_step, bbytes, smem_u32(full + st));
@@ -297,21 +319,23 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
     bool ok = true;
     for (long long ti = blockIdx.x; ti < op.ntiles && ok; ti += gridDim.x) {
       if (!op.tile(ti, t)) continue;
-      const int K = umma::uniform(t.K), n = umma::uniform(t.n), nch = (K + kTKC - 1) / kTKC;
+      const int K = umma::uniform(t.K), n = umma::uniform(t.n), nch = (K + kChunk - 1) / kChunk;
       const uint32_t idesc = idesc_f16(n), b_lo = (uint32_t)(n * umma::kRow) >> 4;
       for (int kc = 0; kc < nch; ++kc, ++c) {
-        const int st = (int)(c % kStages), buf = (int)(c & 1u);
+        const int st = (int)(c % kRing), buf = (int)(c & 1u);
         ok = umma::uniform((c < 2 || umma::mbar_wait(smem_u32(tempty + buf), ((c >> 1) - 1) & 1u)) &&
-                           umma::mbar_wait(smem_u32(full + st), (c / kStages) & 1u) && !*fail);
+                           umma::mbar_wait(smem_u32(full + st), (c / kRing) & 1u) && !*fail);
         if (!ok) {
           if (leader) fail_now(fail, op.status);
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t da = d0 + (uint64_t)((st * kStage) >> 4), db = da + (uint64_t)((2 * kTileA) >> 4);
+        const uint64_t da = d0 + (uint64_t)((st * kStageB) >> 4), db = da + (uint64_t)((2 * kTileA) >> 4);
         const uint32_t d_re = umma::uniform(tmem + (uint32_t)(buf * kAccCols));
         if (leader) {
-          if (K - kc * kTKC > 16)
+          if (R)
+            chunk_mmas_real(d_re, da, (uint32_t)(kTileA >> 4), db, b_lo, (K - kc * kChunk + 15) / 16, idesc);
+          else if (K - kc * kTKC > 16)
             chunk_mmas<Op::kConj, 2>(d_re, d_re + 128u, da, (uint32_t)(kTileA >> 4), db, b_lo, idesc);
           else
             chunk_mmas<Op::kConj, 1>(d_re, d_re + 128u, da, (uint32_t)(kTileA >> 4), db, b_lo, idesc);
@@ -335,7 +359,7 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
     bool ok = true;
     for (long long ti = blockIdx.x; ti < op.ntiles && ok; ti += gridDim.x) {
       if (!op.tile(ti, t)) continue;
-      const int nch = (t.K + kTKC - 1) / kTKC;
+      const int nch = (t.K + kChunk - 1) / kChunk;
       float re[4][16], im[4][16];
 #pragma unroll
       for (int g = 0; g < 4; ++g)
@@ -357,7 +381,7 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
         const uint32_t base = lane_addr + (uint32_t)(buf * kAccCols);
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-          if (c0 + 16 * g >= t.n) break;
+          if (!R && c0 + 16 * g >= t.n) break;
           uint32_t v[16];
           umma::tmem_ld16(base + 16u * g, v);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -376,6 +400,39 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
         unsigned char* xp = xpose + warp * kXpose;
         const int row = (warp & 3) * 32 + lane;
         const float sa = row < t.mvalid ? op.row_scale(t, row) : 0.f;
+        if constexpr (R) {                         // columns c0 + 16 g.. (re) and 128 + c0 + 16 g.. (im), 16 at a time
+#pragma unroll
+          for (int g = 0; g < 8; ++g) {
+            const int cb = (g < 4 ? 0 : 128) + c0 + 16 * (g & 3);
+            if (cb >= t.nvalid) continue;
+            const float(&v)[16] = g < 4 ? re[g & 3] : im[g & 3];
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              *reinterpret_cast<float4*>(xp + lane * 64 + ((i ^ ((lane >> 1) & 3)) << 4)) =
+                  make_float4(v[4 * i] * sa, v[4 * i + 1] * sa, v[4 * i + 2] * sa, v[4 * i + 3] * sa);
+            __syncwarp();
+            const int j = lane & 3, col = cb + 4 * j;
+            float s[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s[i] = col + i < t.nvalid ? op.col_scale(t, col + i) : 0.f;
+#pragma unroll 2
+            for (int r8 = 0; r8 < 4; ++r8) {
+              const int rl = r8 * 8 + (lane >> 2), ro = (warp & 3) * 32 + rl;
+              if (ro >= t.mvalid || col >= t.nvalid) continue;
+              const float4 u = *reinterpret_cast<const float4*>(xp + rl * 64 + ((j ^ ((rl >> 1) & 3)) << 4));
+              float* out = op.row_out(t, ro) + col;
+              const float w[4] = {u.x * s[0], u.y * s[1], u.z * s[2], u.w * s[3]};
+              if (col + 3 < t.nvalid && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+                *reinterpret_cast<float4*>(out) = make_float4(w[0], w[1], w[2], w[3]);
+              } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                  if (col + i < t.nvalid) out[i] = w[i];
+              }
+            }
+          }
+        } else {
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
           if (c0 + 16 * g >= t.nvalid) break;
@@ -394,6 +451,17 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
             if (ro >= t.mvalid || col >= t.nvalid) continue;
             const float4 v = *reinterpret_cast<const float4*>(xp + rl * 128 + ((j ^ (rl & 7)) << 4));
             float2* out = op.row_out(t, ro) + col;
+            if constexpr (Op::kHerm) {             // upper triangle, and its mirror image
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                if (col + i >= t.nvalid || t.m0 + ro > t.n0 + col + i) continue;
+                float2 y = op.value(t, ro, col + i, i ? make_float2(v.z * s1, v.w * s1) : make_float2(v.x * s0, v.y * s0));
+                if (t.m0 + ro == t.n0 + col + i) y.y = 0.f;
+                out[i] = y;
+                if (t.m0 + ro != t.n0 + col + i) *op.mirror_out(t, ro, col + i) = make_float2(y.x, -y.y);
+              }
+              continue;
+            }
             const float2 y0 = op.value(t, ro, col, make_float2(v.x * s0, v.y * s0));
             if (col + 1 < t.nvalid) {
               const float2 y1 = op.value(t, ro, col + 1, make_float2(v.z * s1, v.w * s1));
@@ -408,6 +476,7 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
             }
           }
         }
+        }
       }
     }
   }
@@ -415,7 +484,7 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
   __syncthreads();
   if (tid == 0) {                                  // copies still in flight after a failure
     for (unsigned c = *consumed; c < *issued; ++c)
-      if (!umma::mbar_wait(smem_u32(full + c % kStages), (c / kStages) & 1u)) break;
+      if (!umma::mbar_wait(smem_u32(full + c % kRing), (c / kRing) & 1u)) break;
   }
   __syncthreads();
   if (warp == 0) {

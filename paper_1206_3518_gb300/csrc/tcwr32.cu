@@ -81,7 +81,7 @@ int launch_split(const DevSys& d, const void* rho, const void* W, unsigned char*
 }
 
 struct WrOp {
-  static constexpr bool kConj = false;
+  static constexpr bool kReal = false, kConj = false, kHerm = false;
   DevSys d;
   WrGeo g;
   const unsigned char *As, *Bs;

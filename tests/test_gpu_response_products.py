@@ -1,0 +1,59 @@
+"""Products of the TDDFT response and of the screening on the tensor cores, and the blocked Dyson elimination, at the
+sizes where their tiles end: fewer transitions than a K chunk, frequencies on both sides of a 32-row tile of
+weights and of a 128-frequency group, spheres below one panel and with a ragged last one, more q than one group.
+
+Bound of chi~0 per entry, from the arithmetic, relative to the sum of the magnitudes of its terms: the weights, a and T are
+rounded to FP32 (5 x 2^-24), the split products are within 2^-21, each chunk of 64 adds at most 12 truncations of 2^-23
+and the promotion 2^-24 per chunk.
+"""
+import numpy as np
+import pytest
+
+from synth import SystemSpec
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def bse():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__ as ge
+    ge.build()
+    from paper_1206_3518_gb300 import bse as b
+    return b
+
+
+def _dev(x, dtype):
+    return torch.as_tensor(np.ascontiguousarray(x)).to(device="cuda", dtype=dtype)
+
+
+def _ws(bse, plan, kind, arg=0):
+    return torch.empty(bse.bse_workspace_size(plan, 0, kind, arg) // 8 + 1, dtype=torch.complex64, device="cuda")
+
+
+def _spec(n, nv, nc, ecut, grid):
+    return SystemSpec("cell", "fcc", 10.0, 0.0, (n, n, n), nv, nc, ecut, (grid,) * 3, "3d")
+
+
+def test_screening_range_equals_single_points(bse):
+    """W of a range (more q than one group of split images) is W of each q on its own, bit for bit."""
+    spec = _spec(4, 1, 2, 2.0, 24)
+    plan = bse.Plan([spec])
+    inf = plan.info(0)
+    nq, K, ng = inf["nq"], inf["dim"], inf["ng_max"]
+    rng = np.random.default_rng(1)
+    en = _dev(np.sort(rng.uniform(-0.3, 0.4, (inf["nkpt"], 3)), axis=1), torch.float64)
+    P = _dev(rng.standard_normal(K) + 1j * rng.standard_normal(K), torch.complex128)
+    rho = _dev(0.1 * (rng.standard_normal((nq * K, ng)) + 1j * rng.standard_normal((nq * K, ng))), torch.complex64)
+    W, W1 = [torch.zeros(nq, ng, ng, dtype=torch.complex64, device="cuda") for _ in range(2)]
+    res = torch.zeros(nq, device="cuda")
+    bse.bse_screening(plan, 0, rho.clone(), en, P, 0, nq, 12, W, res, _ws(bse, plan, bse.BSE_WS_SCREEN, nq))
+    for q in (0, 1, 31, 32, 33, nq - 1):
+        one = rho[q * K:(q + 1) * K].clone()
+        bse.bse_screening(plan, 0, one, en, P, q, q + 1, 12, W1, None, _ws(bse, plan, bse.BSE_WS_SCREEN, 1))
+        bse.bse_status_read(plan)
+        assert torch.equal(W1[q], W[q]), q
+    assert float(res.max()) < 1e-4
+    assert torch.equal(W, W.mH)
