@@ -154,7 +154,7 @@ int launch_nonfinite_scan(const void* p, long long n, int elem_bytes, int* statu
 // Macroscopic dielectric function from TDDFT with local fields (tddft.cu).
 size_t chi0_ws_bytes(const DevSys& d);
 int launch_chi0_optical(const DevSys& d, const void* rho_x, const void* P, const double* energies, double delta,
-                        const double* omega, int nw, double eta, void* chi0, void* ws, void* stream);
+                        const double* omega, int nw, double eta, void* chi0, void* ws, int* status, void* stream);
 size_t alda_ws_bytes(const DevSys& d);
 int launch_alda_kernel(const DevSys& d, const void* pair_ws, const int* m, void* F, void* ws, void* stream);
 size_t epsm_ws_bytes(const DevSys& d, long long nw);

@@ -1188,7 +1188,8 @@ bse_status bse_chi0_optical(bse_plan* plan, int s, const void* rho_x, const void
   if ((st = scan_input(plan, P, 2LL * d.dim, 8, stream)) != BSE_OK) return st;
   if ((st = scan_input(plan, energies, (long long)d.nkpt * d.nb, 8, stream)) != BSE_OK) return st;
   if ((st = scan_input(plan, omega, nw, 8, stream)) != BSE_OK) return st;
-  return cuda_check(launch_chi0_optical(d, rho_x, P, energies, delta, omega, nw, eta, chi0, ws, stream), "chi0");
+  return cuda_check(launch_chi0_optical(d, rho_x, P, energies, delta, omega, nw, eta, chi0, ws, plan->d_status, stream),
+                    "chi0");
 }
 
 bse_status bse_xc_kernel_alda(bse_plan* plan, int s, const void* pair_ws, size_t pair_bytes, void* F, void* ws,

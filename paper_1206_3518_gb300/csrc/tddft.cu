@@ -11,9 +11,7 @@
 // f_xc(r) = d^2(n eps_xc)/dn^2 at the density n(r) = 2/(Omega Nk) sum_{k,v} |u_vk(r)|^2 (Slater
 // exchange + Perdew-Zunger correlation), F_GG' = |G| f_xc(G - G') |G'|/(4 pi).
 //
-// Kernels: a_S, abar_S and de_S from rho_x, P and the energies; chi~0(w) as a weighted complex Gram
-// product per frequency (64 x 64 output tiles, 16 transitions per shared-memory stage, FP32); the
-// density, f_xc(r) and its transform onto the difference box of the sphere (three separable direct
+// Kernels (chi~0(w) itself is built in tcchi0.cu): the density, f_xc(r) and its transform onto the difference box of the sphere (three separable direct
 // DFT passes in FP64); the batched Dyson solve: M = I - chi~0 (I + F) augmented with chi~0 e_0, Gaussian
 // elimination with partial pivoting and back substitution, one CTA per frequency (FP32 matrix, FP64
 // result).  No device-side waits; capturable.
@@ -30,106 +28,6 @@ constexpr int kT = 64;            // output tile (G x G')
 constexpr int kKC = 16;           // transitions per shared-memory stage
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-
-// a, abar [dim][ng0] and de [dim]
-__global__ void optical_pairs_kernel(DevSys d, const float2* __restrict__ rho_x, const double2* __restrict__ P,
-                                     const double* __restrict__ e, double delta, float2* __restrict__ a,
-                                     float2* __restrict__ ab, double* __restrict__ de) {
-  const long long n = (long long)d.dim * d.ng0;
-  const float s4pi = 3.5449077018110318f;   // sqrt(4 pi)
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int S = (int)(i / d.ng0), g = (int)(i - (long long)S * d.ng0);
-    float2 x, y;
-    if (g == 0) {
-      const double2 p = P[S];
-      x = make_float2(s4pi * (float)p.x, -s4pi * (float)p.y);
-      y = make_float2(-s4pi * (float)p.x, -s4pi * (float)p.y);
-    } else {
-      const float vs = d.vsq[g];                                   // q = 0 row: sqrt(4 pi)/|G|
-      const float2 r = rho_x[(size_t)S * d.ng_max + g];
-      const float2 rm = rho_x[(size_t)S * d.ng_max + d.gminus0[g]];
-      x = make_float2(vs * r.x, vs * r.y);
-      y = make_float2(vs * rm.x, -vs * rm.y);
-    }
-    a[i] = x;
-    ab[i] = y;
-    if (g == 0) {
-      const int nvc = d.nv * d.nc, k = S / nvc, v = (S / d.nc) % d.nv, c = S % d.nc;
-      de[S] = e[(size_t)k * d.nb + d.nv + c] + delta - e[(size_t)k * d.nb + v];
-    }
-  }
-}
-
-// chi[w][G][G'] for the frequencies of the launch (blockIdx.z); 256 threads, 4 x 4 outputs each
-__global__ void __launch_bounds__(256) chi0_kernel(int dim, int ng, const float2* __restrict__ a,
-                                                   const float2* __restrict__ ab, const double* __restrict__ de,
-                                                   const double* __restrict__ omega, double eta, double pref,
-                                                   float2* __restrict__ chi) {
-  __shared__ float2 sa[kKC][kT], sap[kKC][kT], sb[kKC][kT], sbp[kKC][kT];
-  __shared__ float2 r[kKC], rb[kKC];
-  const int w = blockIdx.z;
-  const int g0 = blockIdx.y * kT, h0 = blockIdx.x * kT;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const double om = omega[w];
-  float2 acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
-  for (int s0 = 0; s0 < dim; s0 += kKC) {
-    for (int t = threadIdx.x; t < kKC * kT; t += 256) {
-      const int kk = t / kT, c = t - kk * kT, S = s0 + kk;
-      const bool sv = S < dim;
-      sa[kk][c] = (sv && g0 + c < ng) ? a[(size_t)S * ng + g0 + c] : make_float2(0.f, 0.f);
-      sb[kk][c] = (sv && g0 + c < ng) ? ab[(size_t)S * ng + g0 + c] : make_float2(0.f, 0.f);
-      sap[kk][c] = (sv && h0 + c < ng) ? a[(size_t)S * ng + h0 + c] : make_float2(0.f, 0.f);
-      sbp[kk][c] = (sv && h0 + c < ng) ? ab[(size_t)S * ng + h0 + c] : make_float2(0.f, 0.f);
-    }
-    if (threadIdx.x < kKC) {
-      const int S = s0 + threadIdx.x;
-      float2 x = make_float2(0.f, 0.f), y = make_float2(0.f, 0.f);
-      if (S < dim) {
-        const double u = om - de[S], v = om + de[S];
-        const double du = u * u + eta * eta, dv = v * v + eta * eta;
-        x = make_float2((float)(u / du), (float)(-eta / du));          // 1/(w - de + i eta)
-        y = make_float2((float)(-v / dv), (float)(eta / dv));          // -1/(w + de + i eta)
-      }
-      r[threadIdx.x] = x;
-      rb[threadIdx.x] = y;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < kKC; ++kk) {
-      float2 x[4], xb[4], y[4], yb[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        x[i] = cmul(sa[kk][ty * 4 + i], r[kk]);
-        xb[i] = cmul(sb[kk][ty * 4 + i], rb[kk]);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        y[j] = sap[kk][tx * 4 + j];
-        yb[j] = sbp[kk][tx * 4 + j];
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {                                  // x conj(y) + xb conj(yb)
-          acc[i][j].x += x[i].x * y[j].x + x[i].y * y[j].y + xb[i].x * yb[j].x + xb[i].y * yb[j].y;
-          acc[i][j].y += x[i].y * y[j].x - x[i].x * y[j].y + xb[i].y * yb[j].x - xb[i].x * yb[j].y;
-        }
-    }
-    __syncthreads();
-  }
-  const float p = (float)pref;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int g = g0 + ty * 4 + i, h = h0 + tx * 4 + j;
-      if (g < ng && h < ng) chi[((size_t)w * ng + g) * ng + h] = make_float2(p * acc[i][j].x, p * acc[i][j].y);
-    }
-}
 
 // C[w] = A[w] B for n x n complex matrices (B shared), 64 x 64 tiles
 __global__ void __launch_bounds__(256) batched_gemm_kernel(int n, const float2* __restrict__ A,
@@ -400,32 +298,6 @@ unsigned blocks_for(long long n, int threads) {
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
-
-size_t chi0_ws_bytes(const DevSys& d) {
-  return 2 * align256((size_t)d.dim * d.ng0 * sizeof(float2)) + align256((size_t)d.dim * sizeof(double));
-}
-
-int launch_chi0_optical(const DevSys& d, const void* rho_x, const void* P, const double* energies, double delta,
-                        const double* omega, int nw, double eta, void* chi0, void* ws, void* stream) {
-  cudaStream_t st = (cudaStream_t)stream;
-  char* base = (char*)ws;
-  float2* a = (float2*)base;
-  float2* ab = (float2*)(base + align256((size_t)d.dim * d.ng0 * sizeof(float2)));
-  double* de = (double*)(base + 2 * align256((size_t)d.dim * d.ng0 * sizeof(float2)));
-  optical_pairs_kernel<<<blocks_for((long long)d.dim * d.ng0, 256), 256, 0, st>>>(
-      d, (const float2*)rho_x, (const double2*)P, energies, delta, a, ab, de);
-  if (int e = (int)cudaGetLastError()) return e;
-  if (nw <= 0) return 0;
-  const int nt = (d.ng0 + kT - 1) / kT;
-  for (int w0 = 0; w0 < nw; w0 += 65535) {
-    const int nwc = nw - w0 < 65535 ? nw - w0 : 65535;
-    dim3 grid(nt, nt, nwc);
-    chi0_kernel<<<grid, 256, 0, st>>>(d.dim, d.ng0, a, ab, de, omega + w0, eta, 2.0 * d.norm,
-                                      (float2*)chi0 + (size_t)w0 * d.ng0 * d.ng0);
-    if (int e = (int)cudaGetLastError()) return e;
-  }
-  return 0;
-}
 
 size_t alda_ws_bytes(const DevSys& d) {
   const size_t nr = (size_t)d.n1 * d.n2 * d.n3;

@@ -37,6 +37,45 @@ def _spec(n, nv, nc, ecut, grid):
     return SystemSpec("cell", "fcc", 10.0, 0.0, (n, n, n), nv, nc, ecut, (grid,) * 3, "3d")
 
 
+@pytest.mark.parametrize("n,nv,nc,ecut,grid,nw", [(2, 1, 1, 1.0, 8, 1), (2, 2, 2, 1.0, 8, 31), (2, 2, 2, 1.0, 8, 33),
+                                                  (3, 2, 2, 4.0, 24, 129), (2, 3, 4, 8.6, 32, 40)])
+def test_chi0_of_random_densities(bse, n, nv, nc, ecut, grid, nw):
+    spec = _spec(n, nv, nc, ecut, grid)
+    plan = bse.Plan([spec])
+    inf = plan.info(0)
+    dim, ng = inf["dim"], inf["ng0"]
+    g = bse.bse_gvectors(plan, 0, 0, True)
+    lut = {tuple(v): i for i, v in enumerate(g)}
+    minus = np.array([lut[tuple(-v)] for v in g])
+    rng = np.random.default_rng(7)
+    rho = np.zeros((dim, inf["ng_max"]), dtype=np.complex64)
+    rho[:, :ng] = (rng.standard_normal((dim, ng)) + 1j * rng.standard_normal((dim, ng))) * 10.0 ** rng.uniform(-3, 1, (1, ng))
+    P = rng.standard_normal(dim) + 1j * rng.standard_normal(dim)
+    en = np.sort(rng.uniform(-0.2, 0.0, (inf["nkpt"], nv)), axis=1)
+    en = np.concatenate([en, np.sort(rng.uniform(0.05, 0.4, (inf["nkpt"], nc)), axis=1)], axis=1)
+    omega, eta = np.linspace(0.0, 0.4, nw), 2e-3
+    chi = torch.full((nw, ng, ng), float("nan"), dtype=torch.complex64, device="cuda")
+    bse.bse_chi0_optical(plan, 0, _dev(rho, torch.complex64), _dev(P, torch.complex128), _dev(en, torch.float64), 0.03,
+                         _dev(omega, torch.float64), eta, chi, _ws(bse, plan, bse.BSE_WS_CHI0))
+    bse.bse_status_read(plan)
+    chi = chi.cpu().numpy()
+    b = 2.0 * np.pi / 10.0 * np.array([[-1.0, 1, 1], [1, -1, 1], [1, 1, -1]])
+    norm = np.linalg.norm(g @ b, axis=1)
+    vh = np.sqrt(4.0 * np.pi) / np.where(norm > 0, norm, 1.0)
+    r = rho[:, :ng].astype(np.complex128)
+    a, ab = r * vh, r[:, minus].conj() * vh
+    a[:, 0], ab[:, 0] = np.sqrt(4.0 * np.pi) * P.conj(), -np.sqrt(4.0 * np.pi) * P
+    de = (en[:, None, nv:] + 0.03 - en[:, :nv, None]).reshape(-1)
+    chunks = (dim + 63) // 64
+    tol = 5 * 2.0 ** -24 + 2.0 ** -21 + 12 * 2.0 ** -23 + chunks * 2.0 ** -24
+    for w in {0, nw // 2, nw - 1}:
+        z = omega[w] + 1j * eta
+        x, y = 1.0 / (z - de), -1.0 / (z + de)
+        ref = 2.0 * inf["norm"] * ((a * x[:, None]).T @ a.conj() + (ab * y[:, None]).T @ ab.conj())
+        size = 4.0 * inf["norm"] * (np.abs(a * x[:, None]).T @ np.abs(a) + np.abs(ab * y[:, None]).T @ np.abs(ab))
+        assert np.all(np.abs(chi[w] - ref) <= tol * size), w
+
+
 def test_screening_range_equals_single_points(bse):
     """W of a range (more q than one group of split images) is W of each q on its own, bit for bit."""
     spec = _spec(4, 1, 2, 2.0, 24)
