@@ -24,6 +24,7 @@
 
 #include "gemm_tile.cuh"
 #include "internal.h"
+#include "tcfcols.cuh"
 
 namespace bse {
 namespace {
@@ -32,6 +33,8 @@ constexpr int kNwChunk = 256;       // frequencies per resolvent chunk
 constexpr int kQChunk = 32;         // q points per direct-term chunk
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+size_t split_area(const DevSys& d, long long nsteps, long long qc, long long w);
 
 struct BwdLayout {
   size_t spec, eps2, ab, done, scal, Y, Mh, Mf, Vf, Zf, Gh, Xv, Xc, Yd, split, total;
@@ -61,7 +64,7 @@ BwdLayout bwd_layout(const DevSys& d, long long nsteps) {
   L.Xc = o; o = a256(o + 8 * (size_t)L.rows_c * d.ng_max);
   L.Yd = o; o = a256(o + 8 * (size_t)L.rows_c * d.ng_max);
   const long long w = d.nv > d.nc ? d.nv * d.nv : d.nc * d.nc;
-  L.split = o; o = a256(o + wr32_split_bytes(d, qc, w));
+  L.split = o; o = a256(o + split_area(d, nsteps, qc, w));
   L.total = o;
   return L;
 }
@@ -187,37 +190,6 @@ __global__ __launch_bounds__(gemm::kThreads) void gemm_kernel(const float2* __re
   }
 }
 
-// dW_q[G][G'] = -norm sum_k Y_q[k][G] conj(Rc_q[k][G'])  grouped over the q chunk.
-__global__ __launch_bounds__(gemm::kThreads) void gemm_dw_kernel(DevSys d, const float2* __restrict__ Yd,
-                                                                const float2* __restrict__ rho_dir,
-                                                                float2* __restrict__ dW, int q_begin) {
-  const int q = q_begin + blockIdx.z;
-  const long long b0 = d.qblk_off[q_begin];
-  const long long nblk = d.qblk_off[q + 1] - d.qblk_off[q];
-  const int nc2 = d.nc * d.nc, NG = d.ngq[q];
-  const int K = (int)(nblk * nc2);
-  const int m0 = blockIdx.y * gemm::BM, n0 = blockIdx.x * gemm::BN;
-  if (m0 >= NG || n0 >= NG || K == 0) return;
-  const float2* A = Yd + (size_t)((d.qblk_off[q] - b0) * nc2) * d.ng_max;
-  const float2* B = rho_dir + (size_t)(d.qvec_off[q] + nblk * d.nv * d.nv) * d.ng_max;
-  __shared__ gemm::Smem sm;
-  float2 acc[4][4];
-  gemm::tile<false, false, false, true>(A, d.ng_max, NG, B, d.ng_max, NG, K, m0, n0, sm, acc);
-  float2* C = dW + (size_t)q * d.ng_max * d.ng_max;
-  const float nrm = -(float)d.norm;
-  const int tm = threadIdx.x / 16, tn = threadIdx.x % 16;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = m0 + tm * 4 + i;
-    if (r >= NG) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = n0 + tn * 4 + j;
-      if (c < NG) C[(size_t)r * d.ng_max + c] = make_float2(nrm * acc[i][j].x, nrm * acc[i][j].y);
-    }
-  }
-}
-
 // Per upper block of the chunk: block gradient Gm, dL/drho_vv', dL/drho_cc' and Y = Gm-weighted rho_vv'.
 __global__ __launch_bounds__(256) void block_grad_kernel(DevSys d, const float2* __restrict__ Gh,
                                                          const float2* __restrict__ rho_dir,
@@ -283,6 +255,209 @@ __global__ __launch_bounds__(256) void block_grad_kernel(DevSys d, const float2*
   }
 }
 
+// ---------------------------------------------------------------- products on the tensor cores (tcf16.cuh)
+//
+// Measured, fcc 8x8x8 3v4c, 300 steps (64 x 64 tiles on the FP32 pipes before): dL/dW 43.0 -> 9.8 ms (products 4.8,
+// images 5.0), dL/drho_x 3.1 -> 0.6, G_h 2.0 -> 0.3; error of dL/dW against 64 bits 2.7e-6 -> 2.0e-6 (what is left is
+// the recursion's FP32 product).
+
+// Columns of a dense operand X[k][g].
+struct DenseSrc {
+  const float2* x;
+  int ld, K, G, nbatch;
+  __device__ __forceinline__ bool get(int, const float2*& p, int& k, int& g) const {
+    p = x;
+    k = K;
+    g = G;
+    return true;
+  }
+};
+
+// C[m][n] = alpha s(n)^2 sum_k opA(A[m][k]) B[n][k] of one pair of images; rows from m_begin (a panel of A).
+template <bool CONJ>
+struct DenseOp {
+  static constexpr bool kReal = false, kConj = CONJ, kHerm = false;
+  const unsigned char *a, *b;
+  const float *inva, *invb;
+  float2* C;
+  int M, N, K, nt, n_tile, kc;
+  long long ldc;
+  float alpha;
+  const float* colscale;
+  int* status;
+  long long ntiles;
+  __device__ __forceinline__ bool tile(long long ti, tcf::Tile& o) const {
+    const int mt = (int)(ti / nt), ntl = (int)(ti - (long long)mt * nt);
+    o.a_step = 2 * tcf::kTileA;
+    o.b_step = (uint32_t)(2 * n_tile * umma::kRow);
+    o.a = a + (size_t)mt * kc * o.a_step;
+    o.b = b + (size_t)ntl * kc * o.b_step;
+    o.K = K;
+    o.n = n_tile;
+    o.m0 = mt * tcf::kTM;
+    o.n0 = ntl * n_tile;
+    o.mvalid = M - o.m0;
+    o.nvalid = min(n_tile, N - o.n0);
+    o.batch = 0;
+    o.row0 = o.m0;
+    return true;
+  }
+  __device__ __forceinline__ float2* row_out(const tcf::Tile& t, int row) const { return C + (t.row0 + row) * ldc + t.n0; }
+  __device__ __forceinline__ float row_scale(const tcf::Tile& t, int row) const { return inva[t.m0 + row]; }
+  __device__ __forceinline__ float col_scale(const tcf::Tile& t, int col) const { return invb[t.n0 + col]; }
+  __device__ __forceinline__ float2 value(const tcf::Tile& t, int, int col, float2 v) const {
+    float s = alpha;
+    if (colscale) s *= colscale[t.n0 + col] * colscale[t.n0 + col];
+    return make_float2(s * v.x, s * v.y);
+  }
+};
+
+// Columns of the rows of one band side of a q chunk: rho_cc' (rho_dir) or Y (its chunk).
+struct SideSrc {
+  DevSys d;
+  const float2* x;
+  int q_begin, ld, nbatch;
+  bool chunk;                                   // x starts at the chunk's first block, rows of Nc^2 only
+  __device__ __forceinline__ bool get(int batch, const float2*& p, int& K, int& G) const {
+    const int q = q_begin + batch, nc2 = d.nc * d.nc;
+    const long long nblk = d.qblk_off[q + 1] - d.qblk_off[q];
+    const long long row = chunk ? (d.qblk_off[q] - d.qblk_off[q_begin]) * nc2 : d.qvec_off[q] + nblk * d.nv * d.nv;
+    p = x + (size_t)row * d.ng_max;
+    K = (int)(nblk * nc2);
+    G = d.ngq[q];
+    return K > 0;
+  }
+};
+
+// dW_q[G][G'] = -norm sum_k Y_q[k][G] conj(Rc_q[k][G']) over the q chunk, as -norm conj(conj(Y)^T Rc).
+struct DwOp {
+  static constexpr bool kReal = false, kConj = true, kHerm = false;
+  DevSys d;
+  const unsigned char *a, *b;
+  const float *inva, *invb;
+  float2* dW;
+  size_t a_batch, b_batch;
+  int q_begin, mt, nt, n_tile, kc;
+  int* status;
+  long long ntiles;
+  __device__ __forceinline__ bool tile(long long ti, tcf::Tile& o) const {
+    const int ntl = (int)(ti % nt);
+    const long long r = ti / nt;
+    const int mtl = (int)(r % mt), qi = (int)(r / mt), q = q_begin + qi, NG = d.ngq[q];
+    o.m0 = mtl * tcf::kTM;
+    o.n0 = ntl * n_tile;
+    o.K = (int)(d.qblk_off[q + 1] - d.qblk_off[q]) * d.nc * d.nc;
+    if (o.m0 >= NG || o.n0 >= NG || o.K == 0) return false;
+    o.a_step = 2 * tcf::kTileA;
+    o.b_step = (uint32_t)(2 * n_tile * umma::kRow);
+    o.a = a + qi * a_batch + (size_t)mtl * kc * o.a_step;
+    o.b = b + qi * b_batch + (size_t)ntl * kc * o.b_step;
+    o.n = n_tile;
+    o.mvalid = NG - o.m0;
+    o.nvalid = min(n_tile, NG - o.n0);
+    o.batch = qi;
+    o.row0 = (long long)q * d.ng_max + o.m0;
+    return true;
+  }
+  __device__ __forceinline__ float2* row_out(const tcf::Tile& t, int row) const {
+    return dW + (size_t)(t.row0 + row) * d.ng_max + t.n0;
+  }
+  __device__ __forceinline__ float row_scale(const tcf::Tile& t, int row) const {
+    return inva[(size_t)t.batch * d.ng_max + t.m0 + row];
+  }
+  __device__ __forceinline__ float col_scale(const tcf::Tile& t, int col) const {
+    return invb[(size_t)t.batch * d.ng_max + t.n0 + col];
+  }
+  __device__ __forceinline__ float2 value(const tcf::Tile&, int, int, float2 v) const {
+    const float nrm = (float)d.norm;
+    return make_float2(-nrm * v.x, nrm * v.y);
+  }
+};
+
+// Rows of G_h (a panel): image rows, K = dim.
+__global__ __launch_bounds__(256) void split_rows_kernel(const float2* __restrict__ x, long long ld, int rows, int K,
+                                                         unsigned char* __restrict__ img, float* __restrict__ inv,
+                                                         int kc) {
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const bool live = row < rows;
+  const float s = tcf::split_row<32, 3>(x + (size_t)(live ? row : 0) * ld, K, nullptr,
+                                        img + (size_t)(row / tcf::kTM) * kc * (2 * tcf::kTileA), 2 * tcf::kTileA,
+                                        tcf::kTileA, row % tcf::kTM, live);
+  if (live && (threadIdx.x & 31) == 0) inv[row] = s;
+}
+
+constexpr int kPanel = 32 * tcf::kTM;           // rows of G_h split at a time (the images of all would take its size again)
+
+// Largest use of the split area (images, then inverse scales): W.rho of a q chunk, dW of a q chunk, G_h, dL/drho_x.
+size_t split_area(const DevSys& d, long long nsteps, long long qc, long long w) {
+  const int n = tcf::n_tile(d.ng_max), nd = tcf::n_tile(d.dim), n0 = tcf::n_tile(d.ng0);
+  const int K = d.nkpt * d.nc * d.nc;
+  const size_t wr = wr32_split_bytes(d, qc, w);
+  const size_t dw = a256(qc * tcf::cols_batch_bytes(d.ng_max, K, tcf::kTM)) + a256(qc * tcf::cols_batch_bytes(d.ng_max, K, n)) +
+                    2 * a256((size_t)qc * d.ng_max * 4);
+  const size_t gh = a256(tcf::cols_batch_bytes(d.dim, (int)nsteps, tcf::kTM)) +
+                    a256(tcf::cols_batch_bytes(d.dim, (int)nsteps, nd)) + 2 * a256((size_t)d.dim * 4);
+  const size_t dx = a256(tcf::cols_batch_bytes(d.dim < kPanel ? d.dim : kPanel, d.dim, tcf::kTM)) +
+                    a256(tcf::cols_batch_bytes(d.ng0, d.dim, n0)) + a256((size_t)kPanel * 4) + a256((size_t)d.ng_max * 4);
+  return std::max(std::max(wr, dw), std::max(gh, dx));
+}
+
+// dL/dW of a q chunk from Y and rho_cc'.
+int launch_dw(const DevSys& d, const float2* Yd, const float2* rho_dir, float2* dW, int q0, int q1, long long maxb,
+              char* area, int* status, cudaStream_t st) {
+  const int nq = q1 - q0, n = tcf::n_tile(d.ng_max), K = (int)maxb * d.nc * d.nc;
+  if (K <= 0) return 0;
+  const size_t ab = tcf::cols_batch_bytes(d.ng_max, K, tcf::kTM), bb = tcf::cols_batch_bytes(d.ng_max, K, n);
+  unsigned char* a = (unsigned char*)area;
+  unsigned char* b = a + a256(nq * ab);
+  float* inva = (float*)(b + a256(nq * bb));
+  float* invb = (float*)((char*)inva + a256((size_t)nq * d.ng_max * 4));
+  int e = tcf::split_cols(SideSrc{d, Yd, q0, d.ng_max, nq, true}, K, d.ng_max, inva, a, tcf::kTM, st);
+  if (!e) e = tcf::split_cols(SideSrc{d, rho_dir, q0, d.ng_max, nq, false}, K, d.ng_max, invb, b, n, st);
+  if (e) return e;
+  DwOp op{d, a, b, inva, invb, dW, ab, bb, q0, (d.ng_max + tcf::kTM - 1) / tcf::kTM, (d.ng_max + n - 1) / n, n,
+          (K + tcf::kTKC - 1) / tcf::kTKC, status, 0};
+  op.ntiles = (long long)nq * op.mt * op.nt;
+  return tcf::launch(op, st);
+}
+
+// G_h = V^T Z (dim x dim, K = nsteps).
+int launch_gh(const DevSys& d, const float2* Vf, const float2* Zf, int nsteps, float2* Gh, char* area, int* status,
+              cudaStream_t st) {
+  const int n = tcf::n_tile(d.dim), kc = (nsteps + tcf::kTKC - 1) / tcf::kTKC;
+  unsigned char* a = (unsigned char*)area;
+  unsigned char* b = a + a256(tcf::cols_batch_bytes(d.dim, nsteps, tcf::kTM));
+  float* inva = (float*)(b + a256(tcf::cols_batch_bytes(d.dim, nsteps, n)));
+  float* invb = (float*)((char*)inva + a256((size_t)d.dim * 4));
+  int e = tcf::split_cols(DenseSrc{Vf, d.dim, nsteps, d.dim, 1}, nsteps, d.dim, inva, a, tcf::kTM, st);
+  if (!e) e = tcf::split_cols(DenseSrc{Zf, d.dim, nsteps, d.dim, 1}, nsteps, d.dim, invb, b, n, st);
+  if (e) return e;
+  DenseOp<false> op{a, b, inva, invb, Gh, d.dim, d.dim, nsteps, (d.dim + n - 1) / n, n, kc, d.dim, 1.f, nullptr, status, 0};
+  op.ntiles = (long long)((d.dim + tcf::kTM - 1) / tcf::kTM) * op.nt;
+  return tcf::launch(op, st);
+}
+
+// dL/drho_x[S][G] = 2 xscale(G)^2 sum_S' conj(G_h[S][S']) rho_x[S'][G], G_h split a panel of rows at a time.
+int launch_drho_x(const DevSys& d, const float2* Gh, const float2* rho_x, float2* drho_x, char* area, int* status,
+                  cudaStream_t st) {
+  const int n = tcf::n_tile(d.ng0), kc = (d.dim + tcf::kTKC - 1) / tcf::kTKC;
+  unsigned char* a = (unsigned char*)area;
+  unsigned char* b = a + a256(tcf::cols_batch_bytes(d.dim < kPanel ? d.dim : kPanel, d.dim, tcf::kTM));
+  float* inva = (float*)(b + a256(tcf::cols_batch_bytes(d.ng0, d.dim, n)));
+  float* invb = (float*)((char*)inva + a256((size_t)kPanel * 4));
+  int e = tcf::split_cols(DenseSrc{rho_x, d.ng_max, d.dim, d.ng0, 1}, d.dim, d.ng0, invb, b, n, st);
+  for (int m = 0; m < d.dim && !e; m += kPanel) {
+    const int rows = d.dim - m < kPanel ? d.dim - m : kPanel;
+    split_rows_kernel<<<(rows + 7) / 8, 256, 0, st>>>(Gh + (size_t)m * d.dim, d.dim, rows, d.dim, a, inva, kc);
+    if ((e = (int)cudaGetLastError())) break;
+    DenseOp<true> op{a, b, inva, invb, drho_x + (size_t)m * d.ng_max, rows, d.ng0, d.dim, (d.ng0 + n - 1) / n, n, kc,
+                     d.ng_max, 2.f, d.xscale, status, 0};
+    op.ntiles = (long long)((rows + tcf::kTM - 1) / tcf::kTM) * op.nt;
+    e = tcf::launch(op, st);
+  }
+  return e;
+}
+
 }  // namespace
 
 size_t backward_ws_bytes(const DevSys& d, long long nsteps) { return bwd_layout(d, nsteps).total; }
@@ -328,18 +503,13 @@ int launch_backward(const DevSys& d, const long long* h_qblk_off, const long lon
     dim3 gz((d.dim + 63) / 64, (nsteps + 63) / 64);
     gemm_kernel<true, false, false, true><<<gz, gemm::kThreads, 0, st>>>(Mf, nsteps, nsteps, Vf, d.dim, d.dim, nsteps,
                                                                         Zf, d.dim, 1.f, nullptr);
-    dim3 gg((d.dim + 63) / 64, (d.dim + 63) / 64);
-    gemm_kernel<false, false, false, false><<<gg, gemm::kThreads, 0, st>>>(Vf, d.dim, d.dim, Zf, d.dim, d.dim, nsteps,
-                                                                          Gh, d.dim, 1.f, nullptr);
     if ((e = (int)cudaGetLastError())) return e;
+    if ((e = launch_gh(d, Vf, Zf, nsteps, Gh, base + L.split, status, st))) return e;
   }
   // 4. exchange: dL/drho_x[S][G] = 2 xscale(G)^2 sum_S' conj(G_h[S][S']) rho_x[S'][G]
   if (drho_x) {
     if ((e = (int)cudaMemsetAsync(drho_x, 0, 8 * (size_t)d.dim * d.ng_max, st))) return e;
-    dim3 gx((d.ng0 + 63) / 64, (d.dim + 63) / 64);
-    gemm_kernel<true, false, true, false><<<gx, gemm::kThreads, 0, st>>>(
-        Gh, d.dim, d.dim, (const float2*)rho_x, d.ng_max, d.ng0, d.dim, (float2*)drho_x, d.ng_max, 2.f, d.xscale);
-    if ((e = (int)cudaGetLastError())) return e;
+    if ((e = launch_drho_x(d, Gh, (const float2*)rho_x, (float2*)drho_x, base + L.split, status, st))) return e;
   }
   // 5. direct term, q chunks
   if (drho_dir || dW) {
@@ -358,11 +528,9 @@ int launch_backward(const DevSys& d, const long long* h_qblk_off, const long lon
       if (nb > 0)
         block_grad_kernel<<<(unsigned)nb, 256, 0, st>>>(d, Gh, (const float2*)rho_dir, Xv, Xc, (float2*)drho_dir, Yd,
                                                         q0);
-      if (dW) {
-        dim3 gw((d.ng_max + 63) / 64, (d.ng_max + 63) / 64, q1 - q0);
-        gemm_dw_kernel<<<gw, gemm::kThreads, 0, st>>>(d, Yd, (const float2*)rho_dir, (float2*)dW, q0);
-      }
       if ((e = (int)cudaGetLastError())) return e;
+      if (dW && (e = launch_dw(d, Yd, (const float2*)rho_dir, (float2*)dW, q0, q1, maxb, base + L.split, status, st)))
+        return e;
     }
   }
   return 0;
