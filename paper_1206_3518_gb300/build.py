@@ -22,7 +22,7 @@ NVCC = os.path.join(CUDA, "bin", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 CU_SOURCES = ["pair.cu", "build.cu", "haydock.cu", "adjoint.cu", "tc.cu", "screen.cu", "coupled.cu", "gcorr.cu", "ritz.cu", "sym.cu", "scan.cu", "tddft.cu", "eig.cu", "tcpair.cu", "tcgram.cu",
-              "tcwr32.cu", "tcchi0.cu"]
+              "tcwr32.cu", "tcgram32.cu", "tcchi0.cu"]
 CPP_SOURCES = ["plan.cpp"]
 
 

@@ -377,7 +377,7 @@ static size_t split_bytes(const DevSys& d, long long qchunk, long long w) {
 size_t kernel_ws_bytes(const DevSys& d, long long qchunk) {
   const long long w = direct_width(d);
   const size_t direct = x_bytes(d, qchunk, w) + split_bytes(d, qchunk, w);
-  const size_t init = gram_ws_bytes(d);
+  const size_t init = gram32_ws_bytes(d) > gram_ws_bytes(d) ? gram32_ws_bytes(d) : gram_ws_bytes(d);
   return direct > init ? direct : init;
 }
 

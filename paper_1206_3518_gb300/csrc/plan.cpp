@@ -933,6 +933,10 @@ bse_status bse_build_kernel(bse_plan* plan, int s, unsigned flags, const void* r
       if ((st = cuda_check(launch_kernel_init_tc(d, rho_x, energies, delta, H, ws, plan->d_status, stream),
                            "kernel init (tensor)")) != BSE_OK)
         return st;
+    } else if (ws && ws_bytes >= gram32_ws_bytes(d)) {
+      if ((st = cuda_check(launch_kernel_init_tc32(d, rho_x, energies, delta, H, ws, plan->d_status, stream),
+                           "kernel init (tensor, FP32)")) != BSE_OK)
+        return st;
     } else if ((st = cuda_check(launch_kernel_init(d, rho_x, energies, delta, H, stream), "kernel init")) != BSE_OK)
       return st;
   }

@@ -185,11 +185,11 @@ __device__ __forceinline__ void chunk_mmas(uint32_t d_re, uint32_t d_im, uint64_
     const uint32_t d = im ? d_im : d_re, sign = (im != 0) == CONJ ? neg : idesc;   // of the product with Im A
     const uint32_t b0 = im ? 4u : 0u, b1 = 4u - b0;                            // plane of B met by Re A, by Im A
 #pragma unroll
-    for (int s = 0; s < 3; ++s)                  // hi.lo, lo.hi, hi.hi
+    for (int s = 0; s < 3; ++s)                  // hi.lo and lo.hi, then hi.hi
 #pragma unroll
       for (int kk = NKK - 1; kk >= 0; --kk) {
-        const uint64_t pa = da + (s == 1 ? a_lo : 0u) + (uint32_t)kk * 2u;
-        const uint64_t pb = db + (s == 0 ? b_lo : 0u) + (uint32_t)kk * 2u;
+        const uint64_t pa = da + (s == (CONJ ? 0 : 1) ? a_lo : 0u) + (uint32_t)kk * 2u;
+        const uint64_t pb = db + (s == (CONJ ? 1 : 0) ? b_lo : 0u) + (uint32_t)kk * 2u;
         umma::mma_bf16(d, pa, pb + b0, idesc, (s != 0 || kk != NKK - 1) ? 1u : 0u);
         umma::mma_bf16(d, pa + 4u, pb + b1, sign, 1u);
       }
