@@ -78,6 +78,10 @@ namespace bse {
 bse_status set_error(bse_status st, const std::string& msg);
 bse_status cuda_check(int err, const char* what);
 
+// Images that bulk copies read start on a 16-byte boundary wherever the caller's workspace does: sizes carry the slack.
+constexpr size_t kWsSlack = 256;
+inline unsigned char* ws_base(void* ws) { return (unsigned char*)(((uintptr_t)ws + 255) & ~(uintptr_t)255); }
+
 // Kernel launchers (defined in the .cu files); all return cudaError_t as int.
 int launch_realspace(const DevSys& d, const void* coef, void* u, void* stream);
 int launch_pair_exchange(const DevSys& d, const void* u, void* rho_x, int* status, void* stream);

@@ -301,7 +301,7 @@ ScreenWs layout(const DevSys& d, long long nq) {
 }
 }  // namespace
 
-size_t screen_ws_bytes(const DevSys& d, long long qchunk) { return layout(d, qchunk).total; }
+size_t screen_ws_bytes(const DevSys& d, long long qchunk) { return kWsSlack + layout(d, qchunk).total; }
 
 int launch_screening(const DevSys& d, void* rho_chi, const double* energies, const void* P, int q_begin, int q_end,
                      int iterations, void* W, float* residual, void* ws, double gap_floor, int* status, void* stream) {
@@ -309,7 +309,7 @@ int launch_screening(const DevSys& d, void* rho_chi, const double* energies, con
   const int nq = q_end - q_begin, K = d.nkpt * d.nv * d.nc;
   const long long rows = (long long)nq * K;
   const ScreenWs L = layout(d, nq);
-  char* base = (char*)ws;
+  unsigned char* base = ws_base(ws);
   float2* E = (float2*)(base + L.E);
   float2* X = (float2*)(base + L.X);
   float2* T = (float2*)(base + L.T);

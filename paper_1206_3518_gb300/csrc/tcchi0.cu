@@ -290,13 +290,13 @@ __global__ __launch_bounds__(256) void combine_kernel(int ng, const int* __restr
 
 }  // namespace
 
-size_t chi0_ws_bytes(const DevSys& d) { return geo_of(d).total; }
+size_t chi0_ws_bytes(const DevSys& d) { return kWsSlack + geo_of(d).total; }
 
 int launch_chi0_optical(const DevSys& d, const void* rho_x, const void* P, const double* energies, double delta,
                         const double* omega, int nw, double eta, void* chi0, void* ws, int* status, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   const Geo g = geo_of(d);
-  char* base = (char*)ws;
+  unsigned char* base = ws_base(ws);
   float2* a = (float2*)(base + g.o_a);
   float* amax = (float*)(base + g.o_amax);
   double* de = (double*)(base + g.o_de);

@@ -93,12 +93,12 @@ void launch_split(const DevSys& d, const void* rho_x, unsigned char* img, float*
 
 }  // namespace
 
-size_t gram32_ws_bytes(const DevSys& d) { return img_bytes(d) + (size_t)d.dim * sizeof(float); }
+size_t gram32_ws_bytes(const DevSys& d) { return kWsSlack + img_bytes(d) + (((size_t)d.dim * sizeof(float) + 255) & ~(size_t)255); }
 
 int launch_kernel_init_tc32(const DevSys& d, const void* rho_x, const double* energies, double delta, void* H, void* ws,
                             int* status, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
-  unsigned char* img = (unsigned char*)ws;
+  unsigned char* img = ws_base(ws);
   float* inv = (float*)(img + img_bytes(d));
   const int nkc = (d.ng0 + kTKC - 1) / kTKC;
   if (nkc < 1) return (int)cudaErrorInvalidValue;

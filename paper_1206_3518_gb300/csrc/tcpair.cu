@@ -786,7 +786,7 @@ int tcpair_preferred(const DevSys& d, int q_begin, int q_end) {
   return (long long)d.nkpt * touched >= 304 && (long long)nqc * d.nb >= 30ll * touched ? 1 : 0;
 }
 
-size_t tcpair_ws_bytes(const DevSys& d) { return tcpair_valid(d) ? tp_ws(d).total : 0; }
+size_t tcpair_ws_bytes(const DevSys& d) { return tcpair_valid(d) ? kWsSlack + tp_ws(d).total : 0; }
 
 // coef: the coefficient copy of the pair workspace; ws: the tensor-route area (tcpair_ws_bytes).
 int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, int q_begin, int q_end,
@@ -809,7 +809,7 @@ int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, in
   }
   cudaStream_t st = (cudaStream_t)stream;
   const TpWs w = tp_ws(d);
-  unsigned char* base = (unsigned char*)ws;
+  unsigned char* base = ws_base(ws);
   unsigned char* bimg = base + w.bimg;
   int* blist = (int*)(base + w.blist);
   int* counter = (int*)(base + w.counter);

@@ -132,7 +132,8 @@ size_t wr32_split_bytes(const DevSys& d, long long qchunk, long long w) {
   const int n = tcf::n_tile(d.ng_max);
   const long long mt = (d.nkpt * w + kTM - 1) / kTM, nt = (d.ng_max + n - 1) / n, kc = (d.ng_max + kTKC - 1) / kTKC;
   const size_t img = (size_t)qchunk * kc * (size_t)(mt * 2 * kTileA + nt * 2 * n * umma::kRow);
-  return a256(img) + a256((size_t)qchunk * d.nkpt * w * sizeof(float)) + a256((size_t)qchunk * d.ng_max * sizeof(float));
+  return kWsSlack + a256(img) + a256((size_t)qchunk * d.nkpt * w * sizeof(float)) +
+         a256((size_t)qchunk * d.ng_max * sizeof(float));
 }
 
 int launch_gemm_wr(const DevSys& d, const void* rho, int q_begin, int q_end, long long vbase, long long max_rows,
@@ -152,7 +153,7 @@ int launch_gemm_wr(const DevSys& d, const void* rho, int q_begin, int q_end, lon
   WrOp op;
   op.d = d;
   op.g = g;
-  unsigned char* As = (unsigned char*)split_ws;
+  unsigned char* As = ws_base(split_ws);
   unsigned char* Bs = As + a_off(g, g.nq, 0);
   float* inva = (float*)(As + a256(a_off(g, g.nq, 0) + b_off(g, g.nq, 0)));
   float* invb = (float*)((unsigned char*)inva + a256((size_t)g.nq * d.nkpt * w * sizeof(float)));
