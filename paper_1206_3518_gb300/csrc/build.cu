@@ -5,7 +5,8 @@
 //   K^d_SS' = (1/(Omega Nk)) sum_{G,G'} conj(rho_vv'^{kk'}(G)) W_GG'(q) rho_cc'^{kk'}(G')  (Eq. W_SS)
 //
 // init_kernel   : 2K^x + diag on every tile that touches the upper block triangle; the
-//                 exchange scale sqrt(2 vbar/(Omega Nk)) is applied to both operands.
+//                 exchange scale sqrt(2 vbar/(Omega Nk)) is applied to both operands (a build
+//                 without a workspace at this step; with one, tcgram32.cu).
 // W.rho         : per q, X = W(q) R for the smaller band side (grouped over the q chunk), stored as
 //                 X^T rows [col][G] (G contiguous); on the tensor cores (tcwr32.cu, FP32 accuracy).
 // block_kernel  : per upper block (k <= k'), M = X^H R of the other side (K = NG_q),
@@ -59,31 +60,56 @@ __global__ __launch_bounds__(kGemmThreads) void init_kernel(DevSys d, const floa
 }
 
 constexpr int kBlkThreads = 256, KC = 32;
-constexpr int kBlkPerCta = 4, kBlkT = kBlkThreads / kBlkPerCta;   // block_kernel: 64 threads per block
+
+constexpr int kBlkWarps = 4;             // block_kernel: blocks (warps) per CTA
+constexpr int kBlkStages = 3;            // K steps in a warp's ring: one in use, two in flight
+constexpr int kBlkK = 16;                // complex K values per step: 128 bytes of a row
+constexpr int kBlkRow = kBlkK + 2;       // entries of a ring row: 16-byte rows four banks apart
+
+__host__ __device__ constexpr int blk_warp_bytes(int rows) { return kBlkStages * rows * kBlkRow * (int)sizeof(float2); }
+
+// `bytes` of 16 (past L1) or of 8 from global to shared memory, the rest zero.
+__device__ __forceinline__ void cp_async16(float2* dst, const float2* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8(float2* dst, const float2* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
 
 // Per upper block: M[a][c] = sum_G conj(L[a][G]) Rr[c][G], a = (v,v'), c = (c,c');
 // side V: L = X (= W R_v), Rr = R_c;  side C: L = R_v, Rr = X (= W R_c).
-// Four blocks per CTA, 64 threads per block, each thread a 2 x 2 patch of the (at most 16 x 16) product:
-// four shared-memory loads per four complex multiply-adds, sixteen global loads per thread in flight
-// per K step.
-__global__ __launch_bounds__(kBlkThreads) void block_kernel(DevSys d, const float2* __restrict__ rho_dir,
-                                                           const float2* __restrict__ X, float2* __restrict__ H,
-                                                           int q_begin, long long vbase, int side_c, long long b_count) {
-  __shared__ float2 Ls[kBlkPerCta][16][KC + 1];
-  __shared__ float2 Rs[kBlkPerCta][16][KC + 1];
-  __shared__ float2 Bs[kBlkPerCta][16][17];
-  __shared__ int ngs[kBlkPerCta];
-  const int grp = threadIdx.x / kBlkT, t = threadIdx.x % kBlkT;
-  const long long bi = (long long)blockIdx.x * kBlkPerCta + grp;
-  const bool live = bi < b_count;
+// One warp per block, so that no barrier couples blocks of different q, and a ring of three K steps per warp filled
+// with 16-byte asynchronous copies past L1 (8-byte ones, which go through L1, hold a line of it each while in flight).
+// LI x (32 / LI) lanes with a PI x PJ patch each, a = i + LI x, c = j + LJ y; the patch is the smallest that covers
+// nv^2 x nc^2 (lanes beyond it read the last row and store nothing).  Each entry is the same chain of fused
+// multiply-adds over G whatever the patch.  EVEN: every row starts on a 16-byte boundary (two values per load).
+// Bound by HBM (every density and X row is read once) and, close to it, by shared-memory reads (LDS of PI + PJ values for
+// 4 PI PJ multiply-adds).  Measured, all q (ms; before: four blocks per CTA of 256 threads, 2 x 2 patches, loads through
+// registers with two CTA barriers a step): fcc 8x8x8 3v4c 1.71 (2.90; 8.2 GB, 0.72 of the copy rate), fcc 12x12x12 4v4c
+// 51.8 (56), 27 x 27 sheet 2v3c 0.91 (2.3).
+template <int LI, int PI, int PJ, bool EVEN>
+__global__ __launch_bounds__(kBlkWarps * 32) void block_kernel(DevSys d, const float2* __restrict__ rho_dir,
+                                                              const float2* __restrict__ X, float2* __restrict__ H,
+                                                              int q_begin, long long vbase, int side_c,
+                                                              long long b_count) {
+  extern __shared__ __align__(16) unsigned char blk_smem[];
+  constexpr int LJ = 32 / LI;
+  const int lane = threadIdx.x % 32;
+  const long long bi = (long long)blockIdx.x * kBlkWarps + threadIdx.x / 32;
+  if (bi >= b_count) return;                          // whole warps; the kernel has no CTA barrier
+  const int nv2 = d.nv * d.nv, nc2 = d.nc * d.nc, rows = nv2 + nc2;
+  float2* ring = reinterpret_cast<float2*>(blk_smem + (threadIdx.x / 32) * blk_warp_bytes(rows));
   const long long b0 = d.qblk_off[q_begin];
-  const long long b = b0 + (live ? bi : 0);
+  const long long b = b0 + bi;
   const int4 blk = d.blocks[b];
   const int k = blk.x, k2 = blk.y, q = blk.z;
   const long long qb = d.qblk_off[q];
   const long long nblk = d.qblk_off[q + 1] - qb;
   const long long local = b - qb;
-  const int nv2 = d.nv * d.nv, nc2 = d.nc * d.nc;
   const long long vbase_q = d.qvec_off[q] - vbase;
   const float2* Rv = rho_dir + (size_t)(vbase_q + local * nv2) * d.ng_max;
   const float2* Rc = rho_dir + (size_t)(vbase_q + nblk * nv2 + local * nc2) * d.ng_max;
@@ -91,84 +117,174 @@ __global__ __launch_bounds__(kBlkThreads) void block_kernel(DevSys d, const floa
   const float2* Xb = X + (size_t)((qb - b0 + local) * w) * d.ng_max;
   const float2* L = side_c ? Rv : Xb;
   const float2* R = side_c ? Xb : Rc;
-  const int NG = live ? d.ngq[q] : 0;
-  if (t == 0) ngs[grp] = NG;
-  __syncthreads();
-  int ngmax = 0;
-#pragma unroll
-  for (int i = 0; i < kBlkPerCta; ++i) ngmax = max(ngmax, ngs[i]);
-  const int i2 = t >> 3, j2 = t & 7;                 // rows a = 2 i2, 2 i2 + 1; columns c = 2 j2, 2 j2 + 1
-  float2 acc[2][2];
-#pragma unroll
-  for (int x = 0; x < 2; ++x)
-#pragma unroll
-    for (int y = 0; y < 2; ++y) acc[x][y] = make_float2(0.f, 0.f);
-  for (int g0 = 0; g0 < ngmax; g0 += KC) {
-    for (int i = t; i < 16 * KC; i += kBlkT) {
-      const int r = i / KC, g = i % KC;
-      const bool in = (g0 + g) < NG;
-      Ls[grp][r][g] = (r < nv2 && in) ? L[(size_t)r * d.ng_max + g0 + g] : make_float2(0.f, 0.f);
-      Rs[grp][r][g] = (r < nc2 && in) ? R[(size_t)r * d.ng_max + g0 + g] : make_float2(0.f, 0.f);
+  const int NG = d.ngq[q], steps = (NG + kBlkK - 1) / kBlkK;
+
+  // Eight lanes per row, four rows at once.  Entry e of a step lies in slot e + odd(row), so that the 16-byte copies keep
+  // their alignment in rows that start on an odd multiple of eight bytes; there the eighth lane brings the first and
+  // the last entry.  A lane's rows are a multiple of four rows apart and share that parity.
+  const int l8 = lane & 7, r0 = lane >> 3;
+  auto load_rows = [&](const float2* src, float2* dst, int n, int left) {
+    src += (size_t)r0 * d.ng_max;
+    const int odd = EVEN ? 0 : (int)(reinterpret_cast<uintptr_t>(src) >> 3) & 1;
+    const int e = odd + 2 * l8;
+    dst += r0 * kBlkRow;
+    for (int r = r0; r < n; r += 4) {
+      if (!EVEN && odd && l8 == 7) {
+        const bool last = left > kBlkK - 1;
+        cp_async8(dst + 1, src, 8);
+        cp_async8(dst + kBlkK, last ? src + kBlkK - 1 : src, last ? 8 : 0);
+      } else {
+        const int m = min(max(left - e, 0), 2);
+        cp_async16(dst + odd + e, src + (m > 0 ? e : -odd), 8 * m);
+      }
+      src += 4 * (size_t)d.ng_max;
+      dst += 4 * kBlkRow;
     }
-    __syncthreads();
-#pragma unroll 8
-    for (int g = 0; g < KC; ++g) {
-      const float2 l0 = Ls[grp][2 * i2][g], l1 = Ls[grp][2 * i2 + 1][g];
-      const float2 r0 = Rs[grp][2 * j2][g], r1 = Rs[grp][2 * j2 + 1][g];
-      const float2 lv[2] = {l0, l1}, rv[2] = {r0, r1};
-#pragma unroll
-      for (int x = 0; x < 2; ++x)
-#pragma unroll
-        for (int y = 0; y < 2; ++y) {
-          acc[x][y].x = fmaf(lv[x].x, rv[y].x, fmaf(lv[x].y, rv[y].y, acc[x][y].x));     // conj(l) r
-          acc[x][y].y = fmaf(lv[x].x, rv[y].y, fmaf(-lv[x].y, rv[y].x, acc[x][y].y));
-        }
+  };
+  auto load = [&](int it) {
+    if (it < steps) {
+      float2* dst = ring + (it % kBlkStages) * rows * kBlkRow;
+      load_rows(L + it * kBlkK, dst, nv2, NG - it * kBlkK);
+      load_rows(R + it * kBlkK, dst + nv2 * kBlkRow, nc2, NG - it * kBlkK);
     }
-    __syncthreads();
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  const int i0 = lane / LJ, j0 = lane % LJ;
+  int lo[PI], ro[PJ];
+  auto slot = [&](const float2* row, int r) {
+    return r * kBlkRow + (EVEN ? 0 : (int)(reinterpret_cast<uintptr_t>(row) >> 3) & 1);
+  };
+#pragma unroll
+  for (int x = 0; x < PI; ++x) {
+    const int r = min(i0 + LI * x, nv2 - 1);
+    lo[x] = slot(L + (size_t)r * d.ng_max, r);
   }
+#pragma unroll
+  for (int y = 0; y < PJ; ++y) {
+    const int r = min(j0 + LJ * y, nc2 - 1);
+    ro[y] = slot(R + (size_t)r * d.ng_max, nv2 + r);
+  }
+  float2 acc[PI][PJ];
+#pragma unroll
+  for (int x = 0; x < PI; ++x)
+#pragma unroll
+    for (int y = 0; y < PJ; ++y) acc[x][y] = make_float2(0.f, 0.f);
+
+#pragma unroll
+  for (int s = 0; s < kBlkStages - 1; ++s) load(s);
+  for (int it = 0; it < steps; ++it) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kBlkStages - 2) : "memory");
+    __syncwarp();                                     // step it has landed; all lanes are done with step it - 1
+    load(it + kBlkStages - 1);
+    const float2* st = ring + (it % kBlkStages) * rows * kBlkRow;
+    auto mac = [&](const float2 (&l)[PI], const float2 (&r)[PJ]) {
+#pragma unroll
+      for (int x = 0; x < PI; ++x)
+#pragma unroll
+        for (int y = 0; y < PJ; ++y) {
+          acc[x][y].x = fmaf(l[x].x, r[y].x, fmaf(l[x].y, r[y].y, acc[x][y].x));         // conj(l) r
+          acc[x][y].y = fmaf(l[x].x, r[y].y, fmaf(-l[x].y, r[y].x, acc[x][y].y));
+        }
+    };
+    if constexpr (EVEN) {
+#pragma unroll 4
+      for (int g = 0; g < kBlkK; g += 2) {
+        float2 l0[PI], l1[PI], r0_[PJ], r1[PJ];
+#pragma unroll
+        for (int x = 0; x < PI; ++x) {
+          const float4 v = *reinterpret_cast<const float4*>(st + lo[x] + g);
+          l0[x] = make_float2(v.x, v.y);
+          l1[x] = make_float2(v.z, v.w);
+        }
+#pragma unroll
+        for (int y = 0; y < PJ; ++y) {
+          const float4 v = *reinterpret_cast<const float4*>(st + ro[y] + g);
+          r0_[y] = make_float2(v.x, v.y);
+          r1[y] = make_float2(v.z, v.w);
+        }
+        mac(l0, r0_);
+        mac(l1, r1);
+      }
+    } else {
+#pragma unroll 8
+      for (int g = 0; g < kBlkK; ++g) {
+        float2 l[PI], r[PJ];
+#pragma unroll
+        for (int x = 0; x < PI; ++x) l[x] = st[lo[x] + g];
+#pragma unroll
+        for (int y = 0; y < PJ; ++y) r[y] = st[ro[y] + g];
+        mac(l, r);
+      }
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+
   const int nv = d.nv, nc = d.nc, nvc = nv * nc;
   const float nrm = (float)d.norm;
-  int rows[2][2], colsv[2][2];
-  float2 vals[2][2];
-  bool act[2][2];
+  float2* Bs = ring;                                  // the diagonal block: nvc (nvc + 1) <= 54 (nv^2 + nc^2)
 #pragma unroll
-  for (int x = 0; x < 2; ++x)
+  for (int x = 0; x < PI; ++x)
 #pragma unroll
-    for (int y = 0; y < 2; ++y) {
-      const int a = 2 * i2 + x, c = 2 * j2 + y;
-      act[x][y] = live && a < nv2 && c < nc2;
-      rows[x][y] = colsv[x][y] = 0;
-      vals[x][y] = make_float2(0.f, 0.f);
-      if (!act[x][y]) continue;
-      const int v = a / nv, vp = a % nv, cc = c / nc, cp = c % nc;
-      const int row = v * nc + cc;                 // (k, v, c) local
-      const int col = vp * nc + cp;                // (k', v', c') local
-      rows[x][y] = row;
-      colsv[x][y] = col;
+    for (int y = 0; y < PJ; ++y) {
+      const int a = i0 + LI * x, c = j0 + LJ * y;
+      if (a >= nv2 || c >= nc2) continue;
+      const int row = (a / nv) * nc + c / nc;          // (k, v, c) local
+      const int col = (a % nv) * nc + c % nc;          // (k', v', c') local
       const size_t hij = (size_t)(k * nvc + row) * d.dim + (size_t)k2 * nvc + col;
       const float2 h = H[hij];
       const float2 val = make_float2(h.x - nrm * acc[x][y].x, h.y - nrm * acc[x][y].y);
-      vals[x][y] = val;
+      acc[x][y] = val;
       if (k != k2) {
         H[hij] = val;
         H[(size_t)(k2 * nvc + col) * d.dim + (size_t)k * nvc + row] = make_float2(val.x, -val.y);
       } else {
-        Bs[grp][row][col] = val;
+        Bs[row * (nvc + 1) + col] = val;
       }
     }
-  __syncthreads();
   if (k == k2) {
+    __syncwarp();
 #pragma unroll
-    for (int x = 0; x < 2; ++x)
+    for (int x = 0; x < PI; ++x)
 #pragma unroll
-      for (int y = 0; y < 2; ++y) {
-        if (!act[x][y]) continue;
-        const int row = rows[x][y], col = colsv[x][y];
-        const float2 o = Bs[grp][col][row];
+      for (int y = 0; y < PJ; ++y) {
+        const int a = i0 + LI * x, c = j0 + LJ * y;
+        if (a >= nv2 || c >= nc2) continue;
+        const int row = (a / nv) * nc + c / nc, col = (a % nv) * nc + c % nc;
+        const float2 o = Bs[col * (nvc + 1) + row];
         H[(size_t)(k * nvc + row) * d.dim + (size_t)k * nvc + col] =
-            make_float2(0.5f * (vals[x][y].x + o.x), 0.5f * (vals[x][y].y - o.y));
+            make_float2(0.5f * (acc[x][y].x + o.x), 0.5f * (acc[x][y].y - o.y));
       }
   }
+}
+
+template <int LI, int PI, int PJ>
+int launch_block(const DevSys& d, const float2* rho, const float2* X, float2* H, int q_begin, long long vbase,
+                 int side_c, long long b_count, cudaStream_t st) {
+  const int smem = kBlkWarps * blk_warp_bytes(d.nv * d.nv + d.nc * d.nc);       // at most 54 KB
+  const bool even = d.ng_max % 2 == 0 && ((reinterpret_cast<uintptr_t>(rho) | reinterpret_cast<uintptr_t>(X)) & 15) == 0;
+  auto kernel = even ? block_kernel<LI, PI, PJ, true> : block_kernel<LI, PI, PJ, false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return (int)e;
+  kernel<<<(unsigned)((b_count + kBlkWarps - 1) / kBlkWarps), kBlkWarps * 32, smem, st>>>(d, rho, X, H, q_begin, vbase,
+                                                                                         side_c, b_count);
+  return (int)cudaGetLastError();
+}
+
+// The longer side takes the eight lanes; nv^2 and nc^2 are 1, 4, 9 or 16.
+int launch_blocks(const DevSys& d, const float2* rho, const float2* X, float2* H, int q_begin, long long vbase,
+                  int side_c, long long b_count, cudaStream_t st) {
+  const int nv = d.nv, nc = d.nc;
+  if (nv <= nc) {
+    if (nc <= 2) return launch_block<4, 1, 1>(d, rho, X, H, q_begin, vbase, side_c, b_count, st);
+    if (nv <= 2) return launch_block<4, 1, 2>(d, rho, X, H, q_begin, vbase, side_c, b_count, st);
+    if (nv == 3) return launch_block<4, 3, 2>(d, rho, X, H, q_begin, vbase, side_c, b_count, st);
+    return launch_block<4, 4, 2>(d, rho, X, H, q_begin, vbase, side_c, b_count, st);
+  }
+  if (nv <= 2) return launch_block<8, 1, 1>(d, rho, X, H, q_begin, vbase, side_c, b_count, st);
+  if (nc <= 2) return launch_block<8, 2, 1>(d, rho, X, H, q_begin, vbase, side_c, b_count, st);
+  return launch_block<8, 2, 3>(d, rho, X, H, q_begin, vbase, side_c, b_count, st);
 }
 
 // Lower blocks from the upper ones, H_k'k = H_kk'^H, and diagonal blocks (B + B^H)/2 (for a build
@@ -414,10 +530,7 @@ int launch_kernel_direct_range(const DevSys& d, const void* rho_dir, int q_begin
     return -1;
   }
   if (e) return e;
-  if (b_count > 0)
-    block_kernel<<<(unsigned)((b_count + kBlkPerCta - 1) / kBlkPerCta), kBlkThreads, 0, st>>>(
-        d, (const float2*)rho_dir, (const float2*)ws, (float2*)H, q_begin, vbase, side_c, b_count);
-  return (int)cudaGetLastError();
+  return launch_blocks(d, (const float2*)rho_dir, (const float2*)ws, (float2*)H, q_begin, vbase, side_c, b_count, st);
 }
 
 int launch_coupling_init(const DevSys& d, const void* rho_x, void* Bm, void* ws, void* stream) {
