@@ -212,7 +212,7 @@ __device__ __forceinline__ void chunk_mmas_real(uint32_t d, uint64_t da, uint32_
 // the first K16 half, + 32 of the second (two FP16 per 32-bit column, lane = row); A as it is (no conjugation).
 template <int NKK>
 __device__ __forceinline__ void chunk_mmas_ts(uint32_t d_re, uint32_t d_im, uint32_t a, uint64_t db, uint32_t b_lo,
-                                              uint32_t idesc) {
+                                              uint32_t b_sub, uint32_t idesc) {
   const uint32_t neg = idesc | umma::kNegA;
 #pragma unroll
   for (int im = 0; im < 2; ++im) {
@@ -223,7 +223,7 @@ __device__ __forceinline__ void chunk_mmas_ts(uint32_t d_re, uint32_t d_im, uint
 #pragma unroll
       for (int kk = NKK - 1; kk >= 0; --kk) {
         const uint32_t pa = a + (uint32_t)kk * 32u + (s == 1 ? 16u : 0u);
-        const uint64_t pb = db + (s == 0 ? b_lo : 0u) + (uint32_t)kk * 2u;
+        const uint64_t pb = db + (s == 0 ? b_lo : 0u) + (uint32_t)(kk >> 1) * b_sub + (uint32_t)(kk & 1) * 2u;
         umma::mma_bf16_ts(d, pa, pb + b0, idesc, (s != 0 || kk != NKK - 1) ? 1u : 0u);
         umma::mma_bf16_ts(d, pa + 8u, pb + b1, sign, 1u);
       }

@@ -22,7 +22,7 @@
 //
 // Arithmetic (FP16x3, tcf16.cuh): the coefficients of every (k, band) are scaled by a power of two and split
 // hi + lo in FP16 (22 bits); each real product is hi.lo + lo.hi + hi.hi, and the tensor core's accumulator holds
-// one K chunk (32 complex values) at a time, which the epilogue warps add to FP32 registers.  The result has the
+// one K chunk (SUB panels of 32 complex values, tp_fit) at a time, which the epilogue warps add to FP32 registers.  The result has the
 // accuracy of the FP32 correlation kernel, so one kernel serves both precisions of the build.  The G = 0 overlaps
 // of the diagonal blocks (k' = k), which meet the q = 0 head of W, are summed again in FP64
 // afterwards (tcpair_diag_kernel).
@@ -32,21 +32,23 @@
 //   0, 1  promote the chunks of the even / odd passes into registers and write the pass's densities while the
 //         other group promotes the next pass (the scattered 8-byte stores, one cache line each, take most of
 //         a pass);
-//   2     gathers the A tile of each K chunk straight into tensor memory (four slots, tcgen05.st);
+//   2     gathers the A tile of each K chunk straight into tensor memory (4 / SUB slots, tcgen05.st);
 //   3     two warps issue the MMAs (12 per 16 complex K, A from tensor memory, B from shared memory; warp-uniform,
 //         umma.cuh), one warp brings the B rows into a ring of shared-memory stages with bulk copies (the region's
-//         panel of the chunk: its hi rows and its lo rows); the columns of a region's points without a block in
+//         panels of the chunk: hi rows and lo rows); the columns of a region's points without a block in
 //         the tile are computed and dropped.
 // At most 64 columns per pass: a group's sums are 2 x 64 registers a thread, and two accumulators (Re | Im, 128 TMEM
 // columns each) and four A slots fill tensor memory.  Every mbarrier wait is bounded (2 s); on expiry the CTA records
 // BSE_ERR_TIMEOUT, stops issuing, waits (bounded) for its MMAs in flight, frees its tensor memory and returns.
 //
-// What bounds it: the MMAs of a chunk (24 of 40 cycles at N = 64) against the gather (~300 cycles of shared-memory
-// bandwidth a chunk) and
-// the promotion; without promotion and stores fcc 8x8x8 3v4c takes 8.2 ms of 10.5.  Measured (ms; before: the FP32
-// correlation kernel / BF16x3 tensor kernel with 96 columns, two lookups an element and one accumulator a pass):
-// fcc 8x8x8 3v4c 10.5 (50.1 / 15.2), fcc 12x12x12 4v4c, 144 q 49.4 (- / 59), 27x27 sheet 2v3c, 64 q 1.33 (1.52 / -).  Error
-// against 64 bits (2-norm): 1.3e-7 to 1.5e-7 (correlation kernel 2.0e-7 to 4.0e-7).
+// What bounds it: no single part.  With a ring of two stages (fcc 8x8x8 3v4c 10.9 ms; fcc 12x12x12 4v4c, 144 q 45.8) a copy
+// without the tensor-memory stores of A takes 8.0 and 35.2 ms, without the lookups 8.7 and 40.5, without the stores of
+// the densities 9.5 and 39.4, with a twelfth of the MMAs 9.0 and 35.7, without the promotion 10.8 and 44.9: the gather's stores meet the
+// accumulators' traffic in tensor memory (the MMAs take 960 of ~1600 cycles per 32 K).  On sheets (K of 160) the
+// set-up of a tile is as long as its passes.  Measured (ms; before: the FP32 correlation kernel / BF16x3 tensor kernel with 96
+// columns, two lookups an element and one accumulator a pass): fcc 8x8x8 3v4c 9.9 (50.1 / 15.2), fcc 12x12x12 4v4c,
+// 144 q 45.3 (- / 59), 27x27 sheet 2v3c, 64 q 1.03 (1.52 / -; 1.33 before the tile list).  Error against 64 bits
+// (2-norm): 1.6e-7 to 2.0e-7 (correlation kernel 1.6e-7 to 4.0e-7).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -72,12 +74,12 @@ constexpr int kMmaWarp = 12, kB0 = 14;         // two MMA issue warps, B produce
 constexpr int kThreads = 512;
 // 128 registers a thread at launch; 168 + 168 + 112 + 64 = 4 x 128
 constexpr int kRegEpi = 168, kRegGather = 112, kRegIssue = 64;
-constexpr int kMaxStages = 6;                  // B ring depth at most
-constexpr int kAStages = 4;                    // A tiles in tensor memory (even, as the ring's depth)
+constexpr int kMaxStages = 6;                  // B ring depth at most, in panels of 32 complex K
+constexpr int kASlots = 4;                     // A tiles of 32 complex K in tensor memory
 constexpr int kGThreads = kGWarps * 32;
 constexpr int kNCols = 64;                     // columns (k', band) of a pass at most
 constexpr int kAcc = 2 * kNCols;               // one accumulator: Re [0, 64), Im [64, 128)
-constexpr int kTKC = 32;                       // complex K values per stage
+constexpr int kTKC = 32;                       // complex K values of a packed panel
 constexpr int kACols = 64;                     // one A tile in TMEM: two K16 halves x (Re hi, Im hi, Re lo, Im lo) x 8
 constexpr int kImgRow = 256;                   // packed image of 32 K values: hi row (128 B), lo row (128 B)
 size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
@@ -85,24 +87,27 @@ size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 struct TpGeo {
   int q_begin, nqc;
   long long vbase;
-  int nkc;                                      // K chunks of the packed images (tc_kpad / 32)
+  int nkc;                                      // K panels of the packed images (tc_kpad / 32)
+  int sub;                                      // panels per stage (a promoted chunk): 1 or 2
   int stages, nmax;                             // ring depth; B rows per stage (max columns, multiple of 16)
   int cap;                                      // rows of the position table
-  int stage_bytes;
+  int sub_bytes, stage_bytes;                   // a panel's B rows; a stage's
   int by, bz, box_n, box_c;                     // difference box of S(k): dims, entries, key of G1 = 0
   int rowbox, nwords, wpl;                      // row box: entries, bit words, words per (x, y) line
   int o_bar, o_box, o_pkey, o_kkey, o_rows, o_bits, o_slot, o_binfo, o_bptr, o_binv, o_ptab;
   size_t smem;                                  // dynamic shared memory incl. 1 KB alignment slack
 };
 
-TpGeo tp_geo(const DevSys& d, int stages, int cap) {
+TpGeo tp_geo(const DevSys& d, int sub, int stages, int cap) {
   TpGeo g{};
+  g.sub = sub;
   g.stages = stages;
   g.cap = cap;
   g.nkc = d.tc_kpad / kTKC;
   const int mb = d.nv > d.nc ? d.nv : d.nc;
   g.nmax = (d.tc_rsize * mb + 15) / 16 * 16;
-  g.stage_bytes = 2 * g.nmax * umma::kRow;      // B hi rows, B lo rows
+  g.sub_bytes = 2 * g.nmax * umma::kRow;        // B hi rows, B lo rows
+  g.stage_bytes = sub * g.sub_bytes;
   const int rx = d.fwf[0] + d.fpair[0], ry = d.fwf[1] + d.fpair[1], rz = d.fwf[2] + d.fpair[2];
   g.by = 2 * ry + 1;
   g.bz = 2 * rz + 1;
@@ -112,7 +117,7 @@ TpGeo tp_geo(const DevSys& d, int stages, int cap) {
   g.wpl = (2 * d.fpair[2] + 1 + 31) / 32;
   g.nwords = (2 * d.fpair[0] + 1) * (2 * d.fpair[1] + 1) * g.wpl;
   size_t o = (size_t)stages * g.stage_bytes;
-  g.o_bar = (int)o; o += align16((size_t)(2 * stages + 2 * kAStages + 2 * kGroups + 4) * 8 + 8 * sizeof(int));
+  g.o_bar = (int)o; o += align16((size_t)(2 * stages + 2 * (kASlots / sub) + 2 * kGroups + 4) * 8 + 8 * sizeof(int));
   g.o_box = (int)o; o += align16((size_t)g.box_n * 8);
   g.o_pkey = (int)o; o += align16((size_t)d.npw_max * 4);
   g.o_kkey = (int)o; o += align16((size_t)d.tc_kpad * 4);
@@ -211,8 +216,10 @@ __global__ void tcpair_pack_kernel(DevSys d, const float2* __restrict__ coef, co
 }
 
 // ---------------------------------------------------------------- tile table of a q range
-// blist[(k nreg + r) rsize + slot] = block (k, k') of the range with k' in region r at its slot, else -1.
-__global__ void tcpair_tiles_kernel(DevSys d, int q_begin, int nqc, int* __restrict__ blist) {
+// blist[(k nreg + r) rsize + slot] = block (k, k') of the range with k' in region r at its slot, else -1;
+// flag[r nkpt + k] = 1 where the tile has a block.
+__global__ void tcpair_tiles_kernel(DevSys d, int q_begin, int nqc, int* __restrict__ blist,
+                                    unsigned char* __restrict__ flag) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)nqc * d.nkpt) return;
   const int q = q_begin + (int)(t / d.nkpt), k = (int)(t % d.nkpt);
@@ -221,6 +228,46 @@ __global__ void tcpair_tiles_kernel(DevSys d, int q_begin, int nqc, int* __restr
   int r, s;
   region_of(d, d.blocks[b].y, r, s);
   blist[((size_t)k * d.tc_nreg + r) * d.tc_rsize + s] = b;
+  flag[(size_t)r * d.nkpt + k] = 1;
+}
+
+// The tiles with a block, region-major (the CTAs in flight share one region's packed B rows, which stay in L2), and
+// their number in counter[1].  One CTA, 16 flags a thread and sweep.  A q chunk touches a few of the regions, and
+// the empty tiles were found one by one before, with an atomic and two barriers of the CTA each: 0.35 of 1.3 ms at 64 q
+// of the 27 x 27 sheet.
+constexpr int kListThreads = 1024;
+__global__ __launch_bounds__(kListThreads) void tcpair_list_kernel(const unsigned char* __restrict__ flag, int ntiles,
+                                                                  int* __restrict__ counter, int* __restrict__ list) {
+  __shared__ int wsum[kListThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int base = 0;
+  for (int t0 = 0; t0 < ntiles; t0 += 16 * kListThreads) {
+    const int t = t0 + 16 * tid;
+    uint4 f = make_uint4(0u, 0u, 0u, 0u);        // flags are zero past the last tile (to a multiple of 16)
+    if (t < ntiles) f = *reinterpret_cast<const uint4*>(flag + t);
+    const unsigned w[4] = {f.x, f.y, f.z, f.w};
+    const int n = __popc(f.x) + __popc(f.y) + __popc(f.z) + __popc(f.w);
+    int incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int i = 0; i < kListThreads / 32; ++i) {
+      before += i < warp ? wsum[i] : 0;
+      all += wsum[i];
+    }
+    int at = base + before + incl - n;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if ((w[i / 4] >> (8 * (i % 4))) & 1u) list[at++] = t + i;
+    base += all;
+    __syncthreads();
+  }
+  if (tid == 0) counter[1] = base;
 }
 
 // ---------------------------------------------------------------- the GEMM tiles
@@ -245,18 +292,21 @@ __device__ __forceinline__ void write_pass(const float (&re)[kNCols], const floa
   }
 }
 
+template <int SUB>
 __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const float2* __restrict__ coef,
                                                              const float* __restrict__ scale,
                                                              const unsigned char* __restrict__ bimg,
                                                              const int* __restrict__ blist, int* __restrict__ counter,
+                                                             const int* __restrict__ list,
                                                              float2* __restrict__ out,
                                                              const __grid_constant__ TpGeo g, int* status) {
+  constexpr int kAStages = kASlots / SUB, kACols_ = SUB * kACols, kChunk = SUB * kTKC;
   extern __shared__ __align__(1024) unsigned char tp_smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)tp_smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full_b = (uint64_t*)(sm + g.o_bar);   // [stages] B rows landed
   uint64_t* empty_b = full_b + g.stages;          // [stages] MMAs done with the B stage
-  uint64_t* full_a = empty_b + g.stages;          // [4] A tile written to tensor memory
-  uint64_t* empty_a = full_a + kAStages;          // [4] MMAs done with the A tile
+  uint64_t* full_a = empty_b + g.stages;          // [slots] A tile written to tensor memory
+  uint64_t* empty_a = full_a + kAStages;          // [slots] MMAs done with the A tile
   uint64_t* tfull = empty_a + kAStages;           // [group][2] accumulator holds a chunk of one of the group's passes
   uint64_t* tempty = tfull + 2 * kGroups;          // [2] accumulator promoted
   uint64_t* drain = tempty + 2;                    // [2] every MMA of an issue warp complete
@@ -274,7 +324,7 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
   short* ptab = (short*)(sm + g.o_ptab);           // [row][slot] sphere position of the row on the slot's block, or -1
 
   const int tid = threadIdx.x, warp = umma::uniform(tid >> 5), lane = tid & 31;
-  const int ntiles = d.nkpt * d.tc_nreg, rs = d.tc_rsize;
+  const int rs = d.tc_rsize;
   const int f0 = d.fwf[0], f1 = d.fwf[1], f2 = d.fwf[2];
   const int kb1 = 2 * f1 + 1, kb2 = 2 * f2 + 1;
   const int p0 = d.fpair[0], p1 = d.fpair[1], p2 = d.fpair[2];
@@ -326,28 +376,18 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
   auto next_tile = [&]() -> bool {
     sc += (unsigned)(nb * nmt * nch);
     pc += (unsigned)(nb * nmt);
-    int tile;
-    while (true) {
-      all_bar();                                 // every role is done with the previous tile
-      if (tid == 0) {
-        iv[2] = *fail ? ntiles : atomicAdd(counter, 1);
-        iv[5] = 0;
-      }
-      all_bar();
-      const int t_ = iv[2];
-      if (t_ >= ntiles) return false;
-      // region-major order: the CTAs in flight share one region's packed B rows, which stay in L2
-      r = t_ / d.nkpt;
-      k = t_ - r * d.nkpt;
-      tile = k * d.tc_nreg + r;
-      for (int i = tid; i < rs; i += kThreads) {
-        const int b = blist[(size_t)tile * rs + i];
-        slot[i] = b;
-        if (b >= 0) iv[5] = 1;
-      }
-      all_bar();
-      if (iv[5]) break;
+    all_bar();                                   // every role is done with the previous tile
+    if (tid == 0) {
+      const int i = *fail ? -1 : atomicAdd(counter, 1);
+      iv[2] = i >= 0 && i < counter[1] ? list[i] : -1;
     }
+    all_bar();
+    const int t_ = iv[2];
+    if (t_ < 0) return false;
+    r = t_ / d.nkpt;
+    k = t_ - r * d.nkpt;
+    for (int i = tid; i < rs; i += kThreads) slot[i] = blist[((size_t)k * d.tc_nreg + r) * rs + i];
+    all_bar();
     kc = umma::uniform(d.tc_kcount[r]);
     // ---- tile setup: blocks per slot, K keys, sphere keys of k, rows
     for (int i = tid; i < g.nwords; i += kThreads) bits[i] = 0u;
@@ -426,11 +466,21 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
     all_bar();
     MT = umma::uniform(iv[3]);
     if (MT <= g.cap) {                           // (a larger union: per pass, below)
-      for (int i = tid; i < MT * rs; i += kThreads) ptab[i] = position(rows[i / rs], binfo[i % rs]);
+      for (int i0 = tid; i0 < MT * rs; i0 += 4 * kThreads) {   // four lookups in flight
+        short v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = min(i0 + u * kThreads, MT * rs - 1), row = i / rs;
+          v[u] = position(rows[row], binfo[i - row * rs]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i0 + u * kThreads < MT * rs) ptab[i0 + u * kThreads] = v[u];
+      }
       all_bar();
     }
     nmt = (MT + 127) / 128;
-    nch = (kc + kTKC - 1) / kTKC;
+    nch = (kc + kChunk - 1) / kChunk;
     return true;
   };
 
@@ -443,15 +493,15 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
       const int gt = tid - kG0 * 32, q4 = warp & 3;
       const uint32_t box_u = smem_u32(box);
       uint2 x[16];
-      auto load16 = [&](uint32_t at, int k0) {   // 16 K values of this row
+      auto load16 = [&](uint32_t at_, int k0) {  // 16 K values of this row
         const int4* kp = reinterpret_cast<const int4*>(kkey + k0);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int4 t = kp[q];
-          x[4 * q] = lds64(at + (uint32_t)t.x);
-          x[4 * q + 1] = lds64(at + (uint32_t)t.y);
-          x[4 * q + 2] = lds64(at + (uint32_t)t.z);
-          x[4 * q + 3] = lds64(at + (uint32_t)t.w);
+          x[4 * q] = lds64(at_ + (uint32_t)t.x);
+          x[4 * q + 1] = lds64(at_ + (uint32_t)t.y);
+          x[4 * q + 2] = lds64(at_ + (uint32_t)t.z);
+          x[4 * q + 3] = lds64(at_ + (uint32_t)t.w);
         }
       };
       auto pack16 = [&](uint32_t (&v)[32]) {
@@ -491,14 +541,24 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
             }
             if (ok) {
               asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              const uint32_t ta = tmem + ((uint32_t)(q4 * 32) << 16) + a_col0 + (uint32_t)(sa * kACols);
+              const uint32_t ta = tmem + ((uint32_t)(q4 * 32) << 16) + a_col0 + (uint32_t)(sa * kACols_);
+              const int k0 = c * kChunk, kn = min(c + 1, nch - 1) * kChunk;
+              const bool two = SUB > 1 && kc - k0 > kTKC;
               uint32_t v[32];
               pack16(v);
-              load16(at, c * kTKC + 16);
+              load16(at, k0 + 16);
               umma::tmem_st32(ta, v);
               pack16(v);
-              load16(at, min(c + 1, nch - 1) * kTKC);
+              load16(at, two ? k0 + kTKC : kn);
               umma::tmem_st32(ta + 32u, v);
+              if (two) {
+                pack16(v);
+                load16(at, k0 + kTKC + 16);
+                umma::tmem_st32(ta + 64u, v);
+                pack16(v);
+                load16(at, kn);
+                umma::tmem_st32(ta + 96u, v);
+              }
               asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
               asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
               __syncwarp();
@@ -531,11 +591,14 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
                 ok = false;
               }
               if (!ok) continue;
-              umma::mbar_arrive_expect_tx(smem_u32(full_b + st), 2 * half_bytes);
-              const uint32_t bh = smem_u32(sm + (size_t)st * g.stage_bytes);
-              const unsigned char* p = bimg + panel_off(d, r, set, c, g.nkc);
-              umma::bulk_g2s(bh, p, half_bytes, smem_u32(full_b + st));
-              umma::bulk_g2s(bh + (uint32_t)(g.nmax * umma::kRow), p + half_bytes, half_bytes, smem_u32(full_b + st));
+              const int np = min(SUB, (kc - c * kChunk + kTKC - 1) / kTKC);
+              umma::mbar_arrive_expect_tx(smem_u32(full_b + st), 2 * np * half_bytes);
+              for (int u = 0; u < np; ++u) {
+                const uint32_t bh = smem_u32(sm + (size_t)st * g.stage_bytes + (size_t)u * g.sub_bytes);
+                const unsigned char* p = bimg + panel_off(d, r, set, c * SUB + u, g.nkc);
+                umma::bulk_g2s(bh, p, half_bytes, smem_u32(full_b + st));
+                umma::bulk_g2s(bh + (uint32_t)(g.nmax * umma::kRow), p + half_bytes, half_bytes, smem_u32(full_b + st));
+              }
               ++copied;
               if (++st == g.stages) {
                 st = 0;
@@ -553,7 +616,7 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
       unsigned p = pc;
       if (umma::uniform(*fail != 0)) ok = false;
       const uint64_t dstage0 = umma::smem_desc(umma::uniform(smem_u32(sm)));   // B stage st: + st stage_bytes / 16
-      const uint32_t blo = (uint32_t)((g.nmax * umma::kRow) >> 4);
+      const uint32_t blo = (uint32_t)((g.nmax * umma::kRow) >> 4), bsub = (uint32_t)(g.sub_bytes >> 4);
       for (int set = 0; set < 2; ++set) {
         const int nset = set ? nc : nv;
         const uint32_t idesc = tcf::idesc_f16((rs * nset + 15) & ~15);
@@ -569,12 +632,17 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
             if (!ok) continue;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t db = dstage0 + (uint64_t)((st * g.stage_bytes) >> 4);
-            const uint32_t a = tmem + a_col0 + (uint32_t)(sa * kACols), d_re = tmem + own * kAcc;
+            const uint32_t a = tmem + a_col0 + (uint32_t)(sa * kACols_), d_re = tmem + own * kAcc;
             if (leader && buf == own) {
-              if (kc - c * kTKC > 16)
-                tcf::chunk_mmas_ts<2>(d_re, d_re + kNCols, a, db, blo, idesc);
+              const int left = kc - c * kChunk;
+              if (SUB > 1 && left > 48)
+                tcf::chunk_mmas_ts<2 * SUB>(d_re, d_re + kNCols, a, db, blo, bsub, idesc);
+              else if (SUB > 1 && left > 32)
+                tcf::chunk_mmas_ts<2 * SUB - 1>(d_re, d_re + kNCols, a, db, blo, bsub, idesc);
+              else if (left > 16)
+                tcf::chunk_mmas_ts<2>(d_re, d_re + kNCols, a, db, blo, bsub, idesc);
               else
-                tcf::chunk_mmas_ts<1>(d_re, d_re + kNCols, a, db, blo, idesc);
+                tcf::chunk_mmas_ts<1>(d_re, d_re + kNCols, a, db, blo, bsub, idesc);
               mma_commit(smem_u32(empty_a + sa));
               mma_commit(smem_u32(empty_b + st));
               mma_commit(smem_u32(tf + own));
@@ -616,11 +684,11 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
           }
           const int row = mt * 128 + q4 * 32 + lane;
           const bool valid = row < MT;
-          const short* pt = ptab + (size_t)(MT <= g.cap ? row : role * 128 + q4 * 32 + lane) * rs;
+          short* pt = ptab + (size_t)(MT <= g.cap ? row : role * 128 + q4 * 32 + lane) * rs;
           if (MT > g.cap && valid) {
             const char4 G = rows[row];
 #pragma unroll 4
-            for (int b = 0; b < rs; ++b) ptab[(size_t)(role * 128 + q4 * 32 + lane) * rs + b] = position(G, binfo[b]);
+            for (int b = 0; b < rs; ++b) pt[b] = position(G, binfo[b]);
           }
           float re[kNCols], im[kNCols];
 #pragma unroll
@@ -722,22 +790,29 @@ __global__ void tcpair_diag_kernel(DevSys d, const float2* __restrict__ coef, fl
   }
 }
 
-// Ring depth and position-table rows: at least four stages, then a table for up to 1024 rows of a tile (256 serve
-// the two groups' passes), then more stages.  The depth is even, so that a stage's slot always belongs to the same
-// issue warp (which then sees every phase of the slot's barriers).  Depth 0: does not fit shared memory.
+// Panels per stage, ring depth and position-table rows.  Two panels (64 complex K per promotion and per hand-over of a
+// stage) where two such stages and the table of the two groups' passes (256 rows) fit; one panel otherwise.  Two against
+// one, ms: 27x27 sheet 1.03 / 1.13, 32x32 sheet 1.41 / 1.51, 5x5x5 4v4c 1.87 / 2.00, 12x12x12 144 q 45.3 / 47.9, 8x8x8 3v4c
+// 9.9 / 10.6.  The table holds one and a half spheres of rows (512 to 1024) if it can: the rows are the union of
+// spheres whose centres lie within a region of each other, and a larger union is looked up pass by pass.  The depth is
+// even, so that a stage's slot always belongs to the same issue warp (which then sees every phase of the slot's
+// barriers).  Depth 0: does not fit shared memory.
 TpGeo tp_fit(const DevSys& d) {
-  for (int cap = 1024; cap >= 256; cap -= 128)
-    for (int st = kMaxStages; st >= 4; st -= 2) {
-      const TpGeo g = tp_geo(d, st, cap);
-      if (g.smem <= 227 * 1024) return g;
-    }
-  TpGeo g = tp_geo(d, 2, 256);
+  int cap0 = (d.ng_max * 3 / 2 + 127) / 128 * 128;
+  cap0 = cap0 < 512 ? 512 : cap0 > 1024 ? 1024 : cap0;
+  for (int sub = 2; sub >= 1; --sub)
+    for (int cap = cap0; cap >= 256; cap -= 128)
+      for (int st = sub == 2 ? 4 : kMaxStages; st >= (sub == 2 ? 2 : 4); st -= 2) {
+        const TpGeo g = tp_geo(d, sub, st, cap);
+        if (g.smem <= 227 * 1024) return g;
+      }
+  TpGeo g = tp_geo(d, 1, 2, 256);
   if (g.smem > 227 * 1024) g.stages = 0;
   return g;
 }
 
 struct TpWs {
-  size_t bimg, blist, counter, scale, total;
+  size_t bimg, blist, counter, flag, list, scale, total;
 };
 
 TpWs tp_ws(const DevSys& d) {
@@ -746,6 +821,8 @@ TpWs tp_ws(const DevSys& d) {
   w.bimg = o; o += ((size_t)d.nkpt * d.nb * (d.tc_kpad / kTKC) * kImgRow + 255) & ~(size_t)255;
   w.blist = o; o += ((size_t)d.nkpt * d.tc_nreg * d.tc_rsize * sizeof(int) + 255) & ~(size_t)255;
   w.counter = o; o += 256;
+  w.flag = o; o += ((size_t)d.nkpt * d.tc_nreg + 255) & ~(size_t)255;
+  w.list = o; o += ((size_t)d.nkpt * d.tc_nreg * sizeof(int) + 255) & ~(size_t)255;
   w.scale = o; o += ((size_t)2 * d.nkpt * d.nb * sizeof(float) + 255) & ~(size_t)255;
   w.total = o;
   return w;
@@ -765,7 +842,7 @@ int tcpair_valid(const DevSys& d) {
 // route needs tiles for every SM and columns in use: at least 304 tiles, and at least 30 of the 2 x 64 columns of a
 // tile's two band sets on average (regions of the mesh k + q touches are counted at one k off the region grid).
 // Measured, this kernel against gcorr_kernel: 7x7x7 2v2c, 49 q (28 columns) 0.49 against 0.41 ms; 27x27 sheet 2v3c, 64 q
-// (32) 1.33 / 1.52; 5x5x5 4v4c (40) 1.98 / 3.91; 32x32 sheet 3v3c, 64 q 1.73 / 2.61; 8x8x8 3v4c (112) 10.5 / 50.1; 4x4x4
+// (32) 1.03 / 1.52; 5x5x5 4v4c (40) 1.87 / 3.91; 32x32 sheet 3v3c, 64 q 1.41 / 2.61; 8x8x8 3v4c (112) 9.9 / 50.1; 4x4x4
 // 3v3c (256 tiles) 0.131 / 0.117; 3x3x3 1v2c (27 tiles) 0.054 / 0.024.  With k-point symmetry only scattered
 // representative blocks are left and the tiles are nearly empty.
 int tcpair_preferred(const DevSys& d, int q_begin, int q_end) {
@@ -792,21 +869,14 @@ size_t tcpair_ws_bytes(const DevSys& d) { return tcpair_valid(d) ? kWsSlack + tp
 int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, int q_begin, int q_end,
                   long long vbase, int* status, void* stream) {
   if (!tcpair_valid(d)) return (int)cudaErrorInvalidValue;
-  static int attr_dev = -1, num_sms = 0;
-  static size_t attr_smem = 0;
   TpGeo g = tp_fit(d);
-  int dev = 0;
+  auto kernel = g.sub == 2 ? tcpair_kernel<2> : tcpair_kernel<1>;
+  int dev = 0, num_sms = 0;
   int e = (int)cudaGetDevice(&dev);
   if (e) return e;
-  if (attr_dev != dev || attr_smem < g.smem) {
-    e = (int)cudaFuncSetAttribute((const void*)tcpair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(227 * 1024));
-    if (e) return e;
-    e = (int)cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e) return e;
-    attr_dev = dev;
-    attr_smem = 227 * 1024;
-  }
+  if ((e = (int)cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev))) return e;
+  if ((e = (int)cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)))
+    return e;
   cudaStream_t st = (cudaStream_t)stream;
   const TpWs w = tp_ws(d);
   unsigned char* base = ws_base(ws);
@@ -824,13 +894,15 @@ int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, in
   if ((e = (int)cudaGetLastError())) return e;
   if ((e = (int)cudaMemsetAsync(blist, 0xFF, w.counter - w.blist, st))) return e;
   const long long nt = (long long)g.nqc * d.nkpt;
-  tcpair_tiles_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(d, q_begin, g.nqc, blist);
-  if ((e = (int)cudaGetLastError())) return e;
-  if ((e = (int)cudaMemsetAsync(counter, 0, sizeof(int), st))) return e;
+  if ((e = (int)cudaMemsetAsync(counter, 0, w.list - w.counter, st))) return e;
+  tcpair_tiles_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(d, q_begin, g.nqc, blist, base + w.flag);
   const int ntiles = d.nkpt * d.tc_nreg;
+  int* list = (int*)(base + w.list);
+  tcpair_list_kernel<<<1, kListThreads, 0, st>>>(base + w.flag, ntiles, counter, list);
+  if ((e = (int)cudaGetLastError())) return e;
   const int grid = ntiles < num_sms ? ntiles : num_sms;
-  tcpair_kernel<<<grid, kThreads, g.smem, st>>>(d, (const float2*)coef, scale, bimg, blist, counter,
-                                                (float2*)rho_dir, g, status);
+  kernel<<<grid, kThreads, g.smem, st>>>(d, (const float2*)coef, scale, bimg, blist, counter, list, (float2*)rho_dir, g,
+                                         status);
   if ((e = (int)cudaGetLastError())) return e;
   if (q_begin == 0) {
     tcpair_diag_kernel<<<d.nkpt, 256, 0, st>>>(d, (const float2*)coef, (float2*)rho_dir, vbase);
