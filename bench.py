@@ -194,7 +194,7 @@ class Step:
                                F.P, None, 0, 0, F.ws_pair)
         mark("realspace+exchange")
         bse.bse_build_kernel(plan, 0, bse.BSE_BK_INIT, F.rho_x, None, 0, 0, None, self.en, spec.delta, prec, F.H,
-                             F.ws_kernel if prec == bse.BSE_PREC_BF16X3 else None)
+                             F.ws_kernel)
         mark("exchange_kernel")
         fdir = bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if self.tensor_pair(prec) else 0)
         for c, (q0, q1) in enumerate(F.chunks):
@@ -216,16 +216,18 @@ class Step:
         return prec == bse.BSE_PREC_BF16X3 and bool(self.F.info["tensor_pair"])
 
     def kernels_per_step(self, prec):
-        """Kernel launches of one step: realspace, exchange densities, dipole, K^x (BF16x3: operand split and
-        Gram kernel); per chunk the direct densities (FP32: the correlation kernel; BF16x3: image packing, tile
-        table and the tcgen05 kernel, plus the FP64 G = 0 overlaps on the chunk holding q = 0) and the direct
-        term (FP32: W.rho GEMM + block kernel; BF16x3: two operand splits, the tcgen05 GEMM and the block
-        kernel); the Haydock kernel."""
-        from paper_1206_3518_gb300 import bse
-        mixed = prec == bse.BSE_PREC_BF16X3
-        pair = 3 if self.tensor_pair(prec) else 1
-        per_chunk = pair + (4 if mixed else 2)
-        return 4 + (1 if mixed else 0) + per_chunk * len(self.F.chunks) + (1 if self.tensor_pair(prec) else 0) + 1
+        """Kernel launches of one step: realspace, exchange densities, dipole, K^x (operand split and Gram kernel);
+        per chunk the direct densities (the correlation kernel, or on the tensor cores scales, image packing, tile
+        table, tile list and the tcgen05 kernel, plus the FP64 G = 0 overlaps on the chunk holding q = 0) and the
+        direct term (two operand splits, the tcgen05 GEMM and the block kernel); the Haydock kernel."""
+        tensor = self.tensor_pair(prec) or tensor_default(self.spec, self.F.info)
+        return 5 + ((5 if tensor else 1) + 4) * len(self.F.chunks) + (1 if tensor else 0) + 1
+
+
+def tensor_default(spec, inf):
+    """Whether a step without BSE_PD_TENSOR takes the direct densities on the tensor cores all the same: a tile (k, region)
+    for every SM twice over, at the q chunks of whole mesh planes that this file uses."""
+    return bool(inf["tensor_pair"]) and not inf["kpoint_symmetry"] and spec.nkpt >= 304
 
 
 def stage_times(marks_per_step):
@@ -534,17 +536,18 @@ def run_tddft(args, dev, spec, s, en, F, peaks):
     torch.cuda.synchronize()
     bse.bse_status_read(plan)
     t = [statistics.mean(m[i].elapsed_time(m[i + 1]) for m in evs) for i in range(4)]
-    flops = 2.0 * 8.0 * nw * ng * ng * dim            # two weighted Gram terms, 8 flops per complex MAC
+    flops = 24.0 * nw * ng * (ng + 1) * dim           # 4 weights x (Re, Im) of the pairs G <= G', 3 split products
     ach = flops / (t[0] / 1e3) / 1e12
-    fp32 = _fp32_peak(peaks)
+    peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
     er = e_rpa.cpu().numpy()
     ea = e_alda.cpu().numpy()
     i = int(abs(s.omega).argmin())
     return {"workload": f"{spec.name}, q -> 0 sphere of {ng} G, {dim} transitions, {nw} w, eta {eta:.4f} Ha",
             "chi0_ms": t[0], "alda_kernel_ms": t[1], "eps_m_rpa_ms": t[2], "eps_m_alda_ms": t[3],
-            "chi0_roofline": {"bound": "alu", "kernel": "chi0_kernel", "achieved": ach, "peak": fp32,
-                              "unit": "TFLOP/s", "frac": ach / fp32,
-                              "work": "2 x 8 FP32 flops per complex MAC of nw ng0^2 dim"},
+            "chi0_roofline": {"bound": "tensor", "kernel": "gemm_kernel (chi~0)", "achieved": ach, "peak": peak,
+                              "unit": "TFLOP/s", "frac": ach / peak,
+                              "work": "issued FP16x3 flops of the real product of the weights (4 per frequency) with "
+                                      "Re, Im of the pairs G <= G' over dim transitions"},
             "eps_m_static_rpa": float(er[i].real), "eps_m_static_alda": float(ea[i].real),
             "static_frequency_ha": float(s.omega[i])}
 
@@ -925,7 +928,7 @@ def pair_work(plan, spec, inf):
         blk, _ = bse.bse_pair_blocks(plan, 0, q)
         cmac += ng * sum(npw[int(k2)] for _, k2 in blk)
     return {"method": "correlation", "variant": current, "cmac": cmac * (spec.nv ** 2 + spec.nc ** 2),
-            "tensor": bool(inf["tensor_pair"])}
+            "tensor": bool(inf["tensor_pair"]), "tensor_default": tensor_default(spec, inf)}
 
 
 def _fp32_peak(peaks):
@@ -940,15 +943,15 @@ def stage_rooflines(st, spec, inf, peaks, src, nchunks, pw, prec):
     fp32 = _fp32_peak(peaks)
     out = {}
     ms = st["pair_direct"]
-    if prec != 0 and pw.get("tensor"):
+    if pw.get("tensor") if prec != 0 else pw.get("tensor_default"):
         useful = 24.0 * pw["cmac"]
         peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
         same = (TCPAIR_TRAFFIC["shape"] == (spec.lattice, spec.nv, spec.nc, spec.ecut)
                 and TCPAIR_TRAFFIC["sha1"] == _tcpair_sources_sha1())
         out["pair_direct"] = {
             "bound": "tensor", "kernel": "tcpair_kernel", "achieved": useful / (ms / 1e3) / 1e12, "peak": peak,
-            "unit": "TFLOP/s", "frac": useful / (ms / 1e3) / 1e12 / peak, "launches_per_step": 3 * nchunks + 1,
-            "work": "BF16x3 split-complex flops of the correlation itself: 3 hi/lo products x 8 real flops per "
+            "unit": "TFLOP/s", "frac": useful / (ms / 1e3) / 1e12 / peak, "launches_per_step": 5 * nchunks + 1,
+            "work": "FP16x3 split-complex flops of the correlation itself: 3 hi/lo products x 8 real flops per "
                     "complex multiply-add, sum over upper blocks of NG(q) |S(k')| (Nv^2 + Nc^2) (the padding of "
                     "a tile's rows and K positions to the union of its spheres is not counted); the stage's "
                     "whole time (image packing and tile table included)",
@@ -982,42 +985,28 @@ def stage_rooflines(st, spec, inf, peaks, src, nchunks, pw, prec):
     ms = st["direct_contract"]
     w = min(spec.nv ** 2, spec.nc ** 2)
     cmac_wr = float(nb) * w * ng * ng
-    cmac_blk = float(nb) * spec.nv ** 2 * spec.nc ** 2 * ng
-    if prec == 0:
-        flops = 8.0 * (cmac_wr + cmac_blk)
-        out["direct_contract"] = {
-            "bound": "alu", "kernel": "gemm_wr + block_kernel", "achieved": flops / (ms / 1e3) / 1e12, "peak": fp32,
-            "unit": "TFLOP/s", "frac": flops / (ms / 1e3) / 1e12 / fp32, "launches_per_step": 2 * nchunks,
-            "work": "8 flops per complex MAC of W.R (ng_max^2 min(Nv^2, Nc^2) per block) and the block products",
-            "traffic": None, "peak_source": "derived FP32 CUDA-core peak"}
-    else:
-        issued = 24.0 * cmac_wr
-        peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
-        out["direct_contract"] = {
-            "bound": "tensor", "kernel": "split_a/split_b + tc_gemm_wr + block_kernel",
-            "achieved": issued / (ms / 1e3) / 1e12, "peak": peak, "unit": "TFLOP/s",
-            "frac": issued / (ms / 1e3) / 1e12 / peak, "launches_per_step": 4 * nchunks,
-            "work": "issued BF16 MMA flops of W.R: 3 hi/lo products x 8 real flops per complex MAC, "
-                    "ng_max^2 min(Nv^2, Nc^2) per block; the whole stage's time (splits and block products "
-                    "included)",
-            "traffic": None, "peak_source": src + " (sustained bf16: timed inside a long step)"}
+    issued = 24.0 * cmac_wr
+    peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
+    out["direct_contract"] = {
+        "bound": "tensor",
+        "kernel": "operand splits + " + ("gemm_kernel (W.rho)" if prec == 0 else "tc_gemm_wr") + " + block_kernel",
+        "achieved": issued / (ms / 1e3) / 1e12, "peak": peak, "unit": "TFLOP/s",
+        "frac": issued / (ms / 1e3) / 1e12 / peak, "launches_per_step": 4 * nchunks,
+        "work": "issued MMA flops of W.R: 3 hi/lo products x 8 real flops per complex MAC, "
+                "ng_max^2 min(Nv^2, Nc^2) per block; the whole stage's time (splits and block products "
+                "included)",
+        "traffic": None, "peak_source": src + " (sustained bf16: timed inside a long step)"}
     ms = st["exchange_kernel"]
     cmac_x = float(dim) * dim * inf["ng0"] / 2
-    if prec == 0:
-        flops = 8.0 * cmac_x
-        out["exchange_kernel"] = {"bound": "alu", "kernel": "init_kernel", "achieved": flops / (ms / 1e3) / 1e12,
-                                  "peak": fp32, "unit": "TFLOP/s", "frac": flops / (ms / 1e3) / 1e12 / fp32,
-                                  "work": "8 flops per complex MAC of rho_x^H vbar rho_x over the upper triangle",
-                                  "traffic": None, "peak_source": "derived FP32 CUDA-core peak", "launches_per_step": 1}
-    else:
-        flops = 24.0 * cmac_x
-        peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
-        out["exchange_kernel"] = {
-            "bound": "tensor", "kernel": "gram_split_kernel + gram_kernel", "achieved": flops / (ms / 1e3) / 1e12,
-            "peak": peak, "unit": "TFLOP/s", "frac": flops / (ms / 1e3) / 1e12 / peak,
-            "work": "BF16x3 split-complex flops (24 per complex MAC) of rho_x^H vbar rho_x over the upper triangle; "
-                    "the stage's whole time (operand split included)",
-            "traffic": None, "peak_source": src + " (sustained bf16: timed inside a long step)", "launches_per_step": 2}
+    flops = 24.0 * cmac_x
+    peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
+    out["exchange_kernel"] = {
+        "bound": "tensor", "kernel": "split_y_kernel + gemm_kernel (exchange)" if prec == 0 else
+        "gram_split_kernel + gram_kernel", "achieved": flops / (ms / 1e3) / 1e12,
+        "peak": peak, "unit": "TFLOP/s", "frac": flops / (ms / 1e3) / 1e12 / peak,
+        "work": "split-complex flops (24 per complex MAC) of rho_x^H vbar rho_x over the upper triangle; "
+                "the stage's whole time (operand split included)",
+        "traffic": None, "peak_source": src + " (sustained bf16: timed inside a long step)", "launches_per_step": 2}
     return out
 
 
