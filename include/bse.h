@@ -86,7 +86,7 @@ typedef enum {
 #define BSE_PD_DIRECT    4u   /* A2 direct set rho_vv', rho_cc' of a q range   */
 #define BSE_PD_CHI0      8u   /* rho_vc^{k,k+q} for all k, q of a range (screening input) */
 #define BSE_PD_COUPLING 16u   /* rho_vc', rho_cv' of the upper blocks of a q range (coupling) */
-#define BSE_PD_TENSOR   32u   /* with DIRECT: the direct set on the tensor cores (BF16x3)      */
+#define BSE_PD_TENSOR   32u   /* with DIRECT: the direct set on the tensor cores (FP16x3)      */
 #define BSE_BK_INIT      1u   /* A3 + A5 diagonal: H = diag + 2 K^x (upper)    */
 #define BSE_BK_DIRECT    2u   /* A4 + A5: H -= K^d for a q range, mirror       */
 #define BSE_BK_MIRROR    4u   /* A5 without A4: lower blocks and (B+B^H)/2      */
@@ -190,7 +190,8 @@ bse_status bse_rho_dir_count(const bse_plan* plan, int s, int q_begin, int q_end
  * Two routes give the same densities to FP32 rounding (bse_pair_variants): the
  * plane-wave correlation kernel (second form; the default wherever its band counts
  * are compiled) and the pruned batched 3D FFT of the products on the real-space
- * grid (first form; the default otherwise).
+ * grid (first form; the default otherwise).  Without a chosen variant a direct set with enough blocks per
+ * region of k' goes to the tensor-core form of the correlation (BSE_PD_TENSOR below), to FP32 rounding as well.
  * coef     complex64 [nkpt][nb][npw_max], c_nk(G) in sphere order (zero padded).
  * energies float64  [nkpt][nb], bands ascending (valence first), Ha.
  * rho_x    complex64 [dim][ng_max]: rho_vc^{kk}(G) on the q = 0 sphere (S = (k,v,c)).
@@ -207,12 +208,11 @@ bse_status bse_rho_dir_count(const bse_plan* plan, int s, int q_begin, int q_end
  *          With BSE_PD_DIRECT | BSE_PD_TENSOR the direct set is computed on the tensor cores: for
  *          each k, the blocks whose k' lie in one region of the k' mesh (bse_info.tc_region points)
  *          form one GEMM per band n, D[G][(k', m)] = sum_{G2} conj(c_nk(G2 - G)) c_mk'(G2), rows G the
- *          union of the blocks' q spheres, K the union of the region's spheres S(k'), operands split
- *          hi + lo in BF16 with hi.hi + hi.lo + lo.hi accumulated in FP32 (relative error ~1e-5 of
- *          the largest density instead of FP32 rounding); the G = 0 overlaps of the diagonal blocks
- *          are summed in FP64.  Same layout and vectors as without the flag.  The precision of the
- *          mixed build (bse_build_kernel with BSE_PREC_BF16X3); no counterpart in the paper, which
- *          computes the densities by FFT.
+ *          union of the blocks' q spheres, K the union of the region's spheres S(k'), operands scaled
+ *          by a power of two per (k, band) and split hi + lo in FP16, hi.lo + lo.hi + hi.hi added to FP32
+ *          registers every 32 or 64 complex K (FP32 rounding); the G = 0 overlaps of the diagonal blocks
+ *          are summed in FP64.  Same layout and vectors as without the flag.  No counterpart in the
+ *          paper, which computes the densities by FFT.
  * Errors: BSE_ERR_ARG (range, NULL for a requested output), BSE_ERR_WORKSPACE, BSE_ERR_UNSUPPORTED
  *         (BSE_PD_TENSOR where bse_info.tensor_pair = 0), BSE_ERR_TIMEOUT (a tensor-route wait that
  *         did not end within 2 s, through the status word).
@@ -228,9 +228,10 @@ bse_status bse_pair_densities(bse_plan* plan, int s, unsigned flags,
  *   H = diag(e_ck + delta - e_vk) + 2 K^x - K^d.
  * BSE_BK_INIT writes diag + 2K^x on the upper block triangle (k <= k') (on 128 x 128 tiles: also the
  * lower entries of the diagonal tiles, which DIRECT, MIRROR or SYMFILL then overwrite).  With
- * BSE_PREC_BF16X3 and a workspace (ws, at least bse_workspace_size(BSE_WS_KERNEL) for any chunk)
- * 2K^x = Y^H Y, Y = rho_x diag(sqrt(2 vbar/(Omega Nk))), is a BF16x3 tcgen05 Gram product; with
- * ws = NULL it is FP32 on CUDA cores.
+ * a workspace (ws, at least bse_workspace_size(BSE_WS_KERNEL) for any chunk) 2K^x = Y^H Y,
+ * Y = rho_x diag(sqrt(2 vbar/(Omega Nk))), is a tcgen05 Gram product: BF16x3 with BSE_PREC_BF16X3, FP16x3
+ * with promoted accumulation (FP32 accuracy) with BSE_PREC_FP32; with ws = NULL (FP32: or a smaller one) it
+ * is FP32 on CUDA cores.
  * BSE_BK_DIRECT subtracts K^d for the upper blocks of q in [q_begin, q_end)
  * (rho_dir laid out as in bse_pair_densities for the same range) and writes the
  * mirrored lower block H_k'k = H_kk'^H; diagonal blocks become (B + B^H)/2.
@@ -249,8 +250,9 @@ bse_status bse_pair_densities(bse_plan* plan, int s, unsigned flags,
  * The coupling build and the adjoint need every block and return BSE_ERR_UNSUPPORTED for such plans.
  * W        complex64 [nq][ng_max][ng_max], W_q[p][p'] Hermitian, including 4 pi.
  * H        complex64 [dim][dim] row-major.
- * prec     BSE_PREC_FP32 (CUDA-core FP32) or BSE_PREC_BF16X3 (tcgen05 BF16
- *          hi/lo split products, FP32 accumulation) for the contractions.
+ * prec     BSE_PREC_FP32 (tcgen05 FP16 hi/lo split products of scaled rows, the accumulator added to FP32
+ *          registers every 32 complex K: FP32 accuracy) or BSE_PREC_BF16X3 (tcgen05 BF16 hi/lo split
+ *          products, FP32 accumulation) for the contractions.
  * Errors: BSE_ERR_ARG, BSE_ERR_UNSUPPORTED (precision not built), BSE_ERR_WORKSPACE.
  */
 bse_status bse_build_kernel(bse_plan* plan, int s, unsigned flags,
