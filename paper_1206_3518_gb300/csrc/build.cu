@@ -489,7 +489,7 @@ static size_t split_bytes(const DevSys& d, long long qchunk, long long w) {
 }
 
 // The direct stage's W.rho rows and split images of a q chunk; at least the exchange stage's split images of
-// rho_x (BSE_BK_INIT with BSE_PREC_BF16X3).
+// rho_x (BSE_BK_INIT).
 size_t kernel_ws_bytes(const DevSys& d, long long qchunk) {
   const long long w = direct_width(d);
   const size_t direct = x_bytes(d, qchunk, w) + split_bytes(d, qchunk, w);

@@ -208,8 +208,9 @@ __device__ __forceinline__ void chunk_mmas_real(uint32_t d, uint64_t da, uint32_
                        idesc, (s | kk) != 0 ? 1u : 0u);
 }
 
-// The MMAs of a complex chunk with the A planes in tensor memory at columns a + 0 (Re hi), a + 8 (Im hi), a + 16 (Re lo), a + 24 (Im lo) of
-// the first K16 half, + 32 of the second (two FP16 per 32-bit column, lane = row); A as it is (no conjugation).
+// The MMAs of a complex chunk of NKK K16 groups with the A planes in tensor memory at columns a + 0 (Re hi), a + 8 (Im
+// hi), a + 16 (Re lo), a + 24 (Im lo) of the first group, + 32 per further one (two FP16 per 32-bit column, lane =
+// row), B panels of two groups b_sub apart; A as it is (no conjugation).
 template <int NKK>
 __device__ __forceinline__ void chunk_mmas_ts(uint32_t d_re, uint32_t d_im, uint32_t a, uint64_t db, uint32_t b_lo,
                                               uint32_t b_sub, uint32_t idesc) {
@@ -235,12 +236,12 @@ __device__ __forceinline__ void fail_now(volatile int* fail, int* status) {
   atomicCAS(status, 0, (int)BSE_ERR_TIMEOUT);
 }
 
-// Op: long long ntiles; int* status; static constexpr bool kReal, kConj, kHerm (tiles m0 <= n0
-// of a Hermitian result: the upper triangle is stored with its mirror image, float2* mirror_out(...)); bool tile(long long t, Tile&) (false: nothing
-// to do); float2* row_out(const Tile&, int row) the address of column 0 of a row of the tile; float row_scale(const
-// Tile&, int row), col_scale(const Tile&, int col) the inverse scales; float2 value(const Tile&, int row, int col,
-// float2 sum) the output from the unscaled sum (real: float* row_out, no value()).  Outputs go out through shared memory, 16 columns
-// at a time, so that eight lanes write 128 contiguous bytes of a row (rows stored lane by lane cost 2.8 times the
+// Op: long long ntiles; int* status; static constexpr bool kReal, kConj, kHerm (tiles m0 <= n0 of a Hermitian
+// result: the upper triangle is stored with its mirror image, float2* mirror_out(...)); bool tile(long long t, Tile&)
+// (false: nothing to do); float2* row_out(const Tile&, int row) the address of column 0 of a row of the tile; float
+// row_scale(const Tile&, int row), col_scale(const Tile&, int col) the inverse scales; float2 value(const Tile&, int
+// row, int col, float2 sum) the output from the unscaled sum (real: float* row_out, no value()).  Outputs go out
+// through shared memory, 16 columns at a time, so that eight lanes write 128 contiguous bytes of a row (rows stored lane by lane cost 2.8 times the
 // time of the whole product at 115 columns: 294 us against 106 us without stores).
 template <class Op>
 __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant__ Op op) {

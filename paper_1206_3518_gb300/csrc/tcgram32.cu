@@ -5,6 +5,8 @@
 // s(G) = sqrt(2 vbar(G) / (Omega Nk)), as FP16x3 products with promoted accumulation (tcf16.cuh) on the 128 x 128
 // tiles (I <= J) of the upper triangle and the tiles (I, I - 1) just below it (a block of Nv Nc rows that
 // straddles the row 128 I has upper entries there).  One image of Y serves both operands.
+// Bound by the MMAs (0.70 of the sustained BF16 rate issued at dim 27648).  Measured with the split (ms; before: init_kernel on
+// the FP32 pipes): fcc 4x4x4 3v3c 0.022 (0.030), fcc 8x8x8 3v4c 0.17 (1.65), fcc 12x12x12 4v4c 4.0 (53).
 #include <cuda_runtime.h>
 
 #include "internal.h"

@@ -22,8 +22,8 @@
 //
 // Arithmetic (FP16x3, tcf16.cuh): the coefficients of every (k, band) are scaled by a power of two and split
 // hi + lo in FP16 (22 bits); each real product is hi.lo + lo.hi + hi.hi, and the tensor core's accumulator holds
-// one K chunk (SUB panels of 32 complex values, tp_fit) at a time, which the epilogue warps add to FP32 registers.  The result has the
-// accuracy of the FP32 correlation kernel, so one kernel serves both precisions of the build.  The G = 0 overlaps
+// one K chunk (SUB panels of 32 complex values, tp_fit) at a time, which the epilogue warps add to FP32
+// registers.  The result has the accuracy of the FP32 correlation kernel, so one kernel serves both precisions of the build.  The G = 0 overlaps
 // of the diagonal blocks (k' = k), which meet the q = 0 head of W, are summed again in FP64
 // afterwards (tcpair_diag_kernel).
 //
