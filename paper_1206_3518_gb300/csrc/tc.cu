@@ -300,6 +300,7 @@ __global__ __launch_bounds__(kTcThreads, 1) void tc_gemm_wr(DevSys d, TcArgs a) 
         if (!ok) fail_now(fail, a.status);
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
+      __syncwarp();                             // orders lane 0's acquire before the warp's loads (a shuffle does not)
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int m0 = t.mt * TM, n0 = t.nt * N;

@@ -374,6 +374,7 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
           if (!good) fail_now(fail, op.status);
         }
         good = __shfl_sync(0xffffffffu, good, 0);
+        __syncwarp();                              // orders lane 0's acquire before the warp's loads (a shuffle does not)
         if (!good) {
           ok = false;
           break;

@@ -241,6 +241,7 @@ __global__ __launch_bounds__(kThreads, 1) void gram_kernel(DevSys d, const unsig
         if (!ok) fail_now(fail, status);
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
+      __syncwarp();                             // orders lane 0's acquire before the warp's loads (a shuffle does not)
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int S = I * kTM + ew * 32 + lane;

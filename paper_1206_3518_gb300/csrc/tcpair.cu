@@ -578,6 +578,7 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
     int st = 0, sa = 0;                          // B stage, A slot and accumulator, and their phases
     uint32_t bph = 0u, aph = 0u, cph = 0u, buf = 0u;
     bool ok = true;
+    const bool leader = umma::elect_one();       // one lane for every MMA and commit of the warp: a commit tracks its own thread
     while (next_tile()) {
     if (warp == kB0) {                           // ---- B producer: the region's panel, two bulk copies per stage
       if (lane == 0) {
@@ -610,8 +611,8 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
       __syncwarp();
     } else if (warp < kB0) {                     // ---- MMA issue: the whole warp runs the loop, one lane issues
       // Two warps, one per accumulator (even and odd stages): a stage's three waits take ~300 cycles even when
-      // everything is there, and run while the other warp's MMAs do.  Lanes 0-2 wait on one barrier each.
-      const bool leader = umma::elect_one();
+      // everything is there, and run while the other warp's MMAs do.  Lanes 0-2 wait on one barrier each; the warp barrier
+      // after the vote orders what they acquired before the MMAs of the issuing lane (a vote orders no memory).
       const uint32_t own = (uint32_t)(warp - kMmaWarp);
       unsigned p = pc;
       if (umma::uniform(*fail != 0)) ok = false;
@@ -628,6 +629,7 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
                                                                                    : smem_u32(tempty + buf);
               ok = __all_sync(0xffffffffu, mbar_wait(bar, lane == 0 ? aph : lane == 1 ? bph : cph ^ 1u)) != 0;
               if (!ok && leader) fail_now(fail, status);
+              __syncwarp();
             }
             if (!ok) continue;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -666,6 +668,11 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
     if (warp == kB0 && lane == 0 && *fail)       // copies still in flight after a failure
       for (unsigned c = copied > (unsigned)g.stages ? copied - g.stages : 0u; c < copied; ++c)
         if (!mbar_wait(smem_u32(full_b + c % (unsigned)g.stages), (c / g.stages) & 1u)) break;
+    if (warp < kB0 && leader) {                  // tracks every MMA that this thread issued above
+      mma_commit(smem_u32(drain + warp - kMmaWarp));
+      if (!mbar_wait(smem_u32(drain + warp - kMmaWarp), 0u)) fail_now(fail, status);
+    }
+    __syncwarp();
   } else {                                       // ---- epilogue group: promote its passes, then write them
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegEpi));
     unsigned mine0 = 0u, mine1 = 0u;             // chunks this group has promoted from each accumulator
@@ -735,10 +742,6 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
         }
       }
     }
-  }
-  if (role == 3 && warp < kB0 && lane == 0) {   // tracks every MMA this thread issued above
-    mma_commit(smem_u32(drain + warp - kMmaWarp));
-    if (!mbar_wait(smem_u32(drain + warp - kMmaWarp), 0u)) fail_now(fail, status);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
