@@ -702,18 +702,19 @@ __global__ __launch_bounds__(kThreads, 1) void haydock_kernel(const __grid_const
       }
     }
     __syncthreads();
-    if (warp == 0) {                        // |H v_j|^2 only sets the breakdown threshold: FP32, one warp
-      float hv2 = 0.f;
+    float hv2 = 0.f;                        // |H v_j|^2 only sets the breakdown threshold: FP32, one warp
+    if (warp == 0) {
       for (int r = lane; r < nrows; r += 32) {
         const float4 w = wsm[r];
         hv2 += w.x * w.x + w.z * w.z;
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) hv2 += __shfl_xor_sync(0xffffffffu, hv2, o);
-      if (lane == 0) A.npart[2 * A.grank + 1] = hv2;
     }
     project_partial(A, Vb, wsm, nrows, j + 1);
     if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
+    // published after the step's first barrier: before it, a slower CTA may still be reading the last step's sum
+    if (threadIdx.x == 0) A.npart[2 * A.grank + 1] = hv2;
     reduce_coeffs(A, A.h1, j + 1);
     if (!grid_barrier(A.bar, arrivals, A.status, (unsigned)A.gsize)) return;
     subtract_projection(Vb, wsm, red, hs, A.h1, nrows, j + 1);
