@@ -265,8 +265,7 @@ int launch_block(const DevSys& d, const float2* rho, const float2* X, float2* H,
   const int smem = kBlkWarps * blk_warp_bytes(d.nv * d.nv + d.nc * d.nc);       // at most 54 KB
   const bool even = d.ng_max % 2 == 0 && ((reinterpret_cast<uintptr_t>(rho) | reinterpret_cast<uintptr_t>(X)) & 15) == 0;
   auto kernel = even ? block_kernel<LI, PI, PJ, true> : block_kernel<LI, PI, PJ, false>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return (int)e;
+  if (int e = allow_smem((const void*)kernel)) return e;
   kernel<<<(unsigned)((b_count + kBlkWarps - 1) / kBlkWarps), kBlkWarps * 32, smem, st>>>(d, rho, X, H, q_begin, vbase,
                                                                                          side_c, b_count);
   return (int)cudaGetLastError();

@@ -355,8 +355,7 @@ int launch_gcorr(const DevSys& d, const void* coef, void* out, int kind, int mod
   const Box bx = box_of(d);
   const size_t sm = kind == 3 ? e->split_smem(d, bx) : e->smem[kind](d, bx);
   const GcFn fn = kind == 3 ? e->split : e->fn[kind][pf ? 1 : 0];
-  int err = (int)cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (err) return err;
+  if (int err = allow_smem((const void*)fn)) return err;
   fn<<<(unsigned)cells, threads_of(d), sm, (cudaStream_t)stream>>>(d, (const float2*)coef, (float2*)out,
                                                                           mode, q0, nqc, vbase, bx);
   return (int)cudaGetLastError();

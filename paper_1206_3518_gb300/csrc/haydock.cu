@@ -913,7 +913,7 @@ int run_haydock_batch(const HayJob* jobs, int n, int nsteps, const double* omega
     S.vsk = (int)(fit < (size_t)nsteps ? fit : (size_t)nsteps);
     if (fixed + (size_t)S.vsk * per_vec > dyn) dyn = fixed + (size_t)S.vsk * per_vec;
   }
-  cudaFuncSetAttribute((const void*)haydock_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  if (int e = allow_smem((const void*)haydock_kernel)) return e;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, haydock_kernel, kThreads, dyn);
   if (occ < 1) return -1;
   void* args[] = {&B};

@@ -82,6 +82,11 @@ bse_status cuda_check(int err, const char* what);
 constexpr size_t kWsSlack = 256;
 inline unsigned char* ws_base(void* ws) { return (unsigned char*)(((uintptr_t)ws + 255) & ~(uintptr_t)255); }
 
+// Lets launches of a kernel use up to the device's shared memory beside its static part.  The limit is process-wide state
+// of the kernel: set to the size of one call, it would refuse a larger launch of another thread that set its own size
+// just before.  Every call sets the same value instead.
+int allow_smem(const void* kernel);
+
 // Kernel launchers (defined in the .cu files); all return cudaError_t as int.
 int launch_realspace(const DevSys& d, const void* coef, void* u, void* stream);
 int launch_pair_exchange(const DevSys& d, const void* u, void* rho_x, int* status, void* stream);

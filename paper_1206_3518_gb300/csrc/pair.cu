@@ -542,7 +542,7 @@ int pair_variant_current(const DevSys& d) {
 int launch_realspace(const DevSys& d, const void* coef, void* u, void* stream) {
   const Variant* v = pick(d);
   if (!v) return (int)cudaErrorInvalidValue;
-  cudaFuncSetAttribute((const void*)v->rs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v->rs_smem);
+  if (int e = allow_smem((const void*)v->rs)) return e;
   v->rs<<<d.nkpt * d.nb, kThreads, v->rs_smem, (cudaStream_t)stream>>>(d, (const float2*)coef, (float2*)u);
   if (int e = (int)cudaGetLastError()) return e;
   return (int)cudaMemcpyAsync((char*)u + u_bytes(d), coef, (size_t)d.nkpt * d.nb * d.npw_max * 8,
@@ -554,7 +554,7 @@ int launch_pair_exchange(const DevSys& d, const void* u, void* rho_x, int* statu
   const Variant* v = pick(d);
   if (!v) return (int)cudaErrorInvalidValue;
   const size_t sm = v->pair_smem(d.ng_max);
-  cudaFuncSetAttribute((const void*)v->pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (int e = allow_smem((const void*)v->pair)) return e;
   CUtensorMap tm;
   if (int e = make_tmap(d, v, u, &tm)) return e;
   v->pair<<<d.nkpt, v->threads, sm, (cudaStream_t)stream>>>(d, (const float2*)u, (float2*)rho_x, 0, 0, 0, 0, status, tm);
@@ -579,7 +579,7 @@ int launch_pair_direct(const DevSys& d, void* u, void* rho_dir, int q_begin, int
   const Variant* v = pick(d);
   if (!v) return (int)cudaErrorInvalidValue;
   const size_t sm = v->pair_smem(d.ng_max);
-  cudaFuncSetAttribute((const void*)v->pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (int e = allow_smem((const void*)v->pair)) return e;
   const int nqc = q_end - q_begin;
   const long long ntk = (d.nkpt + kTK - 1) / kTK, ntq = (nqc + kTQ - 1) / kTQ;
   const long long cells = ntq * ntk * kTQ * kTK * (v->merged ? 1 : 2);
@@ -601,7 +601,7 @@ int launch_pair_coupling(const DevSys& d, const void* u, void* rho_cpl, int q_be
   const Variant* v = pick(d);
   if (!v) return (int)cudaErrorInvalidValue;
   const size_t sm = v->pair_smem(d.ng_max);
-  cudaFuncSetAttribute((const void*)v->pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (int e = allow_smem((const void*)v->pair)) return e;
   const int nqc = q_end - q_begin;
   const long long ntk = (d.nkpt + kTK - 1) / kTK, ntq = (nqc + kTQ - 1) / kTQ;
   const long long cells = ntq * ntk * kTQ * kTK * (v->merged ? 1 : 2);
@@ -621,7 +621,7 @@ int launch_pair_chi0(const DevSys& d, const void* u, void* rho, int q_begin, int
   const Variant* v = pick(d);
   if (!v) return (int)cudaErrorInvalidValue;
   const size_t sm = v->pair_smem(d.ng_max);
-  cudaFuncSetAttribute((const void*)v->pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (int e = allow_smem((const void*)v->pair)) return e;
   const long long cells = (long long)(q_end - q_begin) * d.nkpt;
   if (cells >= (1LL << 31)) return (int)cudaErrorInvalidValue;
   CUtensorMap tm;

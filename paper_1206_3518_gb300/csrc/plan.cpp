@@ -29,6 +29,13 @@ bse_status set_error(bse_status st, const std::string& msg) {
   return st;
 }
 
+int allow_smem(const void* kernel) {
+  cudaFuncAttributes a;
+  if (cudaError_t e = cudaFuncGetAttributes(&a, kernel)) return (int)e;
+  return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   227 * 1024 - (int)a.sharedSizeBytes);
+}
+
 bse_status cuda_check(int err, const char* what) {
   if (err == cudaSuccess) return BSE_OK;
   return set_error(BSE_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString((cudaError_t)err));

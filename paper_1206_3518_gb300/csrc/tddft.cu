@@ -332,9 +332,7 @@ size_t solve_smem(int n, int pb) { return ((size_t)n * (pb + 1) + (size_t)pb * (
 template <int PB>
 int launch_solve(int n, int nw, float2* aug, double2* eps_m, float2* xb, cudaStream_t st) {
   const size_t sm = solve_smem(n, PB);
-  if (int e = (int)cudaFuncSetAttribute((const void*)dyson_solve_kernel<PB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)sm))
-    return e;
+  if (int e = allow_smem((const void*)dyson_solve_kernel<PB>)) return e;
   dyson_solve_kernel<PB><<<nw, kSolveThreads, sm, st>>>(n, aug, eps_m, xb);
   return (int)cudaGetLastError();
 }
