@@ -288,7 +288,7 @@ __global__ __launch_bounds__(kTcThreads, 1) void tc_gemm_wr(DevSys d, TcArgs a) 
     __syncwarp();
   } else if (warp >= 4) {                       // epilogue: TMEM lanes 32(w-4).. -> output rows
     const int ew = warp - 4;
-    const bool even = (d.ng_max & 1) == 0;
+    const bool even = (d.ng_max & 1) == 0 && (reinterpret_cast<uintptr_t>(a.X) & 15) == 0;
     unsigned j = 0;
     Tile t;
     for (long long ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
@@ -385,25 +385,18 @@ size_t tc_split_bytes(const DevSys& d, long long qchunk, long long w) {
   const int N = tc_n_tile(d);
   const long long mt = (d.nkpt * w + TM - 1) / TM, nt = (d.ng_max + N - 1) / N;
   const long long kc = (d.ng_max + TKC - 1) / TKC;
-  return (size_t)qchunk * (size_t)kc * ((size_t)mt * 2 * kTileA + (size_t)nt * 2 * N * kRow);
+  return kWsSlack + (size_t)qchunk * (size_t)kc * ((size_t)mt * 2 * kTileA + (size_t)nt * 2 * N * kRow);
 }
 
 // ws holds the split tiles; X is the FP32 output of the products.
 int launch_gemm_wr_tc(const DevSys& d, const void* rho_dir, int q_begin, int q_end, long long vbase,
                       long long max_rows, const void* W, void* X, void* split_ws, int side_c, int* status,
                       void* stream) {
-  static int attr_dev = -1, num_sms = 0;
-  int dev = 0;
+  int dev = 0, num_sms = 0;
   int e = (int)cudaGetDevice(&dev);
+  if (!e) e = (int)cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
+  if (!e) e = (int)cudaFuncSetAttribute((const void*)tc_gemm_wr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
   if (e) return e;
-  if (attr_dev != dev) {
-    e = (int)cudaFuncSetAttribute((const void*)tc_gemm_wr, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kTcSmem);
-    if (e) return e;
-    e = (int)cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e) return e;
-    attr_dev = dev;
-  }
   cudaStream_t st = (cudaStream_t)stream;
   SplitGeo g;
   g.q_begin = q_begin;
@@ -414,7 +407,7 @@ int launch_gemm_wr_tc(const DevSys& d, const void* rho_dir, int q_begin, int q_e
   g.mt_max = (int)((max_rows + TM - 1) / TM);
   g.nt_max = (d.ng_max + g.n_tile - 1) / g.n_tile;
   g.kc_max = (d.ng_max + TKC - 1) / TKC;
-  unsigned char* As = (unsigned char*)split_ws;
+  unsigned char* As = ws_base(split_ws);        // bulk copies read the images
   unsigned char* Bs = As + (size_t)g.nq * g.mt_max * g.kc_max * 2 * kTileA;
   split_a_kernel<<<dim3(g.kc_max, g.mt_max, g.nq), kTcThreads, 0, st>>>(d, (const float2*)rho_dir, As, g);
   split_b_kernel<<<dim3(g.kc_max, g.nt_max, g.nq), kTcThreads, 0, st>>>(d, (const float2*)W, Bs, g);

@@ -293,27 +293,21 @@ __global__ __launch_bounds__(kThreads, 1) void gram_kernel(DevSys d, const unsig
 
 size_t gram_ws_bytes(const DevSys& d) {
   const GramGeo g = geo_of(d);
-  return (size_t)g.ntr * g.nkc * kImg;
+  return kWsSlack + (size_t)g.ntr * g.nkc * kImg;
 }
 
 // diag + 2 K^x on the upper tiles of H with BF16x3 tensor-core products; ws holds the split images.
 int launch_kernel_init_tc(const DevSys& d, const void* rho_x, const double* energies, double delta, void* H,
                           void* ws, int* status, void* stream) {
-  static int attr_dev = -1, num_sms = 0;
-  int dev = 0;
+  int dev = 0, num_sms = 0;
   int e = (int)cudaGetDevice(&dev);
+  if (!e) e = (int)cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
+  if (!e) e = (int)cudaFuncSetAttribute((const void*)gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
   if (e) return e;
-  if (attr_dev != dev) {
-    e = (int)cudaFuncSetAttribute((const void*)gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-    if (e) return e;
-    e = (int)cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e) return e;
-    attr_dev = dev;
-  }
   const GramGeo g = geo_of(d);
   if (g.nkc < 1) return (int)cudaErrorInvalidValue;
   cudaStream_t st = (cudaStream_t)stream;
-  unsigned char* img = (unsigned char*)ws;
+  unsigned char* img = ws_base(ws);             // bulk copies read the images
   gram_split_kernel<<<dim3(g.nkc, g.ntr), kThreads, 0, st>>>(d, (const float2*)rho_x, img, g.nkc);
   if ((e = (int)cudaGetLastError())) return e;
   const int grid = (int)(g.ntiles < num_sms ? g.ntiles : num_sms);
