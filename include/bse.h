@@ -202,7 +202,10 @@ bse_status bse_rho_dir_count(const bse_plan* plan, int s, int q_begin, int q_end
  *          symmetry only the representatives); entry p is taken at G = g_p(q) - G0,
  *          g_p the p-th vector of the q sphere, so q_unf + G = q + g_p.
  * flags    BSE_PD_* stages; REALSPACE must run (once) before the others, with
- *          the same workspace.  Unused outputs may be NULL.  With BSE_PD_COUPLING (not with
+ *          the same workspace.  The other stages only read it, so calls for different outputs may
+ *          share a workspace and overlap on several streams; only BSE_PD_TENSOR on a system whose whole
+ *          mesh would not take that form by default packs its panels there in every call.  Unused outputs
+ *          may be NULL.  With BSE_PD_COUPLING (not with
  *          DIRECT or CHI0) rho_dir receives the coupling densities of bse_build_coupling,
  *          bse_rho_cpl_count(q_begin, q_end) vectors.
  *          With BSE_PD_DIRECT | BSE_PD_TENSOR the direct set is computed on the tensor cores: for

@@ -103,7 +103,9 @@ int gcorr_valid(const DevSys& d);
 int tcpair_valid(const DevSys& d);
 int tcpair_preferred(const DevSys& d, int q_begin, int q_end);
 size_t tcpair_ws_bytes(const DevSys& d);
-int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, int q_begin, int q_end,
+int tcpair_packed(const DevSys& d);
+int launch_tcpair_pack(const DevSys& d, const void* coef, void* copy, void* ws, void* stream);
+int launch_tcpair(const DevSys& d, const void* coef, const void* ws, void* rho_dir, int q_begin, int q_end,
                   long long vbase, int* status, void* stream);
 int launch_pair_direct_tensor(const DevSys& d, void* ws, void* rho_dir, int q_begin, int q_end, long long vbase,
                               int* status, void* stream);

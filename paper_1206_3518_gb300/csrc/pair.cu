@@ -484,12 +484,15 @@ static size_t pair_base_bytes(const DevSys& d) {
   return (u_bytes(d) + (size_t)d.nkpt * d.nb * d.npw_max * 8 + 255) & ~(size_t)255;
 }
 
-// u(r), the coefficient copy, then the tensor route's packed images and tile table (when valid).
+// u(r), the coefficient copy, then the tensor route's packed panels and scales (when valid).
 size_t pair_ws_bytes(const DevSys& d) { return pair_base_bytes(d) + tcpair_ws_bytes(d); }
 
+// Only reads the workspace where the real-space stage packed the panels (tcpair_packed).
 int launch_pair_direct_tensor(const DevSys& d, void* ws, void* rho_dir, int q_begin, int q_end, long long vbase,
                               int* status, void* stream) {
-  return launch_tcpair(d, coef_copy(d, ws), (char*)ws + pair_base_bytes(d), rho_dir, q_begin, q_end, vbase, status,
+  if (!tcpair_packed(d))
+    if (int e = launch_tcpair_pack(d, coef_copy(d, ws), nullptr, (char*)ws + pair_base_bytes(d), stream)) return e;
+  return launch_tcpair(d, coef_copy(d, ws), (const char*)ws + pair_base_bytes(d), rho_dir, q_begin, q_end, vbase, status,
                        stream);
 }
 
@@ -545,6 +548,8 @@ int launch_realspace(const DevSys& d, const void* coef, void* u, void* stream) {
   if (int e = allow_smem((const void*)v->rs)) return e;
   v->rs<<<d.nkpt * d.nb, kThreads, v->rs_smem, (cudaStream_t)stream>>>(d, (const float2*)coef, (float2*)u);
   if (int e = (int)cudaGetLastError()) return e;
+  if (tcpair_packed(d))
+    return launch_tcpair_pack(d, coef, (char*)u + u_bytes(d), (char*)u + pair_base_bytes(d), stream);
   return (int)cudaMemcpyAsync((char*)u + u_bytes(d), coef, (size_t)d.nkpt * d.nb * d.npw_max * 8,
                               cudaMemcpyDeviceToDevice, (cudaStream_t)stream);
 }

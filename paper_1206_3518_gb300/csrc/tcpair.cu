@@ -27,8 +27,8 @@
 // of the diagonal blocks (k' = k), which meet the q = 0 head of W, are summed again in FP64
 // afterwards (tcpair_diag_kernel).
 //
-// tcpair_kernel is persistent (one CTA per SM) and takes tiles (k, region) from a counter, region-major; a pass is
-// one band n and 128 rows.  Four warpgroups share the registers (setmaxnreg):
+// tcpair_kernel is persistent (one CTA per SM); its CTAs deal the tiles (k, region) among themselves (deal_tiles); a pass
+// is one band n and 128 rows.  Four warpgroups share the registers (setmaxnreg):
 //   0, 1  promote the chunks of the even / odd passes into registers and write the pass's densities while the
 //         other group promotes the next pass (the scattered 8-byte stores, one cache line each, take most of
 //         a pass);
@@ -52,6 +52,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "internal.h"
@@ -86,6 +87,8 @@ size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 struct TpGeo {
   int q_begin, nqc;
+  int table;                                    // the list of differences has room in the ring (deal_tiles)
+  int share;                                    // which kMine kThreads tiles of every CTA's share the launch takes
   long long vbase;
   int nkc;                                      // K panels of the packed images (tc_kpad / 32)
   int sub;                                      // panels per stage (a promoted chunk): 1 or 2
@@ -152,25 +155,6 @@ __device__ __forceinline__ uint32_t split_word(float x) {
   return (uint32_t)__half_as_ushort(h) | ((uint32_t)__half_as_ushort(l) << 16);
 }
 
-// ---------------------------------------------------------------- scales
-// scale[k nb + band]: the power of two that puts the largest component of c_{k,band} into [2^14, 2^15); its inverse
-// in the second half.  One warp per (k, band).
-__global__ void tcpair_scale_kernel(DevSys d, const float2* __restrict__ coef, float* __restrict__ scale) {
-  const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (row >= d.nkpt * d.nb) return;
-  const float2* x = coef + (size_t)row * d.npw_max;
-  const int n = d.npw[row / d.nb];
-  float m = 0.f;
-  for (int i = lane; i < n; i += 32) m = fmaxf(m, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  const int e = tcf::scale_exp(m);
-  if (lane == 0) {
-    scale[row] = tcf::pow2(e);
-    scale[d.nkpt * d.nb + row] = tcf::pow2(-e);
-  }
-}
-
 // ---------------------------------------------------------------- packed coefficient panels
 // Packed B panels: for each region r, set (valence bands, then conduction bands) and K chunk c, the rows
 // j = slot nset + m of every k' of the region (slot: its position in the region, m: its band in the set),
@@ -189,85 +173,222 @@ __device__ __forceinline__ void region_of(const DevSys& d, int k2, int& r, int& 
   slot = ((o0 % d.tc_rg[0]) * d.tc_rg[1] + o1 % d.tc_rg[1]) * d.tc_rg[2] + o2 % d.tc_rg[2];
 }
 
-__global__ void tcpair_pack_kernel(DevSys d, const float2* __restrict__ coef, const float* __restrict__ scale,
-                                   unsigned char* __restrict__ bimg, int nkc) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long total = (long long)d.nkpt * d.nb * d.npw_max;
-  if (t >= total) return;
-  const int i = (int)(t % d.npw_max);
-  const long long kb = t / d.npw_max;           // k' * nb + band
-  const int k2 = (int)(kb / d.nb), band = (int)(kb - (long long)k2 * d.nb);
-  if (i >= d.npw[k2]) return;
-  const int set = band < d.nv ? 0 : 1, m = set ? band - d.nv : band, nset = set ? d.nc : d.nv;
-  int r, slot;
-  region_of(d, k2, r, slot);
-  const int l = d.tc_kpos[(size_t)k2 * d.npw_max + i];
-  const float2 c = coef[t];
-  const float sc = scale[kb];
-  const uint32_t re = split_word(c.x * sc), im = split_word(c.y * sc);
-  const int e = l % kTKC, j = slot * nset + m, ph = j & 7;
-  unsigned short* hi = reinterpret_cast<unsigned short*>(bimg + panel_off(d, r, set, l / kTKC, nkc)) + j * 64;
-  unsigned short* lo = hi + d.tc_rsize * nset * 64;
-  const int cr = ((e >> 3) ^ ph) * 8 + (e & 7), ci = ((4 + (e >> 3)) ^ ph) * 8 + (e & 7);
-  hi[cr] = (unsigned short)(re & 0xFFFFu);
-  hi[ci] = (unsigned short)(im & 0xFFFFu);
-  lo[cr] = (unsigned short)(re >> 16);
-  lo[ci] = (unsigned short)(im >> 16);
-}
-
-// ---------------------------------------------------------------- tile table of a q range
-// blist[(k nreg + r) rsize + slot] = block (k, k') of the range with k' in region r at its slot, else -1;
-// flag[r nkpt + k] = 1 where the tile has a block.
-__global__ void tcpair_tiles_kernel(DevSys d, int q_begin, int nqc, int* __restrict__ blist,
-                                    unsigned char* __restrict__ flag) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)nqc * d.nkpt) return;
-  const int q = q_begin + (int)(t / d.nkpt), k = (int)(t % d.nkpt);
-  const int b = d.blkidx[(size_t)q * d.nkpt + k];
-  if (b < 0) return;
-  int r, s;
-  region_of(d, d.blocks[b].y, r, s);
-  blist[((size_t)k * d.tc_nreg + r) * d.tc_rsize + s] = b;
-  flag[(size_t)r * d.nkpt + k] = 1;
-}
-
-// The tiles with a block, region-major (the CTAs in flight share one region's packed B rows, which stay in L2), and
-// their number in counter[1].  One CTA, 16 flags a thread and sweep.  A q chunk touches a few of the regions, and
-// the empty tiles were found one by one before, with an atomic and two barriers of the CTA each: 0.35 of 1.3 ms at 64 q
-// of the 27 x 27 sheet.
-constexpr int kListThreads = 1024;
-__global__ __launch_bounds__(kListThreads) void tcpair_list_kernel(const unsigned char* __restrict__ flag, int ntiles,
-                                                                  int* __restrict__ counter, int* __restrict__ list) {
-  __shared__ int wsum[kListThreads / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int base = 0;
-  for (int t0 = 0; t0 < ntiles; t0 += 16 * kListThreads) {
-    const int t = t0 + 16 * tid;
-    uint4 f = make_uint4(0u, 0u, 0u, 0u);        // flags are zero past the last tile (to a multiple of 16)
-    if (t < ntiles) f = *reinterpret_cast<const uint4*>(flag + t);
-    const unsigned w[4] = {f.x, f.y, f.z, f.w};
-    const int n = __popc(f.x) + __popc(f.y) + __popc(f.z) + __popc(f.w);
-    int incl = n;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += u;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    int before = 0, all = 0;
-    for (int i = 0; i < kListThreads / 32; ++i) {
-      before += i < warp ? wsum[i] : 0;
-      all += wsum[i];
-    }
-    int at = base + before + incl - n;
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-      if ((w[i / 4] >> (8 * (i % 4))) & 1u) list[at++] = t + i;
-    base += all;
-    __syncthreads();
+// scale[k nb + band]: the power of two that puts the largest component of c_{k,band} into [2^14, 2^15); its inverse
+// in the second half.  One warp per (k, band): the plain copy of the coefficients (the other densities read it), their
+// scale, the row's panels zeroed and its sphere points written.  Part of the real-space stage where the route is the
+// default (tcpair_packed), so that the direct stages only read the workspace and a set of q chunks packs once.
+__global__ __launch_bounds__(256) void tcpair_pack_kernel(DevSys d, const float2* __restrict__ coef,
+                                                          float2* __restrict__ copy, float* __restrict__ scale,
+                                                          unsigned char* __restrict__ bimg, int nkc) {
+  const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;   // k nb + band
+  if (row >= d.nkpt * d.nb) return;
+  const int k = row / d.nb, band = row - k * d.nb, n = d.npw[k];
+  const float2* x = coef + (size_t)row * d.npw_max;
+  float2* y = copy ? copy + (size_t)row * d.npw_max : nullptr;
+  float m = 0.f;
+#pragma unroll 4
+  for (int i = lane; i < d.npw_max; i += 32) {
+    const float2 c = x[i];
+    if (copy) y[i] = c;
+    if (i < n) m = fmaxf(m, fmaxf(fabsf(c.x), fabsf(c.y)));
   }
-  if (tid == 0) counter[1] = base;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int e = tcf::scale_exp(m);
+  const float sc = tcf::pow2(e);
+  if (lane == 0) {
+    scale[row] = sc;
+    scale[d.nkpt * d.nb + row] = tcf::pow2(-e);
+  }
+  const int set = band < d.nv ? 0 : 1, nset = set ? d.nc : d.nv;
+  int r, slot;
+  region_of(d, k, r, slot);
+  const int j = slot * nset + (set ? band - d.nv : band), ph = j & 7;
+  const size_t lo_off = (size_t)d.tc_rsize * nset * umma::kRow;
+  unsigned char* img = bimg + panel_off(d, r, set, 0, nkc) + (size_t)j * umma::kRow;   // chunk c: + 2 c lo_off
+  for (int t = lane; t < nkc * 16; t += 32)     // 2 x 128 bytes per chunk
+    *reinterpret_cast<uint4*>(img + (size_t)(t >> 3) * lo_off + (t & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+  __syncwarp();
+  const short* kpos = d.tc_kpos + (size_t)k * d.npw_max;
+#pragma unroll 4
+  for (int i = lane; i < n; i += 32) {
+    const int l = kpos[i], at = l % kTKC;
+    const float2 c = x[i];
+    const uint32_t re = split_word(c.x * sc), im = split_word(c.y * sc);
+    unsigned short* hi = reinterpret_cast<unsigned short*>(img + (size_t)(2 * (l / kTKC)) * lo_off);
+    unsigned short* lo = reinterpret_cast<unsigned short*>(reinterpret_cast<unsigned char*>(hi) + lo_off);
+    const int cr = ((at >> 3) ^ ph) * 8 + (at & 7), ci = ((4 + (at >> 3)) ^ ph) * 8 + (at & 7);
+    hi[cr] = (unsigned short)(re & 0xFFFFu);
+    hi[ci] = (unsigned short)(im & 0xFFFFu);
+    lo[cr] = (unsigned short)(re >> 16);
+    lo[ci] = (unsigned short)(im >> 16);
+  }
+}
+
+// ---------------------------------------------------------------- tiles of a q range
+// A tile is a region and a k.  It has a block where some k' of the region has q = k' - k in the range and k <= k'; whether
+// the first holds depends on the difference of the region's corner and k alone.  The CTAs list the differences that do
+// and deal the tiles (region, difference) among themselves, the i-th one to CTA i mod grid, from the plan's tables
+// alone: a call keeps nothing in the workspace, so calls that share it may overlap.  Regions in order: the CTAs in
+// flight share one region's packed B rows, which stay in L2.  The rows of a tile, and with them its passes, grow with
+// the number of its blocks, so the fullest tiles (in quarters of the region) are dealt first.
+struct Point {                                   // offsets on the mesh
+  int x, y, z;
+};
+__device__ __forceinline__ int wrap(int x, int n) { return x < 0 ? x + n : x >= n ? x - n : x; }
+__device__ __forceinline__ int index_of(const DevSys& d, Point p) { return (p.x * d.nk2 + p.y) * d.nk3 + p.z; }
+__device__ __forceinline__ Point point_of(const DevSys& d, int i) {
+  return {i / (d.nk2 * d.nk3), (i / d.nk3) % d.nk2, i % d.nk3};
+}
+__device__ __forceinline__ Point plus(const DevSys& d, Point a, Point b) {
+  return {wrap(a.x + b.x, d.nk1), wrap(a.y + b.y, d.nk2), wrap(a.z + b.z, d.nk3)};
+}
+__device__ __forceinline__ Point minus(const DevSys& d, Point a, Point b) {
+  return {wrap(a.x - b.x, d.nk1), wrap(a.y - b.y, d.nk2), wrap(a.z - b.z, d.nk3)};
+}
+__device__ __forceinline__ Point corner_of(const DevSys& d, int r) {
+  return {r / (d.tc_nr[1] * d.tc_nr[2]) * d.tc_rg[0], (r / d.tc_nr[2]) % d.tc_nr[1] * d.tc_rg[1],
+          r % d.tc_nr[2] * d.tc_rg[2]};
+}
+// Block in the q range of k and the slot's point, given the difference of the region's corner and k; -1: none.
+__device__ __forceinline__ int block_of(const DevSys& d, const TpGeo& g, int k, Point diff, int s) {
+  const Point o = {s / (d.tc_rg[1] * d.tc_rg[2]), (s / d.tc_rg[2]) % d.tc_rg[1], s % d.tc_rg[2]};
+  const int q = index_of(d, plus(d, diff, o));
+  return q >= g.q_begin && q < g.q_begin + g.nqc ? d.blkidx[(size_t)q * d.nkpt + k] : -1;
+}
+// Points of a region at difference p whose own difference lies in the q range: runs along the last axis that has more
+// than one point, each one or two intervals of q.
+__device__ __forceinline__ int near_points(const DevSys& d, const TpGeo& g, Point p) {
+  if (g.nqc == d.nkpt) return d.tc_rsize;
+  const bool z = d.nk3 > 1;
+  const int len = z ? d.tc_rg[2] : d.tc_rg[1], nl = z ? d.nk3 : d.nk2, at = z ? p.z : p.y, rows = z ? d.tc_rg[1] : 1;
+  const int qe = g.q_begin + g.nqc;
+  int m = 0;
+  for (int a = 0; a < d.tc_rg[0]; ++a)
+    for (int b = 0; b < rows; ++b) {
+      const int x = wrap(p.x + a, d.nk1), base = z ? (x * d.nk2 + wrap(p.y + b, d.nk2)) * d.nk3 : x * d.nk2;
+      m += max(0, min(qe, base + min(at + len, nl)) - max(g.q_begin, base + at));
+      m += max(0, min(qe, base + at + len - nl) - max(g.q_begin, base));
+    }
+  return m;
+}
+
+// Tiles of this CTA (its share of the launch) as region nkpt + k in the first kList words of scratch; returns their
+// number.  (Not inlined: its registers are not those of the passes.)  After the list: sums of the warps, differences (without
+// room for them every difference of the mesh is tried).  Where k lies within the region only some of its points come after
+// k: such tiles are dealt last, and next_tile passes over one without a block.
+constexpr int kMine = 2, kFill = 4;              // list entries per thread; classes of fullness
+constexpr int kList = kMine * kThreads, kDealSums = kFill * (kThreads / 32);
+__device__ __noinline__ int deal_tiles(const DevSys& d, const TpGeo& g, int* scratch) {
+  constexpr int kWarps = kThreads / 32;
+  int* list = scratch;
+  int* sums = list + kList;                      // [class][warp]
+  unsigned* diffs = (unsigned*)(sums + kDealSums);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // exclusive prefix over the threads of n[class], classes in order; returns the total
+  auto prefix = [&](int (&n)[kFill], int (&start)[kFill + 1]) {
+    int incl[kFill];
+#pragma unroll
+    for (int f = 0; f < kFill; ++f) {
+      incl[f] = n[f];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl[f], o);
+        if (lane >= o) incl[f] += u;
+      }
+      if (lane == 31) sums[f * kWarps + warp] = incl[f];
+    }
+    __syncthreads();
+    start[0] = 0;
+#pragma unroll
+    for (int f = 0; f < kFill; ++f) {
+      int before = 0, all = 0;
+      for (int i = 0; i < kWarps; ++i) {
+        const int u = sums[f * kWarps + i];
+        before += i < warp ? u : 0;
+        all += u;
+      }
+      n[f] = start[f] + before + incl[f] - n[f];
+      start[f + 1] = start[f] + all;
+    }
+    __syncthreads();
+  };
+
+  // the differences with a point in the range, by class
+  const int per_d = (d.nkpt + kThreads - 1) / kThreads, d0 = min(tid * per_d, d.nkpt), d1 = min(d0 + per_d, d.nkpt);
+  auto class_of = [&](int m) { return (d.tc_rsize - m) * kFill / d.tc_rsize; };
+  int n[kFill], start[kFill + 1];
+#pragma unroll
+  for (int f = 0; f < kFill; ++f) n[f] = 0;
+  for (int i = d0; i < d1; ++i) {
+    const int m = near_points(d, g, point_of(d, i));
+#pragma unroll
+    for (int f = 0; f < kFill; ++f) n[f] += m > 0 && class_of(m) == f ? 1 : 0;
+  }
+  prefix(n, start);
+  const bool table = g.table != 0;
+  if (table) {
+    for (int i = d0; i < d1; ++i) {
+      const Point p = point_of(d, i);
+      const int m = near_points(d, g, p);
+#pragma unroll
+      for (int f = 0; f < kFill; ++f)
+        if (m > 0 && class_of(m) == f) diffs[n[f]++] = (unsigned)(p.x | p.y << 10 | p.z << 20);
+    }
+    __syncthreads();
+  } else {                                       // one class of all differences
+#pragma unroll
+    for (int f = 0; f < kFill; ++f) start[f + 1] = d.nkpt;
+  }
+
+  // candidate tiles: class, region, difference
+  const long long cand = (long long)d.tc_nreg * start[kFill], per = (cand + kThreads - 1) / kThreads;
+  const long long i0 = min(tid * per, cand), i1 = min(i0 + per, cand);
+  auto scan = [&](auto&& live) {
+    int f = 0;
+    while (f < kFill - 1 && i0 >= (long long)d.tc_nreg * start[f + 1]) ++f;
+    int size = start[f + 1] - start[f];
+    const long long in = i0 - (long long)d.tc_nreg * start[f];
+    int r = size > 0 ? (int)(in / size) : 0, j = (int)(in - (long long)r * size);
+    Point c = corner_of(d, r);
+    for (long long i = i0; i < i1; ++i) {
+      while (j >= size) {                        // next region, or the next class with any difference
+        j = 0;
+        if (size > 0 && ++r < d.tc_nreg) {
+          c = corner_of(d, r);
+          break;
+        }
+        r = 0;
+        c = corner_of(d, 0);
+        ++f;
+        size = start[f + 1] - start[f];
+      }
+      const int at = start[f] + j++;
+      const unsigned w = table ? diffs[at] : 0u;
+      const Point diff = table ? Point{(int)(w & 1023u), (int)((w >> 10) & 1023u), (int)(w >> 20)} : point_of(d, at);
+      const int k = index_of(d, minus(d, c, diff));
+      bool any = k <= index_of(d, {c.x + d.tc_rg[0] - 1, c.y + d.tc_rg[1] - 1, c.z + d.tc_rg[2] - 1});
+      if (any && d.nfill > 0) {                  // representatives only: look the blocks up
+        any = false;
+        for (int s = 0; s < d.tc_rsize && !any; ++s) any = block_of(d, g, k, diff, s) >= 0;
+      }
+      if (any) live(r, k, k > index_of(d, c) ? 1 : 0);
+    }
+  };
+#pragma unroll
+  for (int f = 0; f < kFill; ++f) n[f] = 0;
+  if (i0 < i1) scan([&](int, int, int part) { part ? ++n[1] : ++n[0]; });
+  const bool some = n[0] + n[1] > 0;
+  int total[kFill + 1];
+  prefix(n, total);                              // the tiles with k within the region (part) after all others
+  const int grid = (int)gridDim.x, own = (int)blockIdx.x, all = total[kFill], e0 = g.share * kList;
+  if (some)
+    scan([&](int r, int k, int part) {
+      const int rank = part ? n[1]++ : n[0]++, e = rank / grid;
+      if (rank - e * grid == own && e >= e0 && e < e0 + kList) list[e - e0] = r * d.nkpt + k;
+    });
+  __syncthreads();
+  return all > own ? min(kList, max(0, (all - 1 - own) / grid + 1 - e0)) : 0;
 }
 
 // ---------------------------------------------------------------- the GEMM tiles
@@ -293,11 +414,9 @@ __device__ __forceinline__ void write_pass(const float (&re)[kNCols], const floa
 }
 
 template <int SUB>
-__global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const float2* __restrict__ coef,
+__global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(const __grid_constant__ DevSys d, const float2* __restrict__ coef,
                                                              const float* __restrict__ scale,
                                                              const unsigned char* __restrict__ bimg,
-                                                             const int* __restrict__ blist, int* __restrict__ counter,
-                                                             const int* __restrict__ list,
                                                              float2* __restrict__ out,
                                                              const __grid_constant__ TpGeo g, int* status) {
   constexpr int kAStages = kASlots / SUB, kACols_ = SUB * kACols, kChunk = SUB * kTKC;
@@ -310,7 +429,7 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
   uint64_t* tfull = empty_a + kAStages;           // [group][2] accumulator holds a chunk of one of the group's passes
   uint64_t* tempty = tfull + 2 * kGroups;          // [2] accumulator promoted
   uint64_t* drain = tempty + 2;                    // [2] every MMA of an issue warp complete
-  int* iv = (int*)(drain + 2);                     // tmem, fail, tile, rows, points in the box, blocks
+  int* iv = (int*)(drain + 2);                     // tmem, fail, tile, rows, points in the box, last tile with a block
   volatile int* fail = iv + 1;
   uint2* box = (uint2*)(sm + g.o_box);
   int* pkey = (int*)(sm + g.o_pkey);
@@ -351,9 +470,16 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
     for (int i = 0; i < 2; ++i) mbar_init(smem_u32(drain + i), 1);
     iv[1] = 0;
     iv[4] = 0;
+    iv[5] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int i = tid; i < g.box_n; i += kThreads) box[i] = make_uint2(0u, 0u);
+  const int nmine = deal_tiles(d, g, (int*)sm);  // (the ring is not in use yet)
+  int mine[kMine];                               // entry e: mine[e / kThreads] of thread e % kThreads
+#pragma unroll
+  for (int i = 0; i < kMine; ++i) mine[i] = ((const int*)sm)[i * kThreads + tid];   // (past the number: not used)
+  asm volatile("fence.proxy.async;" ::: "memory");   // bulk copies write the ring next
+  int taken = 0;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -376,18 +502,23 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(DevSys d, const flo
   auto next_tile = [&]() -> bool {
     sc += (unsigned)(nb * nmt * nch);
     pc += (unsigned)(nb * nmt);
-    all_bar();                                   // every role is done with the previous tile
-    if (tid == 0) {
-      const int i = *fail ? -1 : atomicAdd(counter, 1);
-      iv[2] = i >= 0 && i < counter[1] ? list[i] : -1;
-    }
-    all_bar();
-    const int t_ = iv[2];
-    if (t_ < 0) return false;
-    r = t_ / d.nkpt;
-    k = t_ - r * d.nkpt;
-    for (int i = tid; i < rs; i += kThreads) slot[i] = blist[((size_t)k * d.tc_nreg + r) * rs + i];
-    all_bar();
+    do {                                         // (a tile dealt may turn out to have no block)
+      all_bar();                                 // every role is done with the previous tile
+      if (tid == taken % kThreads) iv[2] = *fail || taken >= nmine ? -1 : taken < kThreads ? mine[0] : mine[1];
+      ++taken;
+      all_bar();
+      const int t_ = iv[2];
+      if (t_ < 0) return false;
+      r = t_ / d.nkpt;
+      k = t_ - r * d.nkpt;
+      const Point diff = minus(d, corner_of(d, r), point_of(d, k));
+      for (int i = tid; i < rs; i += kThreads) {
+        const int b = block_of(d, g, k, diff, i);
+        slot[i] = b;
+        if (b >= 0) iv[5] = taken;
+      }
+      all_bar();
+    } while (iv[5] != taken);
     kc = umma::uniform(d.tc_kcount[r]);
     // ---- tile setup: blocks per slot, K keys, sphere keys of k, rows
     for (int i = tid; i < g.nwords; i += kThreads) bits[i] = 0u;
@@ -815,17 +946,13 @@ TpGeo tp_fit(const DevSys& d) {
 }
 
 struct TpWs {
-  size_t bimg, blist, counter, flag, list, scale, total;
+  size_t bimg, scale, total;
 };
 
 TpWs tp_ws(const DevSys& d) {
   TpWs w;
   size_t o = 0;
   w.bimg = o; o += ((size_t)d.nkpt * d.nb * (d.tc_kpad / kTKC) * kImgRow + 255) & ~(size_t)255;
-  w.blist = o; o += ((size_t)d.nkpt * d.tc_nreg * d.tc_rsize * sizeof(int) + 255) & ~(size_t)255;
-  w.counter = o; o += 256;
-  w.flag = o; o += ((size_t)d.nkpt * d.tc_nreg + 255) & ~(size_t)255;
-  w.list = o; o += ((size_t)d.nkpt * d.tc_nreg * sizeof(int) + 255) & ~(size_t)255;
   w.scale = o; o += ((size_t)2 * d.nkpt * d.nb * sizeof(float) + 255) & ~(size_t)255;
   w.total = o;
   return w;
@@ -836,6 +963,7 @@ TpWs tp_ws(const DevSys& d) {
 // The tensor-core route needs a region of at most one N tile of columns and its tiles in shared memory.
 int tcpair_valid(const DevSys& d) {
   if (d.nv > 4 || d.nc > 4) return 0;            // write_pass
+  if ((long long)d.nkpt * d.tc_nreg >= 1ll << 31) return 0;   // deal_tiles
   if (d.tc_kpad < kTKC || d.tc_rsize < 1 || d.tc_rsize * (d.nv > d.nc ? d.nv : d.nc) > kNCols) return 0;
   return tp_fit(d).stages > 0 ? 1 : 0;
 }
@@ -868,8 +996,23 @@ int tcpair_preferred(const DevSys& d, int q_begin, int q_end) {
 
 size_t tcpair_ws_bytes(const DevSys& d) { return tcpair_valid(d) ? kWsSlack + tp_ws(d).total : 0; }
 
-// coef: the coefficient copy of the pair workspace; ws: the tensor-route area (tcpair_ws_bytes).
-int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, int q_begin, int q_end,
+// Systems whose panels the real-space stage packs: those whose default route over the whole mesh is this kernel (where it
+// is that of a part of the mesh it is that of the whole: the regions are of one size).  In the others a call with
+// BSE_PD_TENSOR packs for itself.
+int tcpair_packed(const DevSys& d) { return tcpair_preferred(d, 0, d.nq); }
+
+// The tensor-route area ws (tcpair_ws_bytes) from coef (nkpt x nb x npw_max), and a copy of coef unless copy is NULL.
+int launch_tcpair_pack(const DevSys& d, const void* coef, void* copy, void* ws, void* stream) {
+  const TpWs w = tp_ws(d);
+  unsigned char* base = ws_base(ws);
+  tcpair_pack_kernel<<<(unsigned)(((long long)d.nkpt * d.nb + 7) / 8), 256, 0, (cudaStream_t)stream>>>(
+      d, (const float2*)coef, (float2*)copy, (float*)(base + w.scale), base + w.bimg, d.tc_kpad / kTKC);
+  return (int)cudaGetLastError();
+}
+
+// coef: the coefficient copy of the pair workspace; ws: the tensor-route area, packed by launch_tcpair_pack.  Both are
+// only read.
+int launch_tcpair(const DevSys& d, const void* coef, const void* ws, void* rho_dir, int q_begin, int q_end,
                   long long vbase, int* status, void* stream) {
   if (!tcpair_valid(d)) return (int)cudaErrorInvalidValue;
   TpGeo g = tp_fit(d);
@@ -882,31 +1025,23 @@ int launch_tcpair(const DevSys& d, const void* coef, void* ws, void* rho_dir, in
     return e;
   cudaStream_t st = (cudaStream_t)stream;
   const TpWs w = tp_ws(d);
-  unsigned char* base = ws_base(ws);
-  unsigned char* bimg = base + w.bimg;
-  int* blist = (int*)(base + w.blist);
-  int* counter = (int*)(base + w.counter);
+  const unsigned char* base = ws_base(const_cast<void*>(ws));
   g.q_begin = q_begin;
   g.nqc = q_end - q_begin;
   g.vbase = vbase;
-  if ((e = (int)cudaMemsetAsync(bimg, 0, w.blist - w.bimg, st))) return e;
-  const long long npk = (long long)d.nkpt * d.nb * d.npw_max;
-  float* scale = (float*)(base + w.scale);
-  tcpair_scale_kernel<<<(unsigned)((d.nkpt * d.nb + 7) / 8), 256, 0, st>>>(d, (const float2*)coef, scale);
-  tcpair_pack_kernel<<<(unsigned)((npk + 255) / 256), 256, 0, st>>>(d, (const float2*)coef, scale, bimg, g.nkc);
-  if ((e = (int)cudaGetLastError())) return e;
-  if ((e = (int)cudaMemsetAsync(blist, 0xFF, w.counter - w.blist, st))) return e;
-  const long long nt = (long long)g.nqc * d.nkpt;
-  if ((e = (int)cudaMemsetAsync(counter, 0, w.list - w.counter, st))) return e;
-  tcpair_tiles_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(d, q_begin, g.nqc, blist, base + w.flag);
-  const int ntiles = d.nkpt * d.tc_nreg;
-  int* list = (int*)(base + w.list);
-  tcpair_list_kernel<<<1, kListThreads, 0, st>>>(base + w.flag, ntiles, counter, list);
-  if ((e = (int)cudaGetLastError())) return e;
-  const int grid = ntiles < num_sms ? ntiles : num_sms;
-  kernel<<<grid, kThreads, g.smem, st>>>(d, (const float2*)coef, scale, bimg, blist, counter, list, (float2*)rho_dir, g,
-                                         status);
-  if ((e = (int)cudaGetLastError())) return e;
+  // a CTA lists kMine kThreads tiles a launch; an upper bound of the tiles with a block says how many launches
+  long long diffs = std::min<long long>(d.nkpt, (long long)g.nqc * d.tc_rsize);
+  g.table = (kList + kDealSums + diffs) * 4 <= (long long)g.stages * g.stage_bytes && d.nk1 <= 1024 && d.nk2 <= 1024 &&
+            d.nk3 <= 1024;
+  if (!g.table) diffs = d.nkpt;
+  const long long most = d.tc_nreg * diffs;
+  const int grid = (int)std::min<long long>(most, num_sms);
+  const long long step = (long long)kList * grid;
+  for (g.share = 0; g.share * step < most; ++g.share) {
+    kernel<<<(unsigned)grid, kThreads, g.smem, st>>>(d, (const float2*)coef, (const float*)(base + w.scale),
+                                                     base + w.bimg, (float2*)rho_dir, g, status);
+    if ((e = (int)cudaGetLastError())) return e;
+  }
   if (q_begin == 0) {
     tcpair_diag_kernel<<<d.nkpt, 256, 0, st>>>(d, (const float2*)coef, (float2*)rho_dir, vbase);
     e = (int)cudaGetLastError();
