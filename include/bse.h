@@ -191,7 +191,9 @@ bse_status bse_rho_dir_count(const bse_plan* plan, int s, int q_begin, int q_end
  * plane-wave correlation kernel (second form; the default wherever its band counts
  * are compiled) and the pruned batched 3D FFT of the products on the real-space
  * grid (first form; the default otherwise).  Without a chosen variant a direct set with enough blocks per
- * region of k' goes to the tensor-core form of the correlation (BSE_PD_TENSOR below), to FP32 rounding as well.
+ * region of k' goes to the tensor-core form of the correlation (BSE_PD_TENSOR below), to FP32 rounding as well
+ * (bse_pair_route).  That depends on the q range: for densities that do not depend on how the mesh is cut into
+ * ranges, pass BSE_PD_TENSOR in every call or in none of them as bse_pair_route says of the whole mesh.
  * coef     complex64 [nkpt][nb][npw_max], c_nk(G) in sphere order (zero padded).
  * energies float64  [nkpt][nb], bands ascending (valence first), Ha.
  * rho_x    complex64 [dim][ng_max]: rho_vc^{kk}(G) on the q = 0 sphere (S = (k,v,c)).
@@ -203,8 +205,8 @@ bse_status bse_rho_dir_count(const bse_plan* plan, int s, int q_begin, int q_end
  *          g_p the p-th vector of the q sphere, so q_unf + G = q + g_p.
  * flags    BSE_PD_* stages; REALSPACE must run (once) before the others, with
  *          the same workspace.  The other stages only read it, so calls for different outputs may
- *          share a workspace and overlap on several streams; only BSE_PD_TENSOR on a system whose whole
- *          mesh would not take that form by default packs its panels there in every call.  Unused outputs
+ *          share a workspace and overlap on several streams; only BSE_PD_TENSOR on a system where
+ *          bse_pair_route of the whole mesh is 0 without a chosen variant packs its panels there in every call.  Unused outputs
  *          may be NULL.  With BSE_PD_COUPLING (not with
  *          DIRECT or CHI0) rho_dir receives the coupling densities of bse_build_coupling,
  *          bse_rho_cpl_count(q_begin, q_end) vectors.
@@ -416,6 +418,9 @@ bse_status bse_spectrum_backward(bse_plan* plan, int s, const void* H, const voi
  * bse_pair_variants lists the valid variants of system s (up to cap entries of out, the
  * total in *count) and the index in use (*current).  bse_set_pair_variant selects one by its
  * index (-1 restores the default); BSE_ERR_ARG if the index is not valid for the system.
+ * bse_pair_route says in *tensor whether bse_pair_densities with BSE_PD_DIRECT alone computes the range
+ * [q_begin, q_end) in the tensor-core form (1) or with the variant in use (0); where it is 1 for a part of the
+ * mesh and no variant is chosen it is 1 for the whole.  Errors: BSE_ERR_ARG.
  * bse_autotune_pair times every valid variant on the direct pair densities of q in
  * [q_begin, q_end) (one warm-up launch, then reps timed launches each, CUDA events on stream),
  * writes the mean milliseconds per launch to ms[i] (i < cap, in bse_pair_variants order),
@@ -438,6 +443,7 @@ typedef struct {
 bse_status bse_pair_variants(const bse_plan* plan, int s, bse_pair_variant* out, int cap, int* count,
                              int* current);
 bse_status bse_set_pair_variant(bse_plan* plan, int s, int index);
+bse_status bse_pair_route(const bse_plan* plan, int s, int q_begin, int q_end, int* tensor);
 bse_status bse_autotune_pair(bse_plan* plan, int s, void* ws, size_t ws_bytes, void* rho_dir, int q_begin,
                              int q_end, int reps, float* ms, int cap, int* chosen, void* stream);
 

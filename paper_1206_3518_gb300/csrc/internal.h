@@ -107,6 +107,7 @@ int tcpair_packed(const DevSys& d);
 int launch_tcpair_pack(const DevSys& d, const void* coef, void* copy, void* ws, void* stream);
 int launch_tcpair(const DevSys& d, const void* coef, const void* ws, void* rho_dir, int q_begin, int q_end,
                   long long vbase, int* status, void* stream);
+int pair_direct_route(const DevSys& d, int q_begin, int q_end);
 int launch_pair_direct_tensor(const DevSys& d, void* ws, void* rho_dir, int q_begin, int q_end, long long vbase,
                               int* status, void* stream);
 int gcorr_split_valid(const DevSys& d);

@@ -858,6 +858,15 @@ bse_status bse_pair_variants(const bse_plan* plan, int s, bse_pair_variant* out,
   return BSE_OK;
 }
 
+bse_status bse_pair_route(const bse_plan* plan, int s, int q_begin, int q_end, int* tensor) {
+  bse_status st = check_plan(plan, s);
+  if (st != BSE_OK) return st;
+  const DevSys& d = plan->sys[s].d;
+  if (!tensor || q_begin < 0 || q_end > d.nq || q_begin >= q_end) return set_error(BSE_ERR_ARG, "bad q range or output");
+  *tensor = pair_direct_route(d, q_begin, q_end);
+  return BSE_OK;
+}
+
 bse_status bse_set_pair_variant(bse_plan* plan, int s, int index) {
   bse_status st = check_plan(plan, s);
   if (st != BSE_OK) return st;

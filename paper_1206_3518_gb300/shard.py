@@ -6,9 +6,11 @@ Haydock recursion needs only products H x and inner products.  The split is ther
 1. Build.  Rank 0 owns q = 0 (the diagonal blocks) and writes diag + 2 K^x with the mirrored lower
    triangle (bse_build_kernel INIT | MIRROR); every other rank starts from H = 0.  The q points are
    assigned by ``q_groups`` (balanced by the direct-term work of each q, the same on every rank); each
-   rank computes the pair densities and K^d of its own q points only (bse_pair_densities DIRECT +
+   rank computes the pair densities and K^d of its own q points only (bse_pair_densities ``direct_flags`` +
    bse_build_kernel DIRECT over its q list), which subtracts the blocks and writes their mirrors.  Every
-   step is linear in the blocks, so sum_r H_r is the single-GPU H exactly.  W is needed only for the
+   step is linear in the blocks, every block is of one rank and ``direct_flags`` names the route of the whole
+   mesh (a flagless DIRECT of a few q may take another FP32 route), so sum_r H_r is the single-GPU H (but that
+   diag + 2 K^x is added after K^d was rounded).  W is needed only for the
    rank's own q points, u and rho_x are replicated.
 2. Exchange.  ``reduce_rows`` sums the partial H over ranks and leaves each rank its row range
    (``row_ranges``: whole k blocks, balanced rows) - one reduce-scatter of dim^2 complex64.
@@ -53,6 +55,13 @@ def direct_work(plan, s: int = 0) -> List[float]:
         blk, _ = bse.bse_pair_blocks(plan, s, q)
         out.append(float(sum(ng * ng + ng * npw[int(k2)] for _, k2 in blk)))
     return out
+
+
+def direct_flags(plan, s: int = 0) -> int:
+    """bse_pair_densities flags of a rank's direct densities: those of the single-GPU FP32 build, whatever the rank's
+    q ranges."""
+    from . import bse
+    return bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if bse.bse_pair_route(plan, s, 0, plan.info(s)["nq"]) else 0)
 
 
 def row_ranges(nkpt: int, nvc: int, world: int) -> List[Tuple[int, int]]:
