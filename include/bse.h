@@ -417,14 +417,17 @@ bse_status bse_spectrum_backward(bse_plan* plan, int s, const void* H, const voi
  *
  * bse_pair_variants lists the valid variants of system s (up to cap entries of out, the
  * total in *count) and the index in use (*current).  bse_set_pair_variant selects one by its
- * index (-1 restores the default); BSE_ERR_ARG if the index is not valid for the system.
+ * index (-1 restores the default); BSE_ERR_ARG if the index is not valid for the system.  A selected variant
+ * also computes the direct sets that would take the tensor-core form by default; bse_set_pair_tensor(on = 1)
+ * lets those take it again, beside the variant for all other sets.
  * bse_pair_route says in *tensor whether bse_pair_densities with BSE_PD_DIRECT alone computes the range
  * [q_begin, q_end) in the tensor-core form (1) or with the variant in use (0); where it is 1 for a part of the
- * mesh and no variant is chosen it is 1 for the whole.  Errors: BSE_ERR_ARG.
+ * mesh it is 1 for the whole.  Errors: BSE_ERR_ARG.
  * bse_autotune_pair times every valid variant on the direct pair densities of q in
  * [q_begin, q_end) (one warm-up launch, then reps timed launches each, CUDA events on stream),
  * writes the mean milliseconds per launch to ms[i] (i < cap, in bse_pair_variants order),
- * selects the fastest and returns its index in *chosen.  It needs the pair workspace of
+ * selects the fastest and returns its index in *chosen.  Where the range takes the tensor-core form by default
+ * that form is timed too, and direct sets keep it (as after bse_set_pair_tensor) unless a variant was faster.  It needs the pair workspace of
  * bse_pair_densities (its contents only feed the timed launches) and rho_dir with room for
  * bse_rho_dir_count(q_begin, q_end) vectors, whose contents it overwrites.  It synchronises
  * the stream (not capturable).  Errors: BSE_ERR_ARG, BSE_ERR_WORKSPACE, BSE_ERR_UNSUPPORTED,
@@ -443,6 +446,7 @@ typedef struct {
 bse_status bse_pair_variants(const bse_plan* plan, int s, bse_pair_variant* out, int cap, int* count,
                              int* current);
 bse_status bse_set_pair_variant(bse_plan* plan, int s, int index);
+bse_status bse_set_pair_tensor(bse_plan* plan, int s, int on);
 bse_status bse_pair_route(const bse_plan* plan, int s, int q_begin, int q_end, int* tensor);
 bse_status bse_autotune_pair(bse_plan* plan, int s, void* ws, size_t ws_bytes, void* rho_dir, int q_begin,
                              int q_end, int reps, float* ms, int cap, int* chosen, void* stream);

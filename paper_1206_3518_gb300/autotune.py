@@ -2,10 +2,11 @@
 
 The choice for a shape (device name, real-space grid, band counts, sphere sizes) is measured
 once by bse_autotune_pair on a range of q points and stored in a JSON file; later plans of the
-same shape reuse it without timing.  For a mixed-precision build the tensor-core route of the
-direct densities (BSE_PD_TENSOR) can be a further candidate: it is timed on the same q range,
-through the same C ABI call the build makes, against the fastest variant.  Marshalling and
-bookkeeping only: every kernel runs in the CUDA library.
+same shape reuse it without timing.  The tensor-core form of the direct densities is a further
+candidate: where the library takes it by default it is timed and kept unless a variant is faster,
+and with ``with_tensor`` it is timed wherever the system has it, through the same C ABI call the
+build makes, against the fastest variant.  Marshalling and bookkeeping only: every kernel runs in
+the CUDA library.
 """
 from __future__ import annotations
 
@@ -57,9 +58,10 @@ def tune(plan, s, forward, q_begin=0, q_end=None, reps=3, cache_path=DEFAULT_CAC
 
     forward: a pipeline.Forward of this system (its pair workspace and rho_dir buffer are used;
     rho_dir's contents are overwritten; the real-space and coefficient images must be in the pair
-    workspace).  with_tensor (mixed-precision builds): also time the tensor-core route where the
-    system has it and record the faster of the two in forward.tensor_choice, which Forward.build
-    then follows.  Returns a dict with the chosen variant, the per-variant times (empty when taken
+    workspace).  Where the direct set takes the tensor cores by default it keeps them beside the chosen
+    variant, unless a variant was faster.  with_tensor: time the tensor-core route wherever the system has it
+    and record the faster of the two in forward.tensor_choice, which Forward.build then follows in either
+    precision.  Returns a dict with the chosen variant, the per-variant times (empty when taken
     from the cache), whether the cache was used and, with with_tensor, "tensor" (the route chosen).
     """
     import torch
@@ -74,17 +76,22 @@ def tune(plan, s, forward, q_begin=0, q_end=None, reps=3, cache_path=DEFAULT_CAC
         for v in variants:
             if all(v[f] == hit["variant"].get(f) for f in _FIELDS):
                 bse.bse_set_pair_variant(plan, s, v["index"])
+                bse.bse_set_pair_tensor(plan, s, hit.get("default_tensor", True))   # older entries: the library's rule
                 out = {"variant": v, "ms": {}, "cached": True}
                 if with_tensor:
                     forward.tensor_choice = bool(hit.get("tensor", False))
                     out["tensor"] = forward.tensor_choice
+                    bse.bse_set_pair_tensor(plan, s, forward.tensor_choice)
                 return out
     if q_end is None:
         q_end = min(plan.info(s)["nq"], q_begin + forward.qchunk)
+    bse.bse_set_pair_tensor(plan, s, True)
+    by_default = bse.bse_pair_route(plan, s, q_begin, q_end)
     ms, chosen = bse.bse_autotune_pair(plan, s, forward.ws_pair, forward.rho_dir, q_begin, q_end, reps)
     best = next(v for v in variants if v["index"] == chosen)
     times = {str(v["index"]): t for v, t in zip(variants, ms)}
-    entry = {"variant": {f: best[f] for f in _FIELDS}, "ms": times}
+    entry = {"variant": {f: best[f] for f in _FIELDS}, "ms": times,
+             "default_tensor": not by_default or bse.bse_pair_route(plan, s, q_begin, q_end)}
     tensor = False
     if tensor_ok:
         t_tensor = _time_tensor(plan, s, forward, q_begin, q_end, reps)
@@ -93,6 +100,7 @@ def tune(plan, s, forward, q_begin=0, q_end=None, reps=3, cache_path=DEFAULT_CAC
         entry["tensor"] = tensor
     if with_tensor:
         forward.tensor_choice = tensor
+        bse.bse_set_pair_tensor(plan, s, tensor)
     cache[key] = entry
     os.makedirs(os.path.dirname(cache_path), exist_ok=True)
     tmp = cache_path + ".tmp"

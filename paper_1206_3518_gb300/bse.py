@@ -31,7 +31,7 @@ EXPORTED = [
     "bse_last_error", "bse_plan_create", "bse_plan_create_host", "bse_plan_destroy", "bse_plan_info", "bse_gvectors",
     "bse_pair_blocks", "bse_workspace_size", "bse_rho_dir_count", "bse_pair_densities",
     "bse_build_kernel", "bse_apply_H", "bse_spectrum", "bse_spectrum_static", "bse_spectrum_batch", "bse_spectrum_backward", "bse_status_read",
-    "bse_pair_variants", "bse_set_pair_variant", "bse_pair_route", "bse_autotune_pair", "bse_set_wait_limit", "bse_screening",
+    "bse_pair_variants", "bse_set_pair_variant", "bse_set_pair_tensor", "bse_pair_route", "bse_autotune_pair", "bse_set_wait_limit", "bse_screening",
     "bse_rho_cpl_count", "bse_build_coupling", "bse_spectrum_coupled", "bse_ritz", "bse_symmetry", "bse_unfold_w",
     "bse_chi0_optical", "bse_xc_kernel_alda", "bse_epsilon_macro", "bse_exciton_states",
 ]
@@ -99,6 +99,7 @@ def load():
     lib.bse_status_read.argtypes = [vp, vp]
     lib.bse_pair_variants.argtypes = [vp, i, ctypes.POINTER(BsePairVariant), i, ctypes.POINTER(i), ctypes.POINTER(i)]
     lib.bse_set_pair_variant.argtypes = [vp, i, i]
+    lib.bse_set_pair_tensor.argtypes = [vp, i, i]
     lib.bse_pair_route.argtypes = [vp, i, i, i, ctypes.POINTER(i)]
     lib.bse_set_wait_limit.argtypes = [ctypes.c_ulonglong]
     lib.bse_screening.argtypes = [vp, i, vp, vp, vp, i, i, i, vp, vp, vp, sz, vp]
@@ -297,6 +298,11 @@ def bse_pair_variants(plan, s):
 
 def bse_set_pair_variant(plan, s, index):
     _check(load().bse_set_pair_variant(plan.handle, s, int(index)))
+
+
+def bse_set_pair_tensor(plan, s, on):
+    """Whether direct sets that ask for no route may take the tensor cores beside a chosen variant."""
+    _check(load().bse_set_pair_tensor(plan.handle, s, int(bool(on))))
 
 
 def bse_pair_route(plan, s, q_begin, q_end) -> bool:

@@ -33,6 +33,7 @@ struct DevSys {
   const float* vsq;               // [nq][ng_max] sqrt(4 pi)/|q+G| (0 at q+G = 0 and beyond ngq)
   long long nblocks;
   int pair_variant;               // index of the pair-kernel variant chosen for this system, -1 = first valid
+  int pair_tensor;                // 1: direct sets that ask for no route may take the tensor cores (pair_direct_route)
   const int* gminus0;             // [ng0] index of -G on the q = 0 sphere (-1 if absent)
   const int* qperm;               // [nq][ng_max] sphere map of q onto its irreducible point (-1 padded)
   const int2* qsym;               // [nq] (irreducible index, time reversal)

@@ -571,11 +571,11 @@ static long long job_cells(const DevSys& d, int nqc, bool merged) {
   return ntq * ntk * kTQ * kTK * (merged ? 1 : 2);
 }
 
-// 1: a direct set of the range that asks for no route goes to the tensor cores (no variant chosen, and enough blocks per
-// region).  Where that holds for a part of the mesh it holds for the whole: the regions are of one size, so a part has
+// 1: a direct set of the range that asks for no route goes to the tensor cores (no variant chosen, or the tuner found them
+// faster than every variant; and enough blocks per region).  Where that holds for a part of the mesh it holds for the whole: the regions are of one size, so a part has
 // at most as many q per region touched.
 int pair_direct_route(const DevSys& d, int q_begin, int q_end) {
-  return d.pair_variant == -1 && use_gcorr(d) && tcpair_preferred(d, q_begin, q_end) ? 1 : 0;
+  return d.pair_tensor && gcorr_valid(d) && tcpair_preferred(d, q_begin, q_end) ? 1 : 0;
 }
 
 int launch_pair_direct(const DevSys& d, void* u, void* rho_dir, int q_begin, int q_end, long long vbase,

@@ -146,6 +146,7 @@ bse_status build_system(const bse_system& in, SysPlan& sp, bool device) {
   d.n2 = s.fft[1];
   d.n3 = s.fft[2];
   d.pair_variant = -1;
+  d.pair_tensor = 1;
   d.nk1 = nk1;
   d.nk2 = nk2;
   d.nk3 = nk3;
@@ -879,6 +880,14 @@ bse_status bse_set_pair_variant(bse_plan* plan, int s, int index) {
     if (!found) return set_error(BSE_ERR_ARG, "pair variant not valid for this system");
   }
   d.pair_variant = index;
+  d.pair_tensor = index == -1 ? 1 : 0;
+  return BSE_OK;
+}
+
+bse_status bse_set_pair_tensor(bse_plan* plan, int s, int on) {
+  bse_status st = check_plan(plan, s);
+  if (st != BSE_OK) return st;
+  plan->sys[s].d.pair_tensor = on ? 1 : 0;
   return BSE_OK;
 }
 
@@ -904,31 +913,43 @@ bse_status bse_autotune_pair(bse_plan* plan, int s, void* ws, size_t ws_bytes, v
     cudaEventDestroy(e0);
     return st;
   }
-  const int saved = d.pair_variant;
+  const int saved = d.pair_variant, saved_tensor = d.pair_tensor;
+  d.pair_tensor = 0;                             // the variants' own kernels are timed
   const long long vb = sp.qvec_off[q_begin];
   float best = 0.f;
   int besti = -1;
+  auto timed = [&](auto&& launch, float& t) {
+    bse_status e = cuda_check(launch(), "autotune warm-up");
+    if (e != BSE_OK) return e;
+    cudaEventRecord(e0, stm);
+    for (int r = 0; r < reps && e == BSE_OK; ++r) e = cuda_check(launch(), "autotune");
+    cudaEventRecord(e1, stm);
+    if (e == BSE_OK) e = cuda_check(cudaEventSynchronize(e1), "autotune sync");
+    if (e == BSE_OK) e = cuda_check(cudaEventElapsedTime(&t, e0, e1), "autotune timing");
+    t /= (float)reps;
+    return e;
+  };
   for (int i = 0; i < n && i < 64 && st == BSE_OK; ++i) {
     d.pair_variant = buf[7 * i];
-    st = cuda_check(launch_pair_direct(d, ws, rho_dir, q_begin, q_end, vb, plan->d_status, stream), "autotune warm-up");
-    if (st != BSE_OK) break;
-    cudaEventRecord(e0, stm);
-    for (int r = 0; r < reps && st == BSE_OK; ++r)
-      st = cuda_check(launch_pair_direct(d, ws, rho_dir, q_begin, q_end, vb, plan->d_status, stream), "autotune");
-    cudaEventRecord(e1, stm);
-    if (st == BSE_OK) st = cuda_check(cudaEventSynchronize(e1), "autotune sync");
     float t = 0.f;
-    if (st == BSE_OK) st = cuda_check(cudaEventElapsedTime(&t, e0, e1), "autotune timing");
-    t /= (float)reps;
+    st = timed([&] { return launch_pair_direct(d, ws, rho_dir, q_begin, q_end, vb, plan->d_status, stream); }, t);
     if (i < cap) ms[i] = t;
     if (st == BSE_OK && (besti < 0 || t < best)) {
       best = t;
       besti = buf[7 * i];
     }
   }
+  // the tensor-core form where the range takes it by default: it stays the default unless a variant beats it
+  int tensor = 1;
+  if (st == BSE_OK && gcorr_valid(d) && tcpair_preferred(d, q_begin, q_end)) {
+    float t = 0.f;
+    st = timed([&] { return launch_pair_direct_tensor(d, ws, rho_dir, q_begin, q_end, vb, plan->d_status, stream); }, t);
+    tensor = t <= best ? 1 : 0;
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   d.pair_variant = (st == BSE_OK) ? besti : saved;
+  d.pair_tensor = (st == BSE_OK) ? tensor : saved_tensor;
   *chosen = d.pair_variant;
   return st;
 }

@@ -50,16 +50,16 @@ class Forward:
         """A1-A6: pair densities, dipole and H (direct term streamed over q chunks).
 
         tensor_pair: direct pair densities on the tensor cores (BSE_PD_TENSOR); by default with the
-        mixed precision where the system has that route, or as the autotuner chose for this system, and in FP32
-        where the library takes it for the whole mesh.  One choice for every chunk: H does not depend on qchunk.
+        mixed precision where the system has that route, in FP32 where the library takes it for the whole
+        mesh, and in both as the autotuner chose for this system.  One choice for every chunk: H does not depend on qchunk.
         """
         p, s = self.plan, self.s
         if tensor_pair is None:
             tensor_pair = prec == bse.BSE_PREC_BF16X3 and bool(self.info["tensor_pair"])
-            if tensor_pair and self.tensor_choice is not None:
-                tensor_pair = self.tensor_choice
             if prec == bse.BSE_PREC_FP32:
                 tensor_pair = bse.bse_pair_route(p, s, 0, self.nq)
+            if self.tensor_choice is not None and bool(self.info["tensor_pair"]):
+                tensor_pair = self.tensor_choice
         fdir = bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if tensor_pair else 0)
         bse.bse_pair_densities(p, s, bse.BSE_PD_REALSPACE | bse.BSE_PD_EXCHANGE, coef, energies, self.rho_x, self.P,
                                None, 0, 0, self.ws_pair)

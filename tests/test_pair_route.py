@@ -31,3 +31,15 @@ def test_a_part_on_the_tensor_cores_means_the_whole(lat, n, nv, nc, ecut, grid):
     for a, b in ((-1, 1), (0, nq + 1), (3, 3)):
         with pytest.raises(bse.BseError):
             bse.bse_pair_route(plan, 0, a, b)
+
+
+def test_chosen_variant_and_the_tensor_form():
+    plan = _plan("fcc", 5, 4, 4, 3.0, (48,) * 3)
+    nq = plan.info(0)["nq"]
+    assert bse.bse_pair_route(plan, 0, 0, nq)
+    bse.bse_set_pair_variant(plan, 0, 64)
+    assert not bse.bse_pair_route(plan, 0, 0, nq)
+    bse.bse_set_pair_tensor(plan, 0, True)
+    assert bse.bse_pair_route(plan, 0, 0, nq) and bse.bse_pair_variants(plan, 0)[1] == 64
+    bse.bse_set_pair_variant(plan, 0, -1)
+    assert bse.bse_pair_route(plan, 0, 0, nq)
