@@ -65,13 +65,20 @@ struct Tile {
   long long row0;                              // the op's index of the tile's first row
 };
 
-// Power-of-two scale of a row whose largest |component| is m: m * 2^s in [2^14, 2^15).
+// Power-of-two scale of a row whose largest |component| is m: m * 2^s in [2^14, 2^15) (below 2^-112 less).
 __device__ __forceinline__ int scale_exp(float m) {
   if (!(m > 0.f)) return 0;
-  const int s = 14 - ilogbf(m);
-  return s > 126 ? 126 : (s < -110 ? -110 : s);
+  const int s = 14 - ilogbf(m);                // at least -113 where m is finite
+  return s > 126 ? 126 : (s < -126 ? -126 : s);
 }
 __device__ __forceinline__ float pow2(int s) { return __int_as_float((s + 127) << 23); }   // |s| <= 126
+// x times two inverse scales, the smaller first: between a large and a small one no product leaves FP32's range that the
+// result does not leave.
+struct Unscale {
+  float lo, hi;
+  __device__ __forceinline__ Unscale(float a, float b) : lo(fminf(a, b)), hi(fmaxf(a, b)) {}
+  __device__ __forceinline__ float operator()(float x) const { return x * lo * hi; }
+};
 
 // x = hi + lo in FP16 (round to nearest), two values per 32-bit word.
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uint32_t& lo) {
@@ -412,7 +419,7 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
 #pragma unroll
             for (int i = 0; i < 4; ++i)
               *reinterpret_cast<float4*>(xp + lane * 64 + ((i ^ ((lane >> 1) & 3)) << 4)) =
-                  make_float4(v[4 * i] * sa, v[4 * i + 1] * sa, v[4 * i + 2] * sa, v[4 * i + 3] * sa);
+                  make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
             __syncwarp();
             const int j = lane & 3, col = cb + 4 * j;
             float s[4];
@@ -421,10 +428,11 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
 #pragma unroll 2
             for (int r8 = 0; r8 < 4; ++r8) {
               const int rl = r8 * 8 + (lane >> 2), ro = (warp & 3) * 32 + rl;
+              const float sr = __shfl_sync(0xffffffffu, sa, rl);
               if (ro >= t.mvalid || col >= t.nvalid) continue;
               const float4 u = *reinterpret_cast<const float4*>(xp + rl * 64 + ((j ^ ((rl >> 1) & 3)) << 4));
               float* out = op.row_out(t, ro) + col;
-              const float w[4] = {u.x * s[0], u.y * s[1], u.z * s[2], u.w * s[3]};
+              const float w[4] = {Unscale(sr, s[0])(u.x), Unscale(sr, s[1])(u.y), Unscale(sr, s[2])(u.z), Unscale(sr, s[3])(u.w)};
               if (col + 3 < t.nvalid && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
                 *reinterpret_cast<float4*>(out) = make_float4(w[0], w[1], w[2], w[3]);
               } else {
@@ -442,7 +450,7 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             *reinterpret_cast<float4*>(xp + lane * 128 + ((i ^ (lane & 7)) << 4)) =
-                make_float4(re[g][2 * i] * sa, im[g][2 * i] * sa, re[g][2 * i + 1] * sa, im[g][2 * i + 1] * sa);
+                make_float4(re[g][2 * i], im[g][2 * i], re[g][2 * i + 1], im[g][2 * i + 1]);
           __syncwarp();
           const int j = lane & 7, col = c0 + 16 * g + 2 * j;
           const float s0 = col < t.nvalid ? op.col_scale(t, col) : 0.f;
@@ -450,23 +458,26 @@ __global__ __launch_bounds__(kThreads, 1) void gemm_kernel(const __grid_constant
 #pragma unroll 2
           for (int r4 = 0; r4 < 8; ++r4) {
             const int rl = r4 * 4 + (lane >> 3), ro = (warp & 3) * 32 + rl;
+            const float sr = __shfl_sync(0xffffffffu, sa, rl);
             if (ro >= t.mvalid || col >= t.nvalid) continue;
-            const float4 v = *reinterpret_cast<const float4*>(xp + rl * 128 + ((j ^ (rl & 7)) << 4));
+            float4 v = *reinterpret_cast<const float4*>(xp + rl * 128 + ((j ^ (rl & 7)) << 4));
+            const Unscale u0(sr, s0), u1(sr, s1);
+            v = make_float4(u0(v.x), u0(v.y), u1(v.z), u1(v.w));
             float2* out = op.row_out(t, ro) + col;
             if constexpr (Op::kHerm) {             // upper triangle, and its mirror image
 #pragma unroll
               for (int i = 0; i < 2; ++i) {
                 if (col + i >= t.nvalid || t.m0 + ro > t.n0 + col + i) continue;
-                float2 y = op.value(t, ro, col + i, i ? make_float2(v.z * s1, v.w * s1) : make_float2(v.x * s0, v.y * s0));
+                float2 y = op.value(t, ro, col + i, i ? make_float2(v.z, v.w) : make_float2(v.x, v.y));
                 if (t.m0 + ro == t.n0 + col + i) y.y = 0.f;
                 out[i] = y;
                 if (t.m0 + ro != t.n0 + col + i) *op.mirror_out(t, ro, col + i) = make_float2(y.x, -y.y);
               }
               continue;
             }
-            const float2 y0 = op.value(t, ro, col, make_float2(v.x * s0, v.y * s0));
+            const float2 y0 = op.value(t, ro, col, make_float2(v.x, v.y));
             if (col + 1 < t.nvalid) {
-              const float2 y1 = op.value(t, ro, col + 1, make_float2(v.z * s1, v.w * s1));
+              const float2 y1 = op.value(t, ro, col + 1, make_float2(v.z, v.w));
               if ((reinterpret_cast<uintptr_t>(out) & 15) == 0) {
                 *reinterpret_cast<float4*>(out) = make_float4(y0.x, y0.y, y1.x, y1.y);
               } else {

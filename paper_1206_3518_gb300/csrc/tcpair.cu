@@ -54,6 +54,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 #include "tcf16.cuh"
@@ -394,8 +395,10 @@ __device__ __noinline__ int deal_tiles(const DevSys& d, const TpGeo& g, int* scr
 // ---------------------------------------------------------------- the GEMM tiles
 // One row of a pass to its blocks: NSET columns per slot, unrolled (a loop over columns with the slot's tables and
 // branches in it took as long as the promotion of the pass; where the stores go makes no difference: consecutive
-// addresses instead of sphere positions measured the same).
-template <int NSET>
+// addresses instead of sphere positions measured the same).  SMALL: the row's inverse scale is below 1 and is taken first,
+// else last, so that no product leaves FP32's range that the result does not leave (the smaller of the two first, chosen
+// per column, took 1% of the build).
+template <int NSET, bool SMALL>
 __device__ __forceinline__ void write_pass(const float (&re)[kNCols], const float (&im)[kNCols], float ia,
                                            const float* ib, float2* const* bptr, const short* pt, int rs, int nb,
                                            size_t first, int ng_max) {
@@ -406,8 +409,8 @@ __device__ __forceinline__ void write_pass(const float (&re)[kNCols], const floa
     float2* dst = bptr[2 * b] + first + pb;
 #pragma unroll
     for (int m = 0; m < NSET; ++m) {
-      const float s = ib[b * nb + m];
-      const float2 v = make_float2(re[b * NSET + m] * ia * s, im[b * NSET + m] * ia * s);
+      const float s = ib[b * nb + m], x = SMALL ? ia : s, y = SMALL ? s : ia;
+      const float2 v = make_float2(re[b * NSET + m] * x * y, im[b * NSET + m] * x * y);
       if (pb >= 0) dst[(size_t)m * ng_max] = v;
     }
   }
@@ -864,12 +867,19 @@ __global__ __launch_bounds__(kThreads, 1) void tcpair_kernel(const __grid_consta
           const float ia = scale[(size_t)d.nkpt * nb + (size_t)k * nb + n];
           const float* ib = binv + (set ? nv : 0);
           const size_t first = (size_t)nn * nset * d.ng_max;
-          switch (nset) {
-            case 1: write_pass<1>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
-            case 2: write_pass<2>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
-            case 3: write_pass<3>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
-            default: write_pass<4>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
-          }
+          auto write = [&](auto small) {
+            constexpr bool S = decltype(small)::value;
+            switch (nset) {
+              case 1: write_pass<1, S>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
+              case 2: write_pass<2, S>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
+              case 3: write_pass<3, S>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
+              default: write_pass<4, S>(re, im, ia, ib, bptr + set, pt, rs, nb, first, d.ng_max); break;
+            }
+          };
+          if (ia < 1.f)
+            write(std::true_type{});
+          else
+            write(std::false_type{});
         }
       }
     }
