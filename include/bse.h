@@ -177,6 +177,11 @@ bse_status bse_pair_blocks(const bse_plan* plan, int s, int iq, int32_t* out, in
  * Workspace bytes for one call kind on system s.  For BSE_WS_KERNEL, arg is
  * the largest q chunk (q_end - q_begin) that will be passed; for
  * BSE_WS_SPECTRUM and BSE_WS_BACKWARD, arg is nsteps.  Ignored otherwise.
+ * The products on the tensor cores keep split images of their operands in the workspace, 8 bytes per complex
+ * value: BSE_WS_KERNEL those of one side of a q chunk's densities and of its W rows; BSE_WS_SCREEN three
+ * matrices per q beside the matrices and at most 1 GiB of pair vectors; BSE_WS_BACKWARD at most 1.5 GiB for the
+ * direct term (or a panel of 4096 rows of dL/dH, where larger); BSE_WS_CHI0 512 MiB of pairs and sums and
+ * 16 KB of weights per transition.
  */
 bse_status bse_workspace_size(const bse_plan* plan, int s, int kind, long long arg, size_t* bytes);
 

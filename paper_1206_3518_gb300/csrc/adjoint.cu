@@ -34,7 +34,7 @@ constexpr int kQChunk = 32;         // q points per direct-term chunk
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-size_t split_area(const DevSys& d, long long nsteps, long long qc, long long w);
+size_t split_area(const DevSys& d, long long nsteps, long long qc);
 
 struct BwdLayout {
   size_t spec, eps2, ab, done, scal, Y, Mh, Mf, Vf, Zf, Gh, Xv, Xc, Yd, split, total;
@@ -63,8 +63,7 @@ BwdLayout bwd_layout(const DevSys& d, long long nsteps) {
   L.Xv = o; o = a256(o + 8 * (size_t)L.rows_v * d.ng_max);
   L.Xc = o; o = a256(o + 8 * (size_t)L.rows_c * d.ng_max);
   L.Yd = o; o = a256(o + 8 * (size_t)L.rows_c * d.ng_max);
-  const long long w = d.nv > d.nc ? d.nv * d.nv : d.nc * d.nc;
-  L.split = o; o = a256(o + split_area(d, nsteps, qc, w));
+  L.split = o; o = a256(o + split_area(d, nsteps, qc));
   L.total = o;
   return L;
 }
@@ -388,13 +387,28 @@ __global__ __launch_bounds__(256) void split_rows_kernel(const float2* __restric
 
 constexpr int kPanel = 32 * tcf::kTM;           // rows of G_h split at a time (the images of all would take its size again)
 
-// Largest use of the split area (images, then inverse scales): W.rho of a q chunk, dW of a q chunk, G_h, dL/drho_x.
-size_t split_area(const DevSys& d, long long nsteps, long long qc, long long w) {
+// q points of a chunk of qc whose images are held at a time: as many as fit in 1.5 GiB, in groups of one size.  (fcc 8x8x8
+// 3v4c: whole chunks, dW 1.5 GB; with 1 GiB and dW in two groups the gradient took 57.4 instead of 56.7 ms.  fcc 12x12x12
+// 4v4c: whole chunks would take 3.7 GB for W.rho and 8.5 GB for dW.)
+constexpr size_t kSplitArea = size_t(3) << 29;
+int split_group(size_t per_q, long long qc) {
+  const long long parts = (long long)((per_q * qc + kSplitArea - 1) / kSplitArea);
+  return (int)((qc + parts - 1) / parts);
+}
+long long wide_side(const DevSys& d) { return d.nv > d.nc ? d.nv * d.nv : d.nc * d.nc; }
+int wr_group(const DevSys& d, long long qc) { return split_group(wr32_split_bytes(d, 1, wide_side(d)), qc); }
+int dw_group(const DevSys& d, long long qc) {
+  const int K = d.nkpt * d.nc * d.nc;
+  return split_group(tcf::cols_batch_bytes(d.ng_max, K, tcf::kTM) + tcf::cols_batch_bytes(d.ng_max, K, tcf::n_tile(d.ng_max)), qc);
+}
+
+// Largest use of the split area (images, then inverse scales): W.rho and dW of a group of q, G_h, dL/drho_x.
+size_t split_area(const DevSys& d, long long nsteps, long long qc) {
   const int n = tcf::n_tile(d.ng_max), nd = tcf::n_tile(d.dim), n0 = tcf::n_tile(d.ng0);
   const int K = d.nkpt * d.nc * d.nc;
-  const size_t wr = wr32_split_bytes(d, qc, w);
-  const size_t dw = a256(qc * tcf::cols_batch_bytes(d.ng_max, K, tcf::kTM)) + a256(qc * tcf::cols_batch_bytes(d.ng_max, K, n)) +
-                    2 * a256((size_t)qc * d.ng_max * 4);
+  const size_t wr = wr32_split_bytes(d, wr_group(d, qc), wide_side(d)), g = dw_group(d, qc);
+  const size_t dw = a256(g * tcf::cols_batch_bytes(d.ng_max, K, tcf::kTM)) + a256(g * tcf::cols_batch_bytes(d.ng_max, K, n)) +
+                    2 * a256(g * d.ng_max * 4);
   const size_t gh = a256(tcf::cols_batch_bytes(d.dim, (int)nsteps, tcf::kTM)) +
                     a256(tcf::cols_batch_bytes(d.dim, (int)nsteps, nd)) + 2 * a256((size_t)d.dim * 4);
   const size_t dx = a256(tcf::cols_batch_bytes(d.dim < kPanel ? d.dim : kPanel, d.dim, tcf::kTM)) +
@@ -402,7 +416,7 @@ size_t split_area(const DevSys& d, long long nsteps, long long qc, long long w) 
   return std::max(std::max(wr, dw), std::max(gh, dx));
 }
 
-// dL/dW of a q chunk from Y and rho_cc'.
+// dL/dW of a group of q from Y (its first row that of q0) and rho_cc'.
 int launch_dw(const DevSys& d, const float2* Yd, const float2* rho_dir, float2* dW, int q0, int q1, long long maxb,
               char* area, int* status, cudaStream_t st) {
   const int nq = q1 - q0, n = tcf::n_tile(d.ng_max), K = (int)maxb * d.nc * d.nc;
@@ -522,15 +536,24 @@ int launch_backward(const DevSys& d, const long long* h_qblk_off, const long lon
       const int q1 = (q0 + kQChunk) < d.nq ? q0 + kQChunk : d.nq;
       long long maxb = 0;
       for (int q = q0; q < q1; ++q) maxb = std::max(maxb, h_qblk_off[q + 1] - h_qblk_off[q]);
-      if ((e = launch_gemm_wr(d, rho_dir, q0, q1, 0, maxb * d.nv * d.nv, W, Xv, base + L.split, 0, status, stream))) return e;
-      if ((e = launch_gemm_wr(d, rho_dir, q0, q1, 0, maxb * d.nc * d.nc, W, Xc, base + L.split, 1, status, stream))) return e;
+      const int gw = wr_group(d, kQChunk < d.nq ? kQChunk : d.nq), gd = dw_group(d, kQChunk < d.nq ? kQChunk : d.nq);
+      for (int side = 0; side < 2; ++side)
+        for (int qa = q0; qa < q1; qa += gw) {
+          const int qb = std::min(q1, qa + gw), w = side ? d.nc * d.nc : d.nv * d.nv;
+          float2* X = (side ? Xc : Xv) + (size_t)((h_qblk_off[qa] - h_qblk_off[q0]) * w) * d.ng_max;
+          if ((e = launch_gemm_wr(d, rho_dir, qa, qb, 0, maxb * w, W, X, base + L.split, side, status, stream))) return e;
+        }
       const long long nb = h_qblk_off[q1] - h_qblk_off[q0];
       if (nb > 0)
         block_grad_kernel<<<(unsigned)nb, 256, 0, st>>>(d, Gh, (const float2*)rho_dir, Xv, Xc, (float2*)drho_dir, Yd,
                                                         q0);
       if ((e = (int)cudaGetLastError())) return e;
-      if (dW && (e = launch_dw(d, Yd, (const float2*)rho_dir, (float2*)dW, q0, q1, maxb, base + L.split, status, st)))
-        return e;
+      for (int qa = q0; dW && qa < q1; qa += gd) {
+        const float2* Y = Yd + (size_t)((h_qblk_off[qa] - h_qblk_off[q0]) * d.nc * d.nc) * d.ng_max;
+        if ((e = launch_dw(d, Y, (const float2*)rho_dir, (float2*)dW, qa, std::min(q1, qa + gd), maxb, base + L.split, status,
+                           st)))
+          return e;
+      }
     }
   }
   return 0;

@@ -31,7 +31,8 @@ namespace {
 using tcf::kTileA;
 using tcf::kTKC;
 using tcf::kTM;
-constexpr int kQImg = 32;                        // q points whose pair vectors are split at a time
+constexpr size_t kImgBytes = size_t(1) << 30;     // images of pair vectors at a time,
+constexpr int kQImg = 32;                        // of at most so many q points
 
 // sw[row] = sqrt(|w_S|), row = ((qi Nk + k) Nv + v) Nc + c.
 __global__ void weight_kernel(DevSys d, const double* __restrict__ e, int q_begin, long long rows, double gap_floor,
@@ -111,6 +112,11 @@ QGeo qgeo(const DevSys& d, int K, int tile) {
   g.kc = (K + kTKC - 1) / kTKC;
   g.batch = (size_t)g.nt * g.kc * (2 * (size_t)tile * umma::kRow);
   return g;
+}
+
+int q_images(const DevSys& d) {
+  const size_t n = kImgBytes / qgeo(d, d.nkpt * d.nv * d.nc, kTM).batch;
+  return n < 1 ? 1 : (int)std::min<size_t>(n, kQImg);
 }
 
 // C_q = f(sum_k A_mk conj(B_nk)) over the q of a range.
@@ -277,7 +283,7 @@ __global__ void w_kernel(DevSys d, const float2* __restrict__ X, float2* __restr
 namespace {
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-struct ScreenWs {                                 // eps, X, T; images of eps, X (128-row tiles), T; of the pair vectors of kQImg q
+struct ScreenWs {                                 // eps, X, T; images of eps, X (128-row tiles), T; of the pair vectors of q_images q
   size_t E, X, T, img[3], inv[3], vimg, vinv, sw, R, total;
 };
 ScreenWs layout(const DevSys& d, long long nq) {
@@ -292,7 +298,7 @@ ScreenWs layout(const DevSys& d, long long nq) {
     w.img[i] = o; o += a256(nq * qgeo(d, d.ng_max, i == 1 ? kTM : tcf::n_tile(d.ng_max)).batch);
     w.inv[i] = o; o += vec;
   }
-  w.vimg = o; o += a256((size_t)std::min<long long>(nq, kQImg) * qgeo(d, K, kTM).batch);
+  w.vimg = o; o += a256((size_t)std::min<long long>(nq, q_images(d)) * qgeo(d, K, kTM).batch);
   w.vinv = o; o += vec;
   w.sw = o; o += a256((size_t)nq * K * 4);
   w.R = o; o += a256((size_t)nq * 4);
@@ -333,10 +339,11 @@ int launch_screening(const DevSys& d, void* rho_chi, const double* energies, con
                                                                           (unsigned*)vinv);
   const long long nv = (long long)nq * d.ng_max;
   tcf::inv_scale_kernel<<<(unsigned)((nv + 255) / 256), 256, 0, st>>>((unsigned*)vinv, nv);
-  // eps = I + A^T conj(A), kQImg q at a time
+  // eps = I + A^T conj(A), q_images q at a time
   const QGeo gv = qgeo(d, K, kTM), g = qgeo(d, d.ng_max, kTM), gb = qgeo(d, d.ng_max, tcf::n_tile(d.ng_max));
-  for (int q0 = 0; q0 < nq; q0 += kQImg) {
-    const int nb = std::min(kQImg, nq - q0);
+  const int qi = q_images(d);
+  for (int q0 = 0; q0 < nq; q0 += qi) {
+    const int nb = std::min(qi, nq - q0);
     const float2* aq = a + (size_t)q0 * K * d.ng_max;
     const float* iq = vinv + (size_t)q0 * d.ng_max;
     tcf::split_cols_kernel<<<dim3((d.ng_max + tcf::kColG - 1) / tcf::kColG, gv.kc, nb), tcf::kColThreads, 0, st>>>(

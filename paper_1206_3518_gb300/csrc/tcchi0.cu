@@ -29,7 +29,8 @@ namespace {
 
 constexpr int kW = 1024, kWZ = 128;              // frequencies per weights image, per Z
 constexpr int kWPer = 4;                         // frequencies per thread of combine_kernel
-constexpr size_t kPanelBytes = size_t(1) << 30;  // images of T at a time
+constexpr size_t kPanelBytes = size_t(1) << 29;  // images of T and rows of Z at a time
+constexpr long long kWave = 38 * 128;            // pairs of one tile for every SM (4 kWZ / 128 row tiles each)
 constexpr size_t kRowB = umma::kRow;
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -48,7 +49,9 @@ Geo geo_of(const DevSys& d) {
   g.sp = g.kc * tcf::kRealK;
   g.pairs = (long long)g.ng * (g.ng + 1) / 2;
   const size_t per_pair = (size_t)g.kc * 4 * kRowB;           // two rows, hi and lo
-  g.panel = std::max<long long>(1, (long long)(kPanelBytes / (per_pair * 128))) * 128;
+  const size_t per_z = (size_t)4 * kWZ * 2 * sizeof(float);   // a pair's columns of Z
+  g.panel = std::max<long long>(1, (long long)(kPanelBytes / ((per_pair + per_z) * 128))) * 128;
+  if (g.panel > kWave) g.panel -= g.panel % kWave;            // whole waves of tiles
   g.panel = std::min(g.panel, (g.pairs + 127) / 128 * 128);
   size_t o = 0;
   g.o_a = o; o = a256(o + (size_t)g.ng * g.sp * sizeof(float2));

@@ -472,8 +472,7 @@ int launch_alda_kernel(const DevSys& d, const void* pair_ws, const int* m, void*
 
 size_t epsm_ws_bytes(const DevSys& d, long long nw) {
   const size_t n = d.ng0;
-  return align256((size_t)nw * n * (n + 1) * sizeof(float2)) + align256((size_t)nw * n * n * sizeof(float2)) +
-         align256((size_t)nw * n * sizeof(float2));
+  return align256((size_t)nw * n * (n + 1) * sizeof(float2)) + align256((size_t)nw * n * sizeof(float2));
 }
 
 int launch_epsilon_macro(const DevSys& d, const void* chi0, const void* F, int nw, void* eps_m, void* ws,
@@ -482,8 +481,7 @@ int launch_epsilon_macro(const DevSys& d, const void* chi0, const void* F, int n
   const int n = d.ng0;
   char* base = (char*)ws;
   float2* aug = (float2*)base;
-  float2* xb = (float2*)(base + align256((size_t)nw * n * (n + 1) * sizeof(float2)) +
-                         align256((size_t)nw * n * n * sizeof(float2)));
+  float2* xb = (float2*)(base + align256((size_t)nw * n * (n + 1) * sizeof(float2)));
   if (F) {
     const long long rows = (long long)nw * n, step = 65535LL * gf::TM / n * n;      // whole frequencies per launch
     for (long long r = 0; r < rows; r += step) {
@@ -496,7 +494,7 @@ int launch_epsilon_macro(const DevSys& d, const void* chi0, const void* F, int n
     augment_kernel<<<blocks_for((long long)nw * n * (n + 1), 256), 256, 0, st>>>(n, nw, (const float2*)chi0, aug);
     if (int e = (int)cudaGetLastError()) return e;
   }
-  // the widest panel that leaves two CTAs an SM (n <= 427 for 16 columns, 800 for 8), down to 2 columns at n = 4096
+  // the widest panel that leaves two CTAs an SM (n <= 433 for 16 columns, 842 for 8), down to 2 columns at n = 4096
   double2* out = (double2*)eps_m;
   if (solve_smem(n, 16) <= 112 * 1024) return launch_solve<16>(n, nw, aug, out, xb, st);
   if (solve_smem(n, 8) <= 112 * 1024) return launch_solve<8>(n, nw, aug, out, xb, st);
