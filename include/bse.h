@@ -262,8 +262,11 @@ bse_status bse_pair_densities(bse_plan* plan, int s, unsigned flags,
  * H        complex64 [dim][dim] row-major.
  * prec     BSE_PREC_FP32 (tcgen05 FP16 hi/lo split products of scaled rows, the accumulator added to FP32
  *          registers every 32 complex K: FP32 accuracy) or BSE_PREC_BF16X3 (tcgen05 BF16 hi/lo split
- *          products, FP32 accumulation) for the contractions.
- * Errors: BSE_ERR_ARG, BSE_ERR_UNSUPPORTED (precision not built), BSE_ERR_WORKSPACE.
+ *          products, FP32 accumulation) for the contractions.  The FP16 split keeps 22 bits of the components
+ *          down to 2^-17 of their row's largest and 2^-40 of that largest below.
+ * ws       scratch of this call, one call at a time (INIT uses it in either precision).
+ * Errors: BSE_ERR_ARG, BSE_ERR_UNSUPPORTED (precision not built), BSE_ERR_WORKSPACE, BSE_ERR_TIMEOUT (a wait inside
+ *         a product that did not end within 2 s, through the status word).
  */
 bse_status bse_build_kernel(bse_plan* plan, int s, unsigned flags,
                             const void* rho_x, const void* rho_dir, int q_begin, int q_end,
@@ -395,7 +398,9 @@ bse_status bse_spectrum_static(bse_plan* plan, int s, const void* H, const void*
  *   dL_drho_x complex64 [dim][ng_max], dL_drho_dir as rho_dir for all q,
  *   dL_dW     complex64 [nq][ng_max][ng_max],
  * each stored entry taken as a free variable; complex gradients are
- * dL/dRe + i dL/dIm.  Any of dL_drho_x, dL_drho_dir, dL_dW may be NULL.
+ * dL/dRe + i dL/dIm.  Any of dL_drho_x, dL_drho_dir, dL_dW may be NULL.  The products with G_H, W and the
+ * densities are split FP16 ones with promoted sums (as BSE_PREC_FP32 of bse_build_kernel); a device-side wait that
+ * does not end in time reports BSE_ERR_TIMEOUT through the status word.
  */
 bse_status bse_spectrum_backward(bse_plan* plan, int s, const void* H, const void* P, int nsteps,
                                  const double* omega, int nw, double eta, const double* dL_deps2,
@@ -473,7 +478,9 @@ bse_status bse_autotune_pair(bse_plan* plan, int s, void* ws, size_t ws_bytes, v
  * W        complex64 [Nq][ng_max][ng_max]; the rows of q in the range are written (zero padded).
  * residual float32 [q_end - q_begin] on the device (optional): max |I - eps X| per q.
  * ws       bse_workspace_size(BSE_WS_SCREEN, q_end - q_begin) bytes.
- * Errors: BSE_ERR_ARG, BSE_ERR_WORKSPACE, BSE_ERR_UNSUPPORTED (slab Coulomb).
+ * The products are split FP16 ones with promoted sums, as BSE_PREC_FP32 of bse_build_kernel.
+ * Errors: BSE_ERR_ARG, BSE_ERR_WORKSPACE, BSE_ERR_UNSUPPORTED (slab Coulomb), BSE_ERR_TIMEOUT (through the status
+ *         word, as bse_build_kernel).
  */
 bse_status bse_screening(bse_plan* plan, int s, void* rho_chi, const double* energies, const void* P, int q_begin,
                          int q_end, int iterations, void* W, float* residual, void* ws, size_t ws_bytes,
@@ -550,7 +557,9 @@ bse_status bse_spectrum_coupled(bse_plan* plan, int s, const void* A, const void
  *   energies float64 [Nk][Nb];  omega float64 [nw] (Ha);  eta > 0 (Ha).
  *   chi0     complex64 [nw][ng0][ng0] row-major (row G, column G').
  *   ws       bse_workspace_size(BSE_WS_CHI0) bytes.
- *   FP32 products and sums (64 x 64 output tiles per frequency).
+ *   One real product for all frequencies (the weights times Re, Im of the pairs G <= G'): FP64 weights and FP32
+ *   pairs split hi + lo in FP16, sums promoted to FP32 registers every 64 transitions.  Device-side waits are
+ *   bounded (2 s) and report BSE_ERR_TIMEOUT through bse_status_read.
  * bse_xc_kernel_alda: F = v^-1/2 f_xc v^-1/2 of the adiabatic local-density kernel,
  *   F_GG' = |G| f_xc(G - G') |G'| / (4 pi),  f_xc(G) = (1/N_r) sum_r f_xc(r) exp(-iG.r),
  *   f_xc(r) = d^2(n eps_xc)/dn^2 at n(r) = 2/(Omega Nk) sum_{k,v} |u_vk(r)|^2 (floor 1e-6 bohr^-3), eps_xc
@@ -562,7 +571,7 @@ bse_status bse_spectrum_coupled(bse_plan* plan, int s, const void* A, const void
  *   eps_M(w) = 1/[eps^-1]_00 (F = NULL: the RPA, K = v).  One Dyson system per frequency, solved by
  *   Gaussian elimination with partial pivoting in FP32 (one CTA per frequency); eps_m complex128 [nw].
  *   ws: bse_workspace_size(BSE_WS_EPSM, nw).  Errors: BSE_ERR_UNSUPPORTED for ng0 > 4096.
- * Inputs are scanned for NaN/Inf (BSE_ERR_NONFINITE through bse_status_read).  No device-side waits.
+ * Inputs are scanned for NaN/Inf (BSE_ERR_NONFINITE through bse_status_read).  No device-side waits but those of chi~0.
  */
 bse_status bse_chi0_optical(bse_plan* plan, int s, const void* rho_x, const void* P, const double* energies,
                             double delta, const double* omega, int nw, double eta, void* chi0, void* ws,
