@@ -197,8 +197,8 @@ __device__ __forceinline__ void chunk_mmas(uint32_t d_re, uint32_t d_im, uint64_
       for (int kk = NKK - 1; kk >= 0; --kk) {
         const uint64_t pa = da + (s == (CONJ ? 0 : 1) ? a_lo : 0u) + (uint32_t)kk * 2u;
         const uint64_t pb = db + (s == (CONJ ? 1 : 0) ? b_lo : 0u) + (uint32_t)kk * 2u;
-        umma::mma_bf16(d, pa, pb + b0, idesc, (s != 0 || kk != NKK - 1) ? 1u : 0u);
-        umma::mma_bf16(d, pa + 4u, pb + b1, sign, 1u);
+        umma::mma_f16(d, pa, pb + b0, idesc, (s != 0 || kk != NKK - 1) ? 1u : 0u);
+        umma::mma_f16(d, pa + 4u, pb + b1, sign, 1u);
       }
   }
 }
@@ -211,7 +211,7 @@ __device__ __forceinline__ void chunk_mmas_real(uint32_t d, uint64_t da, uint32_
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk)
       if (kk < nkk)
-        umma::mma_bf16(d, da + (s == 1 ? a_lo : 0u) + (uint32_t)kk * 2u, db + (s == 0 ? b_lo : 0u) + (uint32_t)kk * 2u,
+        umma::mma_f16(d, da + (s == 1 ? a_lo : 0u) + (uint32_t)kk * 2u, db + (s == 0 ? b_lo : 0u) + (uint32_t)kk * 2u,
                        idesc, (s | kk) != 0 ? 1u : 0u);
 }
 
@@ -232,8 +232,8 @@ __device__ __forceinline__ void chunk_mmas_ts(uint32_t d_re, uint32_t d_im, uint
       for (int kk = NKK - 1; kk >= 0; --kk) {
         const uint32_t pa = a + (uint32_t)kk * 32u + (s == 1 ? 16u : 0u);
         const uint64_t pb = db + (s == 0 ? b_lo : 0u) + (uint32_t)(kk >> 1) * b_sub + (uint32_t)(kk & 1) * 2u;
-        umma::mma_bf16_ts(d, pa, pb + b0, idesc, (s != 0 || kk != NKK - 1) ? 1u : 0u);
-        umma::mma_bf16_ts(d, pa + 8u, pb + b1, sign, 1u);
+        umma::mma_f16_ts(d, pa, pb + b0, idesc, (s != 0 || kk != NKK - 1) ? 1u : 0u);
+        umma::mma_f16_ts(d, pa + 8u, pb + b1, sign, 1u);
       }
   }
 }

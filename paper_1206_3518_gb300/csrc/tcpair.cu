@@ -1,5 +1,5 @@
-// Direct pair densities on the 5th-generation tensor cores (step A2 of the mixed build; Eq. pair_density
-// in the plane-wave basis):
+// Direct pair densities on the 5th-generation tensor cores (step A2 of the mixed build, and of the FP32 build where
+// tcpair_preferred says so; Eq. pair_density in the plane-wave basis):
 //
 //   rho_nm^{kk'}(G) = sum_{G2 in S(k')} conj(c_nk(G2 - G)) c_mk'(G2),   G = g_p(q) - G0.
 //

@@ -1,8 +1,8 @@
-// Helpers of the 5th-generation tensor-core kernels (tc.cu, tcpair.cu): bounded mbarrier waits,
-// UMMA shared-memory and instruction descriptors, the BF16 MMA issue and its commit, and the
-// 128-byte swizzle of K-major tile rows.
+// Helpers of the 5th-generation tensor-core kernels (tc.cu and tcgram.cu in BF16; tcf16.cuh and tcpair.cu in FP16): bounded
+// mbarrier waits, UMMA shared-memory and instruction descriptors, the issue of kind::f16 MMAs (the instruction
+// descriptor says BF16 or FP16) and their commit, and the 128-byte swizzle of K-major tile rows.
 //
-// Tile format: 128-byte rows holding 32 complex K values as [Re (32 BF16) | Im (32 BF16)], rows in
+// Tile format: 128-byte rows holding 32 complex K values as [Re (32 x 16 bits) | Im (32 x 16 bits)], rows in
 // 8-row atoms of 1024 bytes with 128B swizzle (16-byte chunk c of row r stored at chunk c ^ (r & 7)).
 #pragma once
 
@@ -72,7 +72,7 @@ __host__ __device__ constexpr uint32_t idesc_of(int n) {
 }
 constexpr uint32_t kNegA = 1u << 13;
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
@@ -116,38 +116,19 @@ __device__ __forceinline__ void mma_cplx_k16_desc(uint32_t d_re, uint32_t d_im, 
     for (int s = 0; s < 3; ++s) {                 // hi.hi, hi.lo, lo.hi
       const uint64_t pa = da + ((s == 2) ? a_lo : 0u) + (uint32_t)kk * 2u;
       const uint64_t pb = db + ((s == 1) ? b_lo : 0u) + (uint32_t)kk * 2u;
-      mma_bf16(d, pa, pb + b0, idesc, (init && s == 0) ? 0u : 1u);
-      mma_bf16(d, pa + 4u, pb + b1, sign, 1u);
+      mma_f16(d, pa, pb + b0, idesc, (init && s == 0) ? 0u : 1u);
+      mma_f16(d, pa + 4u, pb + b1, sign, 1u);
     }
   }
 }
 
 // A from tensor memory (column address a of lane 0), B from shared memory.
-__device__ __forceinline__ void mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_f16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
       "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc)
       : "memory");
-}
-
-// The same with the A planes in tensor memory at columns a + 0 (Re hi), a + 8 (Im hi), a + 16 (Re lo), a + 24 (Im lo)
-// (two BF16 per 32-bit column, lane = row).
-__device__ __forceinline__ void mma_cplx_k16_ts(uint32_t d_re, uint32_t d_im, uint32_t a, uint64_t db, uint32_t b_lo,
-                                                int kk, uint32_t idesc, bool init) {
-  const uint32_t neg = idesc | kNegA;
-#pragma unroll
-  for (int im = 0; im < 2; ++im) {
-    const uint32_t d = im ? d_im : d_re, sign = im ? idesc : neg;
-    const uint32_t b0 = im ? 4u : 0u, b1 = 4u - b0;
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {                 // hi.hi, hi.lo, lo.hi
-      const uint32_t ar = a + ((s == 2) ? 16u : 0u);
-      const uint64_t pb = db + ((s == 1) ? b_lo : 0u) + (uint32_t)kk * 2u;
-      mma_bf16_ts(d, ar, pb + b0, idesc, (init && s == 0) ? 0u : 1u);
-      mma_bf16_ts(d, ar + 8u, pb + b1, sign, 1u);
-    }
-  }
 }
 
 // 32 consecutive TMEM columns of this warp's lane quarter from registers.
