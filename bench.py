@@ -4,7 +4,7 @@ Headline workload: fcc 12x12x12 k mesh, 4 valence + 4 conduction bands (dim 2764
 ~496 plane waves per sphere (max 531), 48^3 grid, 300 Haydock steps, 2000
 frequencies, eta 0.05 eV (synthetic inputs of the paper's 12x12x12 convergence
 shape, Sec. IV C).  The step runs twice on the same inputs: with FP32 contractions
-and with BF16 hi/lo split-complex tensor-core contractions ("mixed", FP32
+and with 16-bit hi/lo split-complex tensor-core contractions ("mixed", FP32
 accumulation); ``value`` is the mixed step's kernel elements/s (dim^2 per step) and
 the FP32 step is reported beside it.  The direct pair densities (203 GB over all q)
 and the W.rho products are streamed in q chunks.  Every input (u store 12.3 GB,
@@ -211,23 +211,23 @@ class Step:
         mark("spectrum")
 
     def tensor_pair(self, prec):
-        """The mixed step takes the direct pair densities on the tensor cores where the system has that route."""
+        """Direct pair densities on the tensor cores: in the mixed step where the system has that route, in the FP32 step
+        where the library takes it for the whole mesh (one route for every chunk, as Forward.build)."""
         from paper_1206_3518_gb300 import bse
-        return prec == bse.BSE_PREC_BF16X3 and bool(self.F.info["tensor_pair"])
+        if prec == bse.BSE_PREC_BF16X3:
+            return bool(self.F.info["tensor_pair"])
+        return bse.bse_pair_route(self.plan, 0, 0, self.F.nq)
 
     def kernels_per_step(self, prec):
-        """Kernel launches of one step: realspace, exchange densities, dipole, K^x (operand split and Gram kernel);
-        per chunk the direct densities (the correlation kernel, or on the tensor cores scales, image packing, tile
-        table, tile list and the tcgen05 kernel, plus the FP64 G = 0 overlaps on the chunk holding q = 0) and the
-        direct term (two operand splits, the tcgen05 GEMM and the block kernel); the Haydock kernel."""
-        tensor = self.tensor_pair(prec) or tensor_default(self.spec, self.F.info)
-        return 5 + ((5 if tensor else 1) + 4) * len(self.F.chunks) + (1 if tensor else 0) + 1
-
-
-def tensor_default(spec, inf):
-    """Whether a step without BSE_PD_TENSOR takes the direct densities on the tensor cores all the same: a tile (k, region)
-    for every SM twice over, at the q chunks of whole mesh planes that this file uses."""
-    return bool(inf["tensor_pair"]) and not inf["kpoint_symmetry"] and spec.nkpt >= 304
+        """Kernel launches of one step: realspace, the coefficient panels (with the real-space stage where the tensor
+        route is the default, else in every direct set that takes it), exchange densities, dipole, K^x (operand split
+        and Gram kernel); per chunk the direct densities (one kernel on either route, plus the FP64 G = 0 overlaps on
+        the chunk holding q = 0 on the tensor cores) and the direct term (two operand splits, the tcgen05 GEMM and
+        the block kernel); the Haydock kernel."""
+        from paper_1206_3518_gb300 import bse
+        packed, n = bse.bse_pair_route(self.plan, 0, 0, self.F.nq), len(self.F.chunks)
+        tensor = self.tensor_pair(prec)
+        return 5 + (1 if packed else n if tensor else 0) + 5 * n + (1 if tensor else 0) + 1
 
 
 def stage_times(marks_per_step):
@@ -361,8 +361,8 @@ def run_ours(args):
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": msmx, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "bf16x3", "data": "synthetic",
         "config": dict(workload_config(spec, inf["ng_max"], qchunk, len(F.chunks)),
-                       precision="headline: BF16 hi/lo split-complex tcgen05 contractions (direct pair "
-                                 "densities, K^x and W.rho), FP32 exchange densities and block products, FP64 "
+                       precision="headline: split-complex tcgen05 contractions (direct pair densities FP16 hi/lo, K^x "
+                                 "and W.rho BF16 hi/lo), FP32 exchange densities and block products, FP64 "
                                  "G = 0 overlaps, Lanczos coefficients and continued fraction; compared with "
                                  "the all-FP32 step",
                        parallelism=f"replicas x{world}"),
@@ -842,12 +842,13 @@ def run_stage(args):
                            F.ws_pair)
     q0, q1 = F.chunks[min(1, len(F.chunks) - 1)]
     prec = bse.BSE_PREC_BF16X3 if args.prec == "bf16x3" else bse.BSE_PREC_FP32
-    ws_init = F.ws_kernel if prec == bse.BSE_PREC_BF16X3 else None
     if args.only == "contract":
         bse.bse_pair_densities(plan, 0, bse.BSE_PD_DIRECT, None, None, None, None, F.rho_dir, q0, q1, F.ws_pair)
-        bse.bse_build_kernel(plan, 0, bse.BSE_BK_INIT, F.rho_x, None, 0, 0, None, en, spec.delta, prec, F.H, ws_init)
+        bse.bse_build_kernel(plan, 0, bse.BSE_BK_INIT, F.rho_x, None, 0, 0, None, en, spec.delta, prec, F.H,
+                             F.ws_kernel)
 
-    fdir = bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if prec == bse.BSE_PREC_BF16X3 and F.info["tensor_pair"] else 0)
+    tensor = bool(F.info["tensor_pair"]) if prec == bse.BSE_PREC_BF16X3 else bse.bse_pair_route(plan, 0, 0, F.nq)
+    fdir = bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if tensor else 0)
 
     def once():
         if args.only == "pair":
@@ -857,7 +858,7 @@ def run_stage(args):
                                  F.ws_kernel)
         elif args.only == "exchange":
             bse.bse_build_kernel(plan, 0, bse.BSE_BK_INIT, F.rho_x, None, 0, 0, None, en, spec.delta, prec, F.H,
-                                 ws_init)
+                                 F.ws_kernel)
         else:
             F.spectrum(om, spec.eta)
 
@@ -894,7 +895,7 @@ GCORR_TRAFFIC = {"sha1": "ebbbbf8406f12035e2778354e7d61fd0fc693ec8", "bytes_per_
 # the fcc 12x12x12 4v4c block shape on a 6x6x6 k mesh, q 72..144 (two whole planes of the q mesh, as the
 # bench's chunks are): 9,072 blocks, 357.2 MB read and 1415.1 MB written (the densities at their sphere
 # positions; the region panels of B mostly from L2).  Valid only for the sources with this SHA-1
-# (tcpair.cu + umma.cuh) and that block shape.
+# (tcpair.cu + tcf16.cuh + umma.cuh) and that block shape.
 TCPAIR_TRAFFIC = {"sha1": "44be08bd79adb79e5e4217dbf94880d38196fef7", "bytes_per_block": 195365.4,
                   "shape": ("fcc", 4, 4, 12.0)}
 
@@ -902,7 +903,7 @@ TCPAIR_TRAFFIC = {"sha1": "44be08bd79adb79e5e4217dbf94880d38196fef7", "bytes_per
 def _tcpair_sources_sha1():
     import hashlib
     base = os.path.join(ROOT, "paper_1206_3518_gb300", "csrc")
-    data = open(os.path.join(base, "tcpair.cu"), "rb").read() + open(os.path.join(base, "umma.cuh"), "rb").read()
+    data = b"".join(open(os.path.join(base, f), "rb").read() for f in ("tcpair.cu", "tcf16.cuh", "umma.cuh"))
     return hashlib.sha1(data).hexdigest()
 
 
@@ -928,7 +929,7 @@ def pair_work(plan, spec, inf):
         blk, _ = bse.bse_pair_blocks(plan, 0, q)
         cmac += ng * sum(npw[int(k2)] for _, k2 in blk)
     return {"method": "correlation", "variant": current, "cmac": cmac * (spec.nv ** 2 + spec.nc ** 2),
-            "tensor": bool(inf["tensor_pair"]), "tensor_default": tensor_default(spec, inf)}
+            "tensor": bool(inf["tensor_pair"]), "tensor_default": bse.bse_pair_route(plan, 0, 0, spec.nkpt)}
 
 
 def _fp32_peak(peaks):
@@ -950,11 +951,11 @@ def stage_rooflines(st, spec, inf, peaks, src, nchunks, pw, prec):
                 and TCPAIR_TRAFFIC["sha1"] == _tcpair_sources_sha1())
         out["pair_direct"] = {
             "bound": "tensor", "kernel": "tcpair_kernel", "achieved": useful / (ms / 1e3) / 1e12, "peak": peak,
-            "unit": "TFLOP/s", "frac": useful / (ms / 1e3) / 1e12 / peak, "launches_per_step": 5 * nchunks + 1,
+            "unit": "TFLOP/s", "frac": useful / (ms / 1e3) / 1e12 / peak, "launches_per_step": nchunks + 1,
             "work": "FP16x3 split-complex flops of the correlation itself: 3 hi/lo products x 8 real flops per "
                     "complex multiply-add, sum over upper blocks of NG(q) |S(k')| (Nv^2 + Nc^2) (the padding of "
                     "a tile's rows and K positions to the union of its spheres is not counted); the stage's "
-                    "whole time (image packing and tile table included)",
+                    "whole time",
             "traffic": TCPAIR_TRAFFIC["bytes_per_block"] * nb / nchunks if same else None,
             "peak_source": src + " (sustained bf16: timed inside a long step)"}
     elif pw["method"] == "correlation":
