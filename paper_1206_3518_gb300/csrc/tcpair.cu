@@ -46,9 +46,10 @@
 // the densities 9.5 and 39.4, with a twelfth of the MMAs 9.0 and 35.7, without the promotion 10.8 and 44.9: the gather's stores meet the
 // accumulators' traffic in tensor memory (the MMAs take 960 of ~1600 cycles per 32 K).  On sheets (K of 160) the
 // set-up of a tile is as long as its passes.  Measured (ms; before: the FP32 correlation kernel / BF16x3 tensor kernel with 96
-// columns, two lookups an element and one accumulator a pass): fcc 8x8x8 3v4c 9.9 (50.1 / 15.2), fcc 12x12x12 4v4c,
-// 144 q 45.3 (- / 59), 27x27 sheet 2v3c, 64 q 1.03 (1.52 / -; 1.33 before the tile list).  Error against 64 bits
-// (2-norm): 1.6e-7 to 2.0e-7 (correlation kernel 1.6e-7 to 4.0e-7).
+// columns, two lookups an element and one accumulator a pass): fcc 8x8x8 3v4c 9.7 (50.1 / 15.2), fcc 12x12x12 4v4c,
+// q 144 to 288 43.6 (363 / 59), 27x27 sheet 2v3c, 64 q 1.07 (1.52 / -).  Error against 64 bits (2-norm of random states'
+// densities, nine systems from 3 to 12 Ha): 1.7e-7 to 2.1e-7 (correlation kernel 1.6e-7 to 5.5e-7, growing with the
+// sphere; below it only at 5x5x5 4v4c, 3 Ha: 1.6e-7 against 1.8e-7).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -982,10 +983,12 @@ int tcpair_valid(const DevSys& d) {
 // a region of k'; it costs the same however few of the region's points have a block in the range, so the
 // route needs tiles for every SM and columns in use: at least 304 tiles, and at least 30 of the 2 x 64 columns of a
 // tile's two band sets on average (regions of the mesh k + q touches are counted at one k off the region grid).
-// Measured, this kernel against gcorr_kernel: 7x7x7 2v2c, 49 q (28 columns) 0.49 against 0.41 ms; 27x27 sheet 2v3c, 64 q
-// (32) 1.03 / 1.52; 5x5x5 4v4c (40) 1.87 / 3.91; 32x32 sheet 3v3c, 64 q 1.41 / 2.61; 8x8x8 3v4c (112) 9.9 / 50.1; 4x4x4
-// 3v3c (256 tiles) 0.131 / 0.117; 3x3x3 1v2c (27 tiles) 0.054 / 0.024.  With k-point symmetry only scattered
-// representative blocks are left and the tiles are nearly empty.
+// Measured, this kernel against gcorr_kernel (ms a call; the systems below the line pack in the call): 27x27 sheet 2v3c, 64 q
+// (32 columns) 1.07 / 1.52; 32x32 sheet 3v3c, 64 q 1.32 / 2.62; 5x5x5 4v4c (40) 3.98 / 12.9 at 12 Ha and 0.33 / 0.30 at 3 Ha
+// (62 points: a tile is mostly set-up); 8x8x8 3v4c (112) 9.7 / 50.1; below the line 4x4x4 3v3c (256 tiles) 0.146 /
+// 0.117, 3x3x3 1v2c (27 tiles) 0.060 / 0.035, 7x7x7 2v2c, 49 q (28) 0.26 / 0.25 at 4 Ha (0.89 / 1.93 at 8.6 Ha: the line is
+// drawn by columns alone).  With k-point symmetry only scattered representative blocks are left and the tiles are
+// nearly empty.
 int tcpair_preferred(const DevSys& d, int q_begin, int q_end) {
   if (!tcpair_valid(d) || d.nfill > 0) return 0;
   const int nqc = q_end - q_begin;
@@ -1044,7 +1047,12 @@ int launch_tcpair(const DevSys& d, const void* coef, const void* ws, void* rho_d
   g.table = (kList + kDealSums + diffs) * 4 <= (long long)g.stages * g.stage_bytes && d.nk1 <= 1024 && d.nk2 <= 1024 &&
             d.nk3 <= 1024;
   if (!g.table) diffs = d.nkpt;
-  const long long most = d.tc_nreg * diffs;
+  long long upto = 0;                            // tiles whose region reaches to k or beyond
+  for (int r = 0; r < d.tc_nreg; ++r) {
+    const int x = r / (d.tc_nr[1] * d.tc_nr[2]), y = (r / d.tc_nr[2]) % d.tc_nr[1], z = r % d.tc_nr[2];
+    upto += (((x + 1) * d.tc_rg[0] - 1) * d.nk2 + (y + 1) * d.tc_rg[1] - 1) * (long long)d.nk3 + (z + 1) * d.tc_rg[2];
+  }
+  const long long most = std::min(d.tc_nreg * diffs, upto);
   const int grid = (int)std::min<long long>(most, num_sms);
   const long long step = (long long)kList * grid;
   for (g.share = 0; g.share * step < most; ++g.share) {
