@@ -105,3 +105,46 @@ def test_pair_densities(bse, big, small):
             for a, b in ((0, 1), (1, 0)):                # large times small
                 assert max(np.abs(v[a, b] - rv[a, b]).max(), np.abs(w[a, b] - rc[a, b]).max()) <= tol, (iq, j)
         at += nb * (nv * nv + nc * nc)
+
+
+@pytest.mark.parametrize("big", [10, 18, 24])
+def test_large_component_meets_zeros(bse, big):
+    """Rows of rho and W whose largest component (G = 0, 2^big above the rest) meets zeros of the other operand, as the head of
+    W and the overlaps do where the wings vanish.  A component a of a row with largest m is kept to 2^-22 |a| + 2^-40 m."""
+    nv, nc = 2, 3
+    plan = bse.Plan([SystemSpec("cell", "fcc", 10.0, 0.0, (2, 2, 2), nv, nc, 2.5, (24,) * 3, "3d")])
+    inf = plan.info(0)
+    nq, ngm, dim, nvc = inf["nq"], inf["ng_max"], inf["dim"], nv * nc
+    rng = np.random.default_rng(31)
+    rho = _cplx(rng, bse.bse_rho_dir_count(plan, 0, 0, nq), ngm)
+    rho[:, 0] *= 2.0 ** big
+    rho = rho.astype(np.complex64)
+    W = _cplx(rng, nq, ngm, ngm)
+    W = W + W.conj().transpose(0, 2, 1)
+    W[:, 0, :] = 0.0
+    W[:, :, 0] = 0.0                                     # the head too: nothing of the large component is left
+    W = W.astype(np.complex64)
+    H = torch.zeros(dim, dim, dtype=torch.complex64, device="cuda")
+    ws = torch.empty(bse.bse_workspace_size(plan, 0, bse.BSE_WS_KERNEL, nq) // 8 + 1, dtype=torch.complex64, device="cuda")
+    bse.bse_build_kernel(plan, 0, bse.BSE_BK_DIRECT, None, torch.as_tensor(rho, device="cuda"), 0, nq,
+                         torch.as_tensor(W, device="cuda"), None, 0.0, bse.BSE_PREC_FP32, H, ws)
+    bse.bse_status_read(plan)
+    H, at = H.cpu().numpy(), 0
+    for iq in range(nq):
+        blk, _ = bse.bse_pair_blocks(plan, 0, iq)
+        ng, nb = len(bse.bse_gvectors(plan, 0, iq, True)), len(blk)
+        rv = rho[at: at + nb * nv * nv, :ng].astype(np.complex128).reshape(nb, nv * nv, ng)
+        rc = rho[at + nb * nv * nv: at + nb * (nv * nv + nc * nc), :ng].astype(np.complex128).reshape(nb, nc * nc, ng)
+        at += nb * (nv * nv + nc * nc)
+        w = W[iq, :ng, :ng].astype(np.complex128)
+        tol = 2.0 ** -21 + 24 * 2.0 ** -23 + (4 * ng + ng / 32) * 2.0 ** -24
+        for b, (k, k2) in enumerate(blk):
+            m = -inf["norm"] * (rv[b].conj() @ w @ rc[b].T)
+            kept = np.abs(rv[b]) * tol + 2.0 ** -39 * np.abs(rv[b]).max(axis=1, keepdims=True)     # W multiplies rho_vv'
+            kept[:, 0] = 0.0                             # meets zeros only
+            err = 2.0 * inf["norm"] * (kept @ np.abs(w) @ np.abs(rc[b]).T)
+            m, err = [x.reshape(nv, nv, nc, nc).transpose(0, 2, 1, 3).reshape(nvc, nvc) for x in (m, err)]
+            if k == k2:
+                m, err = 0.5 * (m + m.conj().T), 0.5 * (err + err.T)
+            got = H[k * nvc:(k + 1) * nvc, k2 * nvc:(k2 + 1) * nvc]
+            assert np.all(np.abs(got - m) <= err), (iq, b)
