@@ -49,6 +49,10 @@ struct DevSys {
   const char4* tc_klist;          // [tc_nreg][tc_kpad] G of each K position
   const int* tc_kcount;           // [tc_nreg]
   const short* tc_kpos;           // [nkpt][npw_max] K position of sphere point i of k in its region's layout
+  // Passes (128 rows each) of the tiles of a region: layers along axis tc_axis, tc_layers of them; entry [d][h - 1] for h
+  // whole layers from difference d of the region's corner and k on.  tc_maxpass: the largest.
+  const unsigned char* tc_passes; // [nkpt][tc_layers]
+  int tc_axis, tc_layers, tc_maxpass;
   const short* tc_pmap;           // [nq][(2 fwf0 + 1)(2 fwf1 + 1)(2 fwf2 + 1)] sphere position of g on q, -1 if absent
 };
 

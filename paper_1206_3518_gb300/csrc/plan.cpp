@@ -461,6 +461,7 @@ bse_status build_system(const bse_system& in, SysPlan& sp, bool device) {
   std::vector<char4> h_klist;
   std::vector<int> h_kcount;
   std::vector<short> h_kpos((size_t)nkpt * npw_max, 0), h_pmap;
+  std::vector<unsigned char> h_passes;
   {
     const int rmax = 64 / std::max(s.nv, s.nc);
     const bool thin = nk2 * nk3 >= rmax;
@@ -531,6 +532,44 @@ bse_status build_system(const bse_system& in, SysPlan& sp, bool device) {
         h_pmap[(size_t)iq * p0 * p1 * p2 + ((size_t)(g[3 * t] + d.fwf[0]) * p1 + g[3 * t + 1] + d.fwf[1]) * p2 +
                g[3 * t + 2] + d.fwf[2]] = (short)t;
     }
+    // rows of h whole layers of a region: the union of their spheres around the differences k' - k as they are (not
+    // folded into the mesh), from every difference on; left at zero where that would take long
+    d.tc_axis = best[0] > 1 || best[1] == 1 ? 0 : 1;
+    d.tc_layers = best[d.tc_axis];
+    d.tc_maxpass = 0;
+    h_passes.assign((size_t)nkpt * d.tc_layers, 0);
+    const int e0 = 2 * d.fwf[0] + 2, e1 = 2 * d.fwf[1] + 2, e2 = 2 * d.fwf[2] + 2;   // g - w, w in {0, 1}
+    if ((double)nkpt * d.tc_rsize * d.ng_max < 2e8) {
+      std::vector<int> seen((size_t)e0 * e1 * e2, -1);
+      for (int iq = 0; iq < nkpt; ++iq) {
+        int o[3], n = 0;
+        offs(iq, o);
+        for (int l = 0; l < d.tc_layers; ++l) {
+          int x[3], ext[3] = {best[0], best[1], best[2]}, from[3] = {0, 0, 0};
+          from[d.tc_axis] = l;
+          ext[d.tc_axis] = l + 1;
+          for (x[0] = from[0]; x[0] < ext[0]; ++x[0])
+            for (x[1] = from[1]; x[1] < ext[1]; ++x[1])
+              for (x[2] = from[2]; x[2] < ext[2]; ++x[2]) {
+                int f[3], w[3];
+                for (int j = 0; j < 3; ++j) {
+                  w[j] = (o[j] + x[j]) / s.nk[j];
+                  f[j] = (o[j] + x[j]) % s.nk[j];
+                }
+                const auto& g = sp.gq[(f[0] * nk2 + f[1]) * nk3 + f[2]];
+                for (size_t t = 0; t < g.size() / 3; ++t) {
+                  int& at = seen[((size_t)(g[3 * t] - w[0] + d.fwf[0] + 1) * e1 + g[3 * t + 1] - w[1] + d.fwf[1] + 1) * e2 +
+                                 g[3 * t + 2] - w[2] + d.fwf[2] + 1];
+                  n += at != iq;
+                  at = iq;
+                }
+              }
+          const int p = std::min(255, (n + 127) / 128);
+          h_passes[(size_t)iq * d.tc_layers + l] = (unsigned char)p;
+          d.tc_maxpass = std::max(d.tc_maxpass, p);
+        }
+      }
+    }
   }
 
   if (!device) return BSE_OK;
@@ -555,6 +594,7 @@ bse_status build_system(const bse_system& in, SysPlan& sp, bool device) {
   const size_t o_tkc = off; off = align256(off + h_kcount.size() * sizeof(int));
   const size_t o_tkp = off; off = align256(off + h_kpos.size() * sizeof(short));
   const size_t o_tpm = off; off = align256(off + h_pmap.size() * sizeof(short));
+  const size_t o_tps = off; off = align256(off + h_passes.size());
   char* base = nullptr;
   bse_status st = cuda_check(cudaMalloc((void**)&base, off), "cudaMalloc(plan tables)");
   if (st != BSE_OK) return st;
@@ -580,6 +620,7 @@ bse_status build_system(const bse_system& in, SysPlan& sp, bool device) {
   if (!err) err = up(o_tkc, h_kcount.data(), h_kcount.size() * sizeof(int));
   if (!err) err = up(o_tkp, h_kpos.data(), h_kpos.size() * sizeof(short));
   if (!err) err = up(o_tpm, h_pmap.data(), h_pmap.size() * sizeof(short));
+  if (!err) err = up(o_tps, h_passes.data(), h_passes.size());
   if ((st = cuda_check(err, "cudaMemcpy(plan tables)")) != BSE_OK) return st;
   d.gk = (const char4*)(base + o_gk);
   d.npw = (const int*)(base + o_npw);
@@ -600,6 +641,7 @@ bse_status build_system(const bse_system& in, SysPlan& sp, bool device) {
   d.tc_kcount = (const int*)(base + o_tkc);
   d.tc_kpos = (const short*)(base + o_tkp);
   d.tc_pmap = (const short*)(base + o_tpm);
+  d.tc_passes = (const unsigned char*)(base + o_tps);
   return BSE_OK;
 }
 

@@ -232,8 +232,8 @@ __global__ __launch_bounds__(256) void tcpair_pack_kernel(DevSys d, const float2
 // the first holds depends on the difference of the region's corner and k alone.  The CTAs list the differences that do
 // and deal the tiles (region, difference) among themselves, the i-th one to CTA i mod grid, from the plan's tables
 // alone: a call keeps nothing in the workspace, so calls that share it may overlap.  Regions in order: the CTAs in
-// flight share one region's packed B rows, which stay in L2.  The rows of a tile, and with them its passes, grow with
-// the number of its blocks, so the fullest tiles (in quarters of the region) are dealt first.
+// flight share one region's packed B rows, which stay in L2.  The tiles of the most passes are dealt first, so that every
+// CTA gets as many of each kind (dealt by the fullness of the region a sheet's chunk took up to 10% longer).
 struct Point {                                   // offsets on the mesh
   int x, y, z;
 };
@@ -258,15 +258,15 @@ __device__ __forceinline__ int block_of(const DevSys& d, const TpGeo& g, int k, 
   const int q = index_of(d, plus(d, diff, o));
   return q >= g.q_begin && q < g.q_begin + g.nqc ? d.blkidx[(size_t)q * d.nkpt + k] : -1;
 }
-// Points of a region at difference p whose own difference lies in the q range: runs along the last axis that has more
-// than one point, each one or two intervals of q.
-__device__ __forceinline__ int near_points(const DevSys& d, const TpGeo& g, Point p) {
-  if (g.nqc == d.nkpt) return d.tc_rsize;
+// Points of a box of (e0, e1, e2) at difference p whose own difference lies in the q range: runs along the last axis that
+// has more than one point, each one or two intervals of q.
+__device__ __forceinline__ int near_points(const DevSys& d, const TpGeo& g, Point p, int e0, int e1, int e2) {
+  if (g.nqc == d.nkpt) return e0 * e1 * e2;
   const bool z = d.nk3 > 1;
-  const int len = z ? d.tc_rg[2] : d.tc_rg[1], nl = z ? d.nk3 : d.nk2, at = z ? p.z : p.y, rows = z ? d.tc_rg[1] : 1;
+  const int len = z ? e2 : e1, nl = z ? d.nk3 : d.nk2, at = z ? p.z : p.y, rows = z ? e1 : 1;
   const int qe = g.q_begin + g.nqc;
   int m = 0;
-  for (int a = 0; a < d.tc_rg[0]; ++a)
+  for (int a = 0; a < e0; ++a)
     for (int b = 0; b < rows; ++b) {
       const int x = wrap(p.x + a, d.nk1), base = z ? (x * d.nk2 + wrap(p.y + b, d.nk2)) * d.nk3 : x * d.nk2;
       m += max(0, min(qe, base + min(at + len, nl)) - max(g.q_begin, base + at));
@@ -275,11 +275,50 @@ __device__ __forceinline__ int near_points(const DevSys& d, const TpGeo& g, Poin
   return m;
 }
 
+// Class of the tiles of difference p, the most passes first; -1: no point in the range.  The passes of a tile follow from
+// the rows of its blocks, those of the layers of the region that are at least half in the range (whole layers are in the
+// plan's table; a range cuts a layer at its ends only).
+constexpr int kMine = 2, kFill = 4;              // list entries per thread; classes
+__device__ __forceinline__ int class_of(const DevSys& d, const TpGeo& g, Point p) {
+  const bool ax = d.tc_axis == 0;
+  const int e0 = ax ? 1 : d.tc_rg[0], e1 = ax ? d.tc_rg[1] : 1, e2 = d.tc_rg[2], half = (e0 * e1 * e2 + 1) / 2;
+  int first = -1, last = -1, any = -1;
+  if (g.nqc == d.nkpt) {
+    first = 0;
+    last = any = d.tc_layers - 1;
+  } else if (!ax && d.nk3 == 1) {                // layers of one point: a run along axis 1 and its part beyond the mesh's end
+    const int base = p.x * d.nk2, end = p.y + d.tc_layers - d.nk2, qe = g.q_begin + g.nqc;
+    const int lo = max(g.q_begin - base, p.y), hi = min(qe - base, min(p.y + d.tc_layers, d.nk2));
+    const int lo2 = max(g.q_begin - base, 0), hi2 = min(qe - base, end);
+    if (hi > lo) {
+      first = lo - p.y;
+      last = hi - 1 - p.y;
+    }
+    if (hi2 > lo2) {
+      first = first < 0 ? lo2 + d.nk2 - p.y : first;
+      last = hi2 - 1 + d.nk2 - p.y;
+    }
+    any = last;
+  } else {
+    for (int l = 0; l < d.tc_layers; ++l) {
+      const int m = near_points(d, g, plus(d, p, ax ? Point{l, 0, 0} : Point{0, l, 0}), e0, e1, e2);
+      if (m >= half) {
+        first = first < 0 ? l : first;
+        last = l;
+      }
+      if (m > 0) any = l;
+    }
+  }
+  if (any < 0) return -1;
+  if (first < 0) first = last = any;
+  const int at = index_of(d, plus(d, p, ax ? Point{first, 0, 0} : Point{0, first, 0}));
+  return min(kFill - 1, d.tc_maxpass - (int)d.tc_passes[(size_t)at * d.tc_layers + last - first]);
+}
+
 // Tiles of this CTA (its share of the launch) as region nkpt + k in the first kList words of scratch; returns their
 // number.  (Not inlined: its registers are not those of the passes.)  After the list: sums of the warps, differences (without
 // room for them every difference of the mesh is tried).  Where k lies within the region only some of its points come after
 // k: such tiles are dealt last, and next_tile passes over one without a block.
-constexpr int kMine = 2, kFill = 4;              // list entries per thread; classes of fullness
 constexpr int kList = kMine * kThreads, kDealSums = kFill * (kThreads / 32);
 __device__ __noinline__ int deal_tiles(const DevSys& d, const TpGeo& g, int* scratch) {
   constexpr int kWarps = kThreads / 32;
@@ -318,24 +357,23 @@ __device__ __noinline__ int deal_tiles(const DevSys& d, const TpGeo& g, int* scr
 
   // the differences with a point in the range, by class
   const int per_d = (d.nkpt + kThreads - 1) / kThreads, d0 = min(tid * per_d, d.nkpt), d1 = min(d0 + per_d, d.nkpt);
-  auto class_of = [&](int m) { return (d.tc_rsize - m) * kFill / d.tc_rsize; };
   int n[kFill], start[kFill + 1];
 #pragma unroll
   for (int f = 0; f < kFill; ++f) n[f] = 0;
   for (int i = d0; i < d1; ++i) {
-    const int m = near_points(d, g, point_of(d, i));
+    const int cls = class_of(d, g, point_of(d, i));
 #pragma unroll
-    for (int f = 0; f < kFill; ++f) n[f] += m > 0 && class_of(m) == f ? 1 : 0;
+    for (int f = 0; f < kFill; ++f) n[f] += cls == f ? 1 : 0;
   }
   prefix(n, start);
   const bool table = g.table != 0;
   if (table) {
     for (int i = d0; i < d1; ++i) {
       const Point p = point_of(d, i);
-      const int m = near_points(d, g, p);
+      const int cls = class_of(d, g, p);
 #pragma unroll
       for (int f = 0; f < kFill; ++f)
-        if (m > 0 && class_of(m) == f) diffs[n[f]++] = (unsigned)(p.x | p.y << 10 | p.z << 20);
+        if (cls == f) diffs[n[f]++] = (unsigned)(p.x | p.y << 10 | p.z << 20);
     }
     __syncthreads();
   } else {                                       // one class of all differences
