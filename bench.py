@@ -893,10 +893,10 @@ GCORR_TRAFFIC = {"sha1": "ebbbbf8406f12035e2778354e7d61fd0fc693ec8", "bytes_per_
 
 # The same for the tensor-core route's kernel (tcpair_kernel): one ncu capture (--set full, one launch) of
 # the fcc 12x12x12 4v4c block shape on a 6x6x6 k mesh, q 72..144 (two whole planes of the q mesh, as the
-# bench's chunks are): 9,072 blocks, 762.8 MB read and 1826.0 MB written (the densities at their sphere
+# bench's chunks are): 9,072 blocks, 763.3 MB read and 1825.8 MB written (the densities at their sphere
 # positions; the region panels of B mostly from L2).  Valid only for the sources with this SHA-1
 # (tcpair.cu + tcf16.cuh + umma.cuh) and that block shape.
-TCPAIR_TRAFFIC = {"sha1": "8f52ab8c4dc2db169372478d9b748e82b9f2d950", "bytes_per_block": 285358.7,
+TCPAIR_TRAFFIC = {"sha1": "a2cfad6267175cce80975e86d8230231aa1097f6", "bytes_per_block": 285394.5,
                   "shape": ("fcc", 4, 4, 12.0)}
 
 

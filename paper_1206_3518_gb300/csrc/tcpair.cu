@@ -47,7 +47,7 @@
 // accumulators' traffic in tensor memory (the MMAs take 960 of ~1600 cycles per 32 K).  On sheets (K of 160) the
 // set-up of a tile is as long as its passes.  Measured (ms; before: the FP32 correlation kernel / BF16x3 tensor kernel with 96
 // columns, two lookups an element and one accumulator a pass): fcc 8x8x8 3v4c 9.7 (50.1 / 15.2), fcc 12x12x12 4v4c,
-// q 144 to 288 43.6 (363 / 59), 27x27 sheet 2v3c, 64 q 1.07 (1.52 / -).  Error against 64 bits (2-norm of random states'
+// q 144 to 288 43.2 (363 / 59), 27x27 sheet 2v3c, 64 q 0.96 (1.52 / -).  Error against 64 bits (2-norm of random states'
 // densities, nine systems from 3 to 12 Ha): 1.7e-7 to 2.1e-7 (correlation kernel 1.6e-7 to 5.5e-7, growing with the
 // sphere; below it only at 5x5x5 4v4c, 3 Ha: 1.6e-7 against 1.8e-7).
 #include <cuda_fp16.h>
@@ -975,7 +975,7 @@ __global__ void tcpair_diag_kernel(DevSys d, const float2* __restrict__ coef, fl
 
 // Panels per stage, ring depth and position-table rows.  Two panels (64 complex K per promotion and per hand-over of a
 // stage) where two such stages and the table of the two groups' passes (256 rows) fit; one panel otherwise.  Two against
-// one, ms: 27x27 sheet 1.03 / 1.13, 32x32 sheet 1.41 / 1.51, 5x5x5 4v4c 1.87 / 2.00, 12x12x12 144 q 45.3 / 47.9, 8x8x8 3v4c
+// one, ms (with the tiles from a counter): 27x27 sheet 1.03 / 1.13, 32x32 sheet 1.41 / 1.51, 5x5x5 4v4c 1.87 / 2.00, 12x12x12 144 q 45.3 / 47.9, 8x8x8 3v4c
 // 9.9 / 10.6.  The table holds one and a half spheres of rows (512 to 1024) if it can: the rows are the union of
 // spheres whose centres lie within a region of each other, and a larger union is looked up pass by pass.  The depth is
 // even, so that a stage's slot always belongs to the same issue warp (which then sees every phase of the slot's
@@ -1022,7 +1022,7 @@ int tcpair_valid(const DevSys& d) {
 // route needs tiles for every SM and columns in use: at least 304 tiles, and at least 30 of the 2 x 64 columns of a
 // tile's two band sets on average (regions of the mesh k + q touches are counted at one k off the region grid).
 // Measured, this kernel against gcorr_kernel (ms a call; the systems below the line pack in the call): 27x27 sheet 2v3c, 64 q
-// (32 columns) 1.07 / 1.52; 32x32 sheet 3v3c, 64 q 1.32 / 2.62; 5x5x5 4v4c (40) 3.98 / 12.9 at 12 Ha and 0.33 / 0.30 at 3 Ha
+// (32 columns) 0.96 / 1.52; 32x32 sheet 3v3c, 64 q 1.31 / 2.62; 5x5x5 4v4c (40) 3.98 / 12.9 at 12 Ha and 0.33 / 0.30 at 3 Ha
 // (62 points: a tile is mostly set-up); 8x8x8 3v4c (112) 9.7 / 50.1; below the line 4x4x4 3v3c (256 tiles) 0.146 /
 // 0.117, 3x3x3 1v2c (27 tiles) 0.060 / 0.035, 7x7x7 2v2c, 49 q (28) 0.26 / 0.25 at 4 Ha (0.89 / 1.93 at 8.6 Ha: the line is
 // drawn by columns alone).  With k-point symmetry only scattered representative blocks are left and the tiles are
