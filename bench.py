@@ -196,7 +196,7 @@ class Step:
         bse.bse_build_kernel(plan, 0, bse.BSE_BK_INIT, F.rho_x, None, 0, 0, None, self.en, spec.delta, prec, F.H,
                              F.ws_kernel)
         mark("exchange_kernel")
-        fdir = bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if self.tensor_pair(prec) else 0)
+        fdir = bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if self.tensor_pair(prec) else bse.BSE_PD_VARIANT)
         for c, (q0, q1) in enumerate(F.chunks):
             bse.bse_pair_densities(plan, 0, fdir, None, None, None, None, F.rho_dir, q0, q1, F.ws_pair)
             mark("pair_direct")

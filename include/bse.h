@@ -87,6 +87,7 @@ typedef enum {
 #define BSE_PD_CHI0      8u   /* rho_vc^{k,k+q} for all k, q of a range (screening input) */
 #define BSE_PD_COUPLING 16u   /* rho_vc', rho_cv' of the upper blocks of a q range (coupling) */
 #define BSE_PD_TENSOR   32u   /* with DIRECT: the direct set on the tensor cores (FP16x3)      */
+#define BSE_PD_VARIANT  64u   /* with DIRECT: the direct set by the variant in use, not on the tensor cores */
 #define BSE_BK_INIT      1u   /* A3 + A5 diagonal: H = diag + 2 K^x (upper)    */
 #define BSE_BK_DIRECT    2u   /* A4 + A5: H -= K^d for a q range, mirror       */
 #define BSE_BK_MIRROR    4u   /* A5 without A4: lower blocks and (B+B^H)/2      */
@@ -198,7 +199,8 @@ bse_status bse_rho_dir_count(const bse_plan* plan, int s, int q_begin, int q_end
  * grid (first form; the default otherwise).  Without a chosen variant a direct set with enough blocks per
  * region of k' goes to the tensor-core form of the correlation (BSE_PD_TENSOR below), to FP32 rounding as well
  * (bse_pair_route).  That depends on the q range: for densities that do not depend on how the mesh is cut into
- * ranges, pass BSE_PD_TENSOR in every call or in none of them as bse_pair_route says of the whole mesh.
+ * ranges, pass BSE_PD_TENSOR in every call, or BSE_PD_VARIANT in every call (bse_pair_route of the whole mesh says which
+ * is the default).
  * coef     complex64 [nkpt][nb][npw_max], c_nk(G) in sphere order (zero padded).
  * energies float64  [nkpt][nb], bands ascending (valence first), Ha.
  * rho_x    complex64 [dim][ng_max]: rho_vc^{kk}(G) on the q = 0 sphere (S = (k,v,c)).
@@ -223,8 +225,8 @@ bse_status bse_rho_dir_count(const bse_plan* plan, int s, int q_begin, int q_end
  *          registers every 32 or 64 complex K (FP32 rounding); the G = 0 overlaps of the diagonal blocks
  *          are summed in FP64.  Same layout and vectors as without the flag.  No counterpart in the
  *          paper, which computes the densities by FFT.
- * Errors: BSE_ERR_ARG (range, NULL for a requested output), BSE_ERR_WORKSPACE, BSE_ERR_UNSUPPORTED
- *         (BSE_PD_TENSOR where bse_info.tensor_pair = 0), BSE_ERR_TIMEOUT (a tensor-route wait that
+ * Errors: BSE_ERR_ARG (range, NULL for a requested output, BSE_PD_TENSOR with BSE_PD_VARIANT), BSE_ERR_WORKSPACE,
+ *         BSE_ERR_UNSUPPORTED (BSE_PD_TENSOR where bse_info.tensor_pair = 0), BSE_ERR_TIMEOUT (a tensor-route wait that
  *         did not end within 2 s, through the status word).
  */
 bse_status bse_pair_densities(bse_plan* plan, int s, unsigned flags,

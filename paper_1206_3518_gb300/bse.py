@@ -24,6 +24,7 @@ BSE_WS_PAIR, BSE_WS_KERNEL, BSE_WS_SPECTRUM, BSE_WS_BACKWARD, BSE_WS_SCREEN = 0,
 BSE_WS_COUPLING, BSE_WS_COUPLED, BSE_WS_RITZ = 5, 6, 7
 BSE_WS_CHI0, BSE_WS_ALDA, BSE_WS_EPSM, BSE_WS_STATES = 8, 9, 10, 11
 BSE_PD_REALSPACE, BSE_PD_EXCHANGE, BSE_PD_DIRECT, BSE_PD_CHI0, BSE_PD_COUPLING, BSE_PD_TENSOR = 1, 2, 4, 8, 16, 32
+BSE_PD_VARIANT = 64
 BSE_BK_INIT, BSE_BK_DIRECT, BSE_BK_MIRROR, BSE_BK_SYMFILL = 1, 2, 4, 8
 BSE_BC_INIT, BSE_BC_DIRECT, BSE_BC_MIRROR = 1, 2, 4
 

@@ -97,6 +97,8 @@ int launch_realspace(const DevSys& d, const void* coef, void* u, void* stream);
 int launch_pair_exchange(const DevSys& d, const void* u, void* rho_x, int* status, void* stream);
 int launch_pair_direct(const DevSys& d, void* u, void* rho_dir, int q_begin, int q_end, long long vbase,
                        int* status, void* stream);
+int launch_pair_direct_variant(const DevSys& d, const void* u, void* rho_dir, int q_begin, int q_end, long long vbase,
+                               int* status, void* stream);
 int launch_dipole(const DevSys& d, const void* coef, const double* energies, double gap_floor, void* P, void* stream);
 int launch_pair_chi0(const DevSys& d, const void* u, void* rho, int q_begin, int q_end, int* status, void* stream);
 size_t screen_ws_bytes(const DevSys& d, long long qchunk);

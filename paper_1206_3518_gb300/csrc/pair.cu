@@ -580,8 +580,13 @@ int pair_direct_route(const DevSys& d, int q_begin, int q_end) {
 
 int launch_pair_direct(const DevSys& d, void* u, void* rho_dir, int q_begin, int q_end, long long vbase,
                        int* status, void* stream) {
-  if (pair_direct_route(d, q_begin, q_end))
-    return launch_pair_direct_tensor(d, u, rho_dir, q_begin, q_end, vbase, status, stream);
+  return pair_direct_route(d, q_begin, q_end)
+             ? launch_pair_direct_tensor(d, u, rho_dir, q_begin, q_end, vbase, status, stream)
+             : launch_pair_direct_variant(d, u, rho_dir, q_begin, q_end, vbase, status, stream);
+}
+
+int launch_pair_direct_variant(const DevSys& d, const void* u, void* rho_dir, int q_begin, int q_end, long long vbase,
+                               int* status, void* stream) {
   if (use_gcorr(d))
     return gcorr_split(d)
                ? launch_gcorr(d, coef_copy(d, u), rho_dir, 3, 1, q_begin, q_end - q_begin, vbase,

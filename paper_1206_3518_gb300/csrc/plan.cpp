@@ -873,7 +873,13 @@ bse_status bse_pair_densities(bse_plan* plan, int s, unsigned flags, const void*
   if (flags & BSE_PD_DIRECT) {
     if (!rho_dir || q_begin < 0 || q_end > d.nq || q_begin >= q_end) return set_error(BSE_ERR_ARG, "bad direct range");
     const long long vb = sp.qvec_off[q_begin];
-    if (flags & BSE_PD_TENSOR) {
+    if ((flags & BSE_PD_TENSOR) && (flags & BSE_PD_VARIANT))
+      return set_error(BSE_ERR_ARG, "BSE_PD_TENSOR and BSE_PD_VARIANT name two routes");
+    if (flags & BSE_PD_VARIANT) {
+      if ((st = cuda_check(launch_pair_direct_variant(d, ws, rho_dir, q_begin, q_end, vb, plan->d_status, stream),
+                           "pair direct (variant)")) != BSE_OK)
+        return st;
+    } else if (flags & BSE_PD_TENSOR) {
       if (!tcpair_valid(d)) return set_error(BSE_ERR_UNSUPPORTED, "no tensor-core route for this system");
       if ((st = cuda_check(launch_pair_direct_tensor(d, ws, rho_dir, q_begin, q_end, vb, plan->d_status, stream),
                            "pair direct (tensor)")) != BSE_OK)
@@ -956,7 +962,6 @@ bse_status bse_autotune_pair(bse_plan* plan, int s, void* ws, size_t ws_bytes, v
     return st;
   }
   const int saved = d.pair_variant, saved_tensor = d.pair_tensor;
-  d.pair_tensor = 0;                             // the variants' own kernels are timed
   const long long vb = sp.qvec_off[q_begin];
   float best = 0.f;
   int besti = -1;
@@ -974,7 +979,7 @@ bse_status bse_autotune_pair(bse_plan* plan, int s, void* ws, size_t ws_bytes, v
   for (int i = 0; i < n && i < 64 && st == BSE_OK; ++i) {
     d.pair_variant = buf[7 * i];
     float t = 0.f;
-    st = timed([&] { return launch_pair_direct(d, ws, rho_dir, q_begin, q_end, vb, plan->d_status, stream); }, t);
+    st = timed([&] { return launch_pair_direct_variant(d, ws, rho_dir, q_begin, q_end, vb, plan->d_status, stream); }, t);
     if (i < cap) ms[i] = t;
     if (st == BSE_OK && (besti < 0 || t < best)) {
       best = t;

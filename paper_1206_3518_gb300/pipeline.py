@@ -49,9 +49,10 @@ class Forward:
     def build(self, coef, energies, W, delta, prec=bse.BSE_PREC_FP32, tensor_pair=None):
         """A1-A6: pair densities, dipole and H (direct term streamed over q chunks).
 
-        tensor_pair: direct pair densities on the tensor cores (BSE_PD_TENSOR); by default with the
-        mixed precision where the system has that route, in FP32 where the library takes it for the whole
-        mesh, and in both as the autotuner chose for this system.  One choice for every chunk: H does not depend on qchunk.
+        tensor_pair: direct pair densities on the tensor cores (BSE_PD_TENSOR) or by the pair-kernel variant in use
+        (False, BSE_PD_VARIANT).  By default on the tensor cores in the mixed precision where the system has that
+        route and in FP32 where the library takes it for the whole mesh; in both as the autotuner chose for this
+        system.  One choice for every chunk: H does not depend on qchunk.
         """
         p, s = self.plan, self.s
         if tensor_pair is None:
@@ -60,7 +61,7 @@ class Forward:
                 tensor_pair = bse.bse_pair_route(p, s, 0, self.nq)
             if self.tensor_choice is not None and bool(self.info["tensor_pair"]):
                 tensor_pair = self.tensor_choice
-        fdir = bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if tensor_pair else 0)
+        fdir = bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if tensor_pair else bse.BSE_PD_VARIANT)
         bse.bse_pair_densities(p, s, bse.BSE_PD_REALSPACE | bse.BSE_PD_EXCHANGE, coef, energies, self.rho_x, self.P,
                                None, 0, 0, self.ws_pair)
         bse.bse_build_kernel(p, s, bse.BSE_BK_INIT, self.rho_x, None, 0, 0, None, energies, delta, prec, self.H,

@@ -61,7 +61,8 @@ def direct_flags(plan, s: int = 0) -> int:
     """bse_pair_densities flags of a rank's direct densities: those of the single-GPU FP32 build, whatever the rank's
     q ranges."""
     from . import bse
-    return bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if bse.bse_pair_route(plan, s, 0, plan.info(s)["nq"]) else 0)
+    tensor = bse.bse_pair_route(plan, s, 0, plan.info(s)["nq"])
+    return bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if tensor else bse.BSE_PD_VARIANT)
 
 
 def row_ranges(nkpt: int, nvc: int, world: int) -> List[Tuple[int, int]]:

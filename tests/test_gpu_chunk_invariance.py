@@ -46,3 +46,28 @@ def test_chunked_builds_equal_the_single_pass(bse, lat, n, nv, nc, ecut, grid, c
         ng = len(bse.bse_gvectors(plan, 0, q, 1))
         assert torch.equal(out[:, :ng], F.rho_dir[a:a + n1, :ng]), q
     bse.bse_status_read(plan)
+
+
+def test_no_tensor_cores_asked_for(bse):
+    """tensor_pair=False takes the variant in use in every chunk, also where the tensor cores are the default."""
+    from paper_1206_3518_gb300.pipeline import Forward
+    spec = SystemSpec("cell", "fcc", 10.0, 0.0, (5, 5, 5), 4, 4, 3.0, (48,) * 3, "3d")
+    s = generate(spec, wdtype=np.complex64)
+    plan = bse.Plan([spec])
+    assert bse.bse_pair_route(plan, 0, 0, 125)
+    args = (torch.as_tensor(s.coef, dtype=torch.complex64, device="cuda"),
+            torch.as_tensor(s.energies, dtype=torch.float64, device="cuda"),
+            torch.as_tensor(s.W, dtype=torch.complex64, device="cuda"), spec.delta)
+    for prec in (bse.BSE_PREC_FP32, bse.BSE_PREC_BF16X3):
+        F = Forward(plan, 0, nsteps=8, nw=8)
+        H = F.build(*args, prec, tensor_pair=False).clone()
+        rho = F.rho_dir.clone()
+        bse.bse_set_pair_variant(plan, 0, 64)
+        bse.bse_pair_densities(plan, 0, bse.BSE_PD_DIRECT, None, None, None, None, F.rho_dir, 0, 125, F.ws_pair)
+        assert torch.equal(F.rho_dir, rho)
+        bse.bse_set_pair_variant(plan, 0, -1)
+        assert torch.equal(Forward(plan, 0, nsteps=8, nw=8, qchunk=30).build(*args, prec, tensor_pair=False), H)
+    with pytest.raises(bse.BseError):
+        bse.bse_pair_densities(plan, 0, bse.BSE_PD_DIRECT | bse.BSE_PD_TENSOR | bse.BSE_PD_VARIANT, None, None, None, None,
+                               F.rho_dir, 0, 125, F.ws_pair)
+    bse.bse_status_read(plan)

@@ -24,7 +24,7 @@ def test_a_part_on_the_tensor_cores_means_the_whole(lat, n, nv, nc, ecut, grid):
         for a in range(0, nq - step + 1, max(1, step // 2)):
             assert whole or not bse.bse_pair_route(plan, 0, a, a + step)
     flags = shard.direct_flags(plan)
-    assert flags == (bse.BSE_PD_DIRECT | bse.BSE_PD_TENSOR if whole else bse.BSE_PD_DIRECT)
+    assert flags == (bse.BSE_PD_DIRECT | (bse.BSE_PD_TENSOR if whole else bse.BSE_PD_VARIANT))
     bse.bse_set_pair_variant(plan, 0, 64)
     assert not bse.bse_pair_route(plan, 0, 0, nq)
     bse.bse_set_pair_variant(plan, 0, -1)
